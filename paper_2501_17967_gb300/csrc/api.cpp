@@ -7,6 +7,8 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <new>
+#include <thread>
 
 #include "bc_internal.h"
 
@@ -500,28 +502,32 @@ PassArgs pass_args(const bc_ctx *ctx, const bc_tree *t)
 
 namespace {
 
-// Digits of one FP64 matrix row for the split near field: row scaled by 2^-E
-// into (-1/2, 1/2), rounded to a 40-bit integer, five balanced base-256 digits.
-int split_row(const double *row, int n, int16_t *digits /*[5][n]*/)
+// Digits of one FP64 matrix row: row scaled by 2^-E into (-1/2, 1/2), rounded
+// to an 8 S-bit integer, S balanced base-256 digits.  Returns E and, in *sum,
+// the sum of |digit| over the row (the accumulation bound of Fmt).
+int split_row(const double *row, int n, int S, int16_t *digits /*[S][n]*/, long long *sum)
 {
     double mx = 0.0;
     for (int k = 0; k < n; k++) mx = std::max(mx, std::fabs(row[k]));
+    *sum = 0;
     if (mx == 0.0) {
-        std::fill(digits, digits + size_t(kSplitSlices) * n, int16_t(0));
+        std::fill(digits, digits + size_t(S) * n, int16_t(0));
         return 0;
     }
     int e = 0;
     std::frexp(mx, &e);            // mx < 2^e
     const int E = e + 1;           // mx < 2^(E-1)
     for (int k = 0; k < n; k++) {
-        long long X = std::llround(std::ldexp(row[k], 40 - E));   // |X| < 2^39
-        for (int a = kSplitSlices; a >= 2; a--) {
+        long long X = std::llround(std::ldexp(row[k], 8 * S - E));   // |X| < 2^(8 S - 1)
+        for (int a = S; a >= 2; a--) {
             int d = int(X & 255);
             if (d >= 128) d -= 256;
             X = (X - d) >> 8;
             digits[(a - 1) * n + k] = int16_t(d);
+            *sum += std::abs(d);
         }
         digits[k] = int16_t(X);   // leading digit, |X| <= 128
+        *sum += std::llabs(X);
     }
     return E;
 }
@@ -534,56 +540,136 @@ uint16_t bf16_of_int(int d)
     return uint16_t(u >> 16);
 }
 
-// Appends the BF16 digits of a real operator (rows x K, row-major) to `dig`
-// in the chunk layout [digit a][row half h][K chunk kc] x (128 rows x KC) of
-// canonical K-major core matrices, and its row exponents to `ex`.
-SplitOp add_split_op(std::vector<uint16_t> &dig, std::vector<int32_t> &ex, const std::vector<double> &m, int rows,
-                     int K)
+// Operators of one group in one digit format, as they are uploaded: BF16
+// digits, row exponents and (7 digits) the FP64 entries.
+struct OpGroup {
+    int S = kSplitSlices, K = 0, kvalid = 0;   // digits, padded and valid inner dimension
+    std::vector<uint16_t> dig;
+    std::vector<int32_t> ex;
+    std::vector<double> f;
+    bool exact = true;   // every row keeps the accumulation bound of the format
+};
+
+// Appends the BF16 digits of a real operator (rows x K, row-major) in the
+// chunk layout [digit a][row half h][K chunk kc] x (128 rows x KC) of
+// canonical K-major core matrices, its row exponents and (7 digits) its
+// entries [k][row].
+SplitOp add_split_op(OpGroup &G, const std::vector<double> &m, int rows)
 {
-    const int KC = std::min(K, kSplitKC), nkc = K / KC, mh = rows > 128 ? 2 : 1;
+    const int K = G.K, S = G.S, KC = K > 144 ? kSplitKC : K, nkc = K / KC, mh = rows > 128 ? 2 : 1;
     const size_t chunk = size_t(128) * KC;   // elements per chunk
     SplitOp op;
-    op.a_off = int64_t(dig.size()) * int64_t(sizeof(uint16_t));
+    op.a_off = int64_t(G.dig.size()) * int64_t(sizeof(uint16_t));
     op.rows = rows;
-    op.exp_off = int32_t(ex.size());
-    const size_t base = dig.size();
-    dig.resize(base + size_t(kSplitSlices) * mh * nkc * chunk, 0);
-    ex.resize(ex.size() + size_t(mh) * 128, 0);
-    std::vector<int16_t> dg(size_t(kSplitSlices) * K);
-    for (int i = 0; i < rows; i++) {
-        ex[size_t(op.exp_off) + i] = split_row(&m[size_t(i) * K], K, dg.data());
-        const int h = i / 128, rg = (i % 128) / 8, r = i % 8;
-        for (int a = 0; a < kSplitSlices; a++)
-            for (int k = 0; k < K; k++) {
-                const int kc = k / KC, kg = (k % KC) / 8, e = k % 8;
-                const size_t off = base + ((size_t(a) * mh + h) * nkc + kc) * chunk +
-                                   (size_t(rg) * (KC / 8) + kg) * 64 + size_t(r) * 8 + e;
-                dig[off] = bf16_of_int(dg[size_t(a) * K + k]);
-            }
+    op.exp_off = int32_t(G.ex.size());
+    op.f_off = int64_t(G.f.size());
+    const size_t base = G.dig.size();
+    G.dig.resize(base + size_t(S) * mh * nkc * chunk, 0);
+    G.ex.resize(G.ex.size() + size_t(mh) * 128, 0);
+    if (S == kWideSlices) {
+        G.f.resize(G.f.size() + size_t(G.kvalid) * rows);
+        for (int k = 0; k < G.kvalid; k++)
+            for (int i = 0; i < rows; i++) G.f[size_t(op.f_off) + size_t(k) * rows + i] = m[size_t(i) * K + k];
     }
+    auto part = [&, base](int i0, int i1, bool *ok) {
+        std::vector<int16_t> dg(size_t(S) * K);
+        for (int i = i0; i < i1; i++) {
+            long long sum = 0;
+            G.ex[size_t(op.exp_off) + i] = split_row(&m[size_t(i) * K], K, S, dg.data(), &sum);
+            if (sum > (1ll << 17)) *ok = false;
+            const int h = i / 128, rg = (i % 128) / 8, r = i % 8;
+            for (int a = 0; a < S; a++)
+                for (int k = 0; k < K; k++) {
+                    const int kc = k / KC, kg = (k % KC) / 8, e = k % 8;
+                    const size_t off = base + ((size_t(a) * mh + h) * nkc + kc) * chunk +
+                                       (size_t(rg) * (KC / 8) + kg) * 64 + size_t(r) * 8 + e;
+                    G.dig[off] = bf16_of_int(dg[size_t(a) * K + k]);
+                }
+        }
+    };
+    // the 256 x 256 near tables take a few ms each: the rows in parallel
+    const int nt = size_t(rows) * K > 8192 ? 8 : 1;
+    bool ok[8];
+    std::fill(ok, ok + 8, true);
+    std::vector<std::thread> th;
+    for (int t = 1; t < nt; t++) th.emplace_back(part, rows * t / nt, rows * (t + 1) / nt, &ok[t]);
+    part(0, rows / nt, &ok[0]);
+    for (auto &t : th) t.join();
+    for (bool v : ok) G.exact = G.exact && v;
     return op;
 }
 
-// Real operators of the split path, direction dir (0 forward, 1 adjoint):
-//   group V, K = KV (the p^2 leaf nodes, zero columns up to 64 for p = 8 and
-//     to 256 for p = 12, 16): near tables (p^2 rows), leafA (2 P1 rows: P2M /
-//     L2P^H), X list per code (2 P1 rows: P2L / M2P^H); output rows 2l, 2l+1 =
-//     Re, Im of coefficient l;
+// Device memory of one set-up in a single allocation: the uploaded arrays
+// (one copy) and the uninitialised ones.
+struct DevArena {
+    struct Item { void **dst; const void *src; size_t bytes; };
+    std::vector<Item> items;
+    template <class T> void add(T **dst, const std::vector<T> &v)
+    {
+        items.push_back({reinterpret_cast<void **>(dst), v.data(), v.size() * sizeof(T)});
+    }
+    template <class T> void room(T **dst, size_t n) { items.push_back({reinterpret_cast<void **>(dst), nullptr, n * sizeof(T)}); }
+    cudaError_t commit(std::vector<void *> &allocs, cudaStream_t st)
+    {
+        std::stable_sort(items.begin(), items.end(), [](const Item &a, const Item &b) { return (a.src != nullptr) > (b.src != nullptr); });
+        std::vector<size_t> off;
+        size_t total = 0, up = 0;
+        for (const Item &it : items) {
+            off.push_back(total);
+            total += std::max<size_t>((it.bytes + 255) & ~size_t(255), 256);
+            if (it.src) up = total;
+        }
+        void *base = nullptr;
+        cudaError_t e = cudaMalloc(&base, std::max<size_t>(total, 256));
+        if (e != cudaSuccess) return e;
+        std::vector<uint8_t> host(up);
+        for (size_t i = 0; i < items.size(); i++)
+            if (items[i].src && items[i].bytes) std::memcpy(host.data() + off[i], items[i].src, items[i].bytes);
+        if (up) e = cudaMemcpyAsync(base, host.data(), up, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) { cudaFree(base); return e; }
+        allocs.push_back(base);
+        for (size_t i = 0; i < items.size(); i++) *items[i].dst = static_cast<uint8_t *>(base) + off[i];
+        return cudaSuccess;
+    }
+};
+
+// Real operators of the digit products, direction dir (0 forward, 1 adjoint):
+//   group V, K = KV (the p^2 leaf nodes, zero columns up to KV): near tables
+//     (p^2 rows), leafA (2 P1 rows: P2M / L2P^H), X list per code (2 P1 rows:
+//     P2L / M2P^H); output rows 2l, 2l+1 = Re, Im of coefficient l;
 //   group E, K = 64 (coefficient l at columns 2l, 2l+1 = Re, Im): L2P / P2M^H
 //     and the W list per code (M2P / P2L^H), p^2 rows, output = real part.
-bc_status build_split_tables(bc_ctx *ctx)
+bc_status build_digit_tables(bc_ctx *ctx, SplitTables &T, int slices, bool *ready)
 {
-    // split path: p = 8, 12 or 16, P1 <= 32
-    if ((ctx->p != 8 && ctx->p != 12 && ctx->p != 16) || ctx->device < 0 || 2 * ctx->P1 > kSplitKE) return BC_OK;
+    const bool wide = slices == kWideSlices;
     const HostTables &ht = ctx->ht;
-    const int NP = ctx->NP, KV = NP <= 64 ? 64 : 256, P1 = ctx->P1, R = 2 * P1, KE = kSplitKE;
-    SplitTables &T = ctx->split;
+    const int NP = ctx->NP, P1 = ctx->P1, R = 2 * P1, KE = kSplitKE;
+    const int KV = NP <= 64 ? 64 : wide && NP <= 144 ? 144 : 256;
+    T.slices = slices;
+    T.tileN = wide ? kWideTileN : kSplitTileN;
     T.np = NP;
     T.kv = KV;
+    DevArena arena;
+    OpGroup gv[2], ge[2];
+    std::vector<double> scl[2];
+    // Column scales of group V (7 digits, forward): column k of the operators is
+    // about w_k times the kernel, w_k the node's quadrature weight (down to 1/400
+    // of the largest); dividing it out and multiplying the leaf values by it
+    // (powers of two) keeps the fixed-point rounding in proportion.  The
+    // adjoint operators carry the weights in their rows instead.
+    std::vector<double> vs(NP, 1.0);
+    if (wide) {
+        const double wm = *std::max_element(ht.w.begin(), ht.w.end());
+        for (int k = 0; k < NP; k++) vs[k] = std::ldexp(1.0, int(std::lround(std::log2(std::max(ht.w[k] / wm, 1e-12)))));
+    }
     for (int dir = 0; dir < 2; dir++) {
-        std::vector<uint16_t> dv, de;
-        std::vector<int32_t> xv, xe;
+        OpGroup &V = gv[dir], &E = ge[dir];
+        V.S = E.S = slices;
+        V.K = KV; V.kvalid = NP;
+        E.K = KE; E.kvalid = R;
         std::vector<double> m;
+        auto cscale = [&](int k) { return dir == 0 ? 1.0 / vs[k] : 1.0; };
         // group V
         T.near_op[dir].assign(kNumNear, SplitOp());
         m.assign(size_t(NP) * KV, 0.0);
@@ -592,28 +678,28 @@ bc_status build_split_tables(bc_ctx *ctx)
             if (!g.valid) continue;
             for (int i = 0; i < NP; i++)
                 for (int k = 0; k < NP; k++)
-                    m[size_t(i) * KV + k] = dir == 0 ? ht.T[(size_t(tab) * NP + i) * NP + k]
-                                                     : ht.T[(size_t(g.rev) * NP + k) * NP + i];
-            T.near_op[dir][tab] = add_split_op(dv, xv, m, NP, KV);
+                    m[size_t(i) * KV + k] = cscale(k) * (dir == 0 ? ht.T[(size_t(tab) * NP + i) * NP + k]
+                                                                  : ht.T[(size_t(g.rev) * NP + k) * NP + i]);
+            T.near_op[dir][tab] = add_split_op(V, m, NP);
         }
         m.assign(size_t(R) * KV, 0.0);
         for (int l = 0; l < P1; l++)
             for (int j = 0; j < NP; j++) {
                 cplx z = dir == 0 ? at2(ht.Q, size_t(l) * NP + j) : std::conj(at2(ht.E, size_t(j) * P1 + l));
-                m[size_t(2 * l) * KV + j] = z.real();
-                m[size_t(2 * l + 1) * KV + j] = z.imag();
+                m[size_t(2 * l) * KV + j] = cscale(j) * z.real();
+                m[size_t(2 * l + 1) * KV + j] = cscale(j) * z.imag();
             }
-        T.leafA_op[dir] = add_split_op(dv, xv, m, R, KV);
+        T.leafA_op[dir] = add_split_op(V, m, R);
         T.x_op[dir].assign(kNumWX, SplitOp());
         for (int c = 0; c < kNumWX; c++) {
             for (int l = 0; l < P1; l++)
                 for (int j = 0; j < NP; j++) {
                     cplx z = dir == 0 ? at2(ht.P2L, (size_t(c) * P1 + l) * NP + j)
                                       : std::conj(at2(ht.M2P, (size_t(c) * NP + j) * P1 + l));
-                    m[size_t(2 * l) * KV + j] = z.real();
-                    m[size_t(2 * l + 1) * KV + j] = z.imag();
+                    m[size_t(2 * l) * KV + j] = cscale(j) * z.real();
+                    m[size_t(2 * l + 1) * KV + j] = cscale(j) * z.imag();
                 }
-            T.x_op[dir][c] = add_split_op(dv, xv, m, R, KV);
+            T.x_op[dir][c] = add_split_op(V, m, R);
         }
         // group E: out_j = Re(sum_l Op(j,l) b_l) = sum_l Re Op(j,l) Re b_l - Im Op(j,l) Im b_l;
         // columns rescaled by powers of two (the expansion digits carry the inverse scale)
@@ -649,9 +735,9 @@ bc_status build_split_tables(bc_ctx *ctx)
                 for (int c = 0; c < kNumWX; c++) mw[c][size_t(j) * KE + k] /= sw[k];
             }
         }
-        T.e_op[dir] = add_split_op(de, xe, me, NP, KE);
+        T.e_op[dir] = add_split_op(E, me, NP);
         T.w_op[dir].assign(kNumWX, SplitOp());
-        for (int c = 0; c < kNumWX; c++) T.w_op[dir][c] = add_split_op(de, xe, mw[c], NP, KE);
+        for (int c = 0; c < kNumWX; c++) T.w_op[dir][c] = add_split_op(E, mw[c], NP);
         // Group M: M2L per V code in real form (rows 2l, 2l+1 = Re, Im of
         // output coefficient l; column 2k, 2k+1 = Re, Im of input k):
         //   forward (l,k) = M2L_c[l][k];  adjoint (l,k) = conj(M2L_{-d}[k][l]),
@@ -678,61 +764,78 @@ bc_status build_split_tables(bc_ctx *ctx)
                         mm[size_t(2 * l + 1) * KE + 2 * k] = z.imag() / sw[2 * k];
                         mm[size_t(2 * l + 1) * KE + 2 * k + 1] = z.real() / sw[2 * k + 1];
                     }
-                T.m2l_op[dir][c] = add_split_op(de, xe, mm, R, KE);
+                T.m2l_op[dir][c] = add_split_op(E, mm, R);
             }
         }
         // expA is the W source (first) in the forward apply and the P2M^H input
         // (second) in the adjoint; expB the other way round
-        std::vector<double> scl(2 * KE);
+        scl[dir].resize(2 * KE);
         for (int k = 0; k < KE; k++) {
-            scl[k] = dir == 0 ? sw[k] : se[k];
-            scl[KE + k] = dir == 0 ? se[k] : sw[k];
+            scl[dir][k] = dir == 0 ? sw[k] : se[k];
+            scl[dir][KE + k] = dir == 0 ? se[k] : sw[k];
         }
-        double *dsc = nullptr;
-        uint16_t *d0 = nullptr, *d1 = nullptr;
-        int32_t *e0 = nullptr, *e1 = nullptr;
-        cudaError_t e;
-        if ((e = dev_upload(ctx->split_allocs, &d0, dv.data(), dv.size())) != cudaSuccess ||
-            (e = dev_upload(ctx->split_allocs, &e0, xv.data(), xv.size())) != cudaSuccess ||
-            (e = dev_upload(ctx->split_allocs, &d1, de.data(), de.size())) != cudaSuccess ||
-            (e = dev_upload(ctx->split_allocs, &e1, xe.data(), xe.size())) != cudaSuccess ||
-            (e = dev_upload(ctx->split_allocs, &dsc, scl.data(), scl.size())) != cudaSuccess)
-            return cuda_fail(e, "split tables upload");
-        T.escale[dir] = dsc;
-        T.ops[0][dir] = reinterpret_cast<const uint8_t *>(d0);
-        T.op_exp[0][dir] = e0;
-        T.ops[1][dir] = reinterpret_cast<const uint8_t *>(d1);
-        T.op_exp[1][dir] = e1;
+        if (wide && !(V.exact && E.exact)) return BC_OK;   // not ready: the FP64 kernels serve
     }
-    cudaError_t e = split_prepare();
-    if (e != cudaSuccess) return cuda_fail(e, "split kernel attributes");
-    if (!ctx->side.side) {
-        if ((e = cudaStreamCreateWithFlags(&ctx->side.side, cudaStreamNonBlocking)) != cudaSuccess ||
-            (e = cudaEventCreateWithFlags(&ctx->side.fork, cudaEventDisableTiming)) != cudaSuccess ||
-            (e = cudaEventCreateWithFlags(&ctx->side.join, cudaEventDisableTiming)) != cudaSuccess ||
-            (e = cudaEventCreateWithFlags(&ctx->side.xdone, cudaEventDisableTiming)) != cudaSuccess)
-            return cuda_fail(e, "split side stream");
+    uint16_t *d[2][2];
+    int32_t *x[2][2];
+    double *f[2][2], *sc[2], *pv = nullptr;
+    for (int dir = 0; dir < 2; dir++) {
+        arena.add(&d[0][dir], gv[dir].dig);
+        arena.add(&x[0][dir], gv[dir].ex);
+        arena.add(&f[0][dir], gv[dir].f);
+        arena.add(&d[1][dir], ge[dir].dig);
+        arena.add(&x[1][dir], ge[dir].ex);
+        arena.add(&f[1][dir], ge[dir].f);
+        arena.add(&sc[dir], scl[dir]);
     }
-    ctx->split_ready = true;
+    arena.add(&pv, vs);
+    cudaError_t e = arena.commit(ctx->split_allocs, cudaStreamPerThread);
+    if (e != cudaSuccess) return cuda_fail(e, "digit tables upload");
+    for (int dir = 0; dir < 2; dir++) {
+        T.escale[dir] = sc[dir];
+        for (int g = 0; g < 2; g++) {
+            T.ops[g][dir] = reinterpret_cast<const uint8_t *>(d[g][dir]);
+            T.op_exp[g][dir] = x[g][dir];
+            T.opf[g][dir] = wide ? f[g][dir] : nullptr;
+        }
+    }
+    T.vscale[0] = wide ? pv : nullptr;
+    *ready = true;
     return BC_OK;
 }
 
-// Column lists of the split path for one tree.  Tiles hold up to
-// kSplitTileN columns that share one operator; tiles of 256-row operators
-// come first (longest work first).
+// 5-digit operators for the split modes (p = 8, 12, 16), 7-digit ones for the
+// FP64 mode (every p); nterms <= 32.
+bc_status build_split_tables(bc_ctx *ctx)
+{
+    if (ctx->device < 0 || 2 * ctx->P1 > kSplitKE) return BC_OK;
+    bc_status s = BC_OK;
+    if (ctx->p == 8 || ctx->p == 12 || ctx->p == 16) s = build_digit_tables(ctx, ctx->split, kSplitSlices, &ctx->split_ready);
+    if (s == BC_OK) s = build_digit_tables(ctx, ctx->wide, kWideSlices, &ctx->wide_ready);
+    if (s != BC_OK) return s;
+    cudaError_t e = split_prepare();
+    return e == cudaSuccess ? BC_OK : cuda_fail(e, "split kernel attributes");
+}
+
+// Column lists of the digit products for one tree.  Tiles hold up to `cap`
+// columns that share one operator; tiles of 256-row operators come first
+// (longest work first).
 struct TileBuilder {
+    int cap;
     std::vector<SplitTile> tiles;
     std::vector<SplitCol> cols;
+    explicit TileBuilder(int n) : cap(n) {}
     // one operator, its columns given in order
     void add(const SplitOp &op, const std::vector<SplitCol> &c)
     {
-        for (size_t i = 0; i < c.size(); i += kSplitTileN) {
+        for (size_t i = 0; i < c.size(); i += cap) {
             SplitTile t;
             t.a_off = op.a_off;
+            t.f_off = op.f_off;
             t.rows = op.rows;
             t.exp_off = op.exp_off;
             t.p0 = int32_t(cols.size());
-            t.cnt = int32_t(std::min<size_t>(kSplitTileN, c.size() - i));
+            t.cnt = int32_t(std::min<size_t>(cap, c.size() - i));
             cols.insert(cols.end(), c.begin() + i, c.begin() + i + t.cnt);
             tiles.push_back(t);
         }
@@ -741,40 +844,97 @@ struct TileBuilder {
 
 inline int32_t col_ctl(int shift, bool inv_alpha) { return int32_t(shift * 2 + (inv_alpha ? 1 : 0)); }
 
-bc_status build_split_tree(bc_tree *t)
+// The internal stream and its events, one set per tree (applies of one tree
+// are serialised by the caller, those of different trees are not).
+cudaError_t ensure_side(bc_tree *t)
 {
-    if (t->split_ready) return BC_OK;
+    if (t->side.xdone) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (!t->side.side) e = cudaStreamCreateWithFlags(&t->side.side, cudaStreamNonBlocking);
+    for (cudaEvent_t *ev : {&t->side.fork, &t->side.join, &t->side.xdone})
+        if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    return e;
+}
+
+void free_side(bc_tree *t)
+{
+    for (cudaEvent_t ev : {t->side.fork, t->side.join, t->side.xdone})
+        if (ev) cudaEventDestroy(ev);
+    if (t->side.side) cudaStreamDestroy(t->side.side);
+    t->side = SideStream();
+}
+
+// V-list tiles (tensor-core M2L, part 32): one column per V pair (source box
+// digits, the result row into Pv; the adjoint digits carry alpha0).
+TileBuilder m2l_tiles(const bc_tree *t, const SplitTables &T, int dir, double2 *Pv)
+{
     const HostTree &h = t->h;
-    const SplitTables &T = t->ctx->split;
-    const int P1 = t->ctx->P1;
+    const int P1 = t->ctx->P1, first_which = dir == 1 ? 1 : 0;   // expA = 0, expB = 1
+    const int64_t nbox = int64_t(h.box_level.size());
+    TileBuilder M(T.tileN);
+    std::vector<std::vector<SplitCol>> by_v(kNumV);
+    for (size_t k = 0; k < h.v_src.size(); k++) {
+        SplitCol c;
+        c.vec = int32_t(first_which * nbox + h.v_src[k]);
+        c.ctl = col_ctl(0, dir == 1);
+        c.out = reinterpret_cast<double *>(Pv + k * size_t(P1));
+        by_v[h.v_code[k]].push_back(c);
+    }
+    for (int c = 0; c < kNumV; c++)
+        if (!by_v[c].empty()) M.add(T.m2l_op[dir][c], by_v[c]);
+    return M;
+}
+
+// Tiles, digit buffers and result rows of a tree in the format of T.  The two
+// formats share the result rows.
+cudaError_t build_digit_tree(bc_tree *t, const SplitTables &T, SplitTree &s, bool m2l)
+{
+    const HostTree &h = t->h;
+    const int P1 = t->ctx->P1, S = T.slices;
     const int64_t nn = int64_t(h.near_src.size()), nx = int64_t(h.x_src.size()), nw = int64_t(h.w_src.size());
     const int64_t nbox = int64_t(h.box_level.size());
-    SplitTree &s = t->sp;
-    std::vector<void *> &al = t->d.allocs;
-    cudaError_t e;
+    cudaError_t e = ensure_side(t);
+    if (e != cudaSuccess) return e;
     const size_t NP = size_t(T.np), KV = size_t(T.kv);   // nodes per leaf, group-V K
-    if ((e = dev_upload<double>(al, &s.Pnear, nullptr, size_t(nn) * NP)) != cudaSuccess ||
-        (e = dev_upload<double>(al, &s.PX, nullptr, size_t(nx) * kSplitKE)) != cudaSuccess ||
-        (e = dev_upload<double>(al, &s.PE, nullptr, size_t(h.nleaf) * NP)) != cudaSuccess ||
-        (e = dev_upload<double>(al, &s.PW, nullptr, size_t(nw) * NP)) != cudaSuccess ||
-        (e = dev_upload<uint16_t>(al, &s.vdig, nullptr, size_t(h.nleaf) * kSplitSlices * KV)) != cudaSuccess ||
-        (e = dev_upload<int32_t>(al, &s.vexp, nullptr, size_t(h.nleaf))) != cudaSuccess ||
-        (e = dev_upload<uint16_t>(al, &s.edig, nullptr, size_t(2 * nbox) * kSplitSlices * kSplitKE)) != cudaSuccess ||
-        (e = dev_upload<int32_t>(al, &s.eexp, nullptr, size_t(2 * nbox))) != cudaSuccess)
-        return cuda_fail(e, "split tree upload");
+    // device room first: the tiles hold the result rows' addresses
+    std::vector<void *> &al = t->d.allocs;
+    const size_t mark = al.size();
+    const SplitTree &o = &s == &t->sp ? t->spw : t->sp;
+    SplitTree n;
+    double2 *Pv = t->d.Pv;
+    {
+        DevArena room;
+        if (o.Pnear) {
+            n.Pnear = o.Pnear; n.PX = o.PX; n.PE = o.PE; n.PW = o.PW;
+        } else {
+            room.room(&n.Pnear, size_t(nn) * NP);
+            room.room(&n.PX, size_t(nx) * kSplitKE);
+            room.room(&n.PE, size_t(h.nleaf) * NP);
+            room.room(&n.PW, size_t(nw) * NP);
+        }
+        if (m2l && !Pv) room.room(&Pv, h.v_src.size() * size_t(P1));
+        room.room(&n.vdig, size_t(h.nleaf) * S * KV);
+        room.room(&n.vexp, size_t(h.nleaf));
+        room.room(&n.edig, size_t(2 * nbox) * S * kSplitKE);
+        room.room(&n.eexp, size_t(2 * nbox));
+        if ((e = room.commit(al, t->side.side)) != cudaSuccess) return e;
+    }
     // owners of the near and W entries, box of each X entry
     std::vector<int32_t> near_owner(nn), w_owner(nw), x_box(nx);
-    for (int64_t o = 0; o < h.nleaf; o++) {
-        for (int32_t k = h.near_ptr[o]; k < h.near_ptr[o + 1]; k++) near_owner[k] = int32_t(o);
-        for (int32_t k = h.w_ptr[o]; k < h.w_ptr[o + 1]; k++) w_owner[k] = int32_t(o);
+    for (int64_t o2 = 0; o2 < h.nleaf; o2++) {
+        for (int32_t k = h.near_ptr[o2]; k < h.near_ptr[o2 + 1]; k++) near_owner[k] = int32_t(o2);
+        for (int32_t k = h.w_ptr[o2]; k < h.w_ptr[o2 + 1]; k++) w_owner[k] = int32_t(o2);
     }
     for (int64_t b = 0; b < nbox; b++)
         for (int32_t k = h.x_ptr[b]; k < h.x_ptr[b + 1]; k++) x_box[k] = int32_t(b);
+    DevArena up;
+    std::vector<TileBuilder> keep;   // [dir]: VN, V, N, E, M (alive until the upload)
+    keep.reserve(10);
     for (int dir = 0; dir < 2; dir++) {
         const bool adj = dir == 1;
         double2 *first = adj ? t->d.expB : t->d.expA;
         const int first_which = adj ? 1 : 0, second_which = adj ? 0 : 1;   // expA = 0, expB = 1
-        TileBuilder V, NV, E;
+        TileBuilder V(T.tileN), NV(T.tileN), E(T.tileN);
         // near entries, by table
         std::vector<std::vector<SplitCol>> by_tab(kNumNear);
         for (int64_t k = 0; k < nn; k++) {
@@ -782,7 +942,7 @@ bc_status build_split_tree(bc_tree *t)
             SplitCol c;
             c.vec = src;
             c.ctl = col_ctl(-2 * (adj ? h.leaf_level[own] : h.leaf_level[src]), false);
-            c.out = s.Pnear + size_t(k) * NP;
+            c.out = n.Pnear + size_t(k) * NP;
             by_tab[h.near_tab[k]].push_back(c);
         }
         for (int tab = 0; tab < kNumNear; tab++)
@@ -790,21 +950,21 @@ bc_status build_split_tree(bc_tree *t)
         // leafA of every leaf (Morton order), then the X entries by code
         std::vector<SplitCol> cl;
         for (int64_t i = 0; i < h.nleaf; i++) {
-            const int32_t o = h.leaf_order[i];
+            const int32_t o2 = h.leaf_order[i];
             SplitCol c;
-            c.vec = o;
-            c.ctl = adj ? col_ctl(0, true) : col_ctl(-2 * h.leaf_level[o], false);
-            c.out = reinterpret_cast<double *>(first + size_t(h.leaf_box[o]) * P1);
+            c.vec = o2;
+            c.ctl = adj ? col_ctl(0, true) : col_ctl(-2 * h.leaf_level[o2], false);
+            c.out = reinterpret_cast<double *>(first + size_t(h.leaf_box[o2]) * P1);
             cl.push_back(c);
         }
         V.add(T.leafA_op[dir], cl);
-        s.ntA[dir] = int(V.tiles.size());
+        n.ntA[dir] = int(V.tiles.size());
         std::vector<std::vector<SplitCol>> by_code(kNumWX);
         for (int64_t k = 0; k < nx; k++) {
             SplitCol c;
             c.vec = h.x_src[k];
             c.ctl = adj ? col_ctl(0, true) : col_ctl(-2 * (h.box_level[x_box[k]] - 1), false);
-            c.out = s.PX + size_t(k) * kSplitKE;
+            c.out = n.PX + size_t(k) * kSplitKE;
             by_code[h.x_code[k]].push_back(c);
         }
         for (int c = 0; c < kNumWX; c++)
@@ -812,22 +972,22 @@ bc_status build_split_tree(bc_tree *t)
         // group E: L2P of the leaves at level >= 2, then the W entries by code
         cl.clear();
         for (int64_t i = 0; i < h.nleaf; i++) {
-            const int32_t o = h.leaf_order[i];
-            if (h.leaf_level[o] < 2) continue;
+            const int32_t o2 = h.leaf_order[i];
+            if (h.leaf_level[o2] < 2) continue;
             SplitCol c;
-            c.vec = int32_t(second_which * nbox + h.leaf_box[o]);
-            c.ctl = col_ctl(adj ? -2 * h.leaf_level[o] : 0, false);
-            c.out = s.PE + size_t(o) * NP;
+            c.vec = int32_t(second_which * nbox + h.leaf_box[o2]);
+            c.ctl = col_ctl(adj ? -2 * h.leaf_level[o2] : 0, false);
+            c.out = n.PE + size_t(o2) * NP;
             cl.push_back(c);
         }
         E.add(T.e_op[dir], cl);
-        s.ntL[dir] = int(E.tiles.size());
+        n.ntL[dir] = int(E.tiles.size());
         for (auto &v : by_code) v.clear();
         for (int64_t k = 0; k < nw; k++) {
             SplitCol c;
             c.vec = int32_t(first_which * nbox + h.w_src[k]);
             c.ctl = col_ctl(adj ? -2 * h.leaf_level[w_owner[k]] : 0, false);
-            c.out = s.PW + size_t(k) * NP;
+            c.out = n.PW + size_t(k) * NP;
             by_code[h.w_code[k]].push_back(c);
         }
         for (int c = 0; c < kNumWX; c++)
@@ -838,61 +998,92 @@ bc_status build_split_tree(bc_tree *t)
             VN.tiles.push_back(tl);
         }
         VN.cols.insert(VN.cols.end(), V.cols.begin(), V.cols.end());
-        if ((e = dev_upload(al, &s.tVN[dir], VN.tiles.data(), VN.tiles.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.cVN[dir], VN.cols.data(), VN.cols.size())) != cudaSuccess)
-            return cuda_fail(e, "split tree upload");
-        s.ntVN[dir] = int(VN.tiles.size());
-        if ((e = dev_upload(al, &s.tV[dir], V.tiles.data(), V.tiles.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.cV[dir], V.cols.data(), V.cols.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.tN[dir], NV.tiles.data(), NV.tiles.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.cN[dir], NV.cols.data(), NV.cols.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.tE[dir], E.tiles.data(), E.tiles.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.cE[dir], E.cols.data(), E.cols.size())) != cudaSuccess)
-            return cuda_fail(e, "split tree upload");
-        s.ntV[dir] = int(V.tiles.size());
-        s.ntN[dir] = int(NV.tiles.size());
-        s.ntE[dir] = int(E.tiles.size());
+        auto put = [&](TileBuilder &&b, SplitTile **tiles, SplitCol **cols, int *nt) {
+            *nt = int(b.tiles.size());
+            keep.push_back(std::move(b));
+            up.add(tiles, keep.back().tiles);
+            up.add(cols, keep.back().cols);
+        };
+        put(std::move(VN), &n.tVN[dir], &n.cVN[dir], &n.ntVN[dir]);
+        put(std::move(V), &n.tV[dir], &n.cV[dir], &n.ntV[dir]);
+        put(std::move(NV), &n.tN[dir], &n.cN[dir], &n.ntN[dir]);
+        put(std::move(E), &n.tE[dir], &n.cE[dir], &n.ntE[dir]);
+        if (m2l) put(m2l_tiles(t, T, dir, Pv), &n.tM[dir], &n.cM[dir], &n.ntM[dir]);
     }
-    s.err = t->ctx->dev_err;
+    if ((e = up.commit(al, t->side.side)) != cudaSuccess) {
+        while (al.size() > mark) { cudaFree(al.back()); al.pop_back(); }
+        return e;
+    }
+    n.err = t->ctx->dev_err;
+    s = n;
+    t->d.Pv = Pv;
+    return cudaSuccess;
+}
+
+bc_status build_split_tree(bc_tree *t)
+{
+    if (t->split_ready) return BC_OK;
+    const cudaError_t e = build_digit_tree(t, t->ctx->split, t->sp, false);
+    if (e != cudaSuccess) return cuda_fail(e, "split tree upload");
     t->split_ready = true;
     return BC_OK;
 }
 
-// Tensor-core M2L (part 32, BC_SPLIT_BF16_ALL): one column per V pair
-// (source box digits, the result row into Pv, allocated here on first use:
-// n_v x nterms x 16 bytes; the adjoint digits carry alpha0).
+// 5-digit M2L tiles (part 32, BC_SPLIT_BF16_ALL) and the rows they write
+// (n_v x nterms x 16 bytes), on first use.
 bc_status build_split_m2l(bc_tree *t)
 {
     if (t->m2l_ready) return BC_OK;
-    const HostTree &h = t->h;
-    const SplitTables &T = t->ctx->split;
-    const int P1 = t->ctx->P1;
-    const int64_t nbox = int64_t(h.box_level.size());
     SplitTree &s = t->sp;
     std::vector<void *> &al = t->d.allocs;
-    cudaError_t e = dev_upload<double2>(al, &t->d.Pv, nullptr, h.v_src.size() * size_t(P1));
-    if (e != cudaSuccess) return cuda_fail(e, "tensor-core M2L rows");
-    for (int dir = 0; dir < 2; dir++) {
-        const int first_which = dir == 1 ? 1 : 0;   // expA = 0, expB = 1
-        TileBuilder M;
-        std::vector<std::vector<SplitCol>> by_v(kNumV);
-        for (size_t k = 0; k < h.v_src.size(); k++) {
-            SplitCol c;
-            c.vec = int32_t(first_which * nbox + h.v_src[k]);
-            c.ctl = col_ctl(0, dir == 1);
-            c.out = reinterpret_cast<double *>(t->d.Pv + k * size_t(P1));
-            by_v[h.v_code[k]].push_back(c);
-        }
-        for (int c = 0; c < kNumV; c++)
-            if (!by_v[c].empty()) M.add(T.m2l_op[dir][c], by_v[c]);
-        if ((e = dev_upload(al, &s.tM[dir], M.tiles.data(), M.tiles.size())) != cudaSuccess ||
-            (e = dev_upload(al, &s.cM[dir], M.cols.data(), M.cols.size())) != cudaSuccess)
-            return cuda_fail(e, "tensor-core M2L tiles");
-        s.ntM[dir] = int(M.tiles.size());
+    cudaError_t e = cudaSuccess;
+    if (!t->d.Pv) {
+        DevArena room;
+        room.room(&t->d.Pv, t->h.v_src.size() * size_t(t->ctx->P1));
+        if ((e = room.commit(al, t->side.side)) != cudaSuccess) return cuda_fail(e, "tensor-core M2L rows");
     }
+    TileBuilder M0 = m2l_tiles(t, t->ctx->split, 0, t->d.Pv), M1 = m2l_tiles(t, t->ctx->split, 1, t->d.Pv);
+    DevArena up;
+    up.add(&s.tM[0], M0.tiles);
+    up.add(&s.cM[0], M0.cols);
+    up.add(&s.tM[1], M1.tiles);
+    up.add(&s.cM[1], M1.cols);
+    if ((e = up.commit(al, t->side.side)) != cudaSuccess) return cuda_fail(e, "tensor-core M2L tiles");
+    s.ntM[0] = int(M0.tiles.size());
+    s.ntM[1] = int(M1.tiles.size());
     t->m2l_ready = true;
     return BC_OK;
 }
+
+// 7-digit tiles of the FP64 mode, on first use.  They take device memory that
+// the FP64 kernels do not need; where that is not to be had the FP64 kernels
+// serve (and are asked for again only with another tree).  The set-up runs on
+// the tree's own stream, so it neither joins nor breaks a stream capture.
+bool build_wide_tree(bc_tree *t)
+{
+    if (t->wide_ready) return true;
+    if (t->wide_off || !t->ctx->wide_ready) return false;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return false; }
+    cudaError_t e;
+    try {
+        e = build_digit_tree(t, t->ctx->wide, t->spw, true);
+    } catch (const std::bad_alloc &) {
+        e = cudaErrorMemoryAllocation;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        t->wide_off = true;
+        return false;
+    }
+    t->wide_ready = true;
+    return true;
+}
+
+// Parts of an FP64 apply on 7-digit products: all of them, the M2L only in its
+// default form (the options that choose another one keep the FP64 kernels).
+int wide_parts(const bc_ctx *ctx) { return ctx->m2l_tri || ctx->m2l_kind ? kSplitTableParts : kWideParts; }
 
 // CTAs of the near-field launch on the internal stream: the option, else all
 // SMs when it runs beside the FP64 M2L (one tensor CTA per SM next to the M2L
@@ -930,20 +1121,28 @@ bc_status apply_impl(bc_ctx *ctx, const bc_tree *tree, const double *vin, double
     // apply only, 3 the adjoint only, 0 neither
     const int ov = ctx->split_overlap;
     const bool side = ov == 1 || (ov == 2 && !adj) || (ov == 3 && adj);
-    SplitLaunch sl{&ctx->split, nullptr, parts, side ? &ctx->side : nullptr, near_ctas_for(ctx, parts)};
+    SplitLaunch sl{&ctx->split, nullptr, parts, nullptr, near_ctas_for(ctx, parts)};
     const SplitLaunch *split = nullptr;
     bc_tree *tw = const_cast<bc_tree *>(tree);
-    if (is_split(prec)) {
-        if (!ctx->split_ready) {
-            set_error("apply: split precision is provided for p = 8, 12 and 16 with nterms <= 32 only");
-            return BC_ERR_UNSUPPORTED;
-        }
+    if (is_split(prec) && !ctx->split_ready) {
+        set_error("apply: split precision is provided for p = 8, 12 and 16 with nterms <= 32 only");
+        return BC_ERR_UNSUPPORTED;
+    }
+    // (a split apply without any 5-digit product is the FP64 apply)
+    if ((prec == BC_FP64 || parts == 0) && build_wide_tree(tw)) {
+        sl.tables = &ctx->wide;
+        sl.tree = &tw->spw;
+        sl.parts = wide_parts(ctx);
+        sl.near_ctas = near_ctas_for(ctx, sl.parts);
+        split = &sl;
+    } else if (is_split(prec)) {
         s = build_split_tree(tw);
         if (s == BC_OK && (parts & 32)) s = build_split_m2l(tw);
         if (s != BC_OK) return s;
         sl.tree = &tw->sp;
         split = &sl;
     }
+    if (split && side) sl.side = &tw->side;
     if (din) {
         e = launch_apply(a, tree->h, tree->d, ctx->dt, adj, vin, vout, st, ctx->pass_mask, ctx->timing ? ctx->ev[adj ? 1 : 0] : nullptr, ctx->m2l_tri, split);
         if (e != cudaSuccess) return cuda_fail(e, "apply launch");
@@ -957,7 +1156,7 @@ bc_status apply_impl(bc_ctx *ctx, const bc_tree *tree, const double *vin, double
     // Otherwise they are staged through the tree's device buffers.
     const double *pin_in = static_cast<const double *>(pinned_device_ptr(vin));
     double *pin_out = static_cast<double *>(const_cast<void *>(pinned_device_ptr(vout)));
-    if (split && (parts & 7) == 7 && pin_in && pin_out) {
+    if (split && (sl.parts & 7) == 7 && pin_in && pin_out) {
         e = launch_apply(a, tree->h, tree->d, ctx->dt, adj, pin_in, pin_out, st, ctx->pass_mask,
                          ctx->timing ? ctx->ev[adj ? 1 : 0] : nullptr, ctx->m2l_tri, split);
         if (e != cudaSuccess) return cuda_fail(e, "apply launch");
@@ -987,6 +1186,7 @@ bc_status apply_impl(bc_ctx *ctx, const bc_tree *tree, const double *vin, double
 }  // namespace
 
 bc_status prepare_split_tree(bc_tree *t) { return build_split_tree(t); }
+bool prepare_wide_tree(bc_tree *t) { return build_wide_tree(t); }
 
 void set_error(const char *fmt, ...)
 {
@@ -1031,15 +1231,23 @@ bc_status batch_capture(bc_batch *b, int prec, int adj, int leaf_bps, int m2l_bp
     const int parts = split_parts_for(prec, ctx->split_parts);
     const int ov = ctx->split_overlap;
     const bool side = ov == 1 || (ov == 2 && !adj) || (ov == 3 && adj);
-    SplitLaunch sl{&ctx->split, &b->u->sp, parts, side ? &ctx->side : nullptr, near_ctas_for(ctx, parts)};
-    if (is_split(prec) && (parts & 32)) {   // before the capture: it allocates
+    SplitLaunch sl{&ctx->split, &b->u->sp, parts, nullptr, near_ctas_for(ctx, parts)};
+    // before the capture: they allocate
+    const bool wide = (prec == BC_FP64 || parts == 0) && build_wide_tree(b->u);
+    if (wide) {
+        sl.tables = &ctx->wide;
+        sl.tree = &b->u->spw;
+        sl.parts = wide_parts(ctx);
+        sl.near_ctas = near_ctas_for(ctx, sl.parts);
+    } else if (is_split(prec) && (parts & 32)) {
         bc_status s = build_split_m2l(b->u);
         if (s != BC_OK) return s;
     }
+    if (side && (wide || is_split(prec))) sl.side = &b->u->side;
     cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "batch: begin capture");
     cudaError_t le = launch_apply(a, b->u->h, b->u->d, ctx->dt, adj != 0, b->in_buf, b->out_buf, b->cap, 3, nullptr,
-                                  ctx->m2l_tri, is_split(prec) ? &sl : nullptr);
+                                  ctx->m2l_tri, wide || is_split(prec) ? &sl : nullptr);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(b->cap, &graph);
     if (le != cudaSuccess) {
@@ -1114,10 +1322,6 @@ void bc_destroy(bc_ctx *ctx)
     for (auto &dir : ctx->ev)
         for (auto &e : dir)
             if (e) cudaEventDestroy(e);
-    if (ctx->side.fork) cudaEventDestroy(ctx->side.fork);
-    if (ctx->side.join) cudaEventDestroy(ctx->side.join);
-    if (ctx->side.xdone) cudaEventDestroy(ctx->side.xdone);
-    if (ctx->side.side) cudaStreamDestroy(ctx->side.side);
     free_all(ctx->dt.allocs);
     free_all(ctx->split_allocs);
     delete ctx;
@@ -1381,7 +1585,10 @@ bc_status bc_tree_boxes(const bc_tree *tree, int32_t *level, int32_t *ix, int32_
 void bc_tree_destroy(bc_tree *tree)
 {
     if (!tree) return;
-    if (tree->ctx->device >= 0) cudaSetDevice(tree->ctx->device);
+    if (tree->ctx->device >= 0) {
+        cudaSetDevice(tree->ctx->device);
+        free_side(tree);
+    }
     free_all(tree->d.allocs);
     delete tree;
 }
@@ -1536,6 +1743,7 @@ void bc_batch_destroy(bc_batch *b)
             if (gr.exec) cudaGraphExecDestroy(gr.exec);
     if (b->cap) cudaStreamDestroy(b->cap);
     if (b->u) {
+        free_side(b->u);
         free_all(b->u->d.allocs);
         delete b->u;
     }
@@ -1700,7 +1908,7 @@ bc_status bc_set_option(bc_ctx *ctx, const char *name, double value)
     }
     if (std::strcmp(name, "wait_limit") == 0) {
         if (!(value >= 1.0 && value <= 1e15)) { set_error("bc_set_option: wait_limit must be in [1, 1e15]"); return BC_ERR_ARG; }
-        ctx->split.wait_limit = (long long)value;
+        ctx->split.wait_limit = ctx->wide.wait_limit = (long long)value;
         return BC_OK;
     }
     if (std::strcmp(name, "split_overlap") == 0) {

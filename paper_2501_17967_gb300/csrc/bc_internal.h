@@ -209,19 +209,29 @@ struct DevTree {
 // An operator is a real matrix of `rows` <= 256 rows; its BF16 digits are
 // stored as chunks [digit a][row half h][K chunk kc] of 128 rows x KC
 // columns (KC = min(K, kSplitKC)) in the canonical K-major core-matrix layout.
-constexpr int kSplitSlices = 5;
+constexpr int kSplitSlices = 5;              // split modes: 5 digits (40 bits), 5 levels, 48 columns per tile
 constexpr int kSplitTileN = 48;
+constexpr int kWideSlices = 7;               // FP64 mode: 7 digits (56 bits), 8 levels, 32 columns per tile
+constexpr int kWideLevels = 8;
+constexpr int kWideTileN = 32;
+constexpr int kWideExp = 0x40000000;         // exponent of a vector without digits (an infinity or a NaN in it)
 constexpr int kSplitKE = 64;                 // K of group E (expansion reals, padded)
 constexpr int kSplitKC = 128;                // K columns per operator chunk (one bulk copy)
 struct SplitOp {
     int64_t a_off = 0;     // byte offset of the operator's first chunk
     int32_t rows = 0;      // valid rows
     int32_t exp_off = 0;   // index of the operator's first row exponent
+    int64_t f_off = 0;     // 7 digits: index of its FP64 entries [k][row]
 };
 struct SplitTables {
+    int slices = kSplitSlices, tileN = kSplitTileN;   // digit format
+
     // [group V, group E][forward, adjoint]
     const uint8_t *ops[2][2] = {};
     const int32_t *op_exp[2][2] = {};
+    // 7 digits: the operators in FP64 (with the column scales divided out), for
+    // vectors that have no digits
+    const double *opf[2][2] = {};
     std::vector<SplitOp> near_op[2], x_op[2], w_op[2];   // [dir][code]
     std::vector<SplitOp> m2l_op[2];                       // [dir][V code] (group E, 2 P1 rows)
     SplitOp leafA_op[2], e_op[2];
@@ -230,15 +240,20 @@ struct SplitTables {
     // taken and column k of the operator is divided by s_k (exact rescaling
     // that balances the fixed-point rounding of operator and input).
     const double *escale[2] = {nullptr, nullptr};
+    // 7 digits: group V column scales (powers of two near the quadrature
+    // weights of the nodes) in the forward direction, whose operators carry
+    // the weights in their columns; null: 1
+    const double *vscale[2] = {nullptr, nullptr};
     // group V's inner dimension: the p^2 leaf nodes, zero-padded to one of
-    // the tensor kernel's K (64 for p = 8, 256 for p = 12 and 16)
+    // the tensor kernel's K (5 digits: 64 for p = 8, 256 for p = 12 and 16;
+    // 7 digits: 64 for p <= 8, 144 for p <= 12, else 256)
     int np = 256, kv = 256;
     long long wait_limit = 1ll << 26;            // polls of a bounded mbarrier wait
     int withhold_copy = 0;                       // diagnostics: never start the operator copies (forces a timeout)
 };
-// One tile = one operator times up to kSplitTileN columns.
+// One tile = one operator times up to tileN columns.
 struct SplitTile {
-    int64_t a_off;
+    int64_t a_off, f_off;
     int32_t rows, exp_off;
     int32_t p0, cnt;       // columns [p0, p0 + cnt)
 };
@@ -257,6 +272,12 @@ struct SplitGemm {
     const uint16_t *dig = nullptr;     // [nvec][5][K] BF16 digit bits
     const int32_t *dexp = nullptr;     // [nvec]
     int max_ctas = 0;                  // CTAs of the launch at most (0: one per SM)
+    // 7 digits: the vectors in FP64 (vec < nsplit: src0 + vec kvalid, scales
+    // cs0; else src1, cs1) and the operators, for vectors without digits
+    const double *opf = nullptr, *src0 = nullptr, *src1 = nullptr, *cs0 = nullptr, *cs1 = nullptr;
+    int64_t nsplit = INT64_MAX;
+    double scale = 1.0;
+    int kvalid = 0;
 };
 struct SplitTree {
     // [forward, adjoint]; group V as far part (leafA, X list: needed by the
@@ -269,17 +290,16 @@ struct SplitTree {
     int ntV[2] = {}, ntN[2] = {}, ntVN[2] = {}, ntE[2] = {}, ntM[2] = {};
     int ntA[2] = {};   // the first ntA tiles of tV: leaf-to-expansion (the rest: X list)
     int ntL[2] = {};   // the first ntL tiles of tE: expansion-to-leaf (the rest: W list)
-    double *Pnear = nullptr;      // [n_near][256] near-field result per entry (scale included)
+    double *Pnear = nullptr;      // [n_near][p^2] near-field result per entry (scale included)
     double *PX = nullptr;         // [n_x][64] X-list result per entry
-    double *PE = nullptr;         // [nleaf][256] L2P (adjoint P2M^H) result per leaf
-    double *PW = nullptr;         // [n_w][256] W-list result per entry
-    uint16_t *vdig = nullptr;     // [nleaf][5][256] digits of the leaf vectors
+    double *PE = nullptr;         // [nleaf][p^2] L2P (adjoint P2M^H) result per leaf
+    double *PW = nullptr;         // [n_w][p^2] W-list result per entry
+    uint16_t *vdig = nullptr;     // [nleaf][slices][kv] digits of the leaf vectors
     int32_t *vexp = nullptr;      // [nleaf]
-    uint16_t *edig = nullptr;     // [2 nbox][5][64] digits of expA (first nbox) and expB
+    uint16_t *edig = nullptr;     // [2 nbox][slices][64] digits of expA (first nbox) and expB
     int32_t *eexp = nullptr;      // [2 nbox]
     int32_t *err = nullptr;       // device error flag (bounded waits)
 };
-size_t split_smem_bytes(int kd);
 cudaError_t split_prepare();   // kernel attributes of the split path (before any capture)
 int split_sm_count();          // SMs of the device (after split_prepare)
 // parts: which products take the tensor-core results (bits: 1 near field,
@@ -294,6 +314,7 @@ int split_sm_count();          // SMs of the device (after split_prepare)
 // shifts, the log terms and the sums stay FP64), BC_SPLIT_BF16_ALL every part.
 constexpr int kSplitAllParts = 127;
 constexpr int kSplitTableParts = 31;
+constexpr int kWideParts = 63;   // FP64 mode: every product but the shifts, on 7 digits
 inline bool is_split(int prec) { return prec == BC_SPLIT_BF16 || prec == BC_SPLIT_BF16_ALL; }
 // parts of a split apply: the mode's set, or the diagnostic override (>= 0)
 inline int split_parts_for(int prec, int override_parts)
@@ -308,19 +329,25 @@ struct SplitLaunch {
     int near_ctas = 0;                          // CTAs of the near-field launch on the side stream (0: all SMs)
 };
 // Digits of the leaf vectors (times scale), of the two expansion arrays
-// (times scale), and the tensor-core operator products of one group.
-// (np nodes per leaf, digits zero-padded to kv per slice)
-cudaError_t launch_split_digits_vec(int64_t nleaf, const double *v, double scale, uint16_t *dig, int32_t *dexp,
-                                    cudaStream_t st, const uint8_t *active, int np, int kv);
+// (times scale), and the tensor-core operator products of one group, in the
+// tables' digit format.  (np nodes per leaf, digits zero-padded to kv per slice)
+cudaError_t launch_split_digits_vec(const SplitTables &T, int dir, int64_t nleaf, const double *v, double scale,
+                                    uint16_t *dig, int32_t *dexp, cudaStream_t st, const uint8_t *active);
 // Expansion digits of vectors [i0, i1) of the pair (expA: 0..nbox-1, expB:
 // nbox..2 nbox-1).
-cudaError_t launch_split_digits_exp(int64_t i0, int64_t i1, int64_t nbox, const double2 *ea, const double2 *eb,
-                                    int P1, double scale, const double *escale, uint16_t *dig, int32_t *dexp,
-                                    cudaStream_t st);
-// intcvt: the epilogue converts its integer sums to FP64 with integer
+cudaError_t launch_split_digits_exp(const SplitTables &T, int dir, int64_t i0, int64_t i1, int64_t nbox,
+                                    const double2 *ea, const double2 *eb, int P1, double scale, uint16_t *dig,
+                                    int32_t *dexp, cudaStream_t st);
+// intcvt (5 digits): the epilogue converts its integer sums to FP64 with integer
 // operations only (same bits), for launches that run beside FP64 kernels.
-cudaError_t launch_split_gemm(const SplitGemm &g, int kd, double inv_alpha0, int32_t *err, long long wait_limit,
-                              int withhold, cudaStream_t st, bool intcvt = false);
+cudaError_t launch_split_gemm(const SplitTables &T, const SplitGemm &g, int kd, double inv_alpha0, int32_t *err,
+                              cudaStream_t st, bool intcvt = false);
+// The launch descriptions of the two groups: tiles [t0, t0 + n) of the list
+// (tiles, cols), input vin / the expansions.
+SplitGemm gemm_group_v(const SplitTables &T, const SplitTree &s, int dir, const SplitTile *tiles, const SplitCol *cols,
+                       int n, const double *vin, double scale);
+SplitGemm gemm_group_e(const SplitTables &T, const SplitTree &s, int dir, const SplitTile *tiles, const SplitCol *cols,
+                       int n, const double2 *ea, const double2 *eb, int64_t nbox, int P1, double scale);
 
 // Launch parameters common to the passes.  leaf_bps / m2l_bps: resident
 // blocks per SM used to size the grids of the leaf kernels and of the M2L
@@ -368,6 +395,8 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
                          cudaEvent_t *ev, int m2l_tri, const struct SplitLaunch *split);
 // Fork/join resources of the split path: the near-field tensor launch runs on
 // `side` between the events.
+// (one set per tree: calls on one tree are serialised by the caller, calls on
+// different trees are not).
 struct SideStream {
     cudaStream_t side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -417,8 +446,11 @@ cudaError_t launch_layer(const PassArgs &a, const HostTree &h, const DevTree &d,
 // layer launch on a device) and a check launch (x, lg, inv device arrays).
 cudaError_t layer_log_init();
 cudaError_t launch_log_inv_check(const double *x, int64_t n, double *lg, double *inv, cudaStream_t st);
-// The split path's tiles of a tree (built on first use; api.cpp).
+// The tiles of a tree in one digit format (built on first use; api.cpp).
 bc_status prepare_split_tree(struct bc_tree *t);
+// The same for the 7-digit products of the FP64 mode; false: not available
+// (the caller takes the FP64 kernels).
+bool prepare_wide_tree(struct bc_tree *t);
 // Strip solve (kernels_strip.cu): nsys block-cyclic-tridiagonal systems,
 // one warp each; workspace strip_work_doubles(N, m, r) per system.
 size_t strip_work_doubles(int64_t N, int m, int r);
@@ -473,12 +505,11 @@ struct bc_ctx {
     int m2l_kind = 0;           // FP64 M2L kernel: 0 FMA, 1 tensor-core MMA (see PassArgs)
     bool timing = false;        // record CUDA events around each stage
     cudaEvent_t ev[2][bc::kNumEvents] = {};   // [forward, adjoint]
-    bc::SideStream side;
     bc::HostTables ht;
     bc::DevTables dt;
-    bc::SplitTables split;
+    bc::SplitTables split, wide;   // 5-digit (split modes) and 7-digit (FP64 mode) operators
     std::vector<void *> split_allocs;
-    bool split_ready = false;
+    bool split_ready = false, wide_ready = false;
     int32_t *dev_err = nullptr;   // device flag set by kernels whose bounded waits gave up
     int up_blocks = 0, shift_blocks = 0, down_blocks = 0;   // grids of the persistent passes
     // launch shapes chosen by the autotuner: key = precision*1024 + adjoint*512 + log2(nleaf)
@@ -491,7 +522,9 @@ struct bc_tree {
     bool is_union = false;   // the union tree of a batch
     bc::HostTree h;
     bc::DevTree d;
-    bc::SplitTree sp;
-    bool split_ready = false;
+    bc::SplitTree sp, spw;    // tiles of the 5-digit and the 7-digit products
+    bc::SideStream side;
+    bool split_ready = false, wide_ready = false;
     bool m2l_ready = false;   // tensor-core M2L tiles and rows (BC_SPLIT_BF16_ALL)
+    bool wide_off = false;    // the 7-digit set-up did not fit: FP64 kernels
 };

@@ -668,6 +668,52 @@ inline int m2l_groups(int P1)
 inline int m2l_threads(int P1) { return (m2l_groups(P1) * P1 + 31) / 32 * 32; }
 
 // -------------------------------------------------------------------------
+// v_sums: each box's V-list sum from the tensor-core M2L's rows (which leave
+// out the log term), one warp per box, lane o = coefficient o:
+//   out[b][o] = sum_{e in V(b)} [ Pv[e][o] + (o = 0) (log|d_e| + log r_b) first[s_e][0] ]
+// Apart from the downward pass, whose chain of boxes would wait for the ~27
+// dependent row loads of each.  Memory bound: 16 P1 bytes per pair.
+// -------------------------------------------------------------------------
+__global__ void __launch_bounds__(256)
+k_v_sums(int64_t b0, int64_t b1, const int32_t *__restrict__ v_ptr, const int32_t *__restrict__ v_src,
+         const int32_t *__restrict__ v_code, const int32_t *__restrict__ box_level, const double *__restrict__ logd,
+         const double *__restrict__ lvtab, const double2 *__restrict__ Pv, const double2 *__restrict__ first,
+         double2 *__restrict__ out, int P1)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    const int lane = threadIdx.x & 31, o = lane;   // P1 <= 32
+    const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t b = b0 + blockIdx.x * int64_t(blockDim.x >> 5) + (threadIdx.x >> 5); b < b1; b += nw) {
+        const int v0 = v_ptr[b], v1 = v_ptr[b + 1];
+        double lr = 0.0, li = 0.0, re = 0.0, im = 0.0;
+        for (int e = v0 + lane; e < v1; e += 32) {
+            const double2 a0 = first[int64_t(v_src[e]) * P1];
+            const double c0 = logd[v_code[e]] + lvtab[kLvTab + box_level[b]];
+            lr = fma(c0, a0.x, lr);
+            li = fma(c0, a0.y, li);
+        }
+        if (o < P1) {
+#pragma unroll 8
+            for (int e = v0; e < v1; e++) {
+                const double2 t = Pv[int64_t(e) * P1 + o];
+                re += t.x;
+                im += t.y;
+            }
+        }
+        for (int m = 16; m > 0; m >>= 1) {
+            lr += __shfl_xor_sync(0xffffffffu, lr, m);
+            li += __shfl_xor_sync(0xffffffffu, li, m);
+        }
+        if (o == 0) {
+            re += lr;
+            im += li;
+        }
+        if (o < P1) out[b * P1 + o] = make_double2(re, im);
+    }
+}
+
+// -------------------------------------------------------------------------
 // x_entries (FP64 path): the X-list products, one block per entry e (target
 // box b, source leaf c at level lv_b - 1):
 //   PX[e][l] = s1 * sum_j OpX[code][j][l] x[c][j]
@@ -1457,11 +1503,20 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
     cudaError_t ce;
     if (ev) cudaEventRecord(ev[0], st);
     const SideStream *sd = split ? split->side : nullptr;
-    SplitGemm gv;   // tensor group V
-    if (split) {
-        gv.ops = sT->ops[0][dir]; gv.op_exp = sT->op_exp[0][dir];
-        gv.dig = sp->vdig; gv.dexp = sp->vexp;
-    }
+    // tensor group V (leaf vectors) and group E (expansions): tiles [t0, t0 + n)
+    auto group_v = [&](const SplitTile *t, const SplitCol *c, int n) {
+        return gemm_group_v(*sT, *sp, dir, t, c, n, vin, alpha0);
+    };
+    const double escl = adj ? alpha0 : 1.0;
+    auto group_e = [&](const SplitTile *t, const SplitCol *c, int n) {
+        return gemm_group_e(*sT, *sp, dir, t, c, n, d.expA, d.expB, a.nbox, P1, escl);
+    };
+    auto digits_vec = [&](cudaStream_t s) {
+        return launch_split_digits_vec(*sT, dir, a.nleaf, vin, alpha0, sp->vdig, sp->vexp, s, d.leaf_active);
+    };
+    auto digits_exp = [&](int64_t i0, int64_t i1, cudaStream_t s) {
+        return launch_split_digits_exp(*sT, dir, i0, i1, a.nbox, d.expA, d.expB, P1, escl, sp->edig, sp->eexp, s);
+    };
     const bool leaf_tc = (parts & 2) != 0;
     // Late fork: with the M2L in FP64 (part 32 off) the internal stream's
     // tensor launches (X list, near field) start after the upward pass and run
@@ -1479,13 +1534,11 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             return e;
         if (ev) cudaEventRecord(ev[8], sd->side);
         if (!leaf_tc) {
-            e = launch_split_digits_vec(a.nleaf, vin, alpha0, sp->vdig, sp->vexp, sd->side, d.leaf_active,
-                                            a.NP, sT->kv);
+            e = digits_vec(sd->side);
             if (e != cudaSuccess) return e;
         }
-        SplitGemm g = gv;
-        g.tiles = sp->tV[dir] + sp->ntA[dir]; g.cols = sp->cV[dir]; g.ntiles = sp->ntV[dir] - sp->ntA[dir];
-        e = launch_split_gemm(g, sT->kv, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, sd->side, late);
+        SplitGemm g = group_v(sp->tV[dir] + sp->ntA[dir], sp->cV[dir], sp->ntV[dir] - sp->ntA[dir]);
+        e = launch_split_gemm(*sT, g, sT->kv, 1.0 / alpha0, sp->err, sd->side, late);
         if (e != cudaSuccess) return e;
         if ((e = cudaEventRecord(sd->xdone, sd->side)) != cudaSuccess) return e;
         if (late) {
@@ -1493,20 +1546,15 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             // tiles here too, beside the FP64 M2L (the downward pass's group E
             // keeps the expansion-to-leaf tiles)
             const int64_t f0 = adj ? a.nbox : 0;
-            e = launch_split_digits_exp(f0, f0 + a.nbox, a.nbox, d.expA, d.expB, P1, adj ? alpha0 : 1.0,
-                                        sT->escale[dir], sp->edig, sp->eexp, sd->side);
+            e = digits_exp(f0, f0 + a.nbox, sd->side);
             if (e != cudaSuccess) return e;
-            SplitGemm gw;
-            gw.tiles = sp->tE[dir] + sp->ntL[dir]; gw.cols = sp->cE[dir]; gw.ntiles = sp->ntE[dir] - sp->ntL[dir];
-            gw.ops = sT->ops[1][dir]; gw.op_exp = sT->op_exp[1][dir];
-            gw.dig = sp->edig; gw.dexp = sp->eexp;
-            e = launch_split_gemm(gw, kSplitKE, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, sd->side,
-                                  true);
+            e = launch_split_gemm(*sT, group_e(sp->tE[dir] + sp->ntL[dir], sp->cE[dir], sp->ntE[dir] - sp->ntL[dir]),
+                                  kSplitKE, 1.0 / alpha0, sp->err, sd->side, true);
             if (e != cudaSuccess) return e;
         }
-        g.tiles = sp->tN[dir]; g.cols = sp->cN[dir]; g.ntiles = sp->ntN[dir];
+        g = group_v(sp->tN[dir], sp->cN[dir], sp->ntN[dir]);
         g.max_ctas = split->near_ctas;
-        e = launch_split_gemm(g, sT->kv, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, sd->side, late);
+        e = launch_split_gemm(*sT, g, sT->kv, 1.0 / alpha0, sp->err, sd->side, late);
         if (e != cudaSuccess) return e;
         if (ev) cudaEventRecord(ev[9], sd->side);
         return cudaEventRecord(sd->join, sd->side);
@@ -1519,12 +1567,10 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
         if (!sd) {
             // one launch: the near-field tiles (two jobs each) first, then the
             // leaf-to-expansion and X-list tiles
-            ce = launch_split_digits_vec(a.nleaf, vin, alpha0, sp->vdig, sp->vexp, st, d.leaf_active, a.NP,
-                                             sT->kv);
+            ce = digits_vec(st);
             if (ce != cudaSuccess) return ce;
-            SplitGemm g = gv;
-            g.tiles = sp->tVN[dir]; g.cols = sp->cVN[dir]; g.ntiles = sp->ntVN[dir];
-            ce = launch_split_gemm(g, sT->kv, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, st);
+            ce = launch_split_gemm(*sT, group_v(sp->tVN[dir], sp->cVN[dir], sp->ntVN[dir]), sT->kv, 1.0 / alpha0,
+                                   sp->err, st);
             if (ce != cudaSuccess) return ce;
             if (ev) {
                 cudaEventRecord(ev[8], st);
@@ -1536,15 +1582,13 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             // double-float inside the upward pass, and then the digits run on
             // the internal stream too.
             if (leaf_tc) {
-                ce = launch_split_digits_vec(a.nleaf, vin, alpha0, sp->vdig, sp->vexp, st, d.leaf_active, a.NP,
-                                             sT->kv);
+                ce = digits_vec(st);
                 if (ce != cudaSuccess) return ce;
             }
             if (!late && (ce = side_launches()) != cudaSuccess) return ce;
             if (leaf_tc) {
-                SplitGemm g = gv;
-                g.tiles = sp->tV[dir]; g.cols = sp->cV[dir]; g.ntiles = sp->ntA[dir];
-                ce = launch_split_gemm(g, sT->kv, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, st);
+                ce = launch_split_gemm(*sT, group_v(sp->tV[dir], sp->cV[dir], sp->ntA[dir]), sT->kv, 1.0 / alpha0,
+                                       sp->err, st);
                 if (ce != cudaSuccess) return ce;
             }
         }
@@ -1585,6 +1629,7 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
     if (late && (ce = side_launches()) != cudaSuccess) return ce;
     if (ev) cudaEventRecord(ev[3], st);
     bool first_digits = false;   // digits of `first` taken (tensor-core M2L)
+    bool summed = false;         // its rows already summed per box
     if (far && h.nlevels > 2) {
         // M2L: per V pair on the tensor cores (part 32; results one row per
         // pair, summed by the downward pass), else every box's V-list sum in
@@ -1595,16 +1640,20 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             // tensor group M: digits of `first` (times alpha0 in the adjoint),
             // then every pair's translation but its log term
             const int64_t f0 = adj ? a.nbox : 0;
-            ce = launch_split_digits_exp(f0, f0 + a.nbox, a.nbox, d.expA, d.expB, P1, adj ? alpha0 : 1.0,
-                                         sT->escale[dir], sp->edig, sp->eexp, st);
+            ce = digits_exp(f0, f0 + a.nbox, st);
             if (ce != cudaSuccess) return ce;
             first_digits = true;
-            SplitGemm g;
-            g.tiles = sp->tM[dir]; g.cols = sp->cM[dir]; g.ntiles = sp->ntM[dir];
-            g.ops = sT->ops[1][dir]; g.op_exp = sT->op_exp[1][dir];
-            g.dig = sp->edig; g.dexp = sp->eexp;
-            ce = launch_split_gemm(g, kSplitKE, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, st);
+            ce = launch_split_gemm(*sT, group_e(sp->tM[dir], sp->cM[dir], sp->ntM[dir]), kSplitKE, 1.0 / alpha0,
+                                   sp->err, st);
             if (ce != cudaSuccess) return ce;
+            if (!dfp) {
+                // the FP64 downward pass takes each box's V-list sum, as the FP64 M2L writes it
+                ce = launch_pdl(k_v_sums, grid_for((a.nbox - h.level_start[2] + 7) / 8, 152 * 8), 256, 0, st,
+                                h.level_start[2], a.nbox, d.v_ptr, d.v_src, d.v_code, d.box_level, tb.logd, d.lvtab,
+                                d.Pv, first, second, P1);
+                if (ce != cudaSuccess) return ce;
+                summed = true;
+            }
         } else if (a.m2l_kind == 1) {
             // FP64 tensor cores, one warp per target box; beside the
             // near-field tensor CTAs (late fork) two warps per SM
@@ -1677,8 +1726,8 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             ce = launch_pdl(k_down_warps, a.down_blocks, 128, down_warps_smem_bytes(P1, op.par_f.T, op.par_f.maxp, 4),
                             st, d.level_start, h.nlevels, d.v_ptr, d.Pv, d.x_ptr, d.x_src, PX, px_stride,
                             d.leaf_box, first, d.box_parent, d.box_ix, d.box_iy, op.par_f, second, P1, d.lvtab,
-                            first_digits ? d.v_src : nullptr, d.v_code, tb.logd, !first_digits, d.flag, glimit,
-                            a.err);
+                            first_digits && !summed ? d.v_src : nullptr, d.v_code, tb.logd, !first_digits || summed,
+                            d.flag, glimit, a.err);
         if (ce != cudaSuccess) return ce;
     } else if (ev) {
         cudaEventRecord(ev[4], st);
@@ -1691,14 +1740,10 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
         // the W list of `first` into PW (late fork: L2P only)
         const bool first_done = first_digits || late;
         const int64_t s0 = first_done ? (adj ? 0 : a.nbox) : 0, s1 = first_done ? s0 + a.nbox : 2 * a.nbox;
-        ce = launch_split_digits_exp(s0, s1, a.nbox, d.expA, d.expB, P1, adj ? alpha0 : 1.0, sT->escale[dir],
-                                     sp->edig, sp->eexp, st);
+        ce = digits_exp(s0, s1, st);
         if (ce != cudaSuccess) return ce;
-        SplitGemm g;
-        g.tiles = sp->tE[dir]; g.cols = sp->cE[dir]; g.ntiles = late ? sp->ntL[dir] : sp->ntE[dir];
-        g.ops = sT->ops[1][dir]; g.op_exp = sT->op_exp[1][dir];
-        g.dig = sp->edig; g.dexp = sp->eexp;
-        ce = launch_split_gemm(g, kSplitKE, 1.0 / alpha0, sp->err, sT->wait_limit, sT->withhold_copy, st);
+        ce = launch_split_gemm(*sT, group_e(sp->tE[dir], sp->cE[dir], late ? sp->ntL[dir] : sp->ntE[dir]), kSplitKE,
+                               1.0 / alpha0, sp->err, st);
         if (ce != cudaSuccess) return ce;
     }
     // the log-term sums of every leaf's W and near lists (they read `first`

@@ -395,15 +395,11 @@ cudaError_t launch_layer(const PassArgs &a, const HostTree &h, const DevTree &d,
         const SplitTables *sT = split->tables;
         const SplitTree *sp = split->tree;
         const int64_t nbox = a.nbox;
-        e = launch_split_digits_exp(nbox, 2 * nbox, nbox, d.expA, d.expB, P1, 1.0, sT->escale[0], sp->edig,
-                                    sp->eexp, st);
+        e = launch_split_digits_exp(*sT, 0, nbox, 2 * nbox, nbox, d.expA, d.expB, P1, 1.0, sp->edig, sp->eexp, st);
         if (e != cudaSuccess) return e;
-        SplitGemm g;
-        g.tiles = sp->tE[0]; g.cols = sp->cE[0]; g.ntiles = sp->ntL[0];
-        g.ops = sT->ops[1][0]; g.op_exp = sT->op_exp[1][0];
-        g.dig = sp->edig; g.dexp = sp->eexp;
-        e = launch_split_gemm(g, kSplitKE, 1.0 / (a.half_L * a.half_L), sp->err, sT->wait_limit, sT->withhold_copy,
-                              st);
+        e = launch_split_gemm(*sT, gemm_group_e(*sT, *sp, 0, sp->tE[0], sp->cE[0], sp->ntL[0], d.expA, d.expB, nbox, P1,
+                                                1.0),
+                              kSplitKE, 1.0 / (a.half_L * a.half_L), sp->err, st);
         if (e != cudaSuccess) return e;
         PE = sp->PE;
     }

@@ -1,12 +1,12 @@
-// Split-precision operator products on the 5th-generation tensor cores
-// (tcgen05), p = 16.
+// Operator products on the 5th-generation tensor cores (tcgen05) as exact
+// products of BF16 digits.
 //
-// The fixed-operator products of a split-precision apply -- the near-field
-// tables, P2M, L2P, the W list (M2P) and the X list (P2L), their adjoints,
-// and in BC_SPLIT_BF16_ALL also the multipole-to-local translations -- are
-// dense real matrices (the operators) times many vectors (leaf values or
-// expansion coefficients).  Each product is evaluated exactly in integer
-// arithmetic on BF16 tensor cores:
+// The fixed-operator products of an apply -- the near-field tables, P2M, L2P,
+// the W list (M2P) and the X list (P2L), their adjoints, and the multipole-to-
+// local translations -- are dense real matrices (the operators) times many
+// vectors (leaf values or expansion coefficients).  Each product is evaluated
+// in integer arithmetic on BF16 tensor cores, with five digits per operand in
+// the split modes (described first) or seven in the FP64 mode (see Fmt):
 //   * each FP64 operand row (operator row, input vector) is scaled by a power
 //     of two 2^E so that its entries lie in (-1/2, 1/2), rounded to a 40-bit
 //     fixed-point integer X and cut into five balanced base-256 digits,
@@ -22,8 +22,8 @@
 //     hardware conversion; the power-of-two scale is then added to the
 //     exponent field of the bit pattern).
 //
-// Work decomposition: a tile is one operator times up to 48 columns, done as
-// one job per 128-row half of the operator.
+// Work decomposition: a tile is one operator times up to 48 (32) columns, done
+// as one job per 128-row half of the operator.
 //   B operand: the columns' digits, gathered into shared memory slice by slice
 //              with 16-byte asynchronous copies (cp.async), resident for the
 //              tile; the next tile's slices are gathered as the current tile's
@@ -35,8 +35,8 @@
 //              order 0, 4, 1, 3, 2 (long and short chunks alternate, so copies
 //              keep up), its last job in the order 0..4 (B slices are freed
 //              earliest);
-//   D:         5 levels x 48 columns of FP32 per job, two TMEM buffers, so one
-//              job's epilogue overlaps the next job's MMAs.
+//   D:         5 levels x 48 (8 x 32) columns of FP32 per job, two TMEM
+//              buffers, so one job's epilogue overlaps the next job's MMAs.
 // One tcgen05.mma of 128 x 48 x 16 takes about as long as one of 128 x 16 x 16
 // (a fixed cost per instruction), which the MMA warp now reaches.  All waits
 // are bounded: a wait that runs out sets the error flag, every role stops at
@@ -55,9 +55,25 @@ namespace bc {
 
 namespace {
 
-constexpr int kS = kSplitSlices;   // 5 digits
-constexpr int kN = kSplitTileN;    // 48 columns per tile
-constexpr int kNBuf = 3;           // operator chunk buffers (32 KB each)
+constexpr int kNBuf = 3;           // operator chunk buffers (32 KB each at K = 256)
+
+// The two digit formats.  S digits per operand, L levels kept (digit pairs
+// a + b <= L + 1, counted from 1), tiles of N columns: L N <= 256, half of
+// the TMEM columns, so that a job's epilogue overlaps the next job's MMAs.
+//   5 digits (split modes): 40 bits, levels 2..6, 15 products.
+//   7 digits (FP64 mode): 56 bits, levels 2..9, 34 products.  What is dropped
+//   (levels >= 10) is below 2^-62 sqrt(K) of max|A'| max|x'|, what is rounded
+//   (the operands to 56 bits) 2^-57 sqrt(K) of it: about a tenth of the
+//   rounding of a chain of K FP64 additions (2^-53 of the running sums), so
+//   the products are no less accurate than the FP64 kernels they stand for.
+//   A level sums up to seven pairs; that each |D_g| <= 128 sum_a sum_k
+//   |theta_a(k)| stays <= 2^24 is checked row by row when the operator's
+//   digits are made (the row's digits used once per level each).
+template <int S> struct Fmt;
+template <> struct Fmt<kSplitSlices> { static constexpr int L = 5, N = kSplitTileN; };
+template <> struct Fmt<kWideSlices> { static constexpr int L = kWideLevels, N = kWideTileN; };
+static_assert(Fmt<kSplitSlices>::L * Fmt<kSplitSlices>::N <= 256 && Fmt<kWideSlices>::L * Fmt<kWideSlices>::N <= 256,
+              "two TMEM job buffers");
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -109,7 +125,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// waits until at most n (0..4) of this thread's cp.async groups are pending
+// waits until at most n (0..6) of this thread's cp.async groups are pending
 __device__ __forceinline__ void cp_async_wait_pending(int n)
 {
     switch (n) {
@@ -117,7 +133,9 @@ __device__ __forceinline__ void cp_async_wait_pending(int n)
     case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
     case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
     case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-    default: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
     }
 }
 
@@ -188,6 +206,26 @@ __device__ __forceinline__ void umma_kchain_warp<4>(uint32_t dtmem, uint64_t ade
         : "memory");
 }
 
+template <>
+__device__ __forceinline__ void umma_kchain_warp<1>(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                    uint32_t first)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;}"
+        ::"r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(first)
+        : "memory");
+}
+template <>
+__device__ __forceinline__ void umma_kchain_warp<9>(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                    uint32_t first)
+{
+    umma_kchain_warp<8>(dtmem, adesc, bdesc, idesc, first);
+    umma_kchain_warp<1>(dtmem, adesc + 8 * 16, bdesc + 8 * 16, idesc, 1u);
+}
+
 __device__ __forceinline__ void umma_commit_warp(uint64_t *bar)
 {
     asm volatile(
@@ -196,6 +234,13 @@ __device__ __forceinline__ void umma_commit_warp(uint64_t *bar)
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
             smem_u32(bar))
         : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
@@ -288,21 +333,43 @@ __device__ __forceinline__ double i64_scaled_int(long long S, int ex)
         static_cast<long long>((sgn | (static_cast<unsigned long long>(e - 1) << 52)) + mant + up));
 }
 
-// Five balanced base-256 digits (BF16 bit patterns) of round(x * 2^(40 - E)),
+// The eight levels of the 7-digit format: sum_g D_g 256^(7-g) (g = 0..7,
+// |D_g| <= 2^24) times 2^ex.  Levels 0-3 and 4-7 are each exact in int64 (and
+// in FP64: below 2^50), so one FMA gives the sum with a single rounding.
+// Results outside the normal range take the general scaling.
+__device__ __noinline__ double scale_wide(double v, int ex) { return scalbn(v, ex); }
+__device__ __forceinline__ double levels_scaled(const int (&D)[kWideLevels], int ex)
+{
+    const long long hi = (long long)D[3] + (long long)D[2] * 256 + (long long)D[1] * 65536 + (long long)D[0] * 16777216;
+    const long long lo = (long long)D[7] + (long long)D[6] * 256 + (long long)D[5] * 65536 + (long long)D[4] * 16777216;
+    const double v = fma(__ll2double_rn(hi), 4294967296.0, __ll2double_rn(lo));
+    const long long b = __double_as_longlong(v);
+    const int e = int((b >> 52) & 0x7FF), es = e + ex;
+    if (e == 0) return 0.0;   // v is zero (a nonzero sum is at least 1)
+    if (es <= 0 || es >= 0x7FF) return scale_wide(v, ex);
+    return __longlong_as_double(b + ((long long)ex << 52));
+}
+
+// S balanced base-256 digits (BF16 bit patterns) of round(x * 2^(8 S - E)),
 // |x| < 2^(E-1), from the FP64 bit pattern by integer operations; written to
-// out[0], out[stride], ... (most significant first).
+// out[0], out[stride], ... (most significant first).  The 5-digit format
+// takes subnormal entries as zero (it rounds at 2^-40 of the largest); the
+// 7-digit format keeps them.
+template <int S>
 __device__ __forceinline__ void digits_of(long long bits, int E, uint16_t *out, int stride)
 {
-    const int e = int((bits >> 52) & 0x7FF);
+    int e = int((bits >> 52) & 0x7FF);
     long long X = 0;
-    if (e != 0) {
-        const long long mant = (bits & ((1ll << 52) - 1)) | (1ll << 52);
-        const int rs = -(e - 1075 + 40 - E);   // >= 14
-        X = rs >= 62 ? 0 : (mant + (1ll << (rs - 1))) >> rs;
+    if (e != 0 || S > 5) {
+        long long mant = bits & ((1ll << 52) - 1);
+        if (e != 0) mant |= 1ll << 52; else e = 1;
+        const int rs = -(e - 1075 + 8 * S - E);   // >= 54 - 8 S
+        if (S > 5 && rs <= 0) X = mant << -rs;
+        else X = rs >= 62 ? 0 : (mant + (1ll << (rs - 1))) >> rs;
         if (bits < 0) X = -X;
     }
 #pragma unroll
-    for (int a = kS; a >= 2; a--) {
+    for (int a = S; a >= 2; a--) {
         int d = int(X & 255);
         if (d >= 128) d -= 256;
         X = (X - d) >> 8;
@@ -311,32 +378,47 @@ __device__ __forceinline__ void digits_of(long long bits, int E, uint16_t *out, 
     out[0] = uint16_t(__float_as_uint(float(int(X))) >> 16);   // leading digit, |X| <= 128
 }
 
+// Magnitude key of a vector's exponent E: the biased exponent of its largest
+// entry.  7-digit format: subnormal entries count as exponent 1, and a vector
+// with an infinity or a NaN has no digits (exponent kWideExp: its products
+// are formed in FP64 by the epilogue).
+template <int S>
+__device__ __forceinline__ int exp_key(long long bits)
+{
+    const int e = int((bits >> 52) & 0x7FF);
+    return (S > 5 && e == 0 && (bits & ((1ll << 52) - 1)) != 0) ? 1 : e;
+}
+
 // ---------------------------------------------------------------------------
-// Digits of scale * (leaf vectors): dig[leaf][a][k], dexp[leaf] = E with
-// max |scale v| < 2^(E-1).  One block of kv threads (kv = 64 or 256) per
-// leaf; the np <= kv nodes of a leaf, then zero digits up to kv.
+// Digits of scale * cs_k * (leaf vectors): dig[leaf][a][k], dexp[leaf] = E with
+// max |scale cs v| < 2^(E-1).  One block of kv threads (kv rounded up to whole
+// warps) per leaf; the np <= kv nodes of a leaf, then zero digits up to kv.
+template <int S>
 __global__ void __launch_bounds__(256) k_split_vec(int64_t nleaf, const double *__restrict__ v, double scale,
-                                                   uint16_t *__restrict__ dig, int32_t *__restrict__ dexp,
-                                                   const uint8_t *__restrict__ active, int np)
+                                                   const double *__restrict__ cs, uint16_t *__restrict__ dig,
+                                                   int32_t *__restrict__ dexp, const uint8_t *__restrict__ active,
+                                                   int np, int kv)
 {
     griddep_wait();
     griddep_launch_dependents();
     __shared__ int wmax[8];
-    const int k = threadIdx.x, kv = blockDim.x;
+    const int k = threadIdx.x, nwp = blockDim.x >> 5;
+    const double sk = (S > 5 && cs && k < np) ? scale * cs[k] : scale;
     for (int64_t leaf = blockIdx.x; leaf < nleaf; leaf += gridDim.x) {
         // a discarded leaf of a truncated tree is no source: zero digits
         const double x = (k >= np || (active && !active[leaf])) ? 0.0 : v[leaf * np + k];
-        const long long bits = __double_as_longlong(scale * x);
-        int m = int((bits >> 52) & 0x7FF);
+        const long long bits = __double_as_longlong(sk * x);
+        int m = exp_key<S>(bits);
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if ((k & 31) == 0) wmax[k >> 5] = m;
         __syncthreads();
         int emax = wmax[0];
-        for (int w = 1; w < (kv >> 5); w++) emax = max(emax, wmax[w]);
+        for (int w = 1; w < nwp; w++) emax = max(emax, wmax[w]);
         __syncthreads();
+        const bool wide = S > 5 && emax == 0x7FF;
         const int E = emax ? emax - 1023 + 2 : 0;
-        digits_of(emax ? bits : 0ll, E, dig + leaf * (kS * kv) + k, kv);
-        if (k == 0) dexp[leaf] = E;
+        if (k < kv) digits_of<S>(emax && !wide ? bits : 0ll, E, dig + leaf * (S * kv) + k, kv);
+        if (k == 0) dexp[leaf] = wide ? kWideExp : E;
     }
 }
 
@@ -344,6 +426,7 @@ __global__ void __launch_bounds__(256) k_split_vec(int64_t nleaf, const double *
 // [i0, i1): vector i < nbox is ea[i] with column scales escale[0..63], else
 // eb[i - nbox] with escale[64..127]; its 2*P1 reals (re, im interleaved)
 // padded with zeros to 64.  One warp per vector: dig[i][a][64], dexp[i].
+template <int S>
 __global__ void __launch_bounds__(256) k_split_exp(int64_t i0, int64_t i1, int64_t nbox,
                                                    const double *__restrict__ ea, const double *__restrict__ eb,
                                                    int nreal, double scale, const double *__restrict__ escale,
@@ -360,62 +443,67 @@ __global__ void __launch_bounds__(256) k_split_exp(int64_t i0, int64_t i1, int64
         const double v0 = lane < nreal ? src[lane] : 0.0, v1 = lane + 32 < nreal ? src[lane + 32] : 0.0;
         const long long b0 = __double_as_longlong(scale * sc[lane] * v0);
         const long long b1 = __double_as_longlong(scale * sc[lane + 32] * v1);
-        int m = max(int((b0 >> 52) & 0x7FF), int((b1 >> 52) & 0x7FF));
+        int m = max(exp_key<S>(b0), exp_key<S>(b1));
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        const bool wide = S > 5 && m == 0x7FF;
         const int E = m ? m - 1023 + 2 : 0;
-        uint16_t *out = dig + i * (kS * kSplitKE);
-        digits_of(m ? b0 : 0ll, E, out + lane, kSplitKE);
-        digits_of(m ? b1 : 0ll, E, out + lane + 32, kSplitKE);
-        if (lane == 0) dexp[i] = E;
+        uint16_t *out = dig + i * (S * kSplitKE);
+        digits_of<S>(m && !wide ? b0 : 0ll, E, out + lane, kSplitKE);
+        digits_of<S>(m && !wide ? b1 : 0ll, E, out + lane + 32, kSplitKE);
+        if (lane == 0) dexp[i] = wide ? kWideExp : E;
     }
 }
 
 // ---------------------------------------------------------------------------
-// Operator x columns on tcgen05.  KD = 256 (leaf vectors) or 64 (expansions).
+// Operator x columns on tcgen05.  KD = 256 or 144 (leaf vectors; 64 for small
+// orders) or 64 (expansions).
 // ---------------------------------------------------------------------------
 struct ColMeta {
     double *out;
-    int32_t exp;    // E_v + shift - 48
-    int32_t flag;   // multiply by 1/alpha0
+    int32_t exp;    // E_v + shift - 8 (L + 1)
+    int32_t flag;   // 1: multiply by 1/alpha0; 2: no digits (infinity or NaN), exp = shift
     int32_t vec;
     int32_t pad;
 };
 
-// Operator digit of the p-th chunk group of a job: the order 0, 4, 1, 3, 2
-// alternates long and short MMA runs (a tile's first row-half job); 0..4 frees
+// Operator digit of the p-th chunk group of a job: the order 0, S-1, 1, S-2, ...
+// alternates long and short MMA runs (a tile's first row-half job); 0..S-1 frees
 // the B slices earliest (a tile's last job).
+template <int S>
 __device__ __forceinline__ int chunk_digit(int p, bool interleave)
 {
-    return interleave ? ((0x23140 >> (4 * p)) & 0xF) : p;
+    if (!interleave) return p;
+    return (p & 1) ? S - 1 - (p >> 1) : (p >> 1);
 }
 
-template <int KD, int NB = kNBuf>
+template <int KD, int S, int NB = kNBuf>
 struct GemmShape {
-    static constexpr int KC = KD < kSplitKC ? KD : kSplitKC;   // K columns per operator chunk
+    static constexpr int N = Fmt<S>::N, L = Fmt<S>::L;
+    static constexpr int KC = KD > 144 ? kSplitKC : KD;   // K columns per operator chunk
     static constexpr int NKC = KD / KC;
-    static constexpr int kChunksPerJob = kS * NKC;     // digit x K chunk
-    static constexpr int kBSlice = kN * KD * 2;        // bytes of one B digit slice
+    static constexpr int kChunksPerJob = S * NKC;      // digit x K chunk
+    static constexpr int kBSlice = N * KD * 2;         // bytes of one B digit slice
     static constexpr int kChunk = 128 * KC * 2;        // bytes of one operator chunk
     static constexpr int kBSBO = (KD / 8) * 128;       // B: bytes between 8-row groups
     static constexpr int kASBO = (KC / 8) * 128;       // A: bytes between 8-row groups
     // B buffers: two for K = 64 (the next tile is gathered while this one's
-    // MMAs run), one for K = 256 (120 KB)
+    // MMAs run), one for the larger K (115 to 120 KB at K = 256)
     static constexpr int kBBuf = KD <= 64 ? 2 : 1;
-    static constexpr int kBTile = kS * kBSlice;         // bytes of one tile's B
-    static constexpr size_t kSmem = size_t(kBBuf) * kBTile + size_t(NB) * kChunk + 2 * kN * sizeof(ColMeta) +
+    static constexpr int kBTile = S * kBSlice;          // bytes of one tile's B
+    static constexpr size_t kSmem = size_t(kBBuf) * kBTile + size_t(NB) * kChunk + 2 * N * sizeof(ColMeta) +
                                     64 * sizeof(uint64_t);
 };
 
 // Roles (16 warps): warp 0 issues the MMAs; warp 1 copies the operator chunks;
 // warps 2-7 stage each tile's column metadata and gather its B digits, slice by
-// slice; warps 8-15 run the epilogues (two warps per TMEM lane quarter, 24
-// columns each).
+// slice; warps 8-15 run the epilogues (two warps per TMEM lane quarter, half of
+// the columns each).
 constexpr int kGemmThreads = 512;
 constexpr int kGatherWarp0 = 2;
 constexpr int kGatherThreads = 192;
 constexpr int kEpiWarp0 = 8;
 constexpr int kEpiWarps = 8;
-constexpr int kTmemBuf = 256;        // TMEM columns per job buffer (5 levels x 48 used)
+constexpr int kTmemBuf = 256;        // TMEM columns per job buffer (5 x 48 or 8 x 32 used)
 constexpr int kNoExp = 0x7FFFFFFF;   // 1/alpha0 is not a power of two
 
 // Barriers (mbarriers in shared memory); counts in brackets:
@@ -426,35 +514,51 @@ constexpr int kNoExp = 0x7FFFFFFF;   // 1/alpha0 is not a power of two
 //   b_full[t][s] (1)   B digit slice s (and the metadata) of tile parity t is ready
 //   b_empty[u][s] (1)  no MMA of the tile last held in B buffer u reads slice s any more (commit)
 //   meta_empty[t] (8)  the epilogue warps are done with metadata buffer t
-// Digit slice s (0-based) of B is read by the chunks of operator digit a <= 4 - s,
+// Digit slice s (0-based) of B is read by the chunks of operator digit a <= L - 1 - s,
 // so in a tile's last job it is free after those chunks; the next tile's B is
-// gathered slice by slice from s = 4 down to 0 and its first chunk issues its
-// MMAs from slice 4 down, so with one B buffer only slice 0 is waited for at
-// the tile change.  Tile k uses B buffer k % kBBuf.
+// gathered slice by slice from s = S - 1 down to 0 and its first chunk issues its
+// MMAs from slice S - 1 down, so with one B buffer only the last slices are
+// waited for at the tile change.  Tile k uses B buffer k % kBBuf.
+template <int S>
 struct GemmBars {
-    uint64_t lbar[kNBuf], mbar[kNBuf], job_full[2], job_empty[2], b_full[2][kS], b_empty[2][kS], meta_empty[2];
+    uint64_t lbar[kNBuf], mbar[kNBuf], job_full[2], job_empty[2], b_full[2][S], b_empty[2][S], meta_empty[2];
     uint32_t tslot;
     int fail;
 };
+static_assert(sizeof(GemmBars<kWideSlices>) <= 64 * sizeof(uint64_t), "barrier space");
 
-// The second launch bound caps the registers at 64 per thread: 16 warps x 64
-// leave room, in each SM sub-partition's register file, for the FP64 M2L
-// blocks that run beside a near-field CTA.  Two CTAs never share an SM (shared
-// memory allows one).
-template <int KD, bool ICVT>
-__global__ void __launch_bounds__(kGemmThreads, 2)
-k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__restrict__ err, long long wait_limit,
+// Row `row` of an operator times a vector without digits (an infinity or a NaN
+// among its entries), in FP64: sum_k opf[k][row] (scale cs_k x_k).
+__device__ __noinline__ double plain_product(const SplitGemm &gm, int64_t f_off, int rows, int row, int vec)
+{
+    const bool lo = vec < gm.nsplit;
+    const double *x = lo ? gm.src0 + int64_t(vec) * gm.kvalid : gm.src1 + int64_t(vec - gm.nsplit) * gm.kvalid;
+    const double *cs = lo ? gm.cs0 : gm.cs1;
+    const double *op = gm.opf + f_off + row;
+    double s = 0.0;
+    for (int k = 0; k < gm.kvalid; k++) s = fma(op[int64_t(k) * rows], gm.scale * (cs ? cs[k] : 1.0) * x[k], s);
+    return s;
+}
+
+// 5 digits: the second launch bound caps the registers at 64 per thread: 16
+// warps x 64 leave room, in each SM sub-partition's register file, for the
+// FP64 M2L blocks that run beside a near-field CTA.  Two CTAs never share an SM
+// (shared memory allows one).
+template <int KD, int S, bool ICVT>
+__global__ void __launch_bounds__(kGemmThreads, S == kSplitSlices ? 2 : 1)
+k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__restrict__ err, long long wait_limit,
              int withhold)
 {
     // the K = 256 launches beside the FP64 M2L (ICVT) keep two operator
     // buffers: 32 KB less shared memory makes room for a fourth M2L block
     constexpr int NB = (KD == 256 && ICVT) ? 2 : kNBuf;
-    using Sh = GemmShape<KD, NB>;
+    using Sh = GemmShape<KD, S, NB>;
+    constexpr int kS = S, kN = Sh::N, kL = Sh::L;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *Bs = smem;                                                      // kBBuf x kS x kBSlice
     uint8_t *As = smem + Sh::kBBuf * Sh::kBTile;                             // NB x kChunk
     ColMeta *meta = reinterpret_cast<ColMeta *>(As + NB * Sh::kChunk);       // [2][kN]
-    GemmBars *bars = reinterpret_cast<GemmBars *>(meta + 2 * kN);
+    GemmBars<S> *bars = reinterpret_cast<GemmBars<S> *>(meta + 2 * kN);
     volatile int *fail = &bars->fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -514,10 +618,12 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
                         break;
                     }
                     tc_fence_after();
-                    const int a = chunk_digit(g / Sh::NKC, !last_job), kc = g % Sh::NKC;   // 0-based digit of A
+                    const int pos = g / Sh::NKC, kc = g % Sh::NKC;
+                    const int a = chunk_digit<S>(pos, !last_job);   // 0-based digit of A
+                    const int nb = min(kS, kL - a);                 // B digit slices 0 .. nb-1 pair with it
                     const uint64_t ad = adesc0 + uint64_t(buf) * (Sh::kChunk >> 4);
                     const uint32_t first = (a == 0 && kc == 0) ? 0u : 1u;
-                    for (int b = kS - 1 - a; b >= 0; b--) {   // B digit slices 0 .. kS-1-a present
+                    for (int b = nb - 1; b >= 0; b--) {   // present
                         if (!(ready >> b & 1u)) {
                             if (!wait_bar(&bars->b_full[k & 1][b], uint32_t((k >> 1) & 1), wait_limit, fail)) {
                                 failed = true;
@@ -528,17 +634,31 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
                         }
                     }
                     if (failed) break;
-                    // slices 0 .. kS-1-a lie one after another (a (kS-a) kN-row B
-                    // operand) and feed levels a .. kS-1, adjacent TMEM column
-                    // blocks: one MMA chain of N = (kS - a) kN per chunk
+                    // slices 0 .. nb-1 lie one after another (an nb kN-row B
+                    // operand) and feed levels a .. a+nb-1, adjacent TMEM
+                    // column blocks: one MMA chain of N = nb kN per chunk.  The
+                    // first chunk (a = 0) starts levels 0 .. S-1; where L > S the
+                    // second one starts level L-1 (its last slice, apart).
                     const uint32_t dcol = tmem + uint32_t(r * kTmemBuf + a * kN);
                     const uint64_t bd = bdesc0 + uint64_t(k % Sh::kBBuf) * (Sh::kBTile >> 4) +
                                         uint64_t(kc) * ((Sh::KC / 8) * 128 >> 4);
-                    umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, (kS - a) * kN), first);
+                    if (kL > kS && pos == 1 && kc == 0) {
+                        umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, (nb - 1) * kN), 1u);
+                        umma_kchain_warp<Sh::KC / 16>(dcol + uint32_t((nb - 1) * kN), ad,
+                                                      bd + uint64_t(nb - 1) * (Sh::kBSlice >> 4),
+                                                      umma_idesc(128, kN), 0u);
+                    } else {
+                        umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, nb * kN), first);
+                    }
                     umma_commit_warp(&bars->mbar[buf]);
                     last_commit = G;
-                    // in the tile's last job, slice kS-1-a is read by no later chunk
-                    if (last_job && kc == Sh::NKC - 1) umma_commit_warp(&bars->b_empty[k % Sh::kBBuf][kS - 1 - a]);
+                    // in the tile's last job, slice L-1-a is read by no later
+                    // chunk, and after the last digit no slice is
+                    if (last_job && kc == Sh::NKC - 1) {
+                        if (kL - 1 - a < kS) umma_commit_warp(&bars->b_empty[k % Sh::kBBuf][kL - 1 - a]);
+                        if (a == kS - 1)
+                            for (int b = 0; b < kL - kS; b++) umma_commit_warp(&bars->b_empty[k % Sh::kBBuf][b]);
+                    }
                 }
                 if (failed) break;
                 umma_commit_warp(&bars->job_full[r]);
@@ -568,7 +688,7 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
                         break;
                     }
                     if (withhold) continue;   // diagnostics: the MMA warp's first wait runs out
-                    const int a = chunk_digit(g / Sh::NKC, h < mh - 1), kc = g % Sh::NKC;
+                    const int a = chunk_digit<S>(g / Sh::NKC, h < mh - 1), kc = g % Sh::NKC;
                     const int rows_h = min(128, tl.rows - 128 * h);
                     const uint32_t bytes = uint32_t((rows_h + 7) / 8) * 8 * Sh::KC * 2;
                     const uint8_t *src = gm.ops + tl.a_off + size_t((a * mh + h) * Sh::NKC + kc) * Sh::kChunk;
@@ -616,12 +736,15 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
                 const SplitCol c = have ? ncol : gm.cols[tl.p0 + gt];
                 ColMeta m;
                 m.out = c.out;
-                m.exp = (have ? nexp : gm.dexp[c.vec]) + (c.ctl >> 1) - 48;
+                const int ev = have ? nexp : gm.dexp[c.vec];
+                const bool plain = S > 5 && ev == kWideExp;
+                m.exp = (c.ctl >> 1) + (plain ? 0 : ev - 8 * (kL + 1));
                 m.flag = c.ctl & 1;
                 if (m.flag && inv_alpha_exp != kNoExp) {   // 1/alpha0 a power of two: an exponent shift
                     m.exp += inv_alpha_exp;
                     m.flag = 0;
                 }
+                if (plain) m.flag |= 2;
                 m.vec = c.vec;
                 m.pad = 0;
                 M[gt] = m;
@@ -696,9 +819,10 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
         // ---------------- epilogues ----------------
         // warp w reads TMEM lanes 32(w%4)..32(w%4)+31.  Operators of more
         // than 64 rows: rows 32(w%4)+lane of the job's row half, warps 8-11
-        // columns 0-23, warps 12-15 columns 24-47.  Up to 64 rows (held twice):
-        // rows 32(w%2)+lane, lane quarters 0-1 columns 0-23 and 2-3 columns
-        // 24-47, split 12 + 12 between the two warps of a quarter.
+        // the first half of the columns, warps 12-15 the second.  Up to 64
+        // rows (held twice): rows 32(w%2)+lane, lane quarters 0-1 the first
+        // half of the columns and 2-3 the second, split between the two warps
+        // of a quarter.
         const int wq = warp & 3, half = (warp - kEpiWarp0) >> 2;
         int job = 0, k = 0;
         bool failed = false;
@@ -719,25 +843,43 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
                 const int row = small ? (wq & 1) * 32 + lane : h * 128 + wq * 32 + lane;
                 const bool live = row < tl.rows;
                 const int ea = live ? gm.op_exp[tl.exp_off + row] : 0;
-                const int cb = small ? (wq >> 1) * 24 + half * 12 : half * 24;
-                const int ce = min(tl.cnt, cb + (small ? 12 : 24));
-                for (int c0 = cb; c0 < ce; c0 += 8) {   // uniform over the warp
-                    uint32_t d[kS][8];
+                const int cb = small ? (wq >> 1) * (kN / 2) + half * (kN / 4) : half * (kN / 2);
+                const int ce = min(tl.cnt, cb + (small ? kN / 4 : kN / 2));
+                // columns per TMEM read: 8 levels take twice the registers of 5
+                constexpr int kQ = S > 5 ? 4 : 8;
+                for (int c0 = cb; c0 < ce; c0 += kQ) {   // uniform over the warp
+                    uint32_t d[kL][kQ];
 #pragma unroll
-                    for (int g = 0; g < kS; g++)
-                        tmem_ld8(tmem + (uint32_t(wq * 32) << 16) + uint32_t(r * kTmemBuf + g * kN + c0), d[g]);
+                    for (int g = 0; g < kL; g++) {
+                        const uint32_t ta = tmem + (uint32_t(wq * 32) << 16) + uint32_t(r * kTmemBuf + g * kN + c0);
+                        if constexpr (kQ == 4) tmem_ld4(ta, d[g]);
+                        else tmem_ld8(ta, d[g]);
+                    }
                     tmem_ld_wait();
                     if (!live) continue;
 #pragma unroll
-                    for (int q = 0; q < 8; q++) {
+                    for (int q = 0; q < kQ; q++) {
                         const int c = c0 + q;
                         if (c >= ce) continue;
-                        long long S = 0;
+                        double val;
+                        if constexpr (S > 5) {
+                            if (M[c].flag & 2) {
+                                val = scale_wide(plain_product(gm, tl.f_off, tl.rows, row, M[c].vec), M[c].exp);
+                            } else {
+                                int D[kL];
 #pragma unroll
-                        for (int g = 0; g < kS; g++)
-                            S += (long long)__float2int_rn(__uint_as_float(d[g][q])) << (8 * (kS - 1 - g));
-                        double val = ICVT ? i64_scaled_int(S, ea + M[c].exp) : i64_scaled(S, ea + M[c].exp);
-                        if (M[c].flag) val *= inv_alpha0;
+                                for (int g = 0; g < kL; g++) D[g] = __float2int_rn(__uint_as_float(d[g][q]));
+                                val = levels_scaled(D, ea + M[c].exp);
+                            }
+                            if (M[c].flag & 1) val *= inv_alpha0;
+                        } else {
+                            long long sum = 0;
+#pragma unroll
+                            for (int g = 0; g < kL; g++)
+                                sum += (long long)__float2int_rn(__uint_as_float(d[g][q])) << (8 * (kL - 1 - g));
+                            val = ICVT ? i64_scaled_int(sum, ea + M[c].exp) : i64_scaled(sum, ea + M[c].exp);
+                            if (M[c].flag) val *= inv_alpha0;
+                        }
                         M[c].out[row] = val;
                     }
                 }
@@ -758,35 +900,44 @@ k_split_gemm(SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__rest
 }
 
 int g_sms = 0;
-// The K = 64 kernel asks for more shared memory than it uses so that no two
+// The K = 64 kernels ask for more shared memory than they use so that no two
 // CTAs of the tensor-core kernels share an SM (each holds all 512 TMEM columns
-// while it runs): 2 x 130 KB and 130 KB + the K = 256 kernel's both exceed an SM.
+// while it runs): 2 x 130 KB, and 130 KB + that of any other K, exceed an SM.
 constexpr int kSmem64 = 130 * 1024;
-static_assert(GemmShape<64>::kSmem <= size_t(kSmem64), "K = 64 shared memory");
+static_assert(GemmShape<64, kSplitSlices>::kSmem <= size_t(kSmem64) && GemmShape<64, kWideSlices>::kSmem <= size_t(kSmem64),
+              "K = 64 shared memory");
+static_assert(GemmShape<144, kWideSlices>::kSmem >= size_t(kSmem64) && GemmShape<256, kWideSlices>::kSmem <= size_t(227 * 1024),
+              "one tensor CTA per SM");
+
+template <int KD, int S, bool ICVT>
+constexpr size_t gemm_smem()
+{
+    return KD == 64 ? size_t(kSmem64) : GemmShape<KD, S, (KD == 256 && ICVT) ? 2 : kNBuf>::kSmem;
+}
+
+template <int KD, int S, bool ICVT>
+cudaError_t prepare_gemm()
+{
+    return cudaFuncSetAttribute(k_split_gemm<KD, S, ICVT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                int(gemm_smem<KD, S, ICVT>()));
+}
 
 }  // namespace
-
-size_t split_smem_bytes(int kd) { return kd == 256 ? GemmShape<256>::kSmem : GemmShape<64>::kSmem; }
 
 cudaError_t split_prepare()
 {
     cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_split_gemm<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(GemmShape<256>::kSmem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_split_gemm<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(GemmShape<256, 2>::kSmem));
-    for (const void *k : {(const void *)k_split_gemm<64, false>, (const void *)k_split_gemm<64, true>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem64);
+    for (auto f : {prepare_gemm<256, kSplitSlices, false>, prepare_gemm<256, kSplitSlices, true>,
+                   prepare_gemm<64, kSplitSlices, false>, prepare_gemm<64, kSplitSlices, true>,
+                   prepare_gemm<256, kWideSlices, false>, prepare_gemm<144, kWideSlices, false>,
+                   prepare_gemm<64, kWideSlices, false>})
+        if (e == cudaSuccess) e = f();
     // the digit kernels run before and beside the tensor launches: the
     // largest shared-memory carveout (see fp64_prepare)
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_split_vec, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_split_exp, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
+    for (const void *k : {(const void *)k_split_vec<kSplitSlices>, (const void *)k_split_vec<kWideSlices>,
+                          (const void *)k_split_exp<kSplitSlices>, (const void *)k_split_exp<kWideSlices>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -795,39 +946,78 @@ cudaError_t split_prepare()
 
 int split_sm_count() { return g_sms > 0 ? g_sms : 152; }
 
-cudaError_t launch_split_digits_vec(int64_t nleaf, const double *v, double scale, uint16_t *dig, int32_t *dexp,
-                                    cudaStream_t st, const uint8_t *active, int np, int kv)
+SplitGemm gemm_group_v(const SplitTables &T, const SplitTree &s, int dir, const SplitTile *tiles, const SplitCol *cols,
+                       int n, const double *vin, double scale)
 {
-    if (nleaf <= 0) return cudaSuccess;
-    if ((kv != 64 && kv != 256) || np < 1 || np > kv) return cudaErrorInvalidValue;
-    return launch_pdl(k_split_vec, int(std::min<int64_t>(nleaf, 152 * 16)), kv, 0, st, nleaf, v, scale, dig, dexp,
-                      active, np);
+    SplitGemm g;
+    g.tiles = tiles; g.cols = cols; g.ntiles = n;
+    g.ops = T.ops[0][dir]; g.op_exp = T.op_exp[0][dir];
+    g.dig = s.vdig; g.dexp = s.vexp;
+    g.opf = T.opf[0][dir];
+    g.src0 = vin; g.cs0 = T.vscale[dir];
+    g.scale = scale;
+    g.kvalid = T.np;
+    return g;
 }
 
-cudaError_t launch_split_digits_exp(int64_t i0, int64_t i1, int64_t nbox, const double2 *ea, const double2 *eb,
-                                    int P1, double scale, const double *escale, uint16_t *dig, int32_t *dexp,
-                                    cudaStream_t st)
+SplitGemm gemm_group_e(const SplitTables &T, const SplitTree &s, int dir, const SplitTile *tiles, const SplitCol *cols,
+                       int n, const double2 *ea, const double2 *eb, int64_t nbox, int P1, double scale)
+{
+    SplitGemm g;
+    g.tiles = tiles; g.cols = cols; g.ntiles = n;
+    g.ops = T.ops[1][dir]; g.op_exp = T.op_exp[1][dir];
+    g.dig = s.edig; g.dexp = s.eexp;
+    g.opf = T.opf[1][dir];
+    g.src0 = reinterpret_cast<const double *>(ea); g.cs0 = T.escale[dir];
+    g.src1 = reinterpret_cast<const double *>(eb); g.cs1 = T.escale[dir] + kSplitKE;
+    g.nsplit = nbox;
+    g.scale = scale;
+    g.kvalid = 2 * P1;
+    return g;
+}
+
+cudaError_t launch_split_digits_vec(const SplitTables &T, int dir, int64_t nleaf, const double *v, double scale,
+                                    uint16_t *dig, int32_t *dexp, cudaStream_t st, const uint8_t *active)
+{
+    if (nleaf <= 0) return cudaSuccess;
+    const int grid = int(std::min<int64_t>(nleaf, 152 * 16)), nth = (T.kv + 31) / 32 * 32;
+    if (T.slices == kWideSlices)
+        return launch_pdl(k_split_vec<kWideSlices>, grid, nth, 0, st, nleaf, v, scale, T.vscale[dir], dig, dexp, active,
+                          T.np, T.kv);
+    return launch_pdl(k_split_vec<kSplitSlices>, grid, nth, 0, st, nleaf, v, scale, (const double *)nullptr, dig, dexp,
+                      active, T.np, T.kv);
+}
+
+cudaError_t launch_split_digits_exp(const SplitTables &T, int dir, int64_t i0, int64_t i1, int64_t nbox,
+                                    const double2 *ea, const double2 *eb, int P1, double scale, uint16_t *dig,
+                                    int32_t *dexp, cudaStream_t st)
 {
     if (i1 <= i0) return cudaSuccess;
     const int grid = int(std::min<int64_t>((i1 - i0 + 7) / 8, 152 * 16));
-    return launch_pdl(k_split_exp, grid, 256, 0, st, i0, i1, nbox, reinterpret_cast<const double *>(ea),
-                      reinterpret_cast<const double *>(eb), 2 * P1, scale, escale, dig, dexp);
+    return launch_pdl(T.slices == kWideSlices ? k_split_exp<kWideSlices> : k_split_exp<kSplitSlices>, grid, 256, 0, st,
+                      i0, i1, nbox, reinterpret_cast<const double *>(ea), reinterpret_cast<const double *>(eb), 2 * P1,
+                      scale, T.escale[dir], dig, dexp);
 }
 
-cudaError_t launch_split_gemm(const SplitGemm &g, int kd, double inv_alpha0, int32_t *err, long long wait_limit,
-                              int withhold, cudaStream_t st, bool intcvt)
+cudaError_t launch_split_gemm(const SplitTables &T, const SplitGemm &g, int kd, double inv_alpha0, int32_t *err,
+                              cudaStream_t st, bool intcvt)
 {
     if (g.ntiles <= 0) return cudaSuccess;
     const int sms = g_sms > 0 ? g_sms : 152;
     const int grid = std::min(g.ntiles, g.max_ctas > 0 ? std::min(g.max_ctas, sms) : sms);
     int ie = 0;
     const int inv_alpha_exp = std::frexp(inv_alpha0, &ie) == 0.5 ? ie - 1 : kNoExp;
-    if (kd == 256)
-        return launch_pdl(intcvt ? k_split_gemm<256, true> : k_split_gemm<256, false>, grid, kGemmThreads,
-                          intcvt ? GemmShape<256, 2>::kSmem : GemmShape<256>::kSmem, st, g, inv_alpha0, inv_alpha_exp,
-                          err, wait_limit, withhold);
-    return launch_pdl(intcvt ? k_split_gemm<64, true> : k_split_gemm<64, false>, grid, kGemmThreads, size_t(kSmem64),
-                      st, g, inv_alpha0, inv_alpha_exp, err, wait_limit, withhold);
+#define BC_GEMM(KD, S, IC)                                                                                       \
+    launch_pdl(k_split_gemm<KD, S, IC>, grid, kGemmThreads, gemm_smem<KD, S, IC>(), st, g, inv_alpha0,            \
+               inv_alpha_exp, err, T.wait_limit, T.withhold_copy)
+    if (T.slices == kWideSlices) {
+        if (kd == 256) return BC_GEMM(256, kWideSlices, false);
+        if (kd == 144) return BC_GEMM(144, kWideSlices, false);
+        return BC_GEMM(64, kWideSlices, false);
+    }
+    if (kd == 256) return intcvt ? BC_GEMM(256, kSplitSlices, true) : BC_GEMM(256, kSplitSlices, false);
+    return intcvt ? BC_GEMM(64, kSplitSlices, true) : BC_GEMM(64, kSplitSlices, false);
+#undef BC_GEMM
 }
 
 }  // namespace bc
