@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "bc_internal.h"
 #include "pdl.h"
@@ -1317,149 +1318,116 @@ __global__ void k_leaf_out(int64_t nleaf, const int32_t *__restrict__ order,
 }
 
 // -------------------------------------------------------------------------
-// Point evaluation by barycentric Chebyshev interpolation on the containing leaf.
+// Value (and gradient) of the leaf interpolant at points: v_bulk and its
+// gradient off the grid, as the glue step needs them on the fictitious curve.
+// One thread per point: it descends to the point's leaf, forms the Lagrange
+// basis of the p nodes in x and in y as products without divisions,
+//     l_j(t) = c_j P_j S_j,  P_j = prod_{k<j} (t - x_k),  S_j = prod_{k>j} (t - x_k),
+//     l'_j   = c_j (P'_j S_j + P_j S'_j),   (P e)' = P' e + P,
+// c_j = prod_{k != j} 1/(x_j - x_k) (host, extended precision), exact at the
+// nodes up to rounding and without cancellation near them, and contracts the
+// leaf's values:
+//     u = sum l_jy sum l_jx u,  grad u = (1/r) (sum l_jy sum l'_jx u, sum l'_jy sum l_jx u).
+// Bound by the FP64 pipe: at p = 16 about 560 FMAs for the sums and 320 for the
+// bases (barycentric weights would take 32 to 64 divisions of ~10 operations
+// and, without the tables, 64 sines and cosines).  The x basis sits in
+// registers (loops unrolled to PM >= p), the y basis in shared memory
+// [node][thread].  100,003 points, 1,372 leaves, p = 16, value and gradient: 936 us
+// with barycentric weights and the nodes recomputed by each thread, 205 us so
+// (880 FP64 operations a point take 140 us of the pipe).
 // -------------------------------------------------------------------------
-__global__ void k_eval_points(int64_t n, const double *__restrict__ xy, const double *__restrict__ u,
-                              const int32_t *__restrict__ child0, const int32_t *__restrict__ box_leaf,
-                              const int32_t *__restrict__ box_level, const int32_t *__restrict__ box_ix,
-                              const int32_t *__restrict__ box_iy, double x0, double y0, double L, int p,
-                              double *__restrict__ out)
+struct EvalNodes {
+    double x[kMaxP], c[kMaxP];
+};
+constexpr int kEvalThreads = 128;
+
+// basis (and derivative) at t: l[j * st], dl[j * st], j < p
+template <int PM, bool GRAD>
+__device__ __forceinline__ void node_basis(const EvalNodes &nd, int p, double t, double *l, double *dl, int st)
 {
-    const double pi = 3.14159265358979323846;
-    for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-        double x = xy[2 * k], y = xy[2 * k + 1];
-        if (!(x >= x0 && x <= x0 + L && y >= y0 && y <= y0 + L)) { out[k] = nan(""); continue; }
-        int b = 0;
-        while (box_leaf[b] < 0) {
-            int lv = box_level[b];
-            double h = ldexp(L, -lv);
-            double mx = x0 + (box_ix[b] + 0.5) * h, my = y0 + (box_iy[b] + 0.5) * h;
-            b = child0[b] + (x >= mx ? 1 : 0) + (y >= my ? 2 : 0);
+    double P = 1.0, dP = 0.0;
+#pragma unroll
+    for (int j = 0; j < PM; j++) {
+        if (j < p) {
+            const double e = t - nd.x[j];
+            l[j * st] = P;
+            if (GRAD) {
+                dl[j * st] = dP;
+                dP = fma(dP, e, P);
+            }
+            P *= e;
         }
-        int lv = box_level[b];
-        double h = ldexp(L, -lv), r = 0.5 * h;
-        double xi = (x - (x0 + (box_ix[b] + 0.5) * h)) / r, eta = (y - (y0 + (box_iy[b] + 0.5) * h)) / r;
-        double lx[kMaxP], ly[kMaxP], sx = 0.0, sy = 0.0;
-        int hx = -1, hy = -1;
-        for (int m = 0; m < p; m++) {
-            double th = (2.0 * m + 1.0) * pi / (2.0 * p);
-            double xm = -cos(th), lam = ((m & 1) ? -1.0 : 1.0) * sin(th);
-            double dx = xi - xm, dy = eta - xm;
-            if (dx == 0.0) hx = m;
-            if (dy == 0.0) hy = m;
-            lx[m] = dx == 0.0 ? 0.0 : lam / dx;
-            ly[m] = dy == 0.0 ? 0.0 : lam / dy;
-            sx += lx[m];
-            sy += ly[m];
+    }
+    double S = 1.0, dS = 0.0;
+#pragma unroll
+    for (int j = PM - 1; j >= 0; j--) {
+        if (j < p) {
+            const double e = t - nd.x[j], c = nd.c[j], Pj = l[j * st];
+            l[j * st] = c * (Pj * S);
+            if (GRAD) {
+                dl[j * st] = c * fma(dl[j * st], S, Pj * dS);
+                dS = fma(dS, e, S);
+            }
+            S *= e;
         }
-        for (int m = 0; m < p; m++) {
-            lx[m] = hx >= 0 ? (m == hx ? 1.0 : 0.0) : lx[m] / sx;
-            ly[m] = hy >= 0 ? (m == hy ? 1.0 : 0.0) : ly[m] / sy;
-        }
-        const double *ub = u + int64_t(box_leaf[b]) * p * p;
-        double acc = 0.0;
-        for (int jy = 0; jy < p; jy++) {
-            double row = 0.0;
-            for (int jx = 0; jx < p; jx++) row = fma(lx[jx], ub[jy * p + jx], row);
-            acc = fma(ly[jy], row, acc);
-        }
-        out[k] = acc;
     }
 }
 
-// -------------------------------------------------------------------------
-// Value and gradient of the leaf interpolant at points (v_bulk and its
-// gradient off the grid, as the glue step needs them on the fictitious curve):
-// the point's leaf is found as in k_eval_points; with xi its reference
-// coordinate, l_j the barycentric Lagrange basis (weights lam_j) and
-// w_j = lam_j / (xi - x_j), S = sum w_j, T = sum w_j / (xi - x_j):
-//     l_j = w_j / S,   l'_j = l_j (T/S - 1/(xi - x_j))   (j not the nearest node m)
-//     l'_m = l_m sum_{k != m} lam_k (x_k - x_m) / (xi - x_k)^2 / (lam_m + d sum_{k != m} w_k),
-// d = xi - x_m, which is the same quantity without the cancellation of
-// T/S - 1/d as the point nears x_m; at a node the differentiation matrix
-// D_mj = (lam_j / lam_m) / (x_m - x_j), D_mm = -sum_{j != m} D_mj.
-// grad u = (1/r) (sum l_jy sum l'_jx u, sum l'_jy sum l_jx u).
-// -------------------------------------------------------------------------
-__device__ void bary_with_derivative(int p, double xi, double *l, double *dl)
+template <int PM, bool GRAD>
+__global__ void __launch_bounds__(kEvalThreads)
+k_eval_points(int64_t n, const double *__restrict__ xy, const double *__restrict__ u,
+              const int32_t *__restrict__ child0, const int32_t *__restrict__ box_leaf, double x0, double y0, double L,
+              int p, const __grid_constant__ EvalNodes nd, double *__restrict__ val, double *__restrict__ grad)
 {
-    const double pi = 3.14159265358979323846;
-    double xn[kMaxP], lam[kMaxP];
-    int m = 0;
-    for (int k = 0; k < p; k++) {
-        const double th = (2.0 * k + 1.0) * pi / (2.0 * p);
-        xn[k] = -cos(th);
-        lam[k] = ((k & 1) ? -1.0 : 1.0) * sin(th);
-        if (fabs(xi - xn[k]) < fabs(xi - xn[m])) m = k;
-    }
-    const double d = xi - xn[m];
-    if (fabs(d) < 1e-250) {   // at the node (closer than any w_k could be formed without overflow)
-        double dmm = 0.0;
-        for (int j = 0; j < p; j++) {
-            l[j] = j == m ? 1.0 : 0.0;
-            if (j == m) continue;
-            dl[j] = (lam[j] / lam[m]) / (xn[m] - xn[j]);
-            dmm -= dl[j];
-        }
-        dl[m] = dmm;
-        return;
-    }
-    double S = 0.0, T = 0.0, Sr = 0.0, Q = 0.0;   // Sr = sum_{k != m} w_k, Q = sum_{k != m} lam_k (x_k - x_m)/(xi - x_k)^2
-    for (int k = 0; k < p; k++) {
-        const double e = xi - xn[k], w = lam[k] / e;
-        S += w;
-        T += w / e;
-        if (k != m) {
-            Sr += w;
-            Q += lam[k] * (xn[k] - xn[m]) / (e * e);
-        }
-    }
-    for (int j = 0; j < p; j++) {
-        l[j] = (lam[j] / (xi - xn[j])) / S;
-        dl[j] = j == m ? l[j] * Q / (lam[m] + d * Sr) : l[j] * (T / S - 1.0 / (xi - xn[j]));
-    }
-}
-
-__global__ void k_eval_points_grad(int64_t n, const double *__restrict__ xy, const double *__restrict__ u,
-                                   const int32_t *__restrict__ child0, const int32_t *__restrict__ box_leaf,
-                                   const int32_t *__restrict__ box_level, const int32_t *__restrict__ box_ix,
-                                   const int32_t *__restrict__ box_iy, double x0, double y0, double L, int p,
-                                   double *__restrict__ val, double *__restrict__ grad)
-{
+    __shared__ double sy[(GRAD ? 2 : 1) * PM * kEvalThreads];
+    double *ly = sy + threadIdx.x, *dly = ly + (GRAD ? PM * kEvalThreads : 0);   // a thread's own column: no barrier
     for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
         const double x = xy[2 * k], y = xy[2 * k + 1];
         if (!(x >= x0 && x <= x0 + L && y >= y0 && y <= y0 + L)) {
-            val[k] = grad[2 * k] = grad[2 * k + 1] = nan("");
+            val[k] = nan("");
+            if (GRAD) grad[2 * k] = grad[2 * k + 1] = nan("");
             continue;
         }
-        int b = 0;
-        while (box_leaf[b] < 0) {
-            const int lv = box_level[b];
-            const double h = ldexp(L, -lv);
-            const double mx = x0 + (box_ix[b] + 0.5) * h, my = y0 + (box_iy[b] + 0.5) * h;
-            b = child0[b] + (x >= mx ? 1 : 0) + (y >= my ? 2 : 0);
+        // a point on a shared edge belongs to the leaf on its +x / +y side
+        int b = 0, leaf;
+        int64_t ix = 0, iy = 0;
+        double h = L;
+        while ((leaf = box_leaf[b]) < 0) {
+            const double mx = x0 + (ix + 0.5) * h, my = y0 + (iy + 0.5) * h;
+            const int qx = x >= mx ? 1 : 0, qy = y >= my ? 1 : 0;
+            b = child0[b] + qx + 2 * qy;
+            ix = 2 * ix + qx;
+            iy = 2 * iy + qy;
+            h *= 0.5;
         }
-        const int lv = box_level[b];
-        const double h = ldexp(L, -lv), r = 0.5 * h;
-        const double xi = (x - (x0 + (box_ix[b] + 0.5) * h)) / r, eta = (y - (y0 + (box_iy[b] + 0.5) * h)) / r;
-        double lx[kMaxP], ly[kMaxP], dlx[kMaxP], dly[kMaxP];
-        bary_with_derivative(p, xi, lx, dlx);
-        bary_with_derivative(p, eta, ly, dly);
-        const double *ub = u + int64_t(box_leaf[b]) * p * p;
+        const double r = 0.5 * h;
+        const double xi = (x - (x0 + (ix + 0.5) * h)) / r, eta = (y - (y0 + (iy + 0.5) * h)) / r;
+        double lx[PM], dlx[PM];
+        node_basis<PM, GRAD>(nd, p, eta, ly, dly, kEvalThreads);
+        node_basis<PM, GRAD>(nd, p, xi, lx, dlx, 1);
+        const double *ub = u + int64_t(leaf) * p * p;
         double v = 0.0, gx = 0.0, gy = 0.0;
         for (int jy = 0; jy < p; jy++) {
             double row = 0.0, drow = 0.0;
-            for (int jx = 0; jx < p; jx++) {
-                const double uv = ub[jy * p + jx];
-                row = fma(lx[jx], uv, row);
-                drow = fma(dlx[jx], uv, drow);
+#pragma unroll
+            for (int jx = 0; jx < PM; jx++) {
+                if (jx < p) {
+                    const double uv = ub[jy * p + jx];
+                    row = fma(lx[jx], uv, row);
+                    if (GRAD) drow = fma(dlx[jx], uv, drow);
+                }
             }
-            v = fma(ly[jy], row, v);
-            gx = fma(ly[jy], drow, gx);
-            gy = fma(dly[jy], row, gy);
+            v = fma(ly[jy * kEvalThreads], row, v);
+            if (GRAD) {
+                gx = fma(ly[jy * kEvalThreads], drow, gx);
+                gy = fma(dly[jy * kEvalThreads], row, gy);
+            }
         }
         val[k] = v;
-        grad[2 * k] = gx / r;
-        grad[2 * k + 1] = gy / r;
+        if (GRAD) {
+            grad[2 * k] = gx / r;
+            grad[2 * k + 1] = gy / r;
+        }
     }
 }
 
@@ -1903,24 +1871,50 @@ cudaError_t launch_batch_copy(const BatchPtrs &bp, bool gather, double *union_bu
     return cudaGetLastError();
 }
 
+namespace {
+
+EvalNodes eval_nodes(int p)
+{
+    EvalNodes nd{};
+    const long double pi = 3.14159265358979323846264338327950288L;
+    for (int m = 0; m < p; m++) nd.x[m] = double(-std::cos((2.0L * m + 1.0L) * pi / (2.0L * p)));
+    for (int j = 0; j < p; j++) {
+        long double c = 1.0L;
+        for (int k = 0; k < p; k++)
+            if (k != j) c /= static_cast<long double>(nd.x[j]) - nd.x[k];
+        nd.c[j] = double(c);
+    }
+    return nd;
+}
+
+template <bool GRAD>
+cudaError_t launch_eval(const PassArgs &a, const DevTree &d, const double *u, const double *xy, int64_t n, double *val,
+                        double *grad, double x0, double y0, double L, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    const int grid = int(std::min<int64_t>((n + kEvalThreads - 1) / kEvalThreads, 152 * 16));
+    const EvalNodes nd = eval_nodes(a.p);
+#define BC_EVAL(PM)                                                                                              \
+    k_eval_points<PM, GRAD><<<grid, kEvalThreads, 0, st>>>(n, xy, u, d.box_child0, d.box_leaf, x0, y0, L, a.p, nd, val, grad)
+    if (a.p <= 8) BC_EVAL(8);
+    else if (a.p <= 12) BC_EVAL(12);
+    else BC_EVAL(16);
+#undef BC_EVAL
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_eval_points_grad(const PassArgs &a, const DevTree &d, const double *u, const double *xy, int64_t n,
                                     double *val, double *grad, double x0, double y0, double L, cudaStream_t st)
 {
-    if (n <= 0) return cudaSuccess;
-    int grid = int(std::min<int64_t>((n + 127) / 128, 152 * 8));
-    k_eval_points_grad<<<grid, 128, 0, st>>>(n, xy, u, d.box_child0, d.box_leaf, d.box_level, d.box_ix, d.box_iy,
-                                             x0, y0, L, a.p, val, grad);
-    return cudaGetLastError();
+    return launch_eval<true>(a, d, u, xy, n, val, grad, x0, y0, L, st);
 }
 
 cudaError_t launch_eval_points(const PassArgs &a, const DevTree &d, const double *u, const double *xy, int64_t n,
                                double *out, double x0, double y0, double L, cudaStream_t st)
 {
-    if (n <= 0) return cudaSuccess;
-    int grid = int(std::min<int64_t>((n + 255) / 256, 152 * 8));
-    k_eval_points<<<grid, 256, 0, st>>>(n, xy, u, d.box_child0, d.box_leaf, d.box_level, d.box_ix, d.box_iy, x0,
-                                        y0, L, a.p, out);
-    return cudaGetLastError();
+    return launch_eval<false>(a, d, u, xy, n, out, nullptr, x0, y0, L, st);
 }
 
 }  // namespace bc
