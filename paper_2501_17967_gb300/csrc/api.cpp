@@ -822,24 +822,34 @@ bc_status build_split_tables(bc_ctx *ctx)
 // (longest work first).
 struct TileBuilder {
     int cap;
+    bool halves;   // K = 64
     std::vector<SplitTile> tiles;
     std::vector<SplitCol> cols;
-    explicit TileBuilder(int n) : cap(n) {}
+    TileBuilder(const SplitTables &T, int K) : cap(T.tileN), halves(K == 64) {}
     // one operator, its columns given in order
     void add(const SplitOp &op, const std::vector<SplitCol> &c)
     {
-        for (size_t i = 0; i < c.size(); i += cap) {
-            SplitTile t;
-            t.a_off = op.a_off;
-            t.f_off = op.f_off;
-            t.rows = op.rows;
-            t.exp_off = op.exp_off;
-            t.p0 = int32_t(cols.size());
-            t.cnt = int32_t(std::min<size_t>(cap, c.size() - i));
-            cols.insert(cols.end(), c.begin() + i, c.begin() + i + t.cnt);
-            tiles.push_back(t);
+        const int mh = op.rows > 128 ? 2 : 1;
+        for (int h = 0; h < (halves ? mh : 1); h++) {
+            for (size_t i = 0; i < c.size(); i += cap) {
+                SplitTile t;
+                t.a_off = op.a_off + int64_t(h) * kHalfBytes;
+                t.f_off = op.f_off + 128 * h;
+                t.rows = halves ? std::min(128, op.rows - 128 * h) : op.rows;
+                t.exp_off = op.exp_off + 128 * h;
+                t.p0 = int32_t(cols.size());
+                t.cnt = int32_t(std::min<size_t>(cap, c.size() - i));
+                t.astride = mh * kHalfBytes;
+                t.frows = op.rows;
+                for (int q = 0; q < t.cnt; q++) {
+                    cols.push_back(c[i + q]);
+                    cols.back().out += 128 * h;
+                }
+                tiles.push_back(t);
+            }
         }
     }
+    static constexpr int kHalfBytes = 128 * 64 * 2;   // one digit of a 128-row half at K = 64
 };
 
 inline int32_t col_ctl(int shift, bool inv_alpha) { return int32_t(shift * 2 + (inv_alpha ? 1 : 0)); }
@@ -871,7 +881,7 @@ TileBuilder m2l_tiles(const bc_tree *t, const SplitTables &T, int dir, double2 *
     const HostTree &h = t->h;
     const int P1 = t->ctx->P1, first_which = dir == 1 ? 1 : 0;   // expA = 0, expB = 1
     const int64_t nbox = int64_t(h.box_level.size());
-    TileBuilder M(T.tileN);
+    TileBuilder M(T, kSplitKE);
     std::vector<std::vector<SplitCol>> by_v(kNumV);
     for (size_t k = 0; k < h.v_src.size(); k++) {
         SplitCol c;
@@ -934,7 +944,7 @@ cudaError_t build_digit_tree(bc_tree *t, const SplitTables &T, SplitTree &s, boo
         const bool adj = dir == 1;
         double2 *first = adj ? t->d.expB : t->d.expA;
         const int first_which = adj ? 1 : 0, second_which = adj ? 0 : 1;   // expA = 0, expB = 1
-        TileBuilder V(T.tileN), NV(T.tileN), E(T.tileN);
+        TileBuilder V(T, T.kv), NV(T, T.kv), E(T, kSplitKE);
         // near entries, by table
         std::vector<std::vector<SplitCol>> by_tab(kNumNear);
         for (int64_t k = 0; k < nn; k++) {

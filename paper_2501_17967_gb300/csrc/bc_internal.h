@@ -252,10 +252,14 @@ struct SplitTables {
     int withhold_copy = 0;                       // diagnostics: never start the operator copies (forces a timeout)
 };
 // One tile = one operator times up to tileN columns.
+// K = 64: one tile per 128-row half of the operator, consecutive tiles of a half
+// together (the tensor kernel keeps it in shared memory); larger K: the whole
+// operator, its halves done one after the other.
 struct SplitTile {
     int64_t a_off, f_off;
-    int32_t rows, exp_off;
+    int32_t rows, exp_off; // rows of the tile; row exponents
     int32_t p0, cnt;       // columns [p0, p0 + cnt)
+    int32_t astride, frows;   // bytes between digits (K = 64); rows of the operator
 };
 // One column = one input vector and where its result rows go.
 struct SplitCol {

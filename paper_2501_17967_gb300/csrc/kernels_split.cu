@@ -333,20 +333,25 @@ __device__ __forceinline__ double i64_scaled_int(long long S, int ex)
         static_cast<long long>((sgn | (static_cast<unsigned long long>(e - 1) << 52)) + mant + up));
 }
 
-// The eight levels of the 7-digit format: sum_g D_g 256^(7-g) (g = 0..7,
-// |D_g| <= 2^24) times 2^ex.  Levels 0-3 and 4-7 are each exact in int64 (and
-// in FP64: below 2^50), so one FMA gives the sum with a single rounding.
-// Results outside the normal range take the general scaling.
+// The eight levels of the 7-digit format: sum_g D_g 256^(7-g) (g = 0..7) times
+// 2^ex.  The sum is a product of vectors below 2^-1 in magnitude, K <= 256 of
+// them, so it is below 2^78; its last 16 bits are below the rounding of the
+// operands (2^17 and more), so it is rounded to a multiple of 2^16, which int64
+// holds, and converted once (one FP64 operation per element instead of three;
+// the conversions share the FP64 pipe, which bound the epilogue).  Results
+// outside the normal range take the general scaling.
 __device__ __noinline__ double scale_wide(double v, int ex) { return scalbn(v, ex); }
 __device__ __forceinline__ double levels_scaled(const int (&D)[kWideLevels], int ex)
 {
-    const long long hi = (long long)D[3] + (long long)D[2] * 256 + (long long)D[1] * 65536 + (long long)D[0] * 16777216;
-    const long long lo = (long long)D[7] + (long long)D[6] * 256 + (long long)D[5] * 65536 + (long long)D[4] * 16777216;
-    const double v = fma(__ll2double_rn(hi), 4294967296.0, __ll2double_rn(lo));
-    const long long b = __double_as_longlong(v);
-    const int e = int((b >> 52) & 0x7FF), es = e + ex;
-    if (e == 0) return 0.0;   // v is zero (a nonzero sum is at least 1)
-    if (es <= 0 || es >= 0x7FF) return scale_wide(v, ex);
+    const long long top = (long long)D[0] * 65536 + ((long long)D[1] * 256 + D[2]);
+    const long long mid = (long long)D[3] * 65536 + ((long long)D[4] * 256 + D[5]);
+    const long long low = ((long long)D[6] * 256 + (D[7] + 32768)) >> 16;
+    const long long S = (top << 24) + mid + low;
+    ex += 16;
+    const long long b = __double_as_longlong(__ll2double_rn(S));
+    const int es = int((b >> 52) & 0x7FF) + ex;
+    if (S == 0) return 0.0;
+    if (es <= 0 || es >= 0x7FF) return scale_wide(__longlong_as_double(b), ex);
     return __longlong_as_double(b + ((long long)ex << 52));
 }
 
@@ -455,8 +460,7 @@ __global__ void __launch_bounds__(256) k_split_exp(int64_t i0, int64_t i1, int64
 }
 
 // ---------------------------------------------------------------------------
-// Operator x columns on tcgen05.  KD = 256 or 144 (leaf vectors; 64 for small
-// orders) or 64 (expansions).
+// Operator x columns on tcgen05, KD = 256 or 144 (leaf vectors).
 // ---------------------------------------------------------------------------
 struct ColMeta {
     double *out;
@@ -486,11 +490,8 @@ struct GemmShape {
     static constexpr int kChunk = 128 * KC * 2;        // bytes of one operator chunk
     static constexpr int kBSBO = (KD / 8) * 128;       // B: bytes between 8-row groups
     static constexpr int kASBO = (KC / 8) * 128;       // A: bytes between 8-row groups
-    // B buffers: two for K = 64 (the next tile is gathered while this one's
-    // MMAs run), one for the larger K (115 to 120 KB at K = 256)
-    static constexpr int kBBuf = KD <= 64 ? 2 : 1;
-    static constexpr int kBTile = S * kBSlice;          // bytes of one tile's B
-    static constexpr size_t kSmem = size_t(kBBuf) * kBTile + size_t(NB) * kChunk + 2 * N * sizeof(ColMeta) +
+    static constexpr int kBTile = S * kBSlice;          // bytes of one tile's B (115 to 120 KB at K = 256): one buffer
+    static constexpr size_t kSmem = size_t(kBTile) + size_t(NB) * kChunk + 2 * N * sizeof(ColMeta) +
                                     64 * sizeof(uint64_t);
 };
 
@@ -512,16 +513,16 @@ constexpr int kNoExp = 0x7FFFFFFF;   // 1/alpha0 is not a power of two
 //   job_full[r] (1)    the MMAs of the job in TMEM buffer r have completed (commit)
 //   job_empty[r] (8)   the epilogue warps have read TMEM buffer r
 //   b_full[t][s] (1)   B digit slice s (and the metadata) of tile parity t is ready
-//   b_empty[u][s] (1)  no MMA of the tile last held in B buffer u reads slice s any more (commit)
+//   b_empty[s] (1)     no MMA of the previous tile reads B slice s any more (commit)
 //   meta_empty[t] (8)  the epilogue warps are done with metadata buffer t
 // Digit slice s (0-based) of B is read by the chunks of operator digit a <= L - 1 - s,
 // so in a tile's last job it is free after those chunks; the next tile's B is
 // gathered slice by slice from s = S - 1 down to 0 and its first chunk issues its
-// MMAs from slice S - 1 down, so with one B buffer only the last slices are
-// waited for at the tile change.  Tile k uses B buffer k % kBBuf.
+// MMAs from slice S - 1 down, so only the last slices are waited for at the
+// tile change.
 template <int S>
 struct GemmBars {
-    uint64_t lbar[kNBuf], mbar[kNBuf], job_full[2], job_empty[2], b_full[2][S], b_empty[2][S], meta_empty[2];
+    uint64_t lbar[kNBuf], mbar[kNBuf], job_full[2], job_empty[2], b_full[2][S], b_empty[S], meta_empty[2];
     uint32_t tslot;
     int fail;
 };
@@ -529,15 +530,81 @@ static_assert(sizeof(GemmBars<kWideSlices>) <= 64 * sizeof(uint64_t), "barrier s
 
 // Row `row` of an operator times a vector without digits (an infinity or a NaN
 // among its entries), in FP64: sum_k opf[k][row] (scale cs_k x_k).
-__device__ __noinline__ double plain_product(const SplitGemm &gm, int64_t f_off, int rows, int row, int vec)
+__device__ __noinline__ double plain_product(const SplitGemm &gm, const SplitTile &tl, int row, int vec)
 {
     const bool lo = vec < gm.nsplit;
     const double *x = lo ? gm.src0 + int64_t(vec) * gm.kvalid : gm.src1 + int64_t(vec - gm.nsplit) * gm.kvalid;
     const double *cs = lo ? gm.cs0 : gm.cs1;
-    const double *op = gm.opf + f_off + row;
+    const double *op = gm.opf + tl.f_off + row;
     double s = 0.0;
-    for (int k = 0; k < gm.kvalid; k++) s = fma(op[int64_t(k) * rows], gm.scale * (cs ? cs[k] : 1.0) * x[k], s);
+    for (int k = 0; k < gm.kvalid; k++) s = fma(op[int64_t(k) * tl.frows], gm.scale * (cs ? cs[k] : 1.0) * x[k], s);
     return s;
+}
+
+// One warp's share of a job: columns [cb, ce) of its 32 TMEM lanes (row `row`
+// of the tile's operator, valid where live; ea: its row exponent), from the
+// levels' column blocks at ta0.
+template <int S, bool ICVT>
+__device__ __forceinline__ void epilogue_columns(const SplitGemm &gm, const SplitTile &tl, const ColMeta *M, uint32_t ta0,
+                                                 int cb, int ce, int row, bool live, int ea, double inv_alpha0)
+{
+    constexpr int kL = Fmt<S>::L, kN = Fmt<S>::N;
+    // columns per TMEM read: 8 levels take twice the registers of 5
+    constexpr int kQ = S > 5 ? 4 : 8;
+    for (int c0 = cb; c0 < ce; c0 += kQ) {   // uniform over the warp
+        uint32_t d[kL][kQ];
+#pragma unroll
+        for (int g = 0; g < kL; g++) {
+            if constexpr (kQ == 4) tmem_ld4(ta0 + uint32_t(g * kN + c0), d[g]);
+            else tmem_ld8(ta0 + uint32_t(g * kN + c0), d[g]);
+        }
+        tmem_ld_wait();
+        if (!live) continue;
+#pragma unroll
+        for (int q = 0; q < kQ; q++) {
+            const int c = c0 + q;
+            if (c >= ce) continue;
+            double val;
+            if constexpr (S > 5) {
+                if (M[c].flag & 2) {
+                    val = scale_wide(plain_product(gm, tl, row, M[c].vec), M[c].exp);
+                } else {
+                    int D[kL];
+#pragma unroll
+                    for (int g = 0; g < kL; g++) D[g] = __float2int_rn(__uint_as_float(d[g][q]));
+                    val = levels_scaled(D, ea + M[c].exp);
+                }
+                if (M[c].flag & 1) val *= inv_alpha0;
+            } else {
+                long long sum = 0;
+#pragma unroll
+                for (int g = 0; g < kL; g++)
+                    sum += (long long)__float2int_rn(__uint_as_float(d[g][q])) << (8 * (kL - 1 - g));
+                val = ICVT ? i64_scaled_int(sum, ea + M[c].exp) : i64_scaled(sum, ea + M[c].exp);
+                if (M[c].flag) val *= inv_alpha0;
+            }
+            M[c].out[row] = val;
+        }
+    }
+}
+
+// The metadata of a column: digit exponent ev, power-of-two factors folded in.
+template <int S>
+__device__ __forceinline__ ColMeta col_meta(const SplitCol &c, int ev, int inv_alpha_exp)
+{
+    ColMeta m;
+    const bool plain = S > 5 && ev == kWideExp;
+    m.out = c.out;
+    m.exp = (c.ctl >> 1) + (plain ? 0 : ev - 8 * (Fmt<S>::L + 1));
+    m.flag = c.ctl & 1;
+    if (m.flag && inv_alpha_exp != kNoExp) {   // 1/alpha0 a power of two: an exponent shift
+        m.exp += inv_alpha_exp;
+        m.flag = 0;
+    }
+    if (plain) m.flag |= 2;
+    m.vec = c.vec;
+    m.pad = 0;
+    return m;
 }
 
 // 5 digits: the second launch bound caps the registers at 64 per thread: 16
@@ -555,8 +622,8 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
     using Sh = GemmShape<KD, S, NB>;
     constexpr int kS = S, kN = Sh::N, kL = Sh::L;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *Bs = smem;                                                      // kBBuf x kS x kBSlice
-    uint8_t *As = smem + Sh::kBBuf * Sh::kBTile;                             // NB x kChunk
+    uint8_t *Bs = smem;                                                      // kS x kBSlice
+    uint8_t *As = smem + Sh::kBTile;                                         // NB x kChunk
     ColMeta *meta = reinterpret_cast<ColMeta *>(As + NB * Sh::kChunk);       // [2][kN]
     GemmBars<S> *bars = reinterpret_cast<GemmBars<S> *>(meta + 2 * kN);
     volatile int *fail = &bars->fail;
@@ -579,8 +646,7 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
             mbar_init(&bars->meta_empty[i], kEpiWarps);
             for (int sl = 0; sl < kS; sl++) mbar_init(&bars->b_full[i][sl], 1);
         }
-        for (int u = 0; u < 2; u++)
-            for (int sl = 0; sl < kS; sl++) mbar_init(&bars->b_empty[u][sl], 1);
+        for (int sl = 0; sl < kS; sl++) mbar_init(&bars->b_empty[sl], 1);
         bars->fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -640,8 +706,7 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
                     // first chunk (a = 0) starts levels 0 .. S-1; where L > S the
                     // second one starts level L-1 (its last slice, apart).
                     const uint32_t dcol = tmem + uint32_t(r * kTmemBuf + a * kN);
-                    const uint64_t bd = bdesc0 + uint64_t(k % Sh::kBBuf) * (Sh::kBTile >> 4) +
-                                        uint64_t(kc) * ((Sh::KC / 8) * 128 >> 4);
+                    const uint64_t bd = bdesc0 + uint64_t(kc) * ((Sh::KC / 8) * 128 >> 4);
                     if (kL > kS && pos == 1 && kc == 0) {
                         umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, (nb - 1) * kN), 1u);
                         umma_kchain_warp<Sh::KC / 16>(dcol + uint32_t((nb - 1) * kN), ad,
@@ -655,9 +720,9 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
                     // in the tile's last job, slice L-1-a is read by no later
                     // chunk, and after the last digit no slice is
                     if (last_job && kc == Sh::NKC - 1) {
-                        if (kL - 1 - a < kS) umma_commit_warp(&bars->b_empty[k % Sh::kBBuf][kL - 1 - a]);
+                        if (kL - 1 - a < kS) umma_commit_warp(&bars->b_empty[kL - 1 - a]);
                         if (a == kS - 1)
-                            for (int b = 0; b < kL - kS; b++) umma_commit_warp(&bars->b_empty[k % Sh::kBBuf][b]);
+                            for (int b = 0; b < kL - kS; b++) umma_commit_warp(&bars->b_empty[b]);
                     }
                 }
                 if (failed) break;
@@ -716,13 +781,6 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
         // ---------------- column metadata and B gather ----------------
         const int gt = tid - 32 * kGatherWarp0;
         constexpr int kPieces = KD / 8;   // 16-byte pieces per column and slice
-        // two B buffers: the next tile's record, this thread's column of it and
-        // the column's digit exponent are fetched while the current tile's
-        // slices are in flight
-        SplitTile ntl{};
-        SplitCol ncol{};
-        int nexp = 0;
-        bool have = false;
         int k = 0;
         bool stop = false;
         for (int tile = blockIdx.x; tile < gm.ntiles && !stop; tile += gridDim.x, k++) {
@@ -730,87 +788,35 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
             // the epilogues of tile k - 2 no longer read this metadata buffer
             if (k >= 2) ok = wait_bar(&bars->meta_empty[k & 1], uint32_t(((k - 2) >> 1) & 1), wait_limit, fail);
             if (gather_sync_or(kGatherThreads, !ok)) break;   // uniform over the gather warps
-            const SplitTile tl = have ? ntl : gm.tiles[tile];
+            const SplitTile tl = gm.tiles[tile];
             ColMeta *M = meta + (k & 1) * kN;
             if (gt < tl.cnt) {
-                const SplitCol c = have ? ncol : gm.cols[tl.p0 + gt];
-                ColMeta m;
-                m.out = c.out;
-                const int ev = have ? nexp : gm.dexp[c.vec];
-                const bool plain = S > 5 && ev == kWideExp;
-                m.exp = (c.ctl >> 1) + (plain ? 0 : ev - 8 * (kL + 1));
-                m.flag = c.ctl & 1;
-                if (m.flag && inv_alpha_exp != kNoExp) {   // 1/alpha0 a power of two: an exponent shift
-                    m.exp += inv_alpha_exp;
-                    m.flag = 0;
-                }
-                if (plain) m.flag |= 2;
-                m.vec = c.vec;
-                m.pad = 0;
-                M[gt] = m;
+                const SplitCol c = gm.cols[tl.p0 + gt];
+                M[gt] = col_meta<S>(c, gm.dexp[c.vec], inv_alpha_exp);
             }
-            have = false;
             gather_sync(kGatherThreads);
-            uint8_t *Bt = Bs + (k % Sh::kBBuf) * Sh::kBTile;
-            if constexpr (Sh::kBBuf == 2) {
-                // every slice at once: tile k - 2, the last one in this buffer,
-                // has released all of them
-                bool ok2 = true;
-                if (k >= 2)
-                    for (int sl = 0; sl < kS && ok2; sl++)
-                        ok2 = wait_bar(&bars->b_empty[k & 1][sl], uint32_t(((k - 2) >> 1) & 1), wait_limit, fail);
-                if (gather_sync_or(kGatherThreads, !ok2)) break;
-                for (int sl = kS - 1; sl >= 0; sl--) {
+            // one B buffer: two slices in flight, each issued once the
+            // previous tile's MMAs have released it; complete slice sl + 1
+            for (int sl = kS - 1; sl >= -1; sl--) {
+                if (sl >= 0) {
+                    bool ok2 = true;
+                    if (k >= 1) ok2 = wait_bar(&bars->b_empty[sl], uint32_t((k - 1) & 1), wait_limit, fail);
+                    if (gather_sync_or(kGatherThreads, !ok2)) {
+                        stop = true;
+                        break;
+                    }
                     for (int item = gt; item < tl.cnt * kPieces; item += kGatherThreads) {
                         const int c = item / kPieces, kg = item % kPieces;
                         const uint16_t *src = gm.dig + (size_t(M[c].vec) * kS + sl) * KD + kg * 8;
-                        cp_async16(Bt + sl * Sh::kBSlice + ((c >> 3) * kPieces + kg) * 128 + (c & 7) * 16, src);
+                        cp_async16(Bs + sl * Sh::kBSlice + ((c >> 3) * kPieces + kg) * 128 + (c & 7) * 16, src);
                     }
                     cp_async_commit();
                 }
-                const int nt = tile + gridDim.x;
-#pragma unroll
-                for (int j = 0; j < kS; j++) {
-                    cp_async_wait_pending(kS - 1 - j);   // slices kS-1 .. kS-1-j have landed
+                if (sl + 1 <= kS - 1) {
+                    cp_async_wait_pending(sl >= 0 ? 1 : 0);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     gather_sync(kGatherThreads);
-                    if (gt == 0) mbar_arrive(&bars->b_full[k & 1][kS - 1 - j]);
-                    // one step of the next tile's metadata chain per slice
-                    if (nt < gm.ntiles) {
-                        if (j == 0) {
-                            ntl = gm.tiles[nt];
-                        } else if (j == 1) {
-                            if (gt < ntl.cnt) ncol = gm.cols[ntl.p0 + gt];
-                        } else if (j == 2) {
-                            if (gt < ntl.cnt) nexp = gm.dexp[ncol.vec];
-                            have = true;
-                        }
-                    }
-                }
-            } else {
-                // one B buffer: two slices in flight, each issued once the
-                // previous tile's MMAs have released it; complete slice sl + 1
-                for (int sl = kS - 1; sl >= -1; sl--) {
-                    if (sl >= 0) {
-                        bool ok2 = true;
-                        if (k >= 1) ok2 = wait_bar(&bars->b_empty[0][sl], uint32_t((k - 1) & 1), wait_limit, fail);
-                        if (gather_sync_or(kGatherThreads, !ok2)) {
-                            stop = true;
-                            break;
-                        }
-                        for (int item = gt; item < tl.cnt * kPieces; item += kGatherThreads) {
-                            const int c = item / kPieces, kg = item % kPieces;
-                            const uint16_t *src = gm.dig + (size_t(M[c].vec) * kS + sl) * KD + kg * 8;
-                            cp_async16(Bt + sl * Sh::kBSlice + ((c >> 3) * kPieces + kg) * 128 + (c & 7) * 16, src);
-                        }
-                        cp_async_commit();
-                    }
-                    if (sl + 1 <= kS - 1) {
-                        cp_async_wait_pending(sl >= 0 ? 1 : 0);
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        gather_sync(kGatherThreads);
-                        if (gt == 0) mbar_arrive(&bars->b_full[k & 1][sl + 1]);
-                    }
+                    if (gt == 0) mbar_arrive(&bars->b_full[k & 1][sl + 1]);
                 }
             }
         }
@@ -845,44 +851,8 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
                 const int ea = live ? gm.op_exp[tl.exp_off + row] : 0;
                 const int cb = small ? (wq >> 1) * (kN / 2) + half * (kN / 4) : half * (kN / 2);
                 const int ce = min(tl.cnt, cb + (small ? kN / 4 : kN / 2));
-                // columns per TMEM read: 8 levels take twice the registers of 5
-                constexpr int kQ = S > 5 ? 4 : 8;
-                for (int c0 = cb; c0 < ce; c0 += kQ) {   // uniform over the warp
-                    uint32_t d[kL][kQ];
-#pragma unroll
-                    for (int g = 0; g < kL; g++) {
-                        const uint32_t ta = tmem + (uint32_t(wq * 32) << 16) + uint32_t(r * kTmemBuf + g * kN + c0);
-                        if constexpr (kQ == 4) tmem_ld4(ta, d[g]);
-                        else tmem_ld8(ta, d[g]);
-                    }
-                    tmem_ld_wait();
-                    if (!live) continue;
-#pragma unroll
-                    for (int q = 0; q < kQ; q++) {
-                        const int c = c0 + q;
-                        if (c >= ce) continue;
-                        double val;
-                        if constexpr (S > 5) {
-                            if (M[c].flag & 2) {
-                                val = scale_wide(plain_product(gm, tl.f_off, tl.rows, row, M[c].vec), M[c].exp);
-                            } else {
-                                int D[kL];
-#pragma unroll
-                                for (int g = 0; g < kL; g++) D[g] = __float2int_rn(__uint_as_float(d[g][q]));
-                                val = levels_scaled(D, ea + M[c].exp);
-                            }
-                            if (M[c].flag & 1) val *= inv_alpha0;
-                        } else {
-                            long long sum = 0;
-#pragma unroll
-                            for (int g = 0; g < kL; g++)
-                                sum += (long long)__float2int_rn(__uint_as_float(d[g][q])) << (8 * (kL - 1 - g));
-                            val = ICVT ? i64_scaled_int(sum, ea + M[c].exp) : i64_scaled(sum, ea + M[c].exp);
-                            if (M[c].flag) val *= inv_alpha0;
-                        }
-                        M[c].out[row] = val;
-                    }
-                }
+                epilogue_columns<S, ICVT>(gm, tl, M, tmem + (uint32_t(wq * 32) << 16) + uint32_t(r * kTmemBuf), cb, ce,
+                                          row, live, ea, inv_alpha0);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars->job_empty[r]);
@@ -899,26 +869,270 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
-int g_sms = 0;
-// The K = 64 kernels ask for more shared memory than they use so that no two
-// CTAs of the tensor-core kernels share an SM (each holds all 512 TMEM columns
-// while it runs): 2 x 130 KB, and 130 KB + that of any other K, exceed an SM.
-constexpr int kSmem64 = 130 * 1024;
-static_assert(GemmShape<64, kSplitSlices>::kSmem <= size_t(kSmem64) && GemmShape<64, kWideSlices>::kSmem <= size_t(kSmem64),
-              "K = 64 shared memory");
-static_assert(GemmShape<144, kWideSlices>::kSmem >= size_t(kSmem64) && GemmShape<256, kWideSlices>::kSmem <= size_t(227 * 1024),
-              "one tensor CTA per SM");
+// ---------------------------------------------------------------------------
+// K = 64 (expansions, and leaf vectors of small orders): one operator of up to
+// 128 rows is 16 KB per digit, so all its digits stay in shared memory (80 or
+// 112 KB) while a CTA works through its tiles, a contiguous range of the list,
+// in which consecutive tiles share an operator; the operator is fetched again
+// only where it changes.  Streamed through three chunk buffers like the larger
+// ones, a tile took 5.2 us, four times its MMAs: each chunk's copy latency
+// stood between short MMA runs.  17,491 leaves, 30 terms, 7 digits, alone: the
+// M2L's tiles 427 -> 262 us, expansion-to-leaf and W list 168 -> 134 us.
+//   warp 0      MMAs: per tile one chain per operator digit, issued back to back
+//   warp 1      operator copies
+//   warps 2-7   column metadata and digits: 192 / N threads per column, each with
+//               its own column record (the records, columns and exponents of the
+//               next three tiles are in flight), so no barrier among them;
+//               three B buffers
+//   warps 8-15  epilogues, two TMEM buffers
+// Barriers (counts): a_full (1: bulk-copy bytes), a_free (1: commit of the last
+// tile on the operator), b_full[3], meta_full[4] (6: one per gather warp),
+// b_empty[3] (1: commit), job_full[2] (1: commit), job_empty[2], meta_empty[4]
+// (8: one per epilogue warp).
+// ---------------------------------------------------------------------------
+constexpr int kB64 = 3, kM64 = 4;
+template <int S>
+struct Shape64 {
+    static constexpr int N = Fmt<S>::N, L = Fmt<S>::L;
+    static constexpr int kA = 128 * 64 * 2;            // bytes of one operator digit
+    static constexpr int kBSlice = N * 64 * 2, kBTile = S * kBSlice;
+    static constexpr size_t kSmem =
+        size_t(S) * kA + kB64 * size_t(kBTile) + kM64 * N * sizeof(ColMeta) + 32 * sizeof(uint64_t);
+};
+struct Bars64 {
+    uint64_t a_full, a_free, b_full[kB64], b_empty[kB64], meta_full[kM64], meta_empty[kM64], job_full[2], job_empty[2];
+    uint32_t tslot;
+    int fail;
+};
+static_assert(sizeof(Bars64) <= 32 * sizeof(uint64_t), "barrier space");
 
+template <int S, bool ICVT>
+__global__ void __launch_bounds__(kGemmThreads, S == kSplitSlices ? 2 : 1)
+k_gemm64(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__restrict__ err,
+         long long wait_limit, int withhold)
+{
+    using Sh = Shape64<S>;
+    constexpr int kN = Sh::N, kL = Sh::L;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint8_t *As = smem, *Bs = smem + S * Sh::kA;
+    ColMeta *meta = reinterpret_cast<ColMeta *>(Bs + kB64 * Sh::kBTile);   // [kM64][kN]
+    Bars64 *bars = reinterpret_cast<Bars64 *>(meta + kM64 * kN);
+    volatile int *fail = &bars->fail;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tslot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        mbar_init(&bars->a_full, 1);
+        mbar_init(&bars->a_free, 1);
+        for (int i = 0; i < kB64; i++) {
+            mbar_init(&bars->b_full[i], kGatherThreads / 32);
+            mbar_init(&bars->b_empty[i], 1);
+        }
+        for (int i = 0; i < kM64; i++) {
+            mbar_init(&bars->meta_full[i], kGatherThreads / 32);
+            mbar_init(&bars->meta_empty[i], kEpiWarps);
+        }
+        for (int i = 0; i < 2; i++) {
+            mbar_init(&bars->job_full[i], 1);
+            mbar_init(&bars->job_empty[i], kEpiWarps);
+        }
+        bars->fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = bars->tslot;
+    griddep_wait();
+    griddep_launch_dependents();
+    // this CTA's tiles
+    const int t0 = int(int64_t(gm.ntiles) * blockIdx.x / gridDim.x), t1 = int(int64_t(gm.ntiles) * (blockIdx.x + 1) / gridDim.x);
+    const int nt = t1 - t0;
+
+    if (warp == 0) {
+        const uint64_t adesc0 = umma_desc(smem_u32(As), 128, 1024), bdesc0 = umma_desc(smem_u32(Bs), 128, 1024);
+        int ops = 0;          // operators begun
+        int64_t cur = -1;
+        bool ok = true;
+        int k = 0;
+        int64_t a_off = nt > 0 ? gm.tiles[t0].a_off : -1, next = nt > 1 ? gm.tiles[t0 + 1].a_off : -1;
+        for (; k < nt; k++) {
+            const int64_t after = k + 2 < nt ? gm.tiles[t0 + k + 2].a_off : -1;   // used in two tiles' time
+            if (a_off != cur) {
+                ok = wait_bar(&bars->a_full, uint32_t(ops & 1), wait_limit, fail);
+                ops++;
+                cur = a_off;
+            }
+            const int r = k & 1, buf = k % kB64;
+            if (ok && k >= 2) ok = wait_bar(&bars->job_empty[r], uint32_t(((k - 2) >> 1) & 1), wait_limit, fail);
+            if (ok) ok = wait_bar(&bars->b_full[buf], uint32_t((k / kB64) & 1), wait_limit, fail);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t bd = bdesc0 + uint64_t(buf) * (Sh::kBTile >> 4);
+#pragma unroll
+            for (int a = 0; a < S; a++) {   // the chains of k_split_gemm, in the order 0..S-1
+                const int nb = S < kL - a ? S : kL - a;
+                const uint64_t ad = adesc0 + uint64_t(a) * (Sh::kA >> 4);
+                const uint32_t dcol = tmem + uint32_t(r * kTmemBuf + a * kN);
+                if (kL > S && a == 1) {
+                    umma_kchain_warp<4>(dcol, ad, bd, umma_idesc(128, (nb - 1) * kN), 1u);
+                    umma_kchain_warp<4>(dcol + uint32_t((nb - 1) * kN), ad, bd + uint64_t(nb - 1) * (Sh::kBSlice >> 4),
+                                        umma_idesc(128, kN), 0u);
+                } else {
+                    umma_kchain_warp<4>(dcol, ad, bd, umma_idesc(128, nb * kN), a == 0 ? 0u : 1u);
+                }
+            }
+            umma_commit_warp(&bars->b_empty[buf]);
+            umma_commit_warp(&bars->job_full[r]);
+            if (next >= 0 && next != a_off) umma_commit_warp(&bars->a_free);
+            a_off = next;
+            next = after;
+        }
+        if (!ok) {
+            *fail = 1;
+            int dummy = 0;   // MMAs in flight: those of the last tile issued
+            if (k > 0) wait_bar(&bars->job_full[(k - 1) & 1], uint32_t(((k - 1) >> 1) & 1), wait_limit, &dummy);
+        }
+    } else if (warp == 1) {
+        int ops = 0;
+        int64_t cur = -1;
+        for (int k = 0; k < nt && !withhold; k++) {
+            const SplitTile tl = gm.tiles[t0 + k];
+            if (tl.a_off == cur) continue;
+            cur = tl.a_off;
+            if (ops > 0 && !wait_bar(&bars->a_free, uint32_t((ops - 1) & 1), wait_limit, fail)) break;
+            const uint32_t bytes = uint32_t((tl.rows + 7) / 8) * 1024;
+            // an operator of at most 64 rows is held twice, in rows 0-63 and
+            // 64-127, so that every TMEM lane quarter holds a result
+            const int copies = tl.rows <= 64 ? 2 : 1;
+            if (lane == 0) {
+                mbar_expect_tx(&bars->a_full, uint32_t(S) * bytes * copies);
+                for (int a = 0; a < S; a++)
+                    for (int cp = 0; cp < copies; cp++)
+                        bulk_g2s(As + a * Sh::kA + cp * (Sh::kA / 2), gm.ops + tl.a_off + int64_t(a) * tl.astride, bytes,
+                                 &bars->a_full);
+            }
+            __syncwarp();
+            ops++;
+        }
+        if (ops > 0) {   // a copy in flight lands before the CTA ends
+            int dummy = 0;
+            wait_bar(&bars->a_full, uint32_t((ops - 1) & 1), wait_limit, &dummy);
+        }
+    } else if (warp < kEpiWarp0) {
+        // kTPC threads per column, each thread the 16-byte pieces j, j + kTPC, ...
+        constexpr int kTPC = kGatherThreads / kN, kPieces = S * 8;
+        static_assert(kTPC * kN == kGatherThreads, "whole columns");
+        const int gt = tid - 32 * kGatherWarp0, c = gt / kTPC, j = gt % kTPC;
+        SplitTile tl{}, tl1{}, tl2{};
+        SplitCol col{}, col1{};
+        int ev = 0;
+        if (nt > 0) tl = gm.tiles[t0];
+        if (nt > 1) tl1 = gm.tiles[t0 + 1];
+        if (nt > 2) tl2 = gm.tiles[t0 + 2];
+        if (c < tl.cnt) col = gm.cols[tl.p0 + c];
+        if (c < tl1.cnt) col1 = gm.cols[tl1.p0 + c];
+        if (j == 0 && c < tl.cnt) ev = gm.dexp[col.vec];
+        for (int k = 0; k <= nt; k++) {
+            if (k < nt) {
+                bool ok = k < kM64 || wait_bar(&bars->meta_empty[k % kM64], uint32_t(((k - kM64) / kM64) & 1), wait_limit, fail);
+                if (ok && k >= kB64) ok = wait_bar(&bars->b_empty[k % kB64], uint32_t(((k - kB64) / kB64) & 1), wait_limit, fail);
+                if (!ok) break;   // uniform over the warp
+                if (c < tl.cnt) {
+                    if (j == 0) meta[(k % kM64) * kN + c] = col_meta<S>(col, ev, inv_alpha_exp);
+                    const uint16_t *src = gm.dig + size_t(col.vec) * (S * 64);
+                    uint8_t *dst = Bs + (k % kB64) * Sh::kBTile + (c >> 3) * 1024 + (c & 7) * 16;
+                    for (int q = j; q < kPieces; q += kTPC)
+                        cp_async16(dst + (q >> 3) * Sh::kBSlice + (q & 7) * 128, src + q * 8);
+                }
+                cp_async_commit();
+            }
+            if (k > 0) {   // tile k - 1 has landed
+                cp_async_wait_pending(k < nt ? 1 : 0);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&bars->b_full[(k - 1) % kB64]);
+                    mbar_arrive(&bars->meta_full[(k - 1) % kM64]);
+                }
+            }
+            // one step of the following tiles' chains
+            tl = tl1;
+            col = col1;
+            if (j == 0 && c < tl.cnt) ev = gm.dexp[col.vec];
+            tl1 = tl2;
+            if (c < tl1.cnt) col1 = gm.cols[tl1.p0 + c];
+            tl2.cnt = 0;
+            if (k + 3 < nt) tl2 = gm.tiles[t0 + k + 3];
+        }
+        cp_async_wait_all();
+    } else {
+        // rows and columns of a warp as in k_split_gemm
+        const int wq = warp & 3, half = (warp - kEpiWarp0) >> 2;
+        SplitTile tl{}, ntl{};
+        if (nt > 0) ntl = gm.tiles[t0];
+        int exp_off = -1, ea = 0;
+        for (int k = 0; k < nt; k++) {
+            tl = ntl;
+            if (k + 1 < nt) ntl = gm.tiles[t0 + k + 1];   // while this tile is worked on
+            const int r = k & 1;
+            const bool small = tl.rows <= 64;
+            const int row = small ? (wq & 1) * 32 + lane : wq * 32 + lane;
+            const bool live = row < tl.rows;
+            if (tl.exp_off != exp_off) {
+                exp_off = tl.exp_off;
+                ea = live ? gm.op_exp[exp_off + row] : 0;
+            }
+            if (!wait_bar(&bars->meta_full[k % kM64], uint32_t((k / kM64) & 1), wait_limit, fail)) break;
+            const int cb = small ? (wq >> 1) * (kN / 2) + half * (kN / 4) : half * (kN / 2);
+            const int ce = min(tl.cnt, cb + (small ? kN / 4 : kN / 2));
+            if (!wait_bar(&bars->job_full[r], uint32_t((k >> 1) & 1), wait_limit, fail)) break;
+            tc_fence_after();
+            epilogue_columns<S, ICVT>(gm, tl, meta + (k % kM64) * kN, tmem + (uint32_t(wq * 32) << 16) + uint32_t(r * kTmemBuf),
+                                      cb, ce, row, live, ea, inv_alpha0);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&bars->job_empty[r]);
+                mbar_arrive(&bars->meta_empty[k % kM64]);
+            }
+        }
+    }
+    if (*fail && tid == 0) atomicExch(err, 1);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+int g_sms = 0;
+// Every tensor-core launch takes more than half of an SM's shared memory, so
+// that no two of their CTAs share an SM (each holds all 512 TMEM columns while
+// it runs).
+constexpr size_t kSmemMin = 116 * 1024, kSmemMax = 227 * 1024;
 template <int KD, int S, bool ICVT>
 constexpr size_t gemm_smem()
 {
-    return KD == 64 ? size_t(kSmem64) : GemmShape<KD, S, (KD == 256 && ICVT) ? 2 : kNBuf>::kSmem;
+    if constexpr (KD == 64) return Shape64<S>::kSmem;
+    else return GemmShape<KD, S, (KD == 256 && ICVT) ? 2 : kNBuf>::kSmem;
+}
+
+template <int KD, int S, bool ICVT>
+constexpr auto gemm_kernel()
+{
+    static_assert(gemm_smem<KD, S, ICVT>() >= kSmemMin && gemm_smem<KD, S, ICVT>() <= kSmemMax, "one tensor CTA per SM");
+    if constexpr (KD == 64) return k_gemm64<S, ICVT>;
+    else return k_split_gemm<KD, S, ICVT>;
 }
 
 template <int KD, int S, bool ICVT>
 cudaError_t prepare_gemm()
 {
-    return cudaFuncSetAttribute(k_split_gemm<KD, S, ICVT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(gemm_kernel<KD, S, ICVT>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 int(gemm_smem<KD, S, ICVT>()));
 }
 
@@ -1008,7 +1222,7 @@ cudaError_t launch_split_gemm(const SplitTables &T, const SplitGemm &g, int kd, 
     int ie = 0;
     const int inv_alpha_exp = std::frexp(inv_alpha0, &ie) == 0.5 ? ie - 1 : kNoExp;
 #define BC_GEMM(KD, S, IC)                                                                                       \
-    launch_pdl(k_split_gemm<KD, S, IC>, grid, kGemmThreads, gemm_smem<KD, S, IC>(), st, g, inv_alpha0,            \
+    launch_pdl(gemm_kernel<KD, S, IC>(), grid, kGemmThreads, gemm_smem<KD, S, IC>(), st, g, inv_alpha0,            \
                inv_alpha_exp, err, T.wait_limit, T.withhold_copy)
     if (T.slices == kWideSlices) {
         if (kd == 256) return BC_GEMM(256, kWideSlices, false);
