@@ -7,7 +7,9 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <new>
+#include <system_error>
 #include <thread>
 
 #include "bc_internal.h"
@@ -550,6 +552,27 @@ struct OpGroup {
     bool exact = true;   // every row keeps the accumulation bound of the format
 };
 
+// f(0) .. f(n-1), on threads of their own where they can be had; an exception
+// is passed on (the first one) once all have ended.
+template <class F> void in_parallel(int n, const F &f)
+{
+    std::vector<std::exception_ptr> err(n);
+    auto one = [&](int i) {
+        try { f(i); } catch (...) { err[i] = std::current_exception(); }
+    };
+    std::vector<std::thread> th;
+    th.reserve(n);
+    int i = 1;
+    for (; i < n; i++) {
+        try { th.emplace_back(one, i); } catch (const std::system_error &) { break; }
+    }
+    for (int k = i; k < n; k++) one(k);
+    one(0);
+    for (auto &t : th) t.join();
+    for (auto &e : err)
+        if (e) std::rethrow_exception(e);
+}
+
 // Appends the BF16 digits of a real operator (rows x K, row-major) in the
 // chunk layout [digit a][row half h][K chunk kc] x (128 rows x KC) of
 // canonical K-major core matrices, its row exponents and (7 digits) its
@@ -591,10 +614,7 @@ SplitOp add_split_op(OpGroup &G, const std::vector<double> &m, int rows)
     const int nt = size_t(rows) * K > 8192 ? 8 : 1;
     bool ok[8];
     std::fill(ok, ok + 8, true);
-    std::vector<std::thread> th;
-    for (int t = 1; t < nt; t++) th.emplace_back(part, rows * t / nt, rows * (t + 1) / nt, &ok[t]);
-    part(0, rows / nt, &ok[0]);
-    for (auto &t : th) t.join();
+    in_parallel(nt, [&](int t) { part(rows * t / nt, rows * (t + 1) / nt, &ok[t]); });
     for (bool v : ok) G.exact = G.exact && v;
     return op;
 }
@@ -817,42 +837,28 @@ bc_status build_split_tables(bc_ctx *ctx)
     return e == cudaSuccess ? BC_OK : cuda_fail(e, "split kernel attributes");
 }
 
-// Column lists of the digit products for one tree.  Tiles hold up to `cap`
-// columns that share one operator; tiles of 256-row operators come first
-// (longest work first).
-struct TileBuilder {
-    int cap;
-    bool halves;   // K = 64
-    std::vector<SplitTile> tiles;
-    std::vector<SplitCol> cols;
-    TileBuilder(const SplitTables &T, int K) : cap(T.tileN), halves(K == 64) {}
-    // one operator, its columns given in order
-    void add(const SplitOp &op, const std::vector<SplitCol> &c)
-    {
-        const int mh = op.rows > 128 ? 2 : 1;
-        for (int h = 0; h < (halves ? mh : 1); h++) {
-            for (size_t i = 0; i < c.size(); i += cap) {
-                SplitTile t;
-                t.a_off = op.a_off + int64_t(h) * kHalfBytes;
-                t.f_off = op.f_off + 128 * h;
-                t.rows = halves ? std::min(128, op.rows - 128 * h) : op.rows;
-                t.exp_off = op.exp_off + 128 * h;
-                t.p0 = int32_t(cols.size());
-                t.cnt = int32_t(std::min<size_t>(cap, c.size() - i));
-                t.astride = mh * kHalfBytes;
-                t.frows = op.rows;
-                for (int q = 0; q < t.cnt; q++) {
-                    cols.push_back(c[i + q]);
-                    cols.back().out += 128 * h;
-                }
-                tiles.push_back(t);
-            }
+// Tiles of the digit products: up to tileN consecutive columns that share one
+// operator (columns [p0, p0 + n) of a list belong to `op`).
+constexpr int kHalfBytes = 128 * 64 * 2;   // one digit of a 128-row half at K = 64
+void add_tiles(std::vector<SplitTile> &tiles, const SplitOp &op, int64_t p0, int64_t n, int tileN, bool halves)
+{
+    const int mh = op.rows > 128 ? 2 : 1;
+    for (int h = 0; h < (halves ? mh : 1); h++) {
+        for (int64_t i = 0; i < n; i += tileN) {
+            SplitTile t{};
+            t.a_off = op.a_off + int64_t(h) * kHalfBytes;
+            t.f_off = op.f_off + 128 * h;
+            t.rows = halves ? std::min(128, op.rows - 128 * h) : op.rows;
+            t.exp_off = op.exp_off + 128 * h;
+            t.p0 = int32_t(p0 + i);
+            t.cnt = int32_t(std::min<int64_t>(tileN, n - i));
+            t.astride = mh * kHalfBytes;
+            t.frows = op.rows;
+            t.row0 = 128 * h;
+            tiles.push_back(t);
         }
     }
-    static constexpr int kHalfBytes = 128 * 64 * 2;   // one digit of a 128-row half at K = 64
-};
-
-inline int32_t col_ctl(int shift, bool inv_alpha) { return int32_t(shift * 2 + (inv_alpha ? 1 : 0)); }
+}
 
 // The internal stream and its events, one set per tree (applies of one tree
 // are serialised by the caller, those of different trees are not).
@@ -874,160 +880,162 @@ void free_side(bc_tree *t)
     t->side = SideStream();
 }
 
-// V-list tiles (tensor-core M2L, part 32): one column per V pair (source box
-// digits, the result row into Pv; the adjoint digits carry alpha0).
-TileBuilder m2l_tiles(const bc_tree *t, const SplitTables &T, int dir, double2 *Pv)
+// Entries 0..n-1 ordered by code (stable counting sort); counts per code.
+std::vector<int32_t> order_by_code(const std::vector<int32_t> &code, int ncodes, std::vector<int64_t> &count)
 {
-    const HostTree &h = t->h;
-    const int P1 = t->ctx->P1, first_which = dir == 1 ? 1 : 0;   // expA = 0, expB = 1
-    const int64_t nbox = int64_t(h.box_level.size());
-    TileBuilder M(T, kSplitKE);
-    std::vector<std::vector<SplitCol>> by_v(kNumV);
-    for (size_t k = 0; k < h.v_src.size(); k++) {
-        SplitCol c;
-        c.vec = int32_t(first_which * nbox + h.v_src[k]);
-        c.ctl = col_ctl(0, dir == 1);
-        c.out = reinterpret_cast<double *>(Pv + k * size_t(P1));
-        by_v[h.v_code[k]].push_back(c);
-    }
-    for (int c = 0; c < kNumV; c++)
-        if (!by_v[c].empty()) M.add(T.m2l_op[dir][c], by_v[c]);
-    return M;
+    count.assign(ncodes, 0);
+    for (int32_t c : code) count[c]++;
+    std::vector<int64_t> at(ncodes, 0);
+    for (int c = 1; c < ncodes; c++) at[c] = at[c - 1] + count[c - 1];
+    std::vector<int32_t> out(code.size());
+    for (size_t k = 0; k < code.size(); k++) out[at[code[k]]++] = int32_t(k);
+    return out;
 }
 
-// Tiles, digit buffers and result rows of a tree in the format of T.  The two
-// formats share the result rows.
-cudaError_t build_digit_tree(bc_tree *t, const SplitTables &T, SplitTree &s, bool m2l)
+cudaError_t build_tile_order(bc_tree *t)
 {
+    TileOrder &o = t->order;
+    if (o.ready) return cudaSuccess;
+    const HostTree &h = t->h;
+    std::vector<int32_t> near, x, w, v, l2p;
+    auto rest = [&] {
+        near = order_by_code(h.near_tab, kNumNear, o.n_near);
+        x = order_by_code(h.x_code, kNumWX, o.n_x);
+        w = order_by_code(h.w_code, kNumWX, o.n_w);
+        for (int32_t k : h.leaf_order)
+            if (h.leaf_level[k] >= 2) l2p.push_back(k);
+    };
+    auto vlist = [&] { v = order_by_code(h.v_code, kNumV, o.n_v); };   // the longest list, beside the others
+    in_parallel(h.v_code.size() > 50000 ? 2 : 1, [&](int i) { if (i) vlist(); else rest(); });
+    if (h.v_code.size() <= 50000) vlist();
+    o.n_l2p = int64_t(l2p.size());
+    DevArena up;
+    up.add(&o.near, near);
+    up.add(&o.x, x);
+    up.add(&o.w, w);
+    up.add(&o.v, v);
+    up.add(&o.l2p, l2p);
+    const cudaError_t e = up.commit(t->d.allocs, t->side.side);
+    o.ready = e == cudaSuccess;
+    return e;
+}
+
+// Tiles, digit buffers and result rows of a tree in the format of T (the two
+// formats share the result rows), with the M2L's where m2l is set.  The host
+// orders the lists and cuts them into tiles; the columns (16 bytes per entry
+// and direction) are written by the device.
+cudaError_t build_digit_tree(bc_tree *t, const SplitTables &T, SplitTree &s, bool m2l)
+try {
     const HostTree &h = t->h;
     const int P1 = t->ctx->P1, S = T.slices;
     const int64_t nn = int64_t(h.near_src.size()), nx = int64_t(h.x_src.size()), nw = int64_t(h.w_src.size());
-    const int64_t nbox = int64_t(h.box_level.size());
+    const int64_t nv = int64_t(h.v_src.size()), nbox = int64_t(h.box_level.size());
     cudaError_t e = ensure_side(t);
+    if (e == cudaSuccess) e = build_tile_order(t);
     if (e != cudaSuccess) return e;
+    const TileOrder &o = t->order;
     const size_t NP = size_t(T.np), KV = size_t(T.kv);   // nodes per leaf, group-V K
-    // device room first: the tiles hold the result rows' addresses
-    std::vector<void *> &al = t->d.allocs;
-    const size_t mark = al.size();
-    const SplitTree &o = &s == &t->sp ? t->spw : t->sp;
+    std::vector<SplitTile> vn, en, mn;
     SplitTree n;
+    int64_t p0 = 0;
+    for (int c = 0; c < kNumNear; c++) {
+        if (o.n_near[c]) add_tiles(vn, T.near_op[0][c], p0, o.n_near[c], T.tileN, KV == 64);
+        p0 += o.n_near[c];
+    }
+    n.ntN = int(vn.size());
+    add_tiles(vn, T.leafA_op[0], p0, h.nleaf, T.tileN, KV == 64);
+    n.ntA = int(vn.size()) - n.ntN;
+    p0 += h.nleaf;
+    for (int c = 0; c < kNumWX; c++) {
+        if (o.n_x[c]) add_tiles(vn, T.x_op[0][c], p0, o.n_x[c], T.tileN, KV == 64);
+        p0 += o.n_x[c];
+    }
+    n.ntVN = int(vn.size());
+    add_tiles(en, T.e_op[0], 0, o.n_l2p, T.tileN, true);
+    n.ntL = int(en.size());
+    p0 = o.n_l2p;
+    for (int c = 0; c < kNumWX; c++) {
+        if (o.n_w[c]) add_tiles(en, T.w_op[0][c], p0, o.n_w[c], T.tileN, true);
+        p0 += o.n_w[c];
+    }
+    n.ntE = int(en.size());
+    p0 = 0;
+    for (int c = 0; c < kNumV && m2l; c++) {
+        if (o.n_v[c]) add_tiles(mn, T.m2l_op[0][c], p0, o.n_v[c], T.tileN, true);
+        p0 += o.n_v[c];
+    }
+    n.ntM = int(mn.size());
+    const SplitTree &other = &s == &t->sp ? t->spw : t->sp;
     double2 *Pv = t->d.Pv;
-    {
-        DevArena room;
-        if (o.Pnear) {
-            n.Pnear = o.Pnear; n.PX = o.PX; n.PE = o.PE; n.PW = o.PW;
-        } else {
-            room.room(&n.Pnear, size_t(nn) * NP);
-            room.room(&n.PX, size_t(nx) * kSplitKE);
-            room.room(&n.PE, size_t(h.nleaf) * NP);
-            room.room(&n.PW, size_t(nw) * NP);
-        }
-        if (m2l && !Pv) room.room(&Pv, h.v_src.size() * size_t(P1));
-        room.room(&n.vdig, size_t(h.nleaf) * S * KV);
-        room.room(&n.vexp, size_t(h.nleaf));
-        room.room(&n.edig, size_t(2 * nbox) * S * kSplitKE);
-        room.room(&n.eexp, size_t(2 * nbox));
-        if ((e = room.commit(al, t->side.side)) != cudaSuccess) return e;
-    }
-    // owners of the near and W entries, box of each X entry
-    std::vector<int32_t> near_owner(nn), w_owner(nw), x_box(nx);
-    for (int64_t o2 = 0; o2 < h.nleaf; o2++) {
-        for (int32_t k = h.near_ptr[o2]; k < h.near_ptr[o2 + 1]; k++) near_owner[k] = int32_t(o2);
-        for (int32_t k = h.w_ptr[o2]; k < h.w_ptr[o2 + 1]; k++) w_owner[k] = int32_t(o2);
-    }
-    for (int64_t b = 0; b < nbox; b++)
-        for (int32_t k = h.x_ptr[b]; k < h.x_ptr[b + 1]; k++) x_box[k] = int32_t(b);
     DevArena up;
-    std::vector<TileBuilder> keep;   // [dir]: VN, V, N, E, M (alive until the upload)
-    keep.reserve(10);
-    for (int dir = 0; dir < 2; dir++) {
-        const bool adj = dir == 1;
-        double2 *first = adj ? t->d.expB : t->d.expA;
-        const int first_which = adj ? 1 : 0, second_which = adj ? 0 : 1;   // expA = 0, expB = 1
-        TileBuilder V(T, T.kv), NV(T, T.kv), E(T, kSplitKE);
-        // near entries, by table
-        std::vector<std::vector<SplitCol>> by_tab(kNumNear);
-        for (int64_t k = 0; k < nn; k++) {
-            const int32_t src = h.near_src[k], own = near_owner[k];
-            SplitCol c;
-            c.vec = src;
-            c.ctl = col_ctl(-2 * (adj ? h.leaf_level[own] : h.leaf_level[src]), false);
-            c.out = n.Pnear + size_t(k) * NP;
-            by_tab[h.near_tab[k]].push_back(c);
-        }
-        for (int tab = 0; tab < kNumNear; tab++)
-            if (!by_tab[tab].empty()) NV.add(T.near_op[dir][tab], by_tab[tab]);
-        // leafA of every leaf (Morton order), then the X entries by code
-        std::vector<SplitCol> cl;
-        for (int64_t i = 0; i < h.nleaf; i++) {
-            const int32_t o2 = h.leaf_order[i];
-            SplitCol c;
-            c.vec = o2;
-            c.ctl = adj ? col_ctl(0, true) : col_ctl(-2 * h.leaf_level[o2], false);
-            c.out = reinterpret_cast<double *>(first + size_t(h.leaf_box[o2]) * P1);
-            cl.push_back(c);
-        }
-        V.add(T.leafA_op[dir], cl);
-        n.ntA[dir] = int(V.tiles.size());
-        std::vector<std::vector<SplitCol>> by_code(kNumWX);
-        for (int64_t k = 0; k < nx; k++) {
-            SplitCol c;
-            c.vec = h.x_src[k];
-            c.ctl = adj ? col_ctl(0, true) : col_ctl(-2 * (h.box_level[x_box[k]] - 1), false);
-            c.out = n.PX + size_t(k) * kSplitKE;
-            by_code[h.x_code[k]].push_back(c);
-        }
-        for (int c = 0; c < kNumWX; c++)
-            if (!by_code[c].empty()) V.add(T.x_op[dir][c], by_code[c]);
-        // group E: L2P of the leaves at level >= 2, then the W entries by code
-        cl.clear();
-        for (int64_t i = 0; i < h.nleaf; i++) {
-            const int32_t o2 = h.leaf_order[i];
-            if (h.leaf_level[o2] < 2) continue;
-            SplitCol c;
-            c.vec = int32_t(second_which * nbox + h.leaf_box[o2]);
-            c.ctl = col_ctl(adj ? -2 * h.leaf_level[o2] : 0, false);
-            c.out = n.PE + size_t(o2) * NP;
-            cl.push_back(c);
-        }
-        E.add(T.e_op[dir], cl);
-        n.ntL[dir] = int(E.tiles.size());
-        for (auto &v : by_code) v.clear();
-        for (int64_t k = 0; k < nw; k++) {
-            SplitCol c;
-            c.vec = int32_t(first_which * nbox + h.w_src[k]);
-            c.ctl = col_ctl(adj ? -2 * h.leaf_level[w_owner[k]] : 0, false);
-            c.out = n.PW + size_t(k) * NP;
-            by_code[h.w_code[k]].push_back(c);
-        }
-        for (int c = 0; c < kNumWX; c++)
-            if (!by_code[c].empty()) E.add(T.w_op[dir][c], by_code[c]);
-        TileBuilder VN = NV;   // near tiles first (longest), then the far ones
-        for (SplitTile tl : V.tiles) {
-            tl.p0 += int32_t(NV.cols.size());
-            VN.tiles.push_back(tl);
-        }
-        VN.cols.insert(VN.cols.end(), V.cols.begin(), V.cols.end());
-        auto put = [&](TileBuilder &&b, SplitTile **tiles, SplitCol **cols, int *nt) {
-            *nt = int(b.tiles.size());
-            keep.push_back(std::move(b));
-            up.add(tiles, keep.back().tiles);
-            up.add(cols, keep.back().cols);
-        };
-        put(std::move(VN), &n.tVN[dir], &n.cVN[dir], &n.ntVN[dir]);
-        put(std::move(V), &n.tV[dir], &n.cV[dir], &n.ntV[dir]);
-        put(std::move(NV), &n.tN[dir], &n.cN[dir], &n.ntN[dir]);
-        put(std::move(E), &n.tE[dir], &n.cE[dir], &n.ntE[dir]);
-        if (m2l) put(m2l_tiles(t, T, dir, Pv), &n.tM[dir], &n.cM[dir], &n.ntM[dir]);
+    up.add(&n.tVN, vn);
+    up.add(&n.tE, en);
+    if (m2l) up.add(&n.tM, mn);
+    if (s.Pnear) {   // set up before without the M2L
+        n = SplitTree(s);
+        n.ntM = int(mn.size());
+        up.items.clear();
+        up.add(&n.tM, mn);
+    } else if (other.Pnear) {
+        n.Pnear = other.Pnear; n.PX = other.PX; n.PE = other.PE; n.PW = other.PW;
+    } else {
+        up.room(&n.Pnear, size_t(nn) * NP);
+        up.room(&n.PX, size_t(nx) * kSplitKE);
+        up.room(&n.PE, size_t(h.nleaf) * NP);
+        up.room(&n.PW, size_t(nw) * NP);
     }
-    if ((e = up.commit(al, t->side.side)) != cudaSuccess) {
-        while (al.size() > mark) { cudaFree(al.back()); al.pop_back(); }
+    if (!s.Pnear) {
+        up.room(&n.vdig, size_t(h.nleaf) * S * KV);
+        up.room(&n.vexp, size_t(h.nleaf));
+        up.room(&n.edig, size_t(2 * nbox) * S * kSplitKE);
+        up.room(&n.eexp, size_t(2 * nbox));
+        for (int dir = 0; dir < 2; dir++) {
+            up.room(&n.cVN[dir], size_t(nn + h.nleaf + nx));
+            up.room(&n.cE[dir], size_t(o.n_l2p + nw));
+        }
+    }
+    if (m2l) {
+        if (!Pv) up.room(&Pv, size_t(nv) * P1);
+        for (int dir = 0; dir < 2; dir++) up.room(&n.cM[dir], size_t(nv));
+    }
+    if ((e = up.commit(t->d.allocs, t->side.side)) != cudaSuccess) return e;
+    ColLists cl;
+    cl.nleaf = h.nleaf;
+    cl.near_ptr = t->d.near_ptr; cl.near_src = t->d.near_src;
+    cl.w_ptr = t->d.w_ptr; cl.w_src = t->d.w_src;
+    cl.x_src = t->d.x_src; cl.x_box = t->d.x_box;
+    cl.v_src = t->d.v_src;
+    cl.leaf_level = t->d.leaf_level; cl.leaf_box = t->d.leaf_box; cl.box_level = t->d.box_level;
+    auto seg = [&](ColKind k, int dir, int64_t cnt, const int32_t *perm, SplitCol *cols, double *out, int64_t stride,
+                   int64_t vec0) {
+        if (cnt > 0) cl.seg[cl.nseg++] = ColSeg{k, dir, cnt, perm, cols, out, stride, vec0};
+    };
+    for (int dir = 0; dir < 2; dir++) {
+        // expA holds the multipoles (adjoint: the second array), expB the locals
+        double *first = reinterpret_cast<double *>(dir ? t->d.expB : t->d.expA);
+        const int64_t f0 = dir ? nbox : 0, s0 = dir ? 0 : nbox;
+        if (!s.Pnear) {
+            seg(ColKind::Near, dir, nn, o.near, n.cVN[dir], n.Pnear, int64_t(NP), 0);
+            seg(ColKind::LeafA, dir, h.nleaf, t->d.leaf_order, n.cVN[dir] + nn, first, 2 * P1, 0);
+            seg(ColKind::X, dir, nx, o.x, n.cVN[dir] + nn + h.nleaf, n.PX, kSplitKE, 0);
+            seg(ColKind::L2P, dir, o.n_l2p, o.l2p, n.cE[dir], n.PE, int64_t(NP), s0);
+            seg(ColKind::W, dir, nw, o.w, n.cE[dir] + o.n_l2p, n.PW, int64_t(NP), f0);
+        }
+        if (m2l) seg(ColKind::V, dir, nv, o.v, n.cM[dir], reinterpret_cast<double *>(Pv), 2 * P1, f0);
+    }
+    e = launch_make_cols(cl, t->side.side);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(t->side.side);
+    if (e != cudaSuccess) {
+        cudaFree(t->d.allocs.back());
+        t->d.allocs.pop_back();
         return e;
     }
     n.err = t->ctx->dev_err;
     s = n;
     t->d.Pv = Pv;
     return cudaSuccess;
+} catch (const std::bad_alloc &) {
+    return cudaErrorMemoryAllocation;
 }
 
 bc_status build_split_tree(bc_tree *t)
@@ -1044,23 +1052,8 @@ bc_status build_split_tree(bc_tree *t)
 bc_status build_split_m2l(bc_tree *t)
 {
     if (t->m2l_ready) return BC_OK;
-    SplitTree &s = t->sp;
-    std::vector<void *> &al = t->d.allocs;
-    cudaError_t e = cudaSuccess;
-    if (!t->d.Pv) {
-        DevArena room;
-        room.room(&t->d.Pv, t->h.v_src.size() * size_t(t->ctx->P1));
-        if ((e = room.commit(al, t->side.side)) != cudaSuccess) return cuda_fail(e, "tensor-core M2L rows");
-    }
-    TileBuilder M0 = m2l_tiles(t, t->ctx->split, 0, t->d.Pv), M1 = m2l_tiles(t, t->ctx->split, 1, t->d.Pv);
-    DevArena up;
-    up.add(&s.tM[0], M0.tiles);
-    up.add(&s.cM[0], M0.cols);
-    up.add(&s.tM[1], M1.tiles);
-    up.add(&s.cM[1], M1.cols);
-    if ((e = up.commit(al, t->side.side)) != cudaSuccess) return cuda_fail(e, "tensor-core M2L tiles");
-    s.ntM[0] = int(M0.tiles.size());
-    s.ntM[1] = int(M1.tiles.size());
+    const cudaError_t e = build_digit_tree(t, t->ctx->split, t->sp, true);
+    if (e != cudaSuccess) return cuda_fail(e, "tensor-core M2L tiles");
     t->m2l_ready = true;
     return BC_OK;
 }
@@ -1075,12 +1068,7 @@ bool build_wide_tree(bc_tree *t)
     if (t->wide_off || !t->ctx->wide_ready) return false;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return false; }
-    cudaError_t e;
-    try {
-        e = build_digit_tree(t, t->ctx->wide, t->spw, true);
-    } catch (const std::bad_alloc &) {
-        e = cudaErrorMemoryAllocation;
-    }
+    const cudaError_t e = build_digit_tree(t, t->ctx->wide, t->spw, true);
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -260,6 +260,7 @@ struct SplitTile {
     int32_t rows, exp_off; // rows of the tile; row exponents
     int32_t p0, cnt;       // columns [p0, p0 + cnt)
     int32_t astride, frows;   // bytes between digits (K = 64); rows of the operator
+    int32_t row0, pad;        // first row of the tile in the columns' results
 };
 // One column = one input vector and where its result rows go.
 struct SplitCol {
@@ -283,17 +284,43 @@ struct SplitGemm {
     double scale = 1.0;
     int kvalid = 0;
 };
+// One segment of a column list: the entries perm[0..n) of one kind in order,
+// written as columns by the device.
+enum class ColKind : int { Near, LeafA, X, L2P, W, V };
+struct ColSeg {
+    ColKind kind;
+    int dir;                       // 0 forward, 1 adjoint
+    int64_t n;
+    const int32_t *perm;           // entry (near, X, W, V lists) or leaf (LeafA, L2P)
+    SplitCol *cols;
+    double *out;                   // result rows: entry or leaf e at out + e * stride (LeafA: its box)
+    int64_t stride;
+    int64_t vec0;                  // added to the vector index
+};
+constexpr int kMaxColSegs = 12;
+struct ColLists {                  // the tree arrays the columns are made from
+    ColSeg seg[kMaxColSegs];
+    int nseg = 0;
+    int64_t nleaf = 0;
+    const int32_t *near_ptr, *near_src, *w_ptr, *w_src, *x_src, *x_box, *v_src, *leaf_level, *leaf_box, *box_level;
+};
+cudaError_t launch_make_cols(const ColLists &cl, cudaStream_t st);
+// Entries of a tree's lists ordered by operator (device), with the counts per
+// operator (host): the same for both directions and both digit formats.
+struct TileOrder {
+    bool ready = false;
+    int32_t *near = nullptr, *x = nullptr, *w = nullptr, *v = nullptr, *l2p = nullptr;
+    std::vector<int64_t> n_near, n_x, n_w, n_v;
+    int64_t n_l2p = 0;
+};
 struct SplitTree {
-    // [forward, adjoint]; group V as far part (leafA, X list: needed by the
-    // upward and downward passes) and near part (needed at the leaf output),
-    // launched apart when the near part runs on the side stream, and as one
-    // list (near tiles first: two jobs each) otherwise; group E (L2P / P2M^H,
-    // W list); group M: the V-list translations (M2L) by offset code
-    SplitTile *tV[2] = {}, *tN[2] = {}, *tVN[2] = {}, *tE[2] = {}, *tM[2] = {};
-    SplitCol *cV[2] = {}, *cN[2] = {}, *cVN[2] = {}, *cE[2] = {}, *cM[2] = {};
-    int ntV[2] = {}, ntN[2] = {}, ntVN[2] = {}, ntE[2] = {}, ntM[2] = {};
-    int ntA[2] = {};   // the first ntA tiles of tV: leaf-to-expansion (the rest: X list)
-    int ntL[2] = {};   // the first ntL tiles of tE: expansion-to-leaf (the rest: W list)
+    // tiles (the same for both directions) and columns [forward, adjoint].
+    // Group V: the near tiles (ntN, two jobs each: first), then leaf-to-
+    // expansion (ntA) and the X list; group E: expansion-to-leaf (ntL), then the
+    // W list; group M: the V-list translations (M2L) by offset code
+    SplitTile *tVN = nullptr, *tE = nullptr, *tM = nullptr;
+    SplitCol *cVN[2] = {}, *cE[2] = {}, *cM[2] = {};
+    int ntVN = 0, ntN = 0, ntA = 0, ntE = 0, ntL = 0, ntM = 0;
     double *Pnear = nullptr;      // [n_near][p^2] near-field result per entry (scale included)
     double *PX = nullptr;         // [n_x][64] X-list result per entry
     double *PE = nullptr;         // [nleaf][p^2] L2P (adjoint P2M^H) result per leaf
@@ -331,6 +358,9 @@ struct SplitLaunch {
     int parts = kSplitTableParts;
     const struct SideStream *side = nullptr;   // null: the near-field launch stays on the apply's stream
     int near_ctas = 0;                          // CTAs of the near-field launch on the side stream (0: all SMs)
+    // part 32 in another format (the split mode's M2L on 7 digits); null: the same
+    const SplitTables *m2l_tables = nullptr;
+    const SplitTree *m2l_tree = nullptr;
 };
 // Digits of the leaf vectors (times scale), of the two expansion arrays
 // (times scale), and the tensor-core operator products of one group, in the
@@ -526,6 +556,7 @@ struct bc_tree {
     bool is_union = false;   // the union tree of a batch
     bc::HostTree h;
     bc::DevTree d;
+    bc::TileOrder order;      // list entries by operator
     bc::SplitTree sp, spw;    // tiles of the 5-digit and the 7-digit products
     bc::SideStream side;
     bool split_ready = false, wide_ready = false;

@@ -1485,6 +1485,9 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
     auto digits_exp = [&](int64_t i0, int64_t i1, cudaStream_t s) {
         return launch_split_digits_exp(*sT, dir, i0, i1, a.nbox, d.expA, d.expB, P1, escl, sp->edig, sp->eexp, s);
     };
+    // the tensor-core M2L's format
+    const SplitTables *mT = split && split->m2l_tables ? split->m2l_tables : sT;
+    const SplitTree *mp = split && split->m2l_tables ? split->m2l_tree : sp;
     const bool leaf_tc = (parts & 2) != 0;
     // Late fork: with the M2L in FP64 (part 32 off) the internal stream's
     // tensor launches (X list, near field) start after the upward pass and run
@@ -1505,7 +1508,7 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             e = digits_vec(sd->side);
             if (e != cudaSuccess) return e;
         }
-        SplitGemm g = group_v(sp->tV[dir] + sp->ntA[dir], sp->cV[dir], sp->ntV[dir] - sp->ntA[dir]);
+        SplitGemm g = group_v(sp->tVN + sp->ntN + sp->ntA, sp->cVN[dir], sp->ntVN - sp->ntN - sp->ntA);
         e = launch_split_gemm(*sT, g, sT->kv, 1.0 / alpha0, sp->err, sd->side, late);
         if (e != cudaSuccess) return e;
         if ((e = cudaEventRecord(sd->xdone, sd->side)) != cudaSuccess) return e;
@@ -1516,11 +1519,11 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             const int64_t f0 = adj ? a.nbox : 0;
             e = digits_exp(f0, f0 + a.nbox, sd->side);
             if (e != cudaSuccess) return e;
-            e = launch_split_gemm(*sT, group_e(sp->tE[dir] + sp->ntL[dir], sp->cE[dir], sp->ntE[dir] - sp->ntL[dir]),
+            e = launch_split_gemm(*sT, group_e(sp->tE + sp->ntL, sp->cE[dir], sp->ntE - sp->ntL),
                                   kSplitKE, 1.0 / alpha0, sp->err, sd->side, true);
             if (e != cudaSuccess) return e;
         }
-        g = group_v(sp->tN[dir], sp->cN[dir], sp->ntN[dir]);
+        g = group_v(sp->tVN, sp->cVN[dir], sp->ntN);
         g.max_ctas = split->near_ctas;
         e = launch_split_gemm(*sT, g, sT->kv, 1.0 / alpha0, sp->err, sd->side, late);
         if (e != cudaSuccess) return e;
@@ -1537,7 +1540,7 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             // leaf-to-expansion and X-list tiles
             ce = digits_vec(st);
             if (ce != cudaSuccess) return ce;
-            ce = launch_split_gemm(*sT, group_v(sp->tVN[dir], sp->cVN[dir], sp->ntVN[dir]), sT->kv, 1.0 / alpha0,
+            ce = launch_split_gemm(*sT, group_v(sp->tVN, sp->cVN[dir], sp->ntVN), sT->kv, 1.0 / alpha0,
                                    sp->err, st);
             if (ce != cudaSuccess) return ce;
             if (ev) {
@@ -1555,7 +1558,7 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             }
             if (!late && (ce = side_launches()) != cudaSuccess) return ce;
             if (leaf_tc) {
-                ce = launch_split_gemm(*sT, group_v(sp->tV[dir], sp->cV[dir], sp->ntA[dir]), sT->kv, 1.0 / alpha0,
+                ce = launch_split_gemm(*sT, group_v(sp->tVN + sp->ntN, sp->cVN[dir], sp->ntA), sT->kv, 1.0 / alpha0,
                                        sp->err, st);
                 if (ce != cudaSuccess) return ce;
             }
@@ -1608,11 +1611,12 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
             // tensor group M: digits of `first` (times alpha0 in the adjoint),
             // then every pair's translation but its log term
             const int64_t f0 = adj ? a.nbox : 0;
-            ce = digits_exp(f0, f0 + a.nbox, st);
+            ce = launch_split_digits_exp(*mT, dir, f0, f0 + a.nbox, a.nbox, d.expA, d.expB, P1, escl, mp->edig, mp->eexp, st);
             if (ce != cudaSuccess) return ce;
             first_digits = true;
-            ce = launch_split_gemm(*sT, group_e(sp->tM[dir], sp->cM[dir], sp->ntM[dir]), kSplitKE, 1.0 / alpha0,
-                                   sp->err, st);
+            ce = launch_split_gemm(*mT, gemm_group_e(*mT, *mp, dir, mp->tM, mp->cM[dir], mp->ntM, d.expA, d.expB,
+                                                     a.nbox, P1, escl),
+                                   kSplitKE, 1.0 / alpha0, mp->err, st);
             if (ce != cudaSuccess) return ce;
             if (!dfp) {
                 // the FP64 downward pass takes each box's V-list sum, as the FP64 M2L writes it
@@ -1706,11 +1710,11 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
         // adjoint; those of `first` already taken for the M2L or, late fork,
         // on the internal stream), then L2P (P2M^H) of `second` into PE and
         // the W list of `first` into PW (late fork: L2P only)
-        const bool first_done = first_digits || late;
+        const bool first_done = (first_digits && mT == sT) || late;
         const int64_t s0 = first_done ? (adj ? 0 : a.nbox) : 0, s1 = first_done ? s0 + a.nbox : 2 * a.nbox;
         ce = digits_exp(s0, s1, st);
         if (ce != cudaSuccess) return ce;
-        ce = launch_split_gemm(*sT, group_e(sp->tE[dir], sp->cE[dir], late ? sp->ntL[dir] : sp->ntE[dir]), kSplitKE,
+        ce = launch_split_gemm(*sT, group_e(sp->tE, sp->cE[dir], late ? sp->ntL : sp->ntE), kSplitKE,
                                1.0 / alpha0, sp->err, st);
         if (ce != cudaSuccess) return ce;
     }

@@ -397,7 +397,7 @@ cudaError_t launch_layer(const PassArgs &a, const HostTree &h, const DevTree &d,
         const int64_t nbox = a.nbox;
         e = launch_split_digits_exp(*sT, 0, nbox, 2 * nbox, nbox, d.expA, d.expB, P1, 1.0, sp->edig, sp->eexp, st);
         if (e != cudaSuccess) return e;
-        e = launch_split_gemm(*sT, gemm_group_e(*sT, *sp, 0, sp->tE[0], sp->cE[0], sp->ntL[0], d.expA, d.expB, nbox, P1,
+        e = launch_split_gemm(*sT, gemm_group_e(*sT, *sp, 0, sp->tE, sp->cE[0], sp->ntL, d.expA, d.expB, nbox, P1,
                                                 1.0),
                               kSplitKE, 1.0 / (a.half_L * a.half_L), sp->err, st);
         if (e != cudaSuccess) return e;

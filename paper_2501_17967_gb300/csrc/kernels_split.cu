@@ -583,7 +583,7 @@ __device__ __forceinline__ void epilogue_columns(const SplitGemm &gm, const Spli
                 val = ICVT ? i64_scaled_int(sum, ea + M[c].exp) : i64_scaled(sum, ea + M[c].exp);
                 if (M[c].flag) val *= inv_alpha0;
             }
-            M[c].out[row] = val;
+            M[c].out[tl.row0 + row] = val;
         }
     }
 }
@@ -1188,6 +1188,71 @@ SplitGemm gemm_group_e(const SplitTables &T, const SplitTree &s, int dir, const 
     g.scale = scale;
     g.kvalid = 2 * P1;
     return g;
+}
+
+namespace {
+
+// Columns of the segments (blockIdx.y), one entry per thread.
+__global__ void __launch_bounds__(256) k_make_cols(const __grid_constant__ ColLists cl)
+{
+    const ColSeg &s = cl.seg[blockIdx.y];
+    const bool adj = s.dir == 1;
+    // the leaf whose list holds entry e: the last with ptr[leaf] <= e
+    auto owner = [&](const int32_t *ptr, int e) {
+        int64_t lo = 0, hi = cl.nleaf - 1;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (ptr[mid] <= e) lo = mid; else hi = mid - 1;
+        }
+        return int(lo);
+    };
+    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < s.n; i += int64_t(gridDim.x) * blockDim.x) {
+        const int e = s.perm[i];
+        int vec = e, shift = 0, inv = 0;   // power-of-two factor r^2 / r_0^2, or the factor 1/alpha0
+        int64_t at = e;
+        switch (s.kind) {
+        case ColKind::Near:
+            vec = cl.near_src[e];
+            shift = -2 * cl.leaf_level[adj ? owner(cl.near_ptr, e) : vec];
+            break;
+        case ColKind::LeafA:
+            if (adj) inv = 1; else shift = -2 * cl.leaf_level[e];
+            at = cl.leaf_box[e];
+            break;
+        case ColKind::X:
+            vec = cl.x_src[e];
+            if (adj) inv = 1; else shift = -2 * (cl.box_level[cl.x_box[e]] - 1);
+            break;
+        case ColKind::L2P:
+            vec = cl.leaf_box[e];
+            if (adj) shift = -2 * cl.leaf_level[e];
+            break;
+        case ColKind::W:
+            vec = cl.w_src[e];
+            if (adj) shift = -2 * cl.leaf_level[owner(cl.w_ptr, e)];
+            break;
+        case ColKind::V:
+            vec = cl.v_src[e];
+            inv = adj;
+            break;
+        }
+        SplitCol c;
+        c.vec = int32_t(s.vec0 + vec);
+        c.ctl = shift * 2 + inv;
+        c.out = s.out + at * s.stride;
+        s.cols[i] = c;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_make_cols(const ColLists &cl, cudaStream_t st)
+{
+    int64_t n = 0;
+    for (int i = 0; i < cl.nseg; i++) n = std::max(n, cl.seg[i].n);
+    if (n <= 0) return cudaSuccess;
+    k_make_cols<<<dim3(unsigned(std::min<int64_t>((n + 255) / 256, 152 * 4)), unsigned(cl.nseg)), 256, 0, st>>>(cl);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_split_digits_vec(const SplitTables &T, int dir, int64_t nleaf, const double *v, double scale,
