@@ -57,29 +57,38 @@ typedef enum {
     BC_ERR_STATE = -7        /* call order violated (e.g. apply before tables) */
 } bc_status;
 
-/* Arithmetic of an apply.  "BF16 digits" means: each FP64 operand row (an
- * operator row, an input vector) is scaled by a power of two, rounded to a
- * 40-bit fixed-point integer and cut into five BF16 digits; the digit
- * products run on the tensor cores (tcgen05, FP32 accumulation, exact), and
- * the recombination is integer/FP64.  The rounding of the operands to 40 bits
- * is the only error (about 2^-40 of sum |A_ik v_k| per output). */
+/* Arithmetic of an apply.  "n digits" means: each FP64 operand row (an operator
+ * row, an input vector) is scaled by a power of two, rounded to an 8n-bit
+ * fixed-point integer and cut into n BF16 digits; the digit products run on
+ * the tensor cores (tcgen05, FP32 accumulation, exact), and the recombination
+ * is integer/FP64.  The rounding of the operands is the only error: with 5
+ * digits about 2^-40 of sum |A_ik v_k| per output, with 7 digits about a tenth
+ * of the rounding of the same sum in FP64 arithmetic. */
 typedef enum {
-    BC_FP64 = 0,           /* every step in native FP64 */
-    BC_SPLIT_BF16 = 1,     /* BF16 digits for the fixed-operator products: the
+    BC_FP64 = 0,           /* FP64 accuracy throughout: every operator product
+                              (near-field tables, P2M, L2P, W and X lists, the
+                              multipole-to-local translations) on 7 digits,
+                              vectors with an infinity or a NaN in FP64; the
+                              M2M and L2L shifts, the log terms and all sums in
+                              native FP64.  Trees whose tiles do not fit in
+                              device memory, and the options m2l_triangular and
+                              m2l_kernel (M2L only), take the native FP64
+                              kernels, as bc_apply_noalloc does (every p) */
+    BC_SPLIT_BF16 = 1,     /* 5 digits for the fixed-operator products: the
                               near-field tables, P2M, L2P, the W list (M2P) and
-                              the X list (P2L), and their adjoints.  Native FP64
-                              for the multipole-to-local translations, the
-                              M2M and L2L shifts, every log-kernel scaling
-                              term and every sum of partial results
-                              (p = 8, 12 and 16, nterms <= 32; other orders
-                              BC_ERR_UNSUPPORTED) */
-    BC_SPLIT_BF16_ALL = 2  /* BC_SPLIT_BF16 plus the multipole-to-local
-                              translations on BF16 digits (their log terms
-                              stay FP64) and the M2M / L2L shifts in
-                              double-float arithmetic (pairs of FP32 numbers,
-                              about 48 bits, on the FP32 units); the V- and
-                              X-list sums and the local expansions handed to
-                              later steps stay FP64 (p = 8, 12, 16) */
+                              the X list (P2L), and their adjoints.  The rest as
+                              in BC_FP64: the multipole-to-local translations on
+                              7 digits, the M2M and L2L shifts, every log-kernel
+                              scaling term and every sum of partial results in
+                              native FP64 (p = 8, 12 and 16, nterms <= 32; other
+                              orders BC_ERR_UNSUPPORTED) */
+    BC_SPLIT_BF16_ALL = 2  /* BC_SPLIT_BF16 with the multipole-to-local
+                              translations on 5 digits (their log terms stay
+                              FP64) and the M2M / L2L shifts in double-float
+                              arithmetic (pairs of FP32 numbers, about 48 bits,
+                              on the FP32 units); the V- and X-list sums and the
+                              local expansions handed to later steps stay FP64
+                              (p = 8, 12, 16) */
 } bc_precision;
 
 typedef struct {

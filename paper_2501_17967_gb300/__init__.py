@@ -22,10 +22,11 @@ from . import build as _build_mod
 __all__ = ["build", "Context", "Tree", "Batch", "BoxCodeError", "FP64", "SPLIT_BF16", "SPLIT_BF16_ALL", "apply",
            "apply_adjoint", "eval_points", "eval_points_grad", "Layer", "strip_solve", "strip_workspace", "BoxCodeApply", "lib_path"]
 
-# precision modes (bc_precision): FP64 everywhere; BF16 digit products for the
-# fixed-operator contractions (near field, P2M, L2P, W and X lists) with the
-# M2L, the shifts, the log terms and every sum in FP64; the same plus the M2L
-# on BF16 digits and the shifts in double-float
+# precision modes (bc_precision): FP64 accuracy throughout (7 BF16 digits for the
+# operator products, FP64 for the rest); 5-digit products for the
+# fixed-operator contractions (near field, P2M, L2P, W and X lists), the rest as
+# in FP64; the same with the M2L
+# on 5 digits and the shifts in double-float
 FP64 = 0
 SPLIT_BF16 = 1
 SPLIT_BF16_ALL = 2

@@ -1083,6 +1083,17 @@ bool build_wide_tree(bc_tree *t)
 // default form (the options that choose another one keep the FP64 kernels).
 int wide_parts(const bc_ctx *ctx) { return ctx->m2l_tri || ctx->m2l_kind ? kSplitTableParts : kWideParts; }
 
+// The split mode's M2L: on 7-digit products (as accurate as the FP64 kernels,
+// which take 0.87 ms of the FP64 pipe where the tiles take 0.25), unless an
+// option chooses the products or another M2L, or the tiles do not fit.
+void split_m2l(bc_ctx *ctx, bc_tree *t, int prec, SplitLaunch &sl)
+{
+    if (prec != BC_SPLIT_BF16 || ctx->split_parts >= 0 || wide_parts(ctx) != kWideParts || !build_wide_tree(t)) return;
+    sl.parts |= 32;
+    sl.m2l_tables = &ctx->wide;
+    sl.m2l_tree = &t->spw;
+}
+
 // CTAs of the near-field launch on the internal stream: the option, else all
 // SMs when it runs beside the FP64 M2L (one tensor CTA per SM next to the M2L
 // blocks), three quarters of them when it runs beside the level passes
@@ -1138,6 +1149,8 @@ bc_status apply_impl(bc_ctx *ctx, const bc_tree *tree, const double *vin, double
         if (s == BC_OK && (parts & 32)) s = build_split_m2l(tw);
         if (s != BC_OK) return s;
         sl.tree = &tw->sp;
+        split_m2l(ctx, tw, int(prec), sl);
+        sl.near_ctas = near_ctas_for(ctx, sl.parts);
         split = &sl;
     }
     if (split && side) sl.side = &tw->side;
@@ -1240,6 +1253,9 @@ bc_status batch_capture(bc_batch *b, int prec, int adj, int leaf_bps, int m2l_bp
     } else if (is_split(prec) && (parts & 32)) {
         bc_status s = build_split_m2l(b->u);
         if (s != BC_OK) return s;
+    } else if (is_split(prec)) {
+        split_m2l(ctx, b->u, prec, sl);
+        sl.near_ctas = near_ctas_for(ctx, sl.parts);
     }
     if (side && (wide || is_split(prec))) sl.side = &b->u->side;
     cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
