@@ -277,19 +277,19 @@ void bc_layer_destroy(bc_layer *layer);
  *
  *     C[k] x[k-1] + A[k] x[k] + B[k] x[k+1] = b[k],   k = 0..N-1, indices mod N
  *
- * (with N = 1 or 2 the blocks meeting at one position add).  Solved as the
- * paper does: block LU of the tridiagonal part, then the Woodbury identity
- * for the corner blocks C[0] and B[N-1] (O(m^3 N) per system).  Batched over
- * nsys independent systems: blocks up to 32 x 32 one warp per system, all
- * systems at once; larger blocks (the paper's elements, 16 x 24 = 384 nodes)
- * one system after another, each step a blocked LU over the whole GPU (rank
- * updates as cuBLAS DGEMMs).  Layout, all FP64 row-major device arrays: A, B,
+ * (with N = 1 or 2 the blocks meeting at one position add).  Solved by
+ * block LU with the corners as a border, the rank-m form of the paper's
+ * Woodbury correction (x[N-1] eliminated last through its Schur complement;
+ * O(m^3 N) per system).  Batched over nsys independent systems: blocks up to
+ * 32 x 32 one thread block per system, all systems at once; larger blocks (the
+ * paper's elements, 16 x 24 = 384 nodes) one system after another, each step a
+ * blocked LU over the whole GPU (rank updates as cuBLAS DGEMMs).  Layout, all FP64 row-major device arrays: A, B,
  * C [nsys][N][m][m]; b, x [nsys][N][m][r].  Shapes: N >= 1, 1 <= m <= 448,
  * 1 <= r <= 32.  work: device scratch of
  * bc_strip_workspace() bytes, owned by the caller.  status: NULL or device
- * int32 [nsys], set to 1 where a pivot of the block LU (every diagonal block
- * D_k and the 2m x 2m capacitance matrix are factored with partial pivoting)
- * was zero or not finite, else 0; no pivoting across blocks, so the systems
+ * int32 [nsys], set to 1 where a pivot of the block LU (the diagonal blocks
+ * D_0 .. D_{N-2} and the Schur complement of x[N-1] are factored with partial
+ * pivoting) was zero or not finite, else 0; no pivoting across blocks, so the systems
  * should be block diagonally dominant, as collocation strips with their
  * continuity rows are.  Host pointers: BC_ERR_ARG.  Stream-ordered. */
 bc_status bc_strip_workspace(int64_t nsys, int64_t N, int m, int r, int64_t *bytes);
