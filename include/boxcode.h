@@ -282,8 +282,9 @@ void bc_layer_destroy(bc_layer *layer);
  * Woodbury correction (x[N-1] eliminated last through its Schur complement;
  * O(m^3 N) per system).  Batched over nsys independent systems: blocks up to
  * 32 x 32 one thread block per system, all systems at once; larger blocks (the
- * paper's elements, 16 x 24 = 384 nodes) one system after another, each step a
- * blocked LU over the whole GPU (rank updates as cuBLAS DGEMMs).  Layout, all FP64 row-major device arrays: A, B,
+ * paper's elements, 16 x 24 = 384 nodes) one system after another, each one
+ * cooperative launch over the whole GPU (all its SMs: a solve on another stream
+ * waits).  Layout, all FP64 row-major device arrays: A, B,
  * C [nsys][N][m][m]; b, x [nsys][N][m][r].  Shapes: N >= 1, 1 <= m <= 448,
  * 1 <= r <= 32.  work: device scratch of
  * bc_strip_workspace() bytes, owned by the caller.  status: NULL or device

@@ -478,9 +478,8 @@ def strip_solve(A, B, C, b, stream=None, return_status=False, out=None, work=Non
     """Batched strip systems of Sec. 3.3 (block tridiagonal with periodic
     corners): C[k] x[k-1] + A[k] x[k] + B[k] x[k+1] = b[k], indices mod N.
     A, B, C: float64 device tensors [nsys, N, m, m]; b: [nsys, N, m, r].
-    Returns x (and the per-system status if asked: 1 = zero pivot).  With
-    the same tensors (out, work and status passed in too) a large-block
-    solve replays its captured launch graph."""
+    Returns x (and the per-system status if asked: 1 = zero pivot); out, work
+    and status may be passed in."""
     import torch
     A, B, C, b = (t.contiguous() for t in (A, B, C, b))
     if b.dim() != 4 or A.shape != B.shape or A.shape != C.shape or A.shape[:3] != b.shape[:3] \

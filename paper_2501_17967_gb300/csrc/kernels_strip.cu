@@ -19,7 +19,7 @@
 // Blocks up to 32 x 32 (interface-sized blocks): one CTA of 1 to 8 warps per
 // system, many systems at once; the blocks of the current step live in shared
 // memory, H_k and X_k in a global workspace.  Larger blocks (the paper's
-// elements of 16 x 24 nodes): one system at a time on the whole GPU, below.
+// elements of 16 x 24 nodes): kernels_strip_large.cu.
 // FP64.
 #include <cuda_runtime.h>
 
@@ -326,246 +326,7 @@ k_strip_small(int64_t N, int m, int r, const double *__restrict__ A, const doubl
     if (status && tid == 0) status[s] = pv.bad;
 }
 
-// ---------------------------------------------------------------------------
-// Large blocks (m > 32, the element blocks of the paper's strip: 16 x 24 =
-// 384 nodes): one system at a time on the whole GPU.  The host loops over
-// the elements; each step factors the augmented block [D_k | B_k | rhs_k]
-// (row-major, Wc = m + m + R columns) by right-looking blocked LU with
-// partial pivoting (panels of kPanel columns: k_strip_panel factors a panel
-// in shared memory in one CTA, k_strip_swap carries its row exchanges to the
-// columns on its right, k_strip_trsm applies L11^-1 to them (one thread per
-// column, so the many columns spread over the SMs), and a DGEMM updates the
-// trailing block), then back-substitutes the right-hand columns (k_strip_trsm
-// with U11 per diagonal block, DGEMM for the rows above).  Narrow panels keep
-// the single-CTA FP64 work of each panel small: one SM's FP64 pipe does 4
-// flop per clock.
-// ---------------------------------------------------------------------------
-constexpr int kPanel = 16;
-constexpr int kPanelThreads = 256;
-
-// Step k's augmented block (k < N - 1): [A_k | B_k (k < N-2) | b_k | E_k].
-__global__ void k_strip_aug(int64_t N, int m, int r, int64_t k, const double *__restrict__ A,
-                            const double *__restrict__ B, const double *__restrict__ C,
-                            const double *__restrict__ b, double *__restrict__ aug, int Wc)
-{
-    const size_t mm = size_t(m) * m;
-    for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < int64_t(m) * Wc;
-         idx += int64_t(gridDim.x) * blockDim.x) {
-        const int i = int(idx / Wc), c = int(idx % Wc);
-        double v = 0.0;
-        if (c < m) v = A[k * mm + size_t(i) * m + c];
-        else if (c < 2 * m) v = k < N - 2 ? B[k * mm + size_t(i) * m + (c - m)] : 0.0;
-        else if (c < 2 * m + r) v = b[(k * m + i) * r + (c - 2 * m)];
-        else {
-            const int q = c - 2 * m - r;
-            if (k == 0) v += C[size_t(i) * m + q];
-            if (k == N - 2) v += B[k * mm + size_t(i) * m + q];
-        }
-        aug[idx] = v;
-    }
-}
-
-// the border system [A_{N-1} | b_{N-1}] (N = 1: [A_0 + B_0 + C_0 | b_0]),
-// before the products with T'^-1 [b | E] are taken off
-__global__ void k_strip_border(int64_t N, int m, int r, const double *__restrict__ A, const double *__restrict__ B,
-                               const double *__restrict__ C, const double *__restrict__ b, double *__restrict__ S)
-{
-    const size_t mm = size_t(m) * m;
-    const int ld = m + r;
-    const int64_t k = N - 1;
-    for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < int64_t(m) * ld;
-         idx += int64_t(gridDim.x) * blockDim.x) {
-        const int i = int(idx / ld), c = int(idx % ld);
-        double v;
-        if (c < m) {
-            v = A[k * mm + size_t(i) * m + c];
-            if (N == 1) v += B[size_t(i) * m + c] + C[size_t(i) * m + c];
-        } else {
-            v = b[(k * m + i) * r + (c - m)];
-        }
-        S[idx] = v;
-    }
-}
-
-// LU with partial pivoting of the panel: rows [j0, n), columns [j0, j0 + jb)
-// of M (row-major, leading dimension ld), staged in shared memory; the pivot
-// rows go to piv[j] (absolute); a zero or non-finite pivot sets *status.
-// Thread t owns the rows t, t + nt, ...: it searches them for the pivot and
-// applies the rank-1 update to them, so a column step needs three barriers
-// (pivot found, pivot row in place, and the next step's search).
-__global__ void __launch_bounds__(kPanelThreads)
-k_strip_panel(double *__restrict__ M, int n, int ld, int j0, int jb, int32_t *__restrict__ piv,
-              int32_t *__restrict__ status)
-{
-    extern __shared__ double sp[];   // [n - j0][jb]
-    __shared__ unsigned long long s_key[kPanelThreads / 32];
-    __shared__ int s_row[kPanelThreads / 32];
-    __shared__ int s_piv;
-    __shared__ double s_inv;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nt = blockDim.x, nw = nt >> 5;
-    const int rows = n - j0;
-    for (int idx = t; idx < rows * jb; idx += nt) sp[idx] = M[size_t(j0 + idx / jb) * ld + j0 + idx % jb];
-    __syncthreads();
-    // |x| compared through its bit pattern (sign cleared): an integer order
-    // that matches the order of the magnitudes, so the search leaves the FP64
-    // pipe to the updates (a NaN sorts above every number and is flagged)
-    constexpr unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
-    for (int jj = 0; jj < jb; jj++) {
-        unsigned long long key = 0;
-        int bi = rows;
-        for (int i = jj + ((t - jj) % nt + nt) % nt; i < rows; i += nt) {   // owned rows >= jj
-            const unsigned long long v = static_cast<unsigned long long>(__double_as_longlong(sp[i * jb + jj])) & kMag;
-            if (bi == rows || v > key) { key = v; bi = i; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (oi < rows && (bi == rows || ok > key || (ok == key && oi < bi))) { key = ok; bi = oi; }
-        }
-        if (lane == 0) { s_key[w] = key; s_row[w] = bi; }
-        __syncthreads();
-        if (w == 0) {
-            key = lane < nw ? s_key[lane] : 0ull;
-            bi = lane < nw ? s_row[lane] : rows;
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (oi < rows && (bi == rows || ok > key || (ok == key && oi < bi))) { key = ok; bi = oi; }
-            }
-            if (lane == 0) {
-                const int p = bi < rows ? bi : jj;
-                const double d = sp[p * jb + jj];
-                const bool good = d != 0.0 && isfinite(d);
-                s_piv = p;
-                s_inv = good ? 1.0 / d : 0.0;
-                piv[j0 + jj] = j0 + p;
-                if (!good) *status = 1;
-            }
-        }
-        __syncthreads();
-        const int p = s_piv;
-        if (p != jj)
-            for (int c = t; c < jb; c += nt) {
-                const double x = sp[jj * jb + c];
-                sp[jj * jb + c] = sp[p * jb + c];
-                sp[p * jb + c] = x;
-            }
-        __syncthreads();
-        const double inv = s_inv;
-        for (int i = jj + 1 + ((t - jj - 1) % nt + nt) % nt; i < rows; i += nt) {   // owned rows > jj
-            const double l = sp[i * jb + jj] * inv;
-            sp[i * jb + jj] = l;
-            for (int c = jj + 1; c < jb; c++) sp[i * jb + c] = fma(-l, sp[jj * jb + c], sp[i * jb + c]);
-        }
-    }
-    __syncthreads();
-    for (int idx = t; idx < rows * jb; idx += nt) M[size_t(j0 + idx / jb) * ld + j0 + idx % jb] = sp[idx];
-}
-
-// the panel's row exchanges on columns [c0, c1)
-__global__ void k_strip_swap(double *__restrict__ M, int ld, int j0, int jb, const int32_t *__restrict__ piv,
-                             int c0, int c1)
-{
-    const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= c1) return;
-    for (int j = j0; j < j0 + jb; j++) {
-        const int p = piv[j];
-        if (p != j) {
-            const double x = M[size_t(j) * ld + c];
-            M[size_t(j) * ld + c] = M[size_t(p) * ld + c];
-            M[size_t(p) * ld + c] = x;
-        }
-    }
-}
-
-// Triangular solve with the jb x jb diagonal block at j0, in place on rows
-// [j0, j0 + jb) of the columns [c0, c1), one thread per column (jb <= kPanel):
-// upper = false: the unit lower block (L11^-1 A12); upper = true: the upper
-// block (U11^-1 Y).  A zero diagonal gives zero (the panel flagged it).
-__global__ void k_strip_trsm(double *__restrict__ M, int ld, int j0, int jb, bool upper, int c0, int c1)
-{
-    __shared__ double sa[kPanel * kPanel];
-    __shared__ double sr[kPanel];   // reciprocals of the diagonal (upper)
-    for (int idx = threadIdx.x; idx < jb * jb; idx += blockDim.x)
-        sa[idx] = M[size_t(j0 + idx / jb) * ld + j0 + idx % jb];
-    __syncthreads();
-    if (upper && threadIdx.x < jb) {
-        const double d = sa[threadIdx.x * jb + threadIdx.x];
-        sr[threadIdx.x] = d != 0.0 ? 1.0 / d : 0.0;
-    }
-    __syncthreads();
-    const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= c1) return;
-    double x[kPanel];
-#pragma unroll
-    for (int i = 0; i < kPanel; i++) x[i] = i < jb ? M[size_t(j0 + i) * ld + c] : 0.0;
-    if (!upper) {
-#pragma unroll
-        for (int i = 1; i < kPanel; i++)
-#pragma unroll
-            for (int q = 0; q < i; q++) x[i] = fma(-sa[i * jb + q], x[q], x[i]);   // x[q] = 0 past jb
-    } else {
-#pragma unroll
-        for (int i = kPanel - 1; i >= 0; i--) {
-            if (i >= jb) continue;
-#pragma unroll
-            for (int q = i + 1; q < kPanel; q++)
-                if (q < jb) x[i] = fma(-sa[i * jb + q], x[q], x[i]);
-            x[i] *= sr[i];
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < kPanel; i++)
-        if (i < jb) M[size_t(j0 + i) * ld + c] = x[i];
-}
-
 }  // namespace
-
-int strip_panel_width() { return kPanel; }
-
-cudaError_t launch_strip_aug(int64_t N, int m, int r, int64_t k, const double *A, const double *B, const double *C,
-                             const double *b, double *aug, int Wc, cudaStream_t st)
-{
-    const int64_t n = int64_t(m) * Wc;
-    k_strip_aug<<<int(std::min<int64_t>((n + 255) / 256, 152 * 8)), 256, 0, st>>>(N, m, r, k, A, B, C, b, aug, Wc);
-    return cudaGetLastError();
-}
-
-cudaError_t strip_prepare(int nmax)
-{
-    return cudaFuncSetAttribute(k_strip_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(sizeof(double) * size_t(nmax) * kPanel));
-}
-
-cudaError_t launch_strip_panel(double *M, int n, int ld, int j0, int jb, int32_t *piv, int32_t *status,
-                               cudaStream_t st)
-{
-    const size_t sm = sizeof(double) * size_t(n - j0) * jb;
-    k_strip_panel<<<1, kPanelThreads, sm, st>>>(M, n, ld, j0, jb, piv, status);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_strip_swap(double *M, int ld, int j0, int jb, const int32_t *piv, int c0, int c1, cudaStream_t st)
-{
-    if (c1 <= c0) return cudaSuccess;
-    k_strip_swap<<<(c1 - c0 + 127) / 128, 128, 0, st>>>(M, ld, j0, jb, piv, c0, c1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_strip_trsm(double *M, int ld, int j0, int jb, bool upper, int c0, int c1, cudaStream_t st)
-{
-    if (c1 <= c0) return cudaSuccess;
-    k_strip_trsm<<<(c1 - c0 + 31) / 32, 32, 0, st>>>(M, ld, j0, jb, upper, c0, c1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_strip_border(int64_t N, int m, int r, const double *A, const double *B, const double *C,
-                                const double *b, double *S, cudaStream_t st)
-{
-    const int64_t n = int64_t(m) * (m + r);
-    k_strip_border<<<int(std::min<int64_t>((n + 255) / 256, 152 * 8)), 256, 0, st>>>(N, m, r, A, B, C, b, S);
-    return cudaGetLastError();
-}
 
 // two augmented blocks and a third buffer of [H | g] (or two C blocks)
 size_t strip_smem_bytes(int m, int r)
