@@ -24,17 +24,14 @@
 //
 // Work decomposition: a tile is one operator times up to 48 (32) columns, done
 // as one job per 128-row half of the operator.
-//   B operand: the columns' digits, gathered into shared memory slice by slice
-//              with 16-byte asynchronous copies (cp.async), resident for the
-//              tile; the next tile's slices are gathered as the current tile's
-//              last job stops reading them;
+//   B operand: the columns' digits, gathered into shared memory with 16-byte
+//              asynchronous copies (cp.async), one buffer per K chunk of 128; the
+//              chunks take turns (kchunk_at), so that the next tile's are gathered
+//              while this tile's MMAs run;
 //   A operand: the operator's digits, 128 rows x 128 columns per chunk (32 KB),
 //              brought in by bulk asynchronous copies through three buffers
-//              (two in the K = 256 launches beside the FP64 M2L);
-//              a tile's first row-half job takes the operator digits in the
-//              order 0, 4, 1, 3, 2 (long and short chunks alternate, so copies
-//              keep up), its last job in the order 0..4 (B slices are freed
-//              earliest);
+//              (two in the launches beside the FP64 M2L), digits in the order
+//              0, 4, 1, 3, 2 (long and short chunks alternate, so copies keep up);
 //   D:         5 levels x 48 (8 x 32) columns of FP32 per job, two TMEM
 //              buffers, so one job's epilogue overlaps the next job's MMAs.
 // One tcgen05.mma of 128 x 48 x 16 takes about as long as one of 128 x 16 x 16
@@ -55,7 +52,7 @@ namespace bc {
 
 namespace {
 
-constexpr int kNBuf = 3;           // operator chunk buffers (32 KB each at K = 256)
+constexpr int kMeta = 4;           // column metadata buffers (tiles)
 
 // The two digit formats.  S digits per operand, L levels kept (digit pairs
 // a + b <= L + 1, counted from 1), tiles of N columns: L N <= 256, half of
@@ -125,18 +122,11 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// waits until at most n (0..6) of this thread's cp.async groups are pending
+// waits until at most n (0 or 1) of this thread's cp.async groups are pending
 __device__ __forceinline__ void cp_async_wait_pending(int n)
 {
-    switch (n) {
-    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
-    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-    case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
-    default: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
-    }
+    if (n == 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    else asm volatile("cp.async.wait_group 1;" ::: "memory");
 }
 
 // NK MMAs along K (16 columns each) issued from one elected lane of a
@@ -277,24 +267,18 @@ __device__ __forceinline__ bool wait_bar(uint64_t *bar, uint32_t parity, long lo
     return false;
 }
 
-// Named barrier over the gather warps (id 1); the _or form returns whether any
-// of them passed a true predicate.
-__device__ __forceinline__ void gather_sync(int nthreads)
+// Whether an mbarrier phase has completed, without waiting (uniform over the warp).
+__device__ __forceinline__ bool test_bar(uint64_t *bar, uint32_t parity)
 {
-    asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
-}
-__device__ __forceinline__ bool gather_sync_or(int nthreads, bool pred)
-{
-    uint32_t r;
+    uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"(uint32_t(pred)), "r"(nthreads)
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
-    return r != 0;
+    return __any_sync(0xffffffffu, ok);
 }
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -470,34 +454,41 @@ struct ColMeta {
     int32_t pad;
 };
 
-// Operator digit of the p-th chunk group of a job: the order 0, S-1, 1, S-2, ...
-// alternates long and short MMA runs (a tile's first row-half job); 0..S-1 frees
-// the B slices earliest (a tile's last job).
+// Operator digit of the p-th chunk of a K chunk's run: the order 0, S-1, 1, S-2, ...
+// alternates long and short MMA runs, so that the copies keep up.
 template <int S>
-__device__ __forceinline__ int chunk_digit(int p, bool interleave)
+__device__ __forceinline__ int chunk_digit(int p)
 {
-    if (!interleave) return p;
     return (p & 1) ? S - 1 - (p >> 1) : (p >> 1);
 }
 
-template <int KD, int S, int NB = kNBuf>
+// The order of the K chunks (KD = 256 has two): a tile's first row-half job takes
+// them as x, 1 - x, its second as 1 - x, x, and the next tile starts with the one
+// that this tile did not end on, so that every chunk of B is used twice in a row
+// and its buffer is free, for the next tile's gather, while the other chunk's
+// MMAs run.  x: the first chunk of a tile; next_first: of the tile after it.
+__device__ __forceinline__ int kchunk_at(int x, int h, int i) { return h == 0 ? x ^ i : x ^ i ^ 1; }
+__device__ __forceinline__ int next_first(int x, bool two_jobs) { return two_jobs ? x ^ 1 : x; }
+
+template <int KD, int S, bool ICVT>
 struct GemmShape {
     static constexpr int N = Fmt<S>::N, L = Fmt<S>::L;
-    static constexpr int KC = KD > 144 ? kSplitKC : KD;   // K columns per operator chunk
+    static constexpr int KC = KD > 144 ? kSplitKC : KD;   // K columns per operator chunk and B buffer
     static constexpr int NKC = KD / KC;
-    static constexpr int kChunksPerJob = S * NKC;      // digit x K chunk
-    static constexpr int kBSlice = N * KD * 2;         // bytes of one B digit slice
+    // operator chunk buffers: three, two where the shared memory is short (KD = 144:
+    // two whole tiles of B) or left to the FP64 M2L's blocks beside (ICVT)
+    static constexpr int NB = KD == 144 || ICVT ? 2 : 3;
+    static constexpr int kBSlice = N * KC * 2;         // bytes of one B digit slice of a chunk
+    static constexpr int kBChunk = S * kBSlice;        // bytes of one chunk of B (two buffers)
     static constexpr int kChunk = 128 * KC * 2;        // bytes of one operator chunk
-    static constexpr int kBSBO = (KD / 8) * 128;       // B: bytes between 8-row groups
-    static constexpr int kASBO = (KC / 8) * 128;       // A: bytes between 8-row groups
-    static constexpr int kBTile = S * kBSlice;          // bytes of one tile's B (115 to 120 KB at K = 256): one buffer
-    static constexpr size_t kSmem = size_t(kBTile) + size_t(NB) * kChunk + 2 * N * sizeof(ColMeta) +
-                                    64 * sizeof(uint64_t);
+    static constexpr int kSBO = (KC / 8) * 128;        // bytes between 8-row groups (A and B)
+    static constexpr size_t kSmem =
+        2 * size_t(kBChunk) + size_t(NB) * kChunk + kMeta * N * sizeof(ColMeta) + 64 * sizeof(uint64_t);
 };
 
 // Roles (16 warps): warp 0 issues the MMAs; warp 1 copies the operator chunks;
-// warps 2-7 stage each tile's column metadata and gather its B digits, slice by
-// slice; warps 8-15 run the epilogues (two warps per TMEM lane quarter, half of
+// warps 2-7 stage each tile's column metadata and gather its B digits, chunk by
+// chunk; warps 8-15 run the epilogues (two warps per TMEM lane quarter, half of
 // the columns each).
 constexpr int kGemmThreads = 512;
 constexpr int kGatherWarp0 = 2;
@@ -512,21 +503,17 @@ constexpr int kNoExp = 0x7FFFFFFF;   // 1/alpha0 is not a power of two
 //   mbar[b] (1)        the MMAs reading buffer b have completed (commit)
 //   job_full[r] (1)    the MMAs of the job in TMEM buffer r have completed (commit)
 //   job_empty[r] (8)   the epilogue warps have read TMEM buffer r
-//   b_full[t][s] (1)   B digit slice s (and the metadata) of tile parity t is ready
-//   b_empty[s] (1)     no MMA of the previous tile reads B slice s any more (commit)
-//   meta_empty[t] (8)  the epilogue warps are done with metadata buffer t
-// Digit slice s (0-based) of B is read by the chunks of operator digit a <= L - 1 - s,
-// so in a tile's last job it is free after those chunks; the next tile's B is
-// gathered slice by slice from s = S - 1 down to 0 and its first chunk issues its
-// MMAs from slice S - 1 down, so only the last slices are waited for at the
-// tile change.
-template <int S>
+//   b_full[u] (6)      B buffer u is filled (one arrival per gather warp)
+//   b_empty[u] (1)     no MMA reads B buffer u any more (commit)
+//   meta_full[t] (6), meta_empty[t] (8)   metadata buffer t (tile % 4) is filled, done with
+// B buffer u holds K chunk u of the current tile (two chunks), or the tiles of
+// parity u (one chunk).
 struct GemmBars {
-    uint64_t lbar[kNBuf], mbar[kNBuf], job_full[2], job_empty[2], b_full[2][S], b_empty[S], meta_empty[2];
+    uint64_t lbar[3], mbar[3], job_full[2], job_empty[2], b_full[2], b_empty[2], meta_full[kMeta], meta_empty[kMeta];
     uint32_t tslot;
     int fail;
 };
-static_assert(sizeof(GemmBars<kWideSlices>) <= 64 * sizeof(uint64_t), "barrier space");
+static_assert(sizeof(GemmBars) <= 64 * sizeof(uint64_t), "barrier space");
 
 // Row `row` of an operator times a vector without digits (an infinity or a NaN
 // among its entries), in FP64: sum_k opf[k][row] (scale cs_k x_k).
@@ -616,16 +603,12 @@ __global__ void __launch_bounds__(kGemmThreads, S == kSplitSlices ? 2 : 1)
 k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_alpha_exp, int32_t *__restrict__ err, long long wait_limit,
              int withhold)
 {
-    // the K = 256 launches beside the FP64 M2L (ICVT) keep two operator
-    // buffers: 32 KB less shared memory makes room for a fourth M2L block
-    constexpr int NB = (KD == 256 && ICVT) ? 2 : kNBuf;
-    using Sh = GemmShape<KD, S, NB>;
-    constexpr int kS = S, kN = Sh::N, kL = Sh::L;
+    using Sh = GemmShape<KD, S, ICVT>;
+    constexpr int kN = Sh::N, kL = Sh::L, NB = Sh::NB, NKC = Sh::NKC;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *Bs = smem;                                                      // kS x kBSlice
-    uint8_t *As = smem + Sh::kBTile;                                         // NB x kChunk
-    ColMeta *meta = reinterpret_cast<ColMeta *>(As + NB * Sh::kChunk);       // [2][kN]
-    GemmBars<S> *bars = reinterpret_cast<GemmBars<S> *>(meta + 2 * kN);
+    uint8_t *Bs = smem, *As = smem + 2 * Sh::kBChunk;                    // 2 x kBChunk, NB x kChunk
+    ColMeta *meta = reinterpret_cast<ColMeta *>(As + NB * Sh::kChunk);   // [kMeta][kN]
+    GemmBars *bars = reinterpret_cast<GemmBars *>(meta + kMeta * kN);
     volatile int *fail = &bars->fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -643,10 +626,13 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
         for (int i = 0; i < 2; i++) {
             mbar_init(&bars->job_full[i], 1);
             mbar_init(&bars->job_empty[i], kEpiWarps);
-            mbar_init(&bars->meta_empty[i], kEpiWarps);
-            for (int sl = 0; sl < kS; sl++) mbar_init(&bars->b_full[i][sl], 1);
+            mbar_init(&bars->b_full[i], kGatherThreads / 32);
+            mbar_init(&bars->b_empty[i], 1);
         }
-        for (int sl = 0; sl < kS; sl++) mbar_init(&bars->b_empty[sl], 1);
+        for (int i = 0; i < kMeta; i++) {
+            mbar_init(&bars->meta_full[i], kGatherThreads / 32);
+            mbar_init(&bars->meta_empty[i], kEpiWarps);
+        }
         bars->fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -657,77 +643,67 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
     // tensor memory and barriers are set up: now wait for the inputs
     griddep_wait();
     griddep_launch_dependents();
+    const int step = gridDim.x;
+    // B buffer and phase parity of chunk kc of the CTA's tile k
+    auto bbuf = [](int k, int kc) { return NKC == 2 ? kc : k & 1; };
+    auto bpar = [](int k) { return uint32_t(NKC == 2 ? k & 1 : (k >> 1) & 1); };
 
     if (warp == 0) {
         // ---------------- MMAs ----------------
-        const uint64_t adesc0 = umma_desc(smem_u32(As), 128, Sh::kASBO);
-        const uint64_t bdesc0 = umma_desc(smem_u32(Bs), 128, Sh::kBSBO);
-        long long G = 0, last_commit = -1;   // chunks consumed
-        int job = 0, k = 0;
+        const uint64_t adesc0 = umma_desc(smem_u32(As), 128, Sh::kSBO);
+        const uint64_t bdesc0 = umma_desc(smem_u32(Bs), 128, Sh::kSBO);
+        long long G = 0, last_commit = -1;   // operator chunks consumed
+        int job = 0, k = 0, x = 0;
         bool failed = false;
-        for (int tile = blockIdx.x; tile < gm.ntiles && !failed; tile += gridDim.x, k++) {
-            const SplitTile tl = gm.tiles[tile];
-            const int mh = tl.rows > 128 ? 2 : 1;
-            uint32_t ready = 0;   // B slices of this tile known to be gathered
-            for (int h = 0; h < mh && !failed; h++, job++) {
+        for (int tile = blockIdx.x; tile < gm.ntiles && !failed; tile += step, k++) {
+            const bool two = gm.tiles[tile].rows > 128;
+            for (int h = 0; h <= int(two) && !failed; h++, job++) {
                 const int r = job & 1;
-                const bool last_job = h == mh - 1;
                 if (job >= 2 && !wait_bar(&bars->job_empty[r], uint32_t(((job - 2) >> 1) & 1), wait_limit, fail)) {
                     failed = true;
                     break;
                 }
-                tc_fence_after();
-                for (int g = 0; g < Sh::kChunksPerJob; g++, G++) {
-                    const int buf = int(G % NB);
-                    if (!wait_bar(&bars->lbar[buf], uint32_t((G / NB) & 1), wait_limit, fail)) {
+                for (int i = 0; i < NKC && !failed; i++) {
+                    const int kc = NKC == 2 ? kchunk_at(x, h, i) : 0, u = bbuf(k, kc);
+                    if (h == 0 && !wait_bar(&bars->b_full[u], bpar(k), wait_limit, fail)) {
                         failed = true;
                         break;
                     }
                     tc_fence_after();
-                    const int pos = g / Sh::NKC, kc = g % Sh::NKC;
-                    const int a = chunk_digit<S>(pos, !last_job);   // 0-based digit of A
-                    const int nb = min(kS, kL - a);                 // B digit slices 0 .. nb-1 pair with it
-                    const uint64_t ad = adesc0 + uint64_t(buf) * (Sh::kChunk >> 4);
-                    const uint32_t first = (a == 0 && kc == 0) ? 0u : 1u;
-                    for (int b = nb - 1; b >= 0; b--) {   // present
-                        if (!(ready >> b & 1u)) {
-                            if (!wait_bar(&bars->b_full[k & 1][b], uint32_t((k >> 1) & 1), wait_limit, fail)) {
-                                failed = true;
-                                break;
-                            }
-                            tc_fence_after();
-                            ready |= 1u << b;
+                    for (int pos = 0; pos < S; pos++, G++) {
+                        const int buf = int(G % NB);
+                        if (!wait_bar(&bars->lbar[buf], uint32_t((G / NB) & 1), wait_limit, fail)) {
+                            failed = true;
+                            break;
                         }
+                        tc_fence_after();
+                        const int a = chunk_digit<S>(pos);   // 0-based digit of A
+                        const int nb = min(S, kL - a);       // B digit slices 0 .. nb-1 pair with it
+                        const uint64_t ad = adesc0 + uint64_t(buf) * (Sh::kChunk >> 4);
+                        const uint64_t bd = bdesc0 + uint64_t(u) * (Sh::kBChunk >> 4);
+                        const uint32_t dcol = tmem + uint32_t(r * kTmemBuf + a * kN);
+                        // slices 0 .. nb-1 lie one after another (an nb kN-row B
+                        // operand) and feed levels a .. a+nb-1, adjacent TMEM
+                        // column blocks: one MMA chain of N = nb kN per chunk.  The
+                        // first chunk (a = 0) starts levels 0 .. S-1; where L > S the
+                        // second one starts level L-1 (its last slice, apart).
+                        if (kL > S && pos == 1 && i == 0) {
+                            umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, (nb - 1) * kN), 1u);
+                            umma_kchain_warp<Sh::KC / 16>(dcol + uint32_t((nb - 1) * kN), ad,
+                                                          bd + uint64_t(nb - 1) * (Sh::kBSlice >> 4),
+                                                          umma_idesc(128, kN), 0u);
+                        } else {
+                            umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, nb * kN), pos == 0 && i == 0 ? 0u : 1u);
+                        }
+                        umma_commit_warp(&bars->mbar[buf]);
+                        last_commit = G;
                     }
-                    if (failed) break;
-                    // slices 0 .. nb-1 lie one after another (an nb kN-row B
-                    // operand) and feed levels a .. a+nb-1, adjacent TMEM
-                    // column blocks: one MMA chain of N = nb kN per chunk.  The
-                    // first chunk (a = 0) starts levels 0 .. S-1; where L > S the
-                    // second one starts level L-1 (its last slice, apart).
-                    const uint32_t dcol = tmem + uint32_t(r * kTmemBuf + a * kN);
-                    const uint64_t bd = bdesc0 + uint64_t(kc) * ((Sh::KC / 8) * 128 >> 4);
-                    if (kL > kS && pos == 1 && kc == 0) {
-                        umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, (nb - 1) * kN), 1u);
-                        umma_kchain_warp<Sh::KC / 16>(dcol + uint32_t((nb - 1) * kN), ad,
-                                                      bd + uint64_t(nb - 1) * (Sh::kBSlice >> 4),
-                                                      umma_idesc(128, kN), 0u);
-                    } else {
-                        umma_kchain_warp<Sh::KC / 16>(dcol, ad, bd, umma_idesc(128, nb * kN), first);
-                    }
-                    umma_commit_warp(&bars->mbar[buf]);
-                    last_commit = G;
-                    // in the tile's last job, slice L-1-a is read by no later
-                    // chunk, and after the last digit no slice is
-                    if (last_job && kc == Sh::NKC - 1) {
-                        if (kL - 1 - a < kS) umma_commit_warp(&bars->b_empty[kL - 1 - a]);
-                        if (a == kS - 1)
-                            for (int b = 0; b < kL - kS; b++) umma_commit_warp(&bars->b_empty[b]);
-                    }
+                    if (!failed && h == int(two)) umma_commit_warp(&bars->b_empty[u]);   // the tile's last use
                 }
                 if (failed) break;
                 umma_commit_warp(&bars->job_full[r]);
             }
+            x = next_first(x, two);
         }
         if (failed) {
             *fail = 1;
@@ -739,12 +715,17 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
     } else if (warp == 1) {
         // ---------------- operator chunk copies ----------------
         long long n = 0;   // chunks issued
+        int x = 0;
         bool failed = false;
-        for (int tile = blockIdx.x; tile < gm.ntiles && !failed; tile += gridDim.x) {
+        for (int tile = blockIdx.x; tile < gm.ntiles && !failed; tile += step) {
             const SplitTile tl = gm.tiles[tile];
             const int mh = tl.rows > 128 ? 2 : 1;
-            for (int h = 0; h < mh && !failed; h++)
-                for (int g = 0; g < Sh::kChunksPerJob; g++, n++) {
+            // an operator of at most 64 rows is copied twice, to rows 0-63
+            // and 64-127, so that every TMEM lane quarter holds a result
+            const int copies = tl.rows <= 64 ? 2 : 1;
+            for (int h = 0; h < mh && !failed; h++) {
+                const uint32_t bytes = uint32_t((min(128, tl.rows - 128 * h) + 7) / 8) * 8 * Sh::KC * 2;
+                for (int g = 0; g < S * NKC; g++, n++) {
                     const int buf = int(n % NB);
                     // buffer free once the MMAs of chunk n - NB have completed
                     if (n >= NB &&
@@ -753,13 +734,8 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
                         break;
                     }
                     if (withhold) continue;   // diagnostics: the MMA warp's first wait runs out
-                    const int a = chunk_digit<S>(g / Sh::NKC, h < mh - 1), kc = g % Sh::NKC;
-                    const int rows_h = min(128, tl.rows - 128 * h);
-                    const uint32_t bytes = uint32_t((rows_h + 7) / 8) * 8 * Sh::KC * 2;
-                    const uint8_t *src = gm.ops + tl.a_off + size_t((a * mh + h) * Sh::NKC + kc) * Sh::kChunk;
-                    // an operator of at most 64 rows is copied twice, to rows 0-63
-                    // and 64-127, so that every TMEM lane quarter holds a result
-                    const int copies = tl.rows <= 64 ? 2 : 1;
+                    const int a = chunk_digit<S>(g % S), kc = NKC == 2 ? kchunk_at(x, h, g / S) : 0;
+                    const uint8_t *src = gm.ops + tl.a_off + size_t((a * mh + h) * NKC + kc) * Sh::kChunk;
                     if (lane == 0) {
                         mbar_expect_tx(&bars->lbar[buf], bytes * copies);
                         for (int cp = 0; cp < copies; cp++) {
@@ -770,6 +746,8 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
                     }
                     __syncwarp();
                 }
+            }
+            x = next_first(x, mh == 2);
         }
         if (failed && !withhold) {
             // copies still in flight: at most the last NB issued
@@ -779,47 +757,78 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
         }
     } else if (warp < kEpiWarp0) {
         // ---------------- column metadata and B gather ----------------
-        const int gt = tid - 32 * kGatherWarp0;
-        constexpr int kPieces = KD / 8;   // 16-byte pieces per column and slice
-        int k = 0;
-        bool stop = false;
-        for (int tile = blockIdx.x; tile < gm.ntiles && !stop; tile += gridDim.x, k++) {
-            bool ok = true;
-            // the epilogues of tile k - 2 no longer read this metadata buffer
-            if (k >= 2) ok = wait_bar(&bars->meta_empty[k & 1], uint32_t(((k - 2) >> 1) & 1), wait_limit, fail);
-            if (gather_sync_or(kGatherThreads, !ok)) break;   // uniform over the gather warps
-            const SplitTile tl = gm.tiles[tile];
-            ColMeta *M = meta + (k & 1) * kN;
-            if (gt < tl.cnt) {
-                const SplitCol c = gm.cols[tl.p0 + gt];
-                M[gt] = col_meta<S>(c, gm.dexp[c.vec], inv_alpha_exp);
+        // kTPC threads per column, each with its own column record (the records,
+        // columns and exponents of the next tiles are in flight) and the 16-byte
+        // pieces j, j + kTPC, ... of the column's chunk; no barrier among them
+        constexpr int kTPC = kGatherThreads / kN, kRow = Sh::KC / 8, kPieces = S * kRow;
+        static_assert(kTPC * kN == kGatherThreads, "whole columns");
+        const int gt = tid - 32 * kGatherWarp0, c = gt / kTPC, j = gt % kTPC;
+        const int nt = blockIdx.x < gm.ntiles ? (gm.ntiles - 1 - int(blockIdx.x)) / step + 1 : 0;
+        auto tile_at = [&](int k) -> SplitTile {
+            SplitTile t{};
+            if (k < nt) t = gm.tiles[blockIdx.x + k * step];
+            return t;
+        };
+        SplitTile tl = tile_at(0), tl1 = tile_at(1), tl2 = tile_at(2);
+        SplitCol col{}, col1{};
+        int ev = 0, x = 0;
+        if (c < tl.cnt) col = gm.cols[tl.p0 + c];
+        if (c < tl1.cnt) col1 = gm.cols[tl1.p0 + c];
+        if (j == 0 && c < tl.cnt) ev = gm.dexp[col.vec];
+        int pend = -1, pend_meta = -1;   // B buffer (and metadata) whose copies are under way
+        bool ok = true;
+        auto complete = [&](int allowed) {
+            if (pend < 0) return;   // uniform
+            if (allowed) cp_async_wait_pending(1);
+            else cp_async_wait_pending(0);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&bars->b_full[pend]);
+                if (pend_meta >= 0) mbar_arrive(&bars->meta_full[pend_meta]);
             }
-            gather_sync(kGatherThreads);
-            // one B buffer: two slices in flight, each issued once the
-            // previous tile's MMAs have released it; complete slice sl + 1
-            for (int sl = kS - 1; sl >= -1; sl--) {
-                if (sl >= 0) {
-                    bool ok2 = true;
-                    if (k >= 1) ok2 = wait_bar(&bars->b_empty[sl], uint32_t((k - 1) & 1), wait_limit, fail);
-                    if (gather_sync_or(kGatherThreads, !ok2)) {
-                        stop = true;
-                        break;
+            pend = -1;
+        };
+        // before a wait that does not end at once, what is under way is completed:
+        // the MMAs that free a buffer may need it first
+        auto wait_for = [&](uint64_t *bar, uint32_t parity) -> bool {
+            if (test_bar(bar, parity)) return true;
+            complete(0);
+            return wait_bar(bar, parity, wait_limit, fail);
+        };
+        for (int k = 0; k < nt && ok; k++) {
+            for (int i = 0; i < NKC; i++) {
+                const int kc = NKC == 2 ? x ^ i : 0, u = bbuf(k, kc), first_use = NKC == 2 ? 1 : 2;
+                if (i == 0 && k >= kMeta)
+                    ok = wait_for(&bars->meta_empty[k % kMeta], uint32_t(((k - kMeta) / kMeta) & 1));
+                if (ok && k >= first_use) ok = wait_for(&bars->b_empty[u], bpar(k - first_use));
+                if (!ok) break;   // uniform over the warp
+                if (c < tl.cnt) {
+                    if (i == 0 && j == 0) meta[(k % kMeta) * kN + c] = col_meta<S>(col, ev, inv_alpha_exp);
+                    const uint16_t *src = gm.dig + size_t(col.vec) * (S * KD) + kc * Sh::KC;
+                    uint8_t *dst = Bs + u * Sh::kBChunk + (c >> 3) * Sh::kSBO + (c & 7) * 16;
+                    for (int q = j; q < kPieces; q += kTPC) {
+                        const int sl = q / kRow, kg = q % kRow;
+                        cp_async16(dst + sl * Sh::kBSlice + kg * 128, src + sl * KD + kg * 8);
                     }
-                    for (int item = gt; item < tl.cnt * kPieces; item += kGatherThreads) {
-                        const int c = item / kPieces, kg = item % kPieces;
-                        const uint16_t *src = gm.dig + (size_t(M[c].vec) * kS + sl) * KD + kg * 8;
-                        cp_async16(Bs + sl * Sh::kBSlice + ((c >> 3) * kPieces + kg) * 128 + (c & 7) * 16, src);
-                    }
-                    cp_async_commit();
                 }
-                if (sl + 1 <= kS - 1) {
-                    cp_async_wait_pending(sl >= 0 ? 1 : 0);
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    gather_sync(kGatherThreads);
-                    if (gt == 0) mbar_arrive(&bars->b_full[k & 1][sl + 1]);
+                cp_async_commit();
+                complete(1);   // the previous unit
+                pend = u;
+                pend_meta = i == 0 ? k % kMeta : -1;
+                if (i == NKC - 1) {
+                    // one step of the following tiles' chains
+                    x = next_first(x, tl.rows > 128);
+                    tl = tl1;
+                    col = col1;
+                    if (j == 0 && c < tl.cnt) ev = gm.dexp[col.vec];
+                    tl1 = tl2;
+                    if (c < tl1.cnt) col1 = gm.cols[tl1.p0 + c];
+                    tl2 = tile_at(k + 3);
                 }
             }
         }
+        if (ok) complete(0);
         cp_async_wait_all();
     } else {
         // ---------------- epilogues ----------------
@@ -832,25 +841,27 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
         const int wq = warp & 3, half = (warp - kEpiWarp0) >> 2;
         int job = 0, k = 0;
         bool failed = false;
-        for (int tile = blockIdx.x; tile < gm.ntiles && !failed; tile += gridDim.x, k++) {
-            // the metadata is staged before the first slice (kS - 1) is gathered
-            if (!wait_bar(&bars->b_full[k & 1][kS - 1], uint32_t((k >> 1) & 1), wait_limit, fail)) break;
-            const SplitTile tl = gm.tiles[tile];
+        SplitTile tl{}, ntl{};
+        if (blockIdx.x < gm.ntiles) ntl = gm.tiles[blockIdx.x];
+        for (int tile = blockIdx.x; tile < gm.ntiles && !failed; tile += step, k++) {
+            tl = ntl;
+            if (tile + step < gm.ntiles) ntl = gm.tiles[tile + step];   // while this tile is worked on
             const int mh = tl.rows > 128 ? 2 : 1;
-            const ColMeta *M = meta + (k & 1) * kN;
+            const ColMeta *M = meta + (k % kMeta) * kN;
+            if (!wait_bar(&bars->meta_full[k % kMeta], uint32_t((k / kMeta) & 1), wait_limit, fail)) break;
             for (int h = 0; h < mh; h++, job++) {
                 const int r = job & 1;
-                if (!wait_bar(&bars->job_full[r], uint32_t((job >> 1) & 1), wait_limit, fail)) {
-                    failed = true;
-                    break;
-                }
-                tc_fence_after();
                 const bool small = tl.rows <= 64;
                 const int row = small ? (wq & 1) * 32 + lane : h * 128 + wq * 32 + lane;
                 const bool live = row < tl.rows;
                 const int ea = live ? gm.op_exp[tl.exp_off + row] : 0;
                 const int cb = small ? (wq >> 1) * (kN / 2) + half * (kN / 4) : half * (kN / 2);
                 const int ce = min(tl.cnt, cb + (small ? kN / 4 : kN / 2));
+                if (!wait_bar(&bars->job_full[r], uint32_t((job >> 1) & 1), wait_limit, fail)) {
+                    failed = true;
+                    break;
+                }
+                tc_fence_after();
                 epilogue_columns<S, ICVT>(gm, tl, M, tmem + (uint32_t(wq * 32) << 16) + uint32_t(r * kTmemBuf), cb, ce,
                                           row, live, ea, inv_alpha0);
                 tc_fence_before();
@@ -859,7 +870,7 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
             }
             if (failed) break;
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars->meta_empty[k & 1]);
+            if (lane == 0) mbar_arrive(&bars->meta_empty[k % kMeta]);
         }
     }
     if (*fail && tid == 0) atomicExch(err, 1);
@@ -890,7 +901,7 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
 // b_empty[3] (1: commit), job_full[2] (1: commit), job_empty[2], meta_empty[4]
 // (8: one per epilogue warp).
 // ---------------------------------------------------------------------------
-constexpr int kB64 = 3, kM64 = 4;
+constexpr int kB64 = 3, kM64 = kMeta;
 template <int S>
 struct Shape64 {
     static constexpr int N = Fmt<S>::N, L = Fmt<S>::L;
@@ -1118,7 +1129,7 @@ template <int KD, int S, bool ICVT>
 constexpr size_t gemm_smem()
 {
     if constexpr (KD == 64) return Shape64<S>::kSmem;
-    else return GemmShape<KD, S, (KD == 256 && ICVT) ? 2 : kNBuf>::kSmem;
+    else return GemmShape<KD, S, ICVT>::kSmem;
 }
 
 template <int KD, int S, bool ICVT>
