@@ -233,13 +233,6 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
                  : "r"(taddr));
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
-
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -285,18 +278,10 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// S * 2^ex as an FP64 value: the conversion rounds S to nearest even and the
-// scaling adds ex to the exponent field (exact; results below the normal
-// range, negligible here, become zero).  |S| < 2^62.
-__device__ __forceinline__ double i64_scaled(long long S, int ex)
-{
-    const long long b = __double_as_longlong(__ll2double_rn(S));
-    const int e = int((b >> 52) & 0x7FF) + ex;
-    return (S == 0 || e <= 0) ? 0.0 : __longlong_as_double(b + ((long long)ex << 52));
-}
-
-// The same value with integer operations only (bit for bit: S rounded to 53
-// bits, nearest with ties to even).  The tensor launches that run beside the
+// S * 2^ex as an FP64 value with integer operations only (bit for bit what the
+// hardware conversion and an exponent add give: S rounded to 53 bits, nearest with
+// ties to even; results below the normal range, negligible in the split modes,
+// become zero).  The tensor launches that run beside the
 // FP64 kernels use it, since the hardware conversion occupies the FP64 pipe,
 // a small fraction of the FP32 rate on this GPU.  The magnitude is
 // normalised so that its leading one is bit 63; its top 53 bits, rounded by
@@ -317,27 +302,30 @@ __device__ __forceinline__ double i64_scaled_int(long long S, int ex)
         static_cast<long long>((sgn | (static_cast<unsigned long long>(e - 1) << 52)) + mant + up));
 }
 
-// The eight levels of the 7-digit format: sum_g D_g 256^(7-g) (g = 0..7) times
-// 2^ex.  The sum is a product of vectors below 2^-1 in magnitude, K <= 256 of
-// them, so it is below 2^78; its last 16 bits are below the rounding of the
-// operands (2^17 and more), so it is rounded to a multiple of 2^16, which int64
-// holds, and converted once (one FP64 operation per element instead of three;
-// the conversions share the FP64 pipe, which bound the epilogue).  Results
-// outside the normal range take the general scaling.
+// v * 2^ex in general (results outside the normal range too).
 __device__ __noinline__ double scale_wide(double v, int ex) { return scalbn(v, ex); }
-__device__ __forceinline__ double levels_scaled(const int (&D)[kWideLevels], int ex)
+
+// The levels of one element as one integer, times 2^kShift of the units that the
+// column's exponent counts in.
+//   5 digits: sum_g D_g 256^(4-g).
+//   7 digits: sum_g D_g 256^(7-g), g = 0..7: a product of vectors below 2^-1 in
+//   magnitude, K <= 256 of them, so below 2^78; its last 16 bits are below the
+//   rounding of the operands (2^17 and more), so it is rounded to a multiple of
+//   2^16, which int64 holds, and converted once.
+template <int S>
+__device__ __forceinline__ long long level_sum(const int (&D)[Fmt<S>::L])
 {
-    const long long top = (long long)D[0] * 65536 + ((long long)D[1] * 256 + D[2]);
-    const long long mid = (long long)D[3] * 65536 + ((long long)D[4] * 256 + D[5]);
-    const long long low = ((long long)D[6] * 256 + (D[7] + 32768)) >> 16;
-    const long long S = (top << 24) + mid + low;
-    ex += 16;
-    const long long b = __double_as_longlong(__ll2double_rn(S));
-    const int es = int((b >> 52) & 0x7FF) + ex;
-    if (S == 0) return 0.0;
-    if (es <= 0 || es >= 0x7FF) return scale_wide(__longlong_as_double(b), ex);
-    return __longlong_as_double(b + ((long long)ex << 52));
+    if constexpr (S > 5) {
+        const long long top = (long long)D[0] * 65536 + ((long long)D[1] * 256 + D[2]);
+        const long long mid = (long long)D[3] * 65536 + ((long long)D[4] * 256 + D[5]);
+        const long long low = ((long long)D[6] * 256 + (D[7] + 32768)) >> 16;
+        return (top << 24) + mid + low;
+    } else {
+        const long long top = (long long)D[0] * 65536 + ((long long)D[1] * 256 + D[2]);
+        return (top << 16) + ((long long)D[3] * 256 + D[4]);
+    }
 }
+template <int S> constexpr int kShift = S > 5 ? 16 : 0;
 
 // S balanced base-256 digits (BF16 bit patterns) of round(x * 2^(8 S - E)),
 // |x| < 2^(E-1), from the FP64 bit pattern by integer operations; written to
@@ -530,47 +518,69 @@ __device__ __noinline__ double plain_product(const SplitGemm &gm, const SplitTil
 
 // One warp's share of a job: columns [cb, ce) of its 32 TMEM lanes (row `row`
 // of the tile's operator, valid where live; ea: its row exponent), from the
-// levels' column blocks at ta0.
+// levels' column blocks at ta0.  A batch of columns is worked on side by side,
+// without branches, where nothing in it is special (a factor 1/alpha0 that is no
+// power of two, a vector without digits, a short batch, a result outside the
+// normal range): element after element, each with its own branches, the latencies
+// of eight conversions stood one after another (660 cycles per element; a 60 x 32
+// tile of the M2L took 5,300 cycles, its MMAs 2,400).
 template <int S, bool ICVT>
 __device__ __forceinline__ void epilogue_columns(const SplitGemm &gm, const SplitTile &tl, const ColMeta *M, uint32_t ta0,
                                                  int cb, int ce, int row, bool live, int ea, double inv_alpha0)
 {
-    constexpr int kL = Fmt<S>::L, kN = Fmt<S>::N;
-    // columns per TMEM read: 8 levels take twice the registers of 5
-    constexpr int kQ = S > 5 ? 4 : 8;
+    constexpr int kL = Fmt<S>::L, kN = Fmt<S>::N, kQ = 4;   // columns per batch
     for (int c0 = cb; c0 < ce; c0 += kQ) {   // uniform over the warp
         uint32_t d[kL][kQ];
 #pragma unroll
-        for (int g = 0; g < kL; g++) {
-            if constexpr (kQ == 4) tmem_ld4(ta0 + uint32_t(g * kN + c0), d[g]);
-            else tmem_ld8(ta0 + uint32_t(g * kN + c0), d[g]);
+        for (int g = 0; g < kL; g++) tmem_ld4(ta0 + uint32_t(g * kN + c0), d[g]);
+        int ex[kQ], flags = c0 + kQ > ce;
+        double *out[kQ];
+#pragma unroll
+        for (int q = 0; q < kQ; q++) {   // (past ce: another column's or stale, not used)
+            ex[q] = M[c0 + q].exp + ea + kShift<S>;
+            out[q] = M[c0 + q].out + tl.row0 + row;
+            if (c0 + q < ce) flags |= M[c0 + q].flag;
         }
         tmem_ld_wait();
         if (!live) continue;
+        long long sum[kQ];
 #pragma unroll
         for (int q = 0; q < kQ; q++) {
-            const int c = c0 + q;
-            if (c >= ce) continue;
-            double val;
-            if constexpr (S > 5) {
-                if (M[c].flag & 2) {
-                    val = scale_wide(plain_product(gm, tl, row, M[c].vec), M[c].exp);
-                } else {
-                    int D[kL];
+            int D[kL];
 #pragma unroll
-                    for (int g = 0; g < kL; g++) D[g] = __float2int_rn(__uint_as_float(d[g][q]));
-                    val = levels_scaled(D, ea + M[c].exp);
-                }
-                if (M[c].flag & 1) val *= inv_alpha0;
+            for (int g = 0; g < kL; g++) D[g] = __float2int_rn(__uint_as_float(d[g][q]));
+            sum[q] = level_sum<S>(D);
+        }
+        double val[kQ];
+        bool odd = flags != 0;
+#pragma unroll
+        for (int q = 0; q < kQ; q++) {
+            if constexpr (ICVT) {
+                val[q] = i64_scaled_int(sum[q], ex[q]);
             } else {
-                long long sum = 0;
-#pragma unroll
-                for (int g = 0; g < kL; g++)
-                    sum += (long long)__float2int_rn(__uint_as_float(d[g][q])) << (8 * (kL - 1 - g));
-                val = ICVT ? i64_scaled_int(sum, ea + M[c].exp) : i64_scaled(sum, ea + M[c].exp);
-                if (M[c].flag) val *= inv_alpha0;
+                const long long bits = __double_as_longlong(__ll2double_rn(sum[q]));
+                const int es = int((bits >> 52) & 0x7FF) + ex[q];
+                val[q] = sum[q] == 0 ? 0.0 : __longlong_as_double(bits + ((long long)ex[q] << 52));
+                if constexpr (S > 5) odd |= sum[q] != 0 && unsigned(es - 1) >= 0x7FEu;   // es <= 0 or >= 0x7FF
+                else if (sum[q] != 0 && es <= 0) val[q] = 0.0;
             }
-            M[c].out[tl.row0 + row] = val;
+        }
+        if (!odd) {
+#pragma unroll
+            for (int q = 0; q < kQ; q++) *out[q] = val[q];
+            continue;
+        }
+#pragma unroll
+        for (int q = 0; q < kQ; q++) {
+            if (c0 + q >= ce) continue;
+            double v = val[q];
+            const int f = M[c0 + q].flag;
+            if constexpr (S > 5) {
+                if (f & 2) v = scale_wide(plain_product(gm, tl, row, M[c0 + q].vec), M[c0 + q].exp);
+                else if (sum[q] != 0) v = scale_wide(__ll2double_rn(sum[q]), ex[q]);
+            }
+            if (f & 1) v *= inv_alpha0;
+            *out[q] = v;
         }
     }
 }
