@@ -248,11 +248,10 @@ bc_status bc_eval_points_grad(bc_ctx *ctx, const bc_tree *tree, const double *u,
  * at every leaf node x_i ([nleaf][p][p], as the applies).  A source that
  * coincides with a node contributes nothing there.  The far field uses the
  * tree's expansions and lists (error of the expansion order, as the volume
- * apply), the near field is summed directly, in FP64.  precision BC_FP64: all
- * of it in FP64; BC_SPLIT_BF16 (p = 8, 12, 16, nterms <= 32, else
- * BC_ERR_UNSUPPORTED): the local-to-node evaluation (L2P) at every leaf runs
- * on the BF16 tensor cores as exact digit products (the volume apply's
- * split-precision L2P), the rest in FP64; other values BC_ERR_ARG.
+ * apply), the near field is summed directly, in FP64.  The local-to-node
+ * evaluation (L2P) at every leaf is the volume apply's of the same precision:
+ * BC_FP64 7 digits, BC_SPLIT_BF16 5 digits (p = 8, 12, 16, nterms <= 32, else
+ * BC_ERR_UNSUPPORTED); other values BC_ERR_ARG.
  *
  * bc_layer_create: the sources xy[n][2] (host, read during the call), inside
  * the root box (else BC_ERR_ARG), are sorted into the tree's leaves, and the

@@ -21,8 +21,9 @@
 //        L_l = sum (-1)^l (2w)^-l [ -c_q / l + (c_m / r_c) / w ]
 //   M2P  (W list) and L2P as for the volume potential, near field direct;
 // with c_q = -q / (2 pi), c_m = -m / (2 pi).  A source that coincides with a
-// target node contributes nothing.  FP64 throughout, except the split option's
-// L2P (the volume apply's group-E tensor tiles over the same locals).
+// target node contributes nothing.  FP64 throughout, except the L2P (the volume
+// apply's group-E tensor tiles over the same locals: 7 digits in the FP64 mode, 5
+// in the split one; 1.86 -> NN ms at 17,584 leaves, 4,096 nodes, FP64).
 #include <cuda_runtime.h>
 
 #include <algorithm>

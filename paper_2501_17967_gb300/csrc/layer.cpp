@@ -231,12 +231,16 @@ bc_status bc_layer_apply(bc_ctx *ctx, bc_layer *layer, const double *q, const do
     const SplitLaunch *split = nullptr;
     if (prec == BC_SPLIT_BF16) {
         if (!ctx->split_ready) {
-            set_error("bc_layer_apply: split precision is provided for p = 16 with nterms <= 32 only");
+            set_error("bc_layer_apply: split precision is provided for p = 8, 12 and 16 with nterms <= 32 only");
             return BC_ERR_UNSUPPORTED;
         }
         const bc_status bs = prepare_split_tree(tree);
         if (bs != BC_OK) return bs;
         sl.tree = &tree->sp;
+        split = &sl;
+    } else if (prepare_wide_tree(tree)) {   // FP64: the L2P on 7 digits (else on the FP64 pipe)
+        sl.tables = &ctx->wide;
+        sl.tree = &tree->spw;
         split = &sl;
     }
     const size_t nu = size_t(tree->h.nleaf) * ctx->NP, n = size_t(layer->n);
