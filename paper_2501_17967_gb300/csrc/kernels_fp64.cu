@@ -669,13 +669,83 @@ inline int m2l_groups(int P1)
 inline int m2l_threads(int P1) { return (m2l_groups(P1) * P1 + 31) / 32 * 32; }
 
 // -------------------------------------------------------------------------
+// RowSum: sum of doubles, a group at a time, by integer operations.  An FP64 addition
+// holds a sub-partition's FP64 pipe for 64 cycles per warp, so a kernel that only
+// sums rows was bound by its additions, not by memory; aligning a significand to
+// the largest exponent so far and adding it as an integer takes about 15 operations
+// of the integer pipe, 30 cycles.  s counts units of 2^(e - 1080), e the largest
+// biased exponent so far (ek its place in the high word): a significand has 5 bits
+// below its last, so 32 terms fit in 63 bits and each loses less than 2^-5 of the
+// last place of the largest term, where an FP64 addition rounds to half of one.
+// Groups with an infinity or a NaN, near the ends of the range, or all zero are added
+// in FP64.  k_v_sums (300,000 pairs, 31 coefficients): 84 -> 53 us.
+// -------------------------------------------------------------------------
+struct RowSum {
+    double v = 0.0;
+    long long s = 0;
+    int ek = 0, n = 0;
+
+    __device__ __forceinline__ void term(double x, int em, long long &t) const
+    {
+        const int hi = __double2hiint(x);
+        const int sh = min((em - (hi & 0x7FF00000)) >> 20, 63);
+        unsigned long long m = (static_cast<unsigned long long>((hi & 0x000FFFFF) | 0x00100000) << 32 |
+                                static_cast<unsigned>(__double2loint(x)))
+                               << 5;
+        m >>= sh;
+        const long long g = hi >> 31;
+        t += (static_cast<long long>(m) ^ g) - g;
+    }
+    __device__ __forceinline__ double part() const   // s as a double (s != 0)
+    {
+        return __longlong_as_double(__double_as_longlong(__ll2double_rn(s)) +
+                                    (static_cast<long long>((ek >> 20) - 1080) << 52));
+    }
+    __device__ __forceinline__ void flush()
+    {
+        if (s != 0) v = __double_as_longlong(v) == 0 ? part() : v + part();
+        s = 0;
+        ek = 0;
+        n = 0;
+    }
+    template <int N>
+    __device__ __forceinline__ void add(const double *x)
+    {
+        constexpr int kExp = 0x7FF00000, kLo = 128 << 20, kHi = 0x7F0 << 20;
+        if (n > 32 - N) flush();
+        int em = ek;
+#pragma unroll
+        for (int q = 0; q < N; q++) em = max(em, __double2hiint(x[q]) & kExp);
+        if (em < kLo || em >= kHi) {
+            flush();
+#pragma unroll
+            for (int q = 0; q < N; q++) v += x[q];
+            return;
+        }
+        s >>= min((em - ek) >> 20, 63);
+        ek = em;
+        n += N;
+#pragma unroll
+        for (int q = 0; q < N; q++) term(x[q], em, s);
+    }
+    __device__ __forceinline__ double total()
+    {
+        flush();
+        return v;
+    }
+};
+
+// -------------------------------------------------------------------------
 // v_sums: each box's V-list sum from the tensor-core M2L's rows (which leave
 // out the log term), one warp per box, lane o = coefficient o:
 //   out[b][o] = sum_{e in V(b)} [ Pv[e][o] + (o = 0) (log|d_e| + log r_b) first[s_e][0] ]
 // Apart from the downward pass, whose chain of boxes would wait for the ~27
-// dependent row loads of each.  Memory bound: 16 P1 bytes per pair.
+// dependent row loads of each.  16 P1 bytes per pair (197 MB at 300,000 pairs, 29 us);
+// bound by the additions: kVRows rows in flight, summed by RowSum, with 64 registers
+// per thread (12 rows took 90, two blocks per SM and 67 us instead of 53).
 // -------------------------------------------------------------------------
-__global__ void __launch_bounds__(256)
+constexpr int kVRows = 8;
+__global__ void __launch_bounds__(256, 4)
 k_v_sums(int64_t b0, int64_t b1, const int32_t *__restrict__ v_ptr, const int32_t *__restrict__ v_src,
          const int32_t *__restrict__ v_code, const int32_t *__restrict__ box_level, const double *__restrict__ logd,
          const double *__restrict__ lvtab, const double2 *__restrict__ Pv, const double2 *__restrict__ first,
@@ -695,20 +765,34 @@ k_v_sums(int64_t b0, int64_t b1, const int32_t *__restrict__ v_ptr, const int32_
             li = fma(c0, a0.y, li);
         }
         if (o < P1) {
-#pragma unroll 8
-            for (int e = v0; e < v1; e++) {
-                const double2 t = Pv[int64_t(e) * P1 + o];
-                re += t.x;
-                im += t.y;
+            RowSum sr, si;
+            for (int e = v0; e < v1; e += kVRows) {   // the rows of a batch in flight together
+                double tr[kVRows], ti[kVRows];
+#pragma unroll
+                for (int q = 0; q < kVRows; q++) {
+                    const double2 t = e + q < v1 ? Pv[int64_t(e + q) * P1 + o] : make_double2(0.0, 0.0);
+                    tr[q] = t.x;
+                    ti[q] = t.y;
+                }
+#pragma unroll
+                for (int q = 0; q < kVRows; q += 4) {
+                    if (e + q >= v1) break;   // uniform over the warp
+                    sr.add<4>(tr + q);
+                    si.add<4>(ti + q);
+                }
             }
+            re = sr.total();
+            im = si.total();
         }
-        for (int m = 16; m > 0; m >>= 1) {
-            lr += __shfl_xor_sync(0xffffffffu, lr, m);
-            li += __shfl_xor_sync(0xffffffffu, li, m);
-        }
+        // both sums in one butterfly: lanes 0..15 go on with the real part, 16..31
+        // with the imaginary one
+        double l = lane < 16 ? lr : li;
+        l += __shfl_xor_sync(0xffffffffu, lane < 16 ? li : lr, 16);
+        for (int m = 8; m > 0; m >>= 1) l += __shfl_xor_sync(0xffffffffu, l, m);
+        const double lim = __shfl_sync(0xffffffffu, l, 16);
         if (o == 0) {
-            re += lr;
-            im += li;
+            re += l;
+            im += lim;
         }
         if (o < P1) out[b * P1 + o] = make_double2(re, im);
     }
@@ -1174,7 +1258,7 @@ __global__ void __launch_bounds__(256)
 k_leaf_logs(int64_t nleaf, const int32_t *__restrict__ leaf_box, const int32_t *__restrict__ leaf_level,
             const int32_t *__restrict__ w_ptr, const int32_t *__restrict__ w_src, const int32_t *__restrict__ n_ptr,
             const int32_t *__restrict__ n_src, const double2 *__restrict__ src, const double2 *__restrict__ aux,
-            const double *__restrict__ lvtab, int P1, double2 *__restrict__ logs)
+            const double *__restrict__ lvtab, int P1, bool fold, double2 *__restrict__ logs)
 {
     griddep_wait();
     griddep_launch_dependents();
@@ -1187,6 +1271,14 @@ k_leaf_logs(int64_t nleaf, const int32_t *__restrict__ leaf_box, const int32_t *
             const int s = n_src[e];
             const double a0 = aux[int64_t(leaf_box[s]) * P1].x;
             ln += ADJ ? a0 : lvtab[kLvTab + leaf_level[s]] * a0;
+        }
+        const int lv = leaf_level[o];
+        const double lg = lvtab[kLvTab + lv];
+        if (fold) {   // one term for k_leaf_sums, times w_j in the adjoint direction
+            double l = ADJ ? lw + ln : fma(lg, lw, ln);
+            for (int m = 16; m > 0; m >>= 1) l += __shfl_xor_sync(0xffffffffu, l, m);
+            if (lane == 0) logs[o] = make_double2(ADJ ? lvtab[lv] * lg * kInvTwoPi * l : l, 0.0);
+            continue;
         }
         for (int m = 16; m > 0; m >>= 1) {
             lw += __shfl_xor_sync(0xffffffffu, lw, m);
@@ -1314,6 +1406,86 @@ __global__ void k_leaf_out(int64_t nleaf, const int32_t *__restrict__ order,
         acc = fma(cO, l0, acc);
         acc = ADJ ? fma(cO, l1, acc) : acc + l1;
         vout[int64_t(o) * NP + j] = acc;
+    }
+}
+
+// -------------------------------------------------------------------------
+// leaf_sums: the leaf output where every product comes as rows from the tensor
+// cores (scales applied): per node PE + the W rows + the near rows + the leaf's
+// log term, one thread per node.  A stream of rows (2 KB each at p = 16, about 13
+// per leaf); kLeafRows of them in flight, the next leaf's lists read before the
+// sums.  Of each four rows one is added in FP64 and three by RowSum: the FP64 pipe
+// and the integer pipe work side by side, neither alone keeps up with memory.
+// 17,491 leaves, p = 16 (500 MB, 74 us at the copy rate): all additions in FP64 139 us
+// (forward) and 161 (adjoint), all by RowSum 137, one in four 99.
+// -------------------------------------------------------------------------
+constexpr int kLeafRows = 12;
+template <bool ADJ>
+__global__ void __launch_bounds__(256)
+k_leaf_sums(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__restrict__ leaf_level,
+            const int32_t *__restrict__ w_ptr, const int32_t *__restrict__ n_ptr, const double *__restrict__ wvec,
+            double *__restrict__ vout, int NP, bool far, const double *__restrict__ Pnear,
+            const double *__restrict__ PE, const double *__restrict__ PW, const uint8_t *__restrict__ active,
+            const double2 *__restrict__ logs)
+{
+    griddep_wait();
+    griddep_launch_dependents();
+    const int j = threadIdx.x;   // blockDim.x == NP
+    const double wj = ADJ ? wvec[j] : 0.0;
+    struct Leaf {
+        int o, lv, w0, w1, n0, n1;
+        double lg;
+        bool on;
+    };
+    auto read = [&](int o) {
+        Leaf l;
+        l.o = o;
+        l.lv = leaf_level[o];
+        l.w0 = w_ptr[o];
+        l.w1 = w_ptr[o + 1];
+        l.n0 = n_ptr[o];
+        l.n1 = n_ptr[o + 1];
+        l.lg = logs[o].x;
+        l.on = !active || active[o];   // off: a discarded leaf of a truncated tree
+        return l;
+    };
+    int64_t li = blockIdx.x;
+    if (li >= nleaf) return;
+    Leaf cur = read(order[li]);
+    int onext = li + gridDim.x < nleaf ? order[li + gridDim.x] : -1;
+    for (;;) {
+        const Leaf l = cur;
+        RowSum acc;
+        auto add_rows = [&](const double *p, int cnt, bool first) {
+            for (;;) {
+                double x[kLeafRows];
+#pragma unroll
+                for (int q = 0; q < kLeafRows; q++) {
+                    x[q] = q < cnt ? *p : 0.0;
+                    p += NP;
+                }
+                if (first && onext >= 0) {
+                    cur = read(onext);
+                    li += gridDim.x;
+                }
+                first = false;
+#pragma unroll
+                for (int q = 0; q < kLeafRows; q += 4) {
+                    if (q >= cnt) break;   // uniform over the block
+                    acc.v += x[q];
+                    if (q + 1 < cnt) acc.add<3>(x + q + 1);
+                }
+                if ((cnt -= kLeafRows) <= 0) break;
+            }
+        };
+        if (l.on && far && l.lv >= 2) acc.v = PE[int64_t(l.o) * NP + j];
+        add_rows(Pnear + int64_t(l.n0) * NP + j, l.on ? l.n1 - l.n0 : 0, true);
+        if (l.on && l.w1 > l.w0) add_rows(PW + int64_t(l.w0) * NP + j, l.w1 - l.w0, false);
+        double u = 0.0;
+        if (l.on) u = ADJ ? fma(wj, l.lg, acc.total()) : acc.total() + l.lg;
+        vout[int64_t(l.o) * NP + j] = u;
+        if (onext < 0) return;
+        onext = li + gridDim.x < nleaf ? order[li + gridDim.x] : -1;
     }
 }
 
@@ -1718,15 +1890,18 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
                                1.0 / alpha0, sp->err, st);
         if (ce != cudaSuccess) return ce;
     }
+    const double *Pnear = (parts & 1) ? sp->Pnear : nullptr, *PE = (parts & 8) ? sp->PE : nullptr,
+                 *PW = (parts & 16) ? sp->PW : nullptr;
+    const bool rows_only = Pnear && PE && PW;
     // the log-term sums of every leaf's W and near lists (they read `first`
     // only), before the join: they run while the near field finishes
     {
         const int32_t *wl = far ? d.w_ptr : d.zero_ptr, *nl = near ? d.near_ptr : d.zero_ptr;
         const int lgrid = grid_for((a.nleaf + 7) / 8, 152 * 8);
         ce = adj ? launch_pdl(k_leaf_logs<true>, lgrid, 256, 0, st, a.nleaf, d.leaf_box, d.leaf_level, wl, d.w_src,
-                              nl, d.near_src, first, first, d.lvtab, P1, d.leaf_logs)
+                              nl, d.near_src, first, first, d.lvtab, P1, rows_only, d.leaf_logs)
                  : launch_pdl(k_leaf_logs<false>, lgrid, 256, 0, st, a.nleaf, d.leaf_box, d.leaf_level, wl, d.w_src,
-                              nl, d.near_src, first, first, d.lvtab, P1, d.leaf_logs);
+                              nl, d.near_src, first, first, d.lvtab, P1, rows_only, d.leaf_logs);
         if (ce != cudaSuccess) return ce;
     }
     if (ev) cudaEventRecord(ev[6], st);
@@ -1735,9 +1910,12 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
     // near log aux = first (multipole / adjoint local)
     size_t shD = sizeof(double2) * P1 + sizeof(double) * NP;
     const int32_t *wp = far ? d.w_ptr : d.zero_ptr, *np_ = near ? d.near_ptr : d.zero_ptr;
-    const double *Pnear = (parts & 1) ? sp->Pnear : nullptr, *PE = (parts & 8) ? sp->PE : nullptr,
-                 *PW = (parts & 16) ? sp->PW : nullptr;
-    if (adj)
+    if (rows_only)
+        ce = adj ? launch_pdl(k_leaf_sums<true>, grid_leaf, NP, 0, st, a.nleaf, d.leaf_order, d.leaf_level, wp, np_,
+                              tb.wvec, vout, NP, far, Pnear, PE, PW, d.leaf_active, d.leaf_logs)
+                 : launch_pdl(k_leaf_sums<false>, grid_leaf, NP, 0, st, a.nleaf, d.leaf_order, d.leaf_level, wp, np_,
+                              tb.wvec, vout, NP, far, Pnear, PE, PW, d.leaf_active, d.leaf_logs);
+    else if (adj)
         ce = launch_pdl(k_leaf_out<true>, grid_leaf, NP, shD, st, a.nleaf, d.leaf_order, d.leaf_box, d.leaf_level,
                         wp, d.w_src, d.w_code, np_, d.near_src, d.near_tab, op.e, op.w, op.t, tb.wvec, second, first,
                         first, vin, vout, NP, P1, d.lvtab, far, Pnear, PE, PW, d.leaf_active, d.leaf_logs);

@@ -368,33 +368,46 @@ __device__ __forceinline__ int exp_key(long long bits)
 
 // ---------------------------------------------------------------------------
 // Digits of scale * cs_k * (leaf vectors): dig[leaf][a][k], dexp[leaf] = E with
-// max |scale cs v| < 2^(E-1).  One block of kv threads (kv rounded up to whole
-// warps) per leaf; the np <= kv nodes of a leaf, then zero digits up to kv.
+// max |scale cs v| < 2^(E-1).  One block per leaf, each thread two neighbouring
+// nodes (their digits go out as one word, 41 -> 33 us at 17,491 leaves of 256 nodes
+// and 7 digits; bound by integer operations); the np <= kv nodes of a leaf, then zero
+// digits up to kv (even).
 template <int S>
-__global__ void __launch_bounds__(256) k_split_vec(int64_t nleaf, const double *__restrict__ v, double scale,
+__global__ void __launch_bounds__(128) k_split_vec(int64_t nleaf, const double *__restrict__ v, double scale,
                                                    const double *__restrict__ cs, uint16_t *__restrict__ dig,
                                                    int32_t *__restrict__ dexp, const uint8_t *__restrict__ active,
                                                    int np, int kv)
 {
     griddep_wait();
     griddep_launch_dependents();
-    __shared__ int wmax[8];
-    const int k = threadIdx.x, nwp = blockDim.x >> 5;
-    const double sk = (S > 5 && cs && k < np) ? scale * cs[k] : scale;
-    for (int64_t leaf = blockIdx.x; leaf < nleaf; leaf += gridDim.x) {
+    __shared__ int wmax[2][4];
+    const int k = 2 * threadIdx.x, nwp = blockDim.x >> 5, w = threadIdx.x >> 5;
+    double sk[2];
+#pragma unroll
+    for (int q = 0; q < 2; q++) sk[q] = (S > 5 && cs && k + q < np) ? scale * cs[k + q] : scale;
+    int par = 0;   // the maxima of consecutive leaves in turn: one barrier per leaf
+    for (int64_t leaf = blockIdx.x; leaf < nleaf; leaf += gridDim.x, par ^= 1) {
         // a discarded leaf of a truncated tree is no source: zero digits
-        const double x = (k >= np || (active && !active[leaf])) ? 0.0 : v[leaf * np + k];
-        const long long bits = __double_as_longlong(sk * x);
-        int m = exp_key<S>(bits);
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if ((k & 31) == 0) wmax[k >> 5] = m;
+        const bool on = !active || active[leaf];
+        long long bits[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+            bits[q] = __double_as_longlong(sk[q] * (on && k + q < np ? v[leaf * np + k + q] : 0.0));
+        const int m = __reduce_max_sync(0xffffffffu, max(exp_key<S>(bits[0]), exp_key<S>(bits[1])));
+        if ((threadIdx.x & 31) == 0) wmax[par][w] = m;
         __syncthreads();
-        int emax = wmax[0];
-        for (int w = 1; w < nwp; w++) emax = max(emax, wmax[w]);
-        __syncthreads();
+        int emax = wmax[par][0];
+        for (int q = 1; q < nwp; q++) emax = max(emax, wmax[par][q]);
         const bool wide = S > 5 && emax == 0x7FF;
         const int E = emax ? emax - 1023 + 2 : 0;
-        if (k < kv) digits_of<S>(emax && !wide ? bits : 0ll, E, dig + leaf * (S * kv) + k, kv);
+        if (k < kv) {
+            uint16_t d[2][S];
+#pragma unroll
+            for (int q = 0; q < 2; q++) digits_of<S>(emax && !wide ? bits[q] : 0ll, E, d[q], 1);
+            uint32_t *out = reinterpret_cast<uint32_t *>(dig + leaf * (S * kv) + k);
+#pragma unroll
+            for (int a = 0; a < S; a++) out[a * (kv / 2)] = uint32_t(d[0][a]) | uint32_t(d[1][a]) << 16;
+        }
         if (k == 0) dexp[leaf] = wide ? kWideExp : E;
     }
 }
@@ -1280,7 +1293,7 @@ cudaError_t launch_split_digits_vec(const SplitTables &T, int dir, int64_t nleaf
                                     uint16_t *dig, int32_t *dexp, cudaStream_t st, const uint8_t *active)
 {
     if (nleaf <= 0) return cudaSuccess;
-    const int grid = int(std::min<int64_t>(nleaf, 152 * 16)), nth = (T.kv + 31) / 32 * 32;
+    const int grid = int(std::min<int64_t>(nleaf, 152 * 16)), nth = (T.kv / 2 + 31) / 32 * 32;
     if (T.slices == kWideSlices)
         return launch_pdl(k_split_vec<kWideSlices>, grid, nth, 0, st, nleaf, v, scale, T.vscale[dir], dig, dexp, active,
                           T.np, T.kv);
