@@ -47,50 +47,67 @@ __device__ __forceinline__ double2 cinv(double2 a)
     return make_double2(a.x * d, -a.y * d);
 }
 // ---------------------------------------------------------------------------
-// log x and 1/x for the direct near sums, written for this GPU's FP64 rate
-// (1/64 of FP32): a table-driven logarithm after Tang (ACM TOMS 16, 1990).
-// With x = 2^e m, m in [1, 2), and j the top kLogBits bits of m's fraction,
-// c_j is a short (9-bit) approximation of 1 / (1 + (j + 1/2) / 2^kLogBits)
-// (c_0 = 1), so that r = m c_j - 1 is one FMA with a single rounding and
-// |r| < 0.008; then
-//     log x = e ln 2 - log c_j + log1p(r),  log1p(r) = r - r^2/2 + ... + r^7/7,
-//     1/x   = 2^-e c_j / (1 + r),           1/(1 + r) = 1 - r + ... - r^7,
-// both series truncated below 2e-17 relative.  ln 2 is split so that e ln2_hi
-// is exact (42 bits); -log c_j is stored as a double-double.  About 13 FP64
-// operations for the logarithm and 8 for the reciprocal.  Valid for normal x
-// with 1/x normal (|e| <= 1021), which the near sums' squared distances meet.
-// Table: g_logtab[4 j + 0..2] = c_j, hi, lo of -log c_j; [4 kLogN + 0..1] =
-// ln2_hi, ln2_lo (set by layer_log_init).
+// log x and 1/x for the direct near sums: a table-driven logarithm after Tang (ACM
+// TOMS 16, 1990) in fixed point.  An FP64 operation holds a sub-partition's FP64
+// pipe for 64 cycles per warp, 30 of them per (node, source) pair bound the sums
+// (13 for the logarithm, 8 for the reciprocal); integer and FP32 operations take 1 or
+// 2 cycles, and only the two conversions are left on the FP64 pipe.  With
+// x = 2^e m, m in [1, 2), and j the top kLogBits bits of m's fraction, c_j is
+// 1 / (1 + (j + 1/2) / 2^kLogBits) rounded to 11 bits, so that m c_j is an exact 64-bit
+// integer and r = m c_j - 1 an exact multiple of 2^-63, |r| < 7.4e-4; then
+//     log x = e ln 2 - log c_j + log1p(r),  log1p(r) = r - r^2/2 + r^3 (1/3 - r/4 + r^2/5),
+//     1/x   = 2^-e c_j / (1 + r),           1/(1+r)  = 1 - r + r^2 + r^3 (-1 + r - r^2),
+// the linear and square terms as 64-bit integers (r^2 to 2^-62), the cubic ones, below
+// 4e-10, in FP32 (2e-17), the series cut below 2e-19.  Errors before the last rounding:
+// logarithm 2^-53 absolute, reciprocal 2^-54 relative.  Valid for normal x with 1/x
+// normal (|e| <= 1021), which the near sums' squared distances meet.  Table:
+// g_logtab[j] = (c_j 2^11 - 1024) in 11 bits, -log c_j in units of 2^-53 in 53 bits (set by
+// layer_log_init).
 // ---------------------------------------------------------------------------
-constexpr int kLogBits = 7, kLogN = 1 << kLogBits, kLogTabLen = 4 * kLogN + 2;
-__device__ double g_logtab[kLogTabLen];
+constexpr int kLogBits = 10, kLogN = 1 << kLogBits;
+__device__ unsigned long long g_logtab[kLogN];
 
-__device__ __forceinline__ void log_inv(double x, const double *__restrict__ tab, double &lg, double &inv)
+// m 2^ex, m > 0 and the result normal, rounded to nearest by integer operations.
+__device__ __forceinline__ long long int_bits(unsigned long long m, int ex)
 {
+    const int lz = __clzll(static_cast<long long>(m));
+    m <<= lz;   // leading one at bit 63: it adds one to the exponent field
+    return (static_cast<long long>(63 - lz + ex + 1022) << 52) + static_cast<long long>(m >> 11) +
+           static_cast<long long>((m >> 10) & 1);
+}
+
+__device__ __forceinline__ void log_inv(double x, const unsigned long long *__restrict__ tab, double &lg, double &inv)
+{
+    constexpr long long kLn2 = 6243314768165359ll;   // ln 2 in units of 2^-53, and the next 32 bits
+    constexpr unsigned kLn2Lo = 897137782u;
     const long long bits = __double_as_longlong(x);
     const int e = int(bits >> 52) - 1023;   // x > 0
-    const int j = int((bits >> (52 - kLogBits)) & (kLogN - 1));
-    const double m = __longlong_as_double((bits & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-    const double c = tab[4 * j], Lh = tab[4 * j + 1], Ll = tab[4 * j + 2];
-    const double r = fma(m, c, -1.0);
-    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);   // log1p(r) = r + r^2 q(r)
-    q = fma(q, r, 0.2);
-    q = fma(q, r, -0.25);
-    q = fma(q, r, 1.0 / 3.0);
-    q = fma(q, r, -0.5);
-    const double ed = double(e);
-    lg = fma(ed, tab[4 * kLogN], Lh) + (fma(r * r, q, fma(ed, tab[4 * kLogN + 1], Ll)) + r);
-    double s = 1.0 - r;   // 1 / (1 + r)
-#pragma unroll
-    for (int k = 0; k < 6; k++) s = fma(s, -r, 1.0);
-    inv = __longlong_as_double(__double_as_longlong(c * s) - (static_cast<long long>(e) << 52));
+    const unsigned long long tw = tab[int(bits >> (52 - kLogBits)) & (kLogN - 1)];
+    const unsigned c = 1024u + unsigned(tw >> 53);
+    const unsigned long long m = (bits & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll;
+    const long long r = static_cast<long long>(m * c - (1ull << 63));   // units 2^-63
+    // r^2 in units of 2^-82, from r = 2^22 rh + rl
+    const int rh = int(r >> 22), rl = int(r) & 0x3FFFFF;
+    const long long w = static_cast<long long>(rh) * rh + ((static_cast<long long>(rh) * rl) >> 21);
+    // the cubic terms in units of 2^-61
+    const float rf = float(rh) * 0x1p-41f, r3 = rf * rf * (rf * 0x1p61f);
+    const int cl = __float2int_rn(r3 * fmaf(rf, fmaf(rf, 0.2f, -0.25f), 1.0f / 3.0f));
+    const int ci = __float2int_rn(r3 * fmaf(rf, 1.0f - rf, -1.0f));
+    const long long l1 = r - (w >> 20) + 4ll * cl;
+    const long long l = static_cast<long long>(tw & ((1ull << 53) - 1)) + ((l1 + 512) >> 10) + e * kLn2 +
+                        ((static_cast<long long>(e) * kLn2Lo) >> 32);
+    const long long lb = int_bits(static_cast<unsigned long long>(l < 0 ? -l : l), -53);
+    lg = l ? __longlong_as_double(lb | (l & (1ll << 63))) : 0.0;
+    const unsigned long long s = (1ull << 63) - r + (w >> 19) + 4ll * ci;   // 1 / (1 + r), units 2^-63
+    const unsigned cw = c << 20;
+    inv = __longlong_as_double(int_bits((s >> 32) * cw + __umulhi(unsigned(s), cw), -62 - e));   // from units 2^-62
 }
 
 __global__ void k_log_inv_check(const double *__restrict__ x, int64_t n, double *__restrict__ lg,
                                 double *__restrict__ inv)
 {
-    __shared__ double tab[kLogTabLen];
-    for (int i = threadIdx.x; i < kLogTabLen; i += blockDim.x) tab[i] = g_logtab[i];
+    __shared__ unsigned long long tab[kLogN];
+    for (int i = threadIdx.x; i < kLogN; i += blockDim.x) tab[i] = g_logtab[i];
     __syncthreads();
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
         double a, b;
@@ -254,8 +271,8 @@ k_layer_out(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
     __shared__ double2 se[32];
     __shared__ double2 s_xy[kSrcChunk], s_m[kSrcChunk];
     __shared__ double s_q[kSrcChunk];
-    __shared__ double s_log[kLogTabLen];
-    for (int i = j; i < kLogTabLen; i += blockDim.x) s_log[i] = g_logtab[i];   // read after the first barrier below
+    __shared__ unsigned long long s_log[kLogN];
+    for (int i = j; i < kLogN; i += blockDim.x) s_log[i] = g_logtab[i];   // read after the first barrier below
     const double pi = 3.14159265358979323846;
     const double xj = -cos((2.0 * (j % p) + 1.0) * pi / (2.0 * p)), yj = -cos((2.0 * (j / p) + 1.0) * pi / (2.0 * p));
     for (int64_t li = blockIdx.x; li < nleaf; li += gridDim.x) {
@@ -313,7 +330,8 @@ k_layer_out(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
                 for (int i = 0; i < cnt; i++) {
                     const double dx = zx - s_xy[i].x, dy = zy - s_xy[i].y;
                     const double r2 = fma(dx, dx, dy * dy);
-                    if (r2 > 0.0) {
+                    // r2 > 0, as integers (no sign bit; NaN is left out, as by the comparison)
+                    if (static_cast<unsigned long long>(__double_as_longlong(r2)) - 1 < 0x7FF0000000000000ull) {
                         double lg, ir2;
                         log_inv(r2, s_log, lg, ir2);
                         near = fma(s_q[i], lg, near);
@@ -332,26 +350,14 @@ inline int grid_cap(int64_t n, int cap) { return int(n < cap ? (n > 0 ? n : 1) :
 
 cudaError_t layer_log_init()
 {
-    // c_j (9 bits), -log c_j as hi + lo from the host's extended-precision
-    // logarithm, and ln 2 split so that its high part has 42 bits
-    double t[kLogTabLen] = {};
+    // c_j to 11 bits, -log c_j from the host's extended-precision logarithm
+    unsigned long long t[kLogN];
     for (int j = 0; j < kLogN; j++) {
-        const double F = 1.0 + (j + 0.5) / kLogN;
-        const double c = j == 0 ? 1.0 : std::nearbyint(512.0 / F) / 512.0;
-        const long double L = -logl(static_cast<long double>(c));
-        t[4 * j] = c;
-        t[4 * j + 1] = static_cast<double>(L);
-        t[4 * j + 2] = static_cast<double>(L - static_cast<long double>(t[4 * j + 1]));
+        const double c = std::nearbyint(2048.0 / (1.0 + (j + 0.5) / kLogN));
+        const long double l = -logl(static_cast<long double>(c) / 2048.0L);
+        t[j] = static_cast<unsigned long long>(c - 1024.0) << 53 |
+               static_cast<unsigned long long>(l * 9007199254740992.0L + 0.5L);
     }
-    const long double ln2 = logl(2.0L);
-    long long b;
-    const double l2 = static_cast<double>(ln2);
-    std::memcpy(&b, &l2, sizeof b);
-    b &= ~((1ll << 11) - 1);
-    double l2h;
-    std::memcpy(&l2h, &b, sizeof b);
-    t[4 * kLogN] = l2h;
-    t[4 * kLogN + 1] = static_cast<double>(ln2 - static_cast<long double>(l2h));
     return cudaMemcpyToSymbol(g_logtab, t, sizeof t);
 }
 
