@@ -224,11 +224,8 @@ UpScheduleHost build_up_schedule(const std::vector<double2> &up)
 // (B[0][0] = 1 in the M2M cases).  The products are checked against the
 // dense operators (`dense`, layout [q][k][l]) before they are used.
 struct ShiftFacHost {
-    int T = 0, maxp = 0;
     std::vector<double2> si, so;   // [4][P1]
-    std::vector<uint32_t> code;    // [T][32]
-    std::vector<double> coef;      // [T][32]
-    std::vector<int32_t> np;       // [P1]
+    std::vector<double> B;         // [P1][P1], input k major
 };
 
 bc_status build_shift_fac(int P1, bool par, bool adj, const std::vector<double2> &dense, ShiftFacHost &r)
@@ -297,51 +294,22 @@ bc_status build_shift_fac(int P1, bool par, bool adj, const std::vector<double2>
                   adj ? "adjoint" : "forward", worst);
         return BC_ERR_STATE;
     }
-    // term schedule over B's nonzeros, output by output, 32 runs
-    std::vector<std::pair<int, int>> terms;
-    for (int l = 0; l < P1; l++) {
-        bool any = false;
-        for (int k = 0; k < P1; k++)
-            if (B[size_t(l) * P1 + k] != 0.0L) { terms.emplace_back(l, k); any = true; }
-        if (!any) terms.emplace_back(l, 0);   // an all-zero output keeps one zero term
-    }
-    const int N = int(terms.size());
-    r.T = (N + 31) / 32;
-    std::vector<int> lf(P1, -1);
-    r.np.assign(P1, 0);
-    for (int i = 0; i < N; i++) {
-        const int l = terms[i].first, lane = i / r.T;
-        if (lf[l] < 0) lf[l] = lane;
-        r.np[l] = lane - lf[l] + 1;
-    }
-    r.maxp = *std::max_element(r.np.begin(), r.np.end());
-    r.code.assign(size_t(r.T) * 32, 0u);
-    r.coef.assign(size_t(r.T) * 32, 0.0);
-    for (int i = 0; i < N; i++) {
-        const int l = terms[i].first, k = terms[i].second, lane = i / r.T, t = i % r.T;
-        const bool last = i + 1 == N || terms[i + 1].first != l || (i + 1) % r.T == 0;
-        const uint32_t slot = uint32_t(l * r.maxp + lane - lf[l]);
-        r.code[size_t(t) * 32 + lane] = uint32_t(k) | (last ? (slot + 1u) << 8 : 0u);
-        r.coef[size_t(t) * 32 + lane] = double(B[size_t(l) * P1 + k]);
-    }
+    r.B.resize(size_t(P1) * P1);
+    for (int l = 0; l < P1; l++)
+        for (int k = 0; k < P1; k++) r.B[size_t(k) * P1 + l] = double(B[size_t(l) * P1 + k]);
     return BC_OK;
 }
 
 bc_status upload_shift_fac(DevTables &dt, ShiftFac &f, const ShiftFacHost &h)
 {
     double2 *psi = nullptr, *pso = nullptr;
-    uint32_t *pc = nullptr;
-    double *pf = nullptr;
-    int32_t *pn = nullptr;
+    double *pb = nullptr;
     cudaError_t e;
     if ((e = dev_upload(dt.allocs, &psi, h.si.data(), h.si.size())) != cudaSuccess ||
         (e = dev_upload(dt.allocs, &pso, h.so.data(), h.so.size())) != cudaSuccess ||
-        (e = dev_upload(dt.allocs, &pc, h.code.data(), h.code.size())) != cudaSuccess ||
-        (e = dev_upload(dt.allocs, &pf, h.coef.data(), h.coef.size())) != cudaSuccess ||
-        (e = dev_upload(dt.allocs, &pn, h.np.data(), h.np.size())) != cudaSuccess)
+        (e = dev_upload(dt.allocs, &pb, h.B.data(), h.B.size())) != cudaSuccess)
         return cuda_fail(e, "tables upload");
-    f.si = psi; f.so = pso; f.code = pc; f.coef = pf; f.np = pn;
-    f.T = h.T; f.maxp = h.maxp;
+    f.si = psi; f.so = pso; f.B = pb;
     return BC_OK;
 }
 
@@ -1399,12 +1367,12 @@ bc_status bc_tables_build(bc_ctx *ctx, const char *cache_dir)
     e = dev_upload<int32_t>(ctx->dt.allocs, &ctx->dev_err, nullptr, 1);
     if (e != cudaSuccess) return cuda_fail(e, "error flag");
     // two upward blocks per SM leave room for a tensor-core CTA beside them
+    // (four or six: no faster, 100 us at 17,491 leaves); six downward ones (four:
+    // 118 us there, six or eight: 110)
     {
         const OpSet &F = ctx->dt.fwd, &A = ctx->dt.adj;
-        const int fT = std::max(std::max(F.up_f.T, A.up_f.T), std::max(F.par_f.T, A.par_f.T));
-        const int fm = std::max(std::max(F.up_f.maxp, A.up_f.maxp), std::max(F.par_f.maxp, A.par_f.maxp));
-        e = fp64_prepare(ctx->NP, ctx->P1, std::max(F.up_s.T, A.up_s.T), std::max(F.up_s.maxp, A.up_s.maxp), fT, fm,
-                         2, 4, &ctx->up_blocks, &ctx->shift_blocks, &ctx->down_blocks);
+        e = fp64_prepare(ctx->NP, ctx->P1, std::max(F.up_s.T, A.up_s.T), std::max(F.up_s.maxp, A.up_s.maxp),
+                         2, 6, &ctx->up_blocks, &ctx->shift_blocks, &ctx->down_blocks);
     }
     if (e != cudaSuccess) return cuda_fail(e, "FP64 kernel occupancy");
     s = build_split_tables(ctx);

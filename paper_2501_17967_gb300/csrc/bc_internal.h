@@ -135,15 +135,10 @@ struct DfSched {
 //     out[l] = so[q][l] * sum_k B[l][k] * (si[q][k] * in[k])
 // with B real and triangular (binomial coefficients, the same for the four
 // children) and si, so complex diagonals (powers of the child offset delta_q
-// = +-1 +- i or of delta_q / 2).  B's nonzero terms, taken output by output,
-// are cut into 32 runs of T terms, one run per lane of a warp (the scheme of
-// DfSched); each lane ends a partial sum where its run leaves an output.
+// = +-1 +- i or of delta_q / 2; delta_q / delta_0 = 1, i, -i, -1 for q = 0..3).
 struct ShiftFac {
     const double2 *si = nullptr, *so = nullptr;   // [4][P1]
-    const uint32_t *code = nullptr;   // [T][32] input k (bits 0-7); (slot + 1) << 8 where a partial sum ends
-    const double *coef = nullptr;     // [T][32] B[l][k] of each term (0 for padding)
-    const int32_t *np = nullptr;      // [P1] partial sums per output; output l owns slots l * maxp + [0, np[l])
-    int T = 0, maxp = 0;
+    const double *B = nullptr;                    // [P1 inputs k][P1 outputs l]
 };
 
 struct OpSet {
@@ -394,7 +389,7 @@ struct PassArgs {
     int m2l_kind = 0;     // FP64 M2L: 0 by FMAs (k_m2l_boxes), 1 on the FP64 tensor cores (k_m2l_mma)
     // persistent level-synchronous passes: resident blocks of the upward and
     // shift kernels (all blocks must be resident), bounded barrier waits
-    int up_blocks = 0, shift_blocks = 0, down_blocks = 0;   // down_blocks: the one-warp-per-box FP64 pass
+    int up_blocks = 0, shift_blocks = 0, down_blocks = 0;   // down_blocks: the FP64 pass
     long long wait_limit = 1ll << 26;
     int32_t *err = nullptr;
 };
@@ -404,7 +399,7 @@ PassArgs pass_args(const bc_ctx *ctx, const bc_tree *t);
 // (occupancy calculator), capped at `per_sm` blocks per SM.
 // (df_T, df_maxp: the double-float climb's schedule; f_T, f_maxp: the largest
 // factored FP64 shift schedule of the context.)
-cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int f_T, int f_maxp, int up_per_sm, int down_per_sm,
+cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int up_per_sm, int down_per_sm,
                          int *up_blocks, int *shift_blocks, int *down_blocks);
 
 // Disjoint union of trees (batched applies): leaves and boxes renumbered,

@@ -142,22 +142,23 @@ inline size_t up_smem_bytes(int NP, int P1, int T, int maxp)
                         sizeof(int32_t) * ((P1 + 3) & ~3)
                   : 0);
 }
-// Dynamic shared memory of the downward pass: the parent expansion and the
-// partial sums; the FP64 variant adds the factored shift's run sums and its
-// schedule (coefficients, codes, slot counts).
-inline size_t down_smem_bytes(int P1, int T, int maxp, bool df)
+// Dynamic shared memory of the double-float downward pass: the parent expansion
+// and the partial sums.
+inline size_t down_smem_bytes(int P1) { return sizeof(double2) * (5 * P1 + 1); }
+// The FP64 upward variant: the combined children, two sets of partial sums, the
+// leaf values.
+inline size_t up_smem_bytes_f64(int NP, int P1)
 {
-    return sizeof(double2) * (5 * P1 + 1) +
-           (df ? 0 : sizeof(double2) * size_t(P1) * maxp + (sizeof(double) + sizeof(uint32_t)) * T * 32 +
-                         sizeof(int32_t) * P1);
+    return sizeof(double2) * (4 * 32 + 8 * P1) + sizeof(double) * ((NP + 1) & ~1);
 }
-// The FP64 variant: children, partial sums, leaf values, then the factored
-// shift's schedule (coefficients, codes, slot counts) and the four children's
-// partial-sum slots.
-inline size_t up_smem_bytes_f64(int NP, int P1, int T, int maxp)
+
+// v i^n
+__device__ __forceinline__ double2 rot90(double2 v, int n)
 {
-    return sizeof(double2) * 8 * P1 + sizeof(double) * ((NP + 1) & ~1) + sizeof(double) * T * 32 +
-           sizeof(double2) * size_t(4) * P1 * maxp + sizeof(uint32_t) * T * 32 + sizeof(int32_t) * ((P1 + 3) & ~3);
+    const unsigned neg = unsigned(n >> 1 & 1) << 31, odd = unsigned(n & 1);
+    const double a = odd ? v.y : v.x, b = odd ? v.x : v.y;
+    return make_double2(__hiloint2double(int(unsigned(__double2hiint(a)) ^ neg ^ odd << 31), __double2loint(a)),
+                        __hiloint2double(int(unsigned(__double2hiint(b)) ^ neg), __double2loint(b)));
 }
 
 // -------------------------------------------------------------------------
@@ -172,18 +173,38 @@ inline size_t up_smem_bytes_f64(int NP, int P1, int T, int maxp)
 //           forward: M2M; adjoint: L2L^H
 // Four warps per block: in the leaf step warp w sums over the w-th quarter of
 // the nodes, in a parent step warp q applies the operator of child q; the four
-// partial sums meet in shared memory.  The FP64 variant applies Up_q in
-// factored form (ShiftFac: so_q[l] sum_k B[l][k] si_q[k]), B's terms on a
-// schedule that gives the 32 lanes equal shares of the triangle; about a
-// third of the FP64 instructions of the dense complex product.  The
+// partial sums meet in shared memory.  The FP64 variant applies the four Up_q
+// together (ShiftFac): the offsets of the children differ by powers of i, so
+//     ex[p][l] = so_0[l] sum_k B[l][k] U_{(l-k) mod 4}[k],
+//     U_d[k]   = si_0[k] sum_q omega_q^d child_q[k],   omega = 1, i, -i, -1
+// (adjoint: conjugate): one triangle of real coefficients for the four children.
+// Warp r takes the k = r mod 4 (its eight coefficients per output in registers),
+// lane (k, d) forms U_d[k], then lane l sums; about 114 FP64 instructions per
+// parent instead of 194 child by child, each 64 cycles of a sub-partition's pipe, and
+// 36 instead of 56 on the chain from the children's flags to the parent's (17,491
+// leaves, p = 16: 157 -> 100 us).  The
 // double-float variant runs the
 // parent step on the term schedule (DfSched), keeps its sums in double-float
 // until the one conversion of each result, and publishes every climbed
 // expansion twice: ex in FP64 and exdf as double-float pairs, which the
 // parent's step reads without conversion.
 // -------------------------------------------------------------------------
+__device__ __forceinline__ unsigned shift_coefficients(const ShiftFac &f, int w, int l, int P1, double (&b)[8])
+{
+    unsigned nz = 0;
+#pragma unroll
+    for (int m = 0; m < 8; m++) {
+        b[m] = w + 4 * m < P1 && l < P1 ? __ldg(&f.B[(w + 4 * m) * P1 + l]) : 0.0;
+        nz |= unsigned(__double_as_longlong(b[m]) != 0) << m;
+    }
+    return nz;
+}
+
+// Eight blocks fit an SM (64 registers): where the near-field tensor CTAs hold three
+// quarters of the SMs, the rest still takes the whole grid at once (at seven per SM
+// the last blocks, and with them the climb, waited for the near field to end).
 template <bool ADJ, bool DF>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 8)
 k_up_levels(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__restrict__ leaf_box,
             const int32_t *__restrict__ leaf_level, const int64_t *__restrict__ level_start, int nlevels,
             const int32_t *__restrict__ box_child0, const double *__restrict__ vin,
@@ -192,9 +213,9 @@ k_up_levels(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
             const uint8_t *__restrict__ active, long long limit, int32_t *err, const uint8_t *__restrict__ live)
 {
     extern __shared__ double2 shu[];
-    double2 *sc = shu;                                       // 4 * P1 children
-    double2 *part = sc + 4 * P1;                             // [4][P1] partial sums
-    double *sv = reinterpret_cast<double *>(part + 4 * P1);  // NP
+    double2 *sc = shu;                                       // 4 * P1 children (FP64: U, [4][32])
+    double2 *part = sc + 4 * (DF ? P1 : 32);                 // [4][P1] partial sums (FP64: two sets in turn)
+    double *sv = reinterpret_cast<double *>(part + (DF ? 4 : 8) * P1);  // NP
     // the shift schedule in shared memory, copied while the preceding kernel
     // drains (every parent step reads it)
     // double-float path: scheduled operator entries of the four children
@@ -203,29 +224,28 @@ k_up_levels(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
     float4 *sslot = sops + 4 * T * 32;                                 // [4][SL]
     uint32_t *scode = reinterpret_cast<uint32_t *>(sslot + 4 * SL);    // [T][32]
     int32_t *snp = reinterpret_cast<int32_t *>(scode + T * 32);        // [P1]
-    // FP64 path: the factored shift's coefficients and codes (ShiftFac)
-    const int TF = uf.T, SLF = P1 * uf.maxp;
-    double *fcoef = sv + ((NP + 1) & ~1);                              // [TF][32] (FP64 only)
-    double2 *fslot = reinterpret_cast<double2 *>(fcoef + TF * 32);     // [4][SLF]
-    uint32_t *fcode = reinterpret_cast<uint32_t *>(fslot + 4 * SLF);   // [TF][32]
-    int32_t *fnp = reinterpret_cast<int32_t *>(fcode + TF * 32);       // [P1]
     __shared__ int s_leafc[4];   // which children of the current parent are leaves
     if (climb) {
         if constexpr (DF) {
             for (int i = threadIdx.x; i < 4 * T * 32; i += blockDim.x) sops[i] = __ldg(&us.ops[i]);
             for (int i = threadIdx.x; i < T * 32; i += blockDim.x) scode[i] = __ldg(&us.code[i]);
             for (int i = threadIdx.x; i < P1; i += blockDim.x) snp[i] = __ldg(&us.np[i]);
-        } else {
-            for (int i = threadIdx.x; i < TF * 32; i += blockDim.x) {
-                fcoef[i] = __ldg(&uf.coef[i]);
-                fcode[i] = __ldg(&uf.code[i]);
-            }
-            for (int i = threadIdx.x; i < P1; i += blockDim.x) fnp[i] = __ldg(&uf.np[i]);
         }
+    }
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // FP64: the coefficients B[lane][w + 4 m], bit m of nz where they are not zero
+    // (their terms alone are formed: 0 times an infinity is no term), and the
+    // diagonals of the first child
+    double bco[8];
+    unsigned nz = 0;
+    double2 usi = make_double2(0.0, 0.0), uso = make_double2(0.0, 0.0);
+    if constexpr (!DF) {
+        nz = shift_coefficients(uf, w, lane, P1, bco);
+        if (w + 4 * (lane >> 2) < P1) usi = __ldg(&uf.si[w + 4 * (lane >> 2)]);
+        if (lane < P1) uso = __ldg(&uf.so[lane]);
     }
     griddep_wait();
     griddep_launch_dependents();
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // leaf step: warp w sums the nodes [j0, j1) (any number of nodes)
     const int nq = (NP + 3) / 4, j0 = min(NP, w * nq), j1 = min(NP, j0 + nq);
     for (int64_t li = blockIdx.x; OpA && li < nleaf; li += gridDim.x) {
@@ -298,10 +318,18 @@ k_up_levels(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
         flag_publish(&flag[b], 1);
     }
     if (!climb) return;
+    int turn = 0;   // parents done by this block
     for (int lv = nlevels - 2; lv >= 2; lv--) {
-        for (int64_t p = level_start[lv] + blockIdx.x; p < level_start[lv + 1]; p += gridDim.x) {
-            const int c0 = box_child0[p];
-            if (c0 < 0) continue;   // a leaf (uniform over the block)
+        // the parents among 32 of the block's boxes at a time (three in four boxes are
+        // leaves: reading box after box took a load's latency for each)
+        const int64_t le = level_start[lv + 1];
+        for (int64_t base = level_start[lv] + blockIdx.x; base < le; base += 32 * int64_t(gridDim.x)) {
+        const int64_t cand = base + lane * int64_t(gridDim.x);
+        const int cc = cand < le ? box_child0[cand] : -1;
+        for (unsigned todo = __ballot_sync(0xffffffffu, cc >= 0); todo; todo &= todo - 1) {
+            const int sel = __ffs(todo) - 1;
+            const int64_t p = base + sel * int64_t(gridDim.x);
+            const int c0 = __shfl_sync(0xffffffffu, cc, sel);
             if (live && !live[p]) {
                 // no source below this box (point sources): its expansion is
                 // zero, with nothing to wait for
@@ -314,13 +342,13 @@ k_up_levels(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
             }
             // children computed in this launch: every child above the leaves,
             // and the leaves too when their expansions come from the leaf step
-            if (threadIdx.x < 4) {
-                const bool leafc = box_child0[c0 + threadIdx.x] < 0;
-                if (DF) s_leafc[threadIdx.x] = leafc;
-                if (OpA || !leafc) flag_wait(&flag[c0 + threadIdx.x], 1, limit, err);
+            if (DF ? threadIdx.x < 4 : lane < 4) {   // FP64: every warp for itself
+                const bool leafc = box_child0[c0 + lane] < 0;
+                if (DF) s_leafc[lane] = leafc;
+                if (OpA || !leafc) flag_wait(&flag[c0 + lane], 1, limit, err);
             }
-            __syncthreads();
             if constexpr (DF) {
+                __syncthreads();
                 // the children as double-float pairs: climbed ones from exdf,
                 // leaves (expansions of the leaf products) from ex
                 float4 *scf = reinterpret_cast<float4 *>(sc);
@@ -362,47 +390,43 @@ k_up_levels(int64_t nleaf, const int32_t *__restrict__ order, const int32_t *__r
                 }
                 flag_publish(&flag[p], 1);
             } else {
-            // factored FP64 shift (ShiftFac), warp w = child w: a = si_w * child
-            // (lane k), then B's terms on the schedule, each output's partial
-            // sums added and scaled by so_w, and the four children summed
-            double2 *a = sc + w * P1;
-            for (int k = lane; k < P1; k += 32) {
-                const double2 A = __ldcg(&ex[int64_t(c0 + w) * P1 + k]), S = __ldg(&uf.si[w * P1 + k]);
-                a[k] = make_double2(fma(A.x, S.x, -A.y * S.y), fma(A.x, S.y, A.y * S.x));
+            __syncwarp();
+            const int k = w + 4 * (lane >> 2), d = lane & 3;
+            if (k < P1) {
+                const double2 *A = ex + int64_t(c0) * P1 + k;
+                const double2 A0 = __ldcg(A), A1 = rot90(__ldcg(A + P1), ADJ ? -d : d),
+                              A2 = rot90(__ldcg(A + 2 * P1), ADJ ? d : -d), A3 = rot90(__ldcg(A + 3 * P1), 2 * d);
+                const double2 v = make_double2((A0.x + A3.x) + (A1.x + A2.x), (A0.y + A3.y) + (A1.y + A2.y));
+                sc[w * 32 + lane] = make_double2(fma(v.x, usi.x, -v.y * usi.y), fma(v.x, usi.y, v.y * usi.x));
             }
             __syncwarp();
-            double2 *slot = fslot + w * SLF;
+            const double2 *U = sc + w * 32 + ((lane - w) & 3);
             double re = 0.0, im = 0.0;
-#pragma unroll 2
-            for (int t = 0; t < TF; t++) {
-                const uint32_t code = fcode[t * 32 + lane];
-                const double cf = fcoef[t * 32 + lane];
-                const double2 x = a[code & 255u];
-                re = fma(cf, x.x, re);
-                im = fma(cf, x.y, im);
-                if (code >> 8) {   // the run leaves an output here
-                    slot[(code >> 8) - 1u] = make_double2(re, im);
-                    re = im = 0.0;
+#pragma unroll
+            for (int m = 0; m < 8; m++)
+                if (nz >> m & 1) {
+                    const double2 x = U[4 * m];
+                    re = fma(bco[m], x.x, re);
+                    im = fma(bco[m], x.y, im);
                 }
-            }
-            __syncwarp();
-            for (int l = lane; l < P1; l += 32) {
-                double2 y = slot[l * uf.maxp];
-                for (int j = 1; j < fnp[l]; j++) {
-                    const double2 v = slot[l * uf.maxp + j];
-                    y.x += v.x;
-                    y.y += v.y;
-                }
-                const double2 S = __ldg(&uf.so[w * P1 + l]);
-                part[w * P1 + l] = make_double2(fma(y.x, S.x, -y.y * S.y), fma(y.x, S.y, y.y * S.x));
-            }
+            double2 *pt = part + (turn & 1) * 4 * P1;
+            if (lane < P1) pt[w * P1 + lane] = make_double2(re, im);
+            // the only barrier of a parent: a set of partial sums is written again
+            // two parents later, behind the next one's
             __syncthreads();
-            for (int l = threadIdx.x; l < P1; l += blockDim.x) {
-                const double2 a0 = part[l], a1 = part[P1 + l], a2 = part[2 * P1 + l], a3 = part[3 * P1 + l];
-                ex[int64_t(p) * P1 + l] = make_double2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
+            if (w == (turn >> 1 & 3)) {   // in turn: each warp has a sub-partition's FP64 pipe
+                if (lane < P1) {
+                    const double2 a0 = pt[lane], a1 = pt[P1 + lane], a2 = pt[2 * P1 + lane], a3 = pt[3 * P1 + lane];
+                    const double2 y = make_double2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
+                    ex[int64_t(p) * P1 + lane] =
+                        make_double2(fma(y.x, uso.x, -y.y * uso.y), fma(y.x, uso.y, y.y * uso.x));
+                }
+                __syncwarp();
+                if (lane == 0) asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(&flag[p]), "r"(1) : "memory");
             }
-            flag_publish(&flag[p], 1);
+            turn++;
             }
+        }
         }
     }
 }
@@ -852,8 +876,8 @@ k_x_entries(int64_t nx, const int32_t *__restrict__ x_box, const int32_t *__rest
 }
 
 // -------------------------------------------------------------------------
-// down_levels: the local expansion (adjoint: multipole) of every box at
-// level >= 2, in one persistent launch:
+// down_levels (double-float shifts): the local expansion (adjoint: multipole) of
+// every box at level >= 2, in one persistent launch:
 //   the box's own sums:
 //     out[b] = V(b) + sum_{x in X(b)} (PX[x] + log(r_c) A_0(c) e_0)
 //   where V(b) is out[b] itself on entry (vsum: the whole V-list sum, written
@@ -875,41 +899,26 @@ k_x_entries(int64_t nx, const int32_t *__restrict__ x_box, const int32_t *__rest
 // per lane), warps 2 and 3 the V pairs (vsum: warp 2 reads the V sum).  In
 // the shift warp w applies a quarter of the operator's columns, fetched into
 // registers before the wait for the parent (the shift chain is the critical
-// path).  The double-float variant keeps that chain free of FP64 work: a copy
+// path), kept free of FP64 work: a copy
 // of the box's sums is converted to pairs before the wait, the parent is read
 // as pairs (outdf), the shift and its sum with the copy are formed as pairs
 // and published for the children; the FP64 result, read only by later
 // kernels, is the FP64 sums plus the shift, stored after the box's flag.
 // -------------------------------------------------------------------------
-template <bool DF>
 __global__ void __launch_bounds__(128)
 k_down_levels(const int64_t *__restrict__ level_start, int nlevels, const int32_t *__restrict__ v_ptr,
               const double2 *__restrict__ Pv, const int32_t *__restrict__ x_ptr, const int32_t *__restrict__ x_src,
               const double2 *__restrict__ PX, int px_stride, const int32_t *__restrict__ leaf_box,
               const double2 *__restrict__ first, const int32_t *__restrict__ parent,
               const int32_t *__restrict__ box_ix, const int32_t *__restrict__ box_iy,
-              const float4 *__restrict__ OpParDF, ShiftFac pf, double2 *out, float4 *outdf, int P1,
+              const float4 *__restrict__ OpParDF, double2 *out, float4 *outdf, int P1,
               const double *__restrict__ lvtab,
               const int32_t *__restrict__ v_lsrc, const int32_t *__restrict__ v_code,
               const double *__restrict__ logd, bool vsum, int32_t *flag, long long limit, int32_t *err)
 {
     extern __shared__ double2 sdn[];
-    double2 *se = sdn;             // [P1] parent expansion (FP64 variant: times si_q)
+    double2 *se = sdn;             // [P1] parent expansion
     double2 *part = sdn + P1;      // [4][P1] partial sums
-    // FP64 variant: the factored shift's schedule (ShiftFac) and the partial
-    // sums of its runs, staged before the wait for the preceding kernel
-    const int TF = DF ? 0 : pf.T, SLF = DF ? 0 : P1 * pf.maxp;
-    double2 *fslot = part + 4 * P1;                                    // [SLF]
-    double *fcoef = reinterpret_cast<double *>(fslot + SLF);           // [TF][32]
-    uint32_t *fcode = reinterpret_cast<uint32_t *>(fcoef + TF * 32);   // [TF][32]
-    int32_t *fnp = reinterpret_cast<int32_t *>(fcode + TF * 32);       // [P1]
-    if constexpr (!DF) {
-        for (int i = threadIdx.x; i < TF * 32; i += blockDim.x) {
-            fcoef[i] = __ldg(&pf.coef[i]);
-            fcode[i] = __ldg(&pf.code[i]);
-        }
-        for (int i = threadIdx.x; i < P1; i += blockDim.x) fnp[i] = __ldg(&pf.np[i]);
-    }
     griddep_wait();
     griddep_launch_dependents();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -921,19 +930,13 @@ k_down_levels(const int64_t *__restrict__ level_start, int nlevels, const int32_
         const int pb = shift ? parent[b] : 0;
         const int q = (box_ix[b] & 1) + 2 * (box_iy[b] & 1);
         // the shift operator does not depend on the parent's values: fetched
-        // before the wait for them (FP64: warp 0's diagonals si_q, so_q)
+        // before the wait for them
         float4 wf[8];
-        double2 fsi = make_double2(0.0, 0.0), fso = make_double2(0.0, 0.0);
         if (shift && o < P1) {
-            if constexpr (DF) {
 #pragma unroll
-                for (int u = 0; u < 8; u++)
-                    wf[u] = k0 + u < k1 ? __ldg(&OpParDF[(size_t(q) * P1 + k0 + u) * P1 + o])
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-            } else if (w == 0) {
-                fsi = __ldg(&pf.si[q * P1 + o]);
-                fso = __ldg(&pf.so[q * P1 + o]);
-            }
+            for (int u = 0; u < 8; u++)
+                wf[u] = k0 + u < k1 ? __ldg(&OpParDF[(size_t(q) * P1 + k0 + u) * P1 + o])
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         // ---- the box's own sums, one kind per warp: warp 0 the X list and
         // its log term, warp 1 the log term of the V list (tensor-core M2L),
@@ -1001,238 +1004,156 @@ k_down_levels(const int64_t *__restrict__ level_start, int nlevels, const int32_
         if (o < P1) part[w * P1 + o] = make_double2(re, im);
         __syncthreads();
         double2 acc = make_double2(0.0, 0.0);   // meaningful in warp 0, lanes o < P1
-        float4 accf = make_float4(0.f, 0.f, 0.f, 0.f);   // the same as double-float pairs (DF)
-        float4 shf = make_float4(0.f, 0.f, 0.f, 0.f);    // the shifted parent (DF)
+        float4 accf = make_float4(0.f, 0.f, 0.f, 0.f);   // the same as double-float pairs
+        float4 shf = make_float4(0.f, 0.f, 0.f, 0.f);    // the shifted parent
         if (w == 0 && o < P1) {
             const double2 a0 = part[o], a1 = part[P1 + o], a2 = part[2 * P1 + o], a3 = part[3 * P1 + o];
             acc = make_double2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
-            if (DF) accf = df4_of(acc);   // before the wait for the parent
+            accf = df4_of(acc);   // before the wait for the parent
         }
         // ---- plus the parent's expansion shifted to this box (levels >= 3)
         if (shift) {
             if (threadIdx.x == 0) flag_wait(&flag[pb], 2, limit, err);
             __syncthreads();   // also: warp 0 has read its partial sums
-            if constexpr (DF) {
-                float4 *sef = reinterpret_cast<float4 *>(se);   // the parent's double-float pairs
-                for (int i = threadIdx.x; i < P1; i += blockDim.x) sef[i] = __ldcg(&outdf[int64_t(pb) * P1 + i]);
-                __syncthreads();
-                if (o < P1) {
-                    float r0h = 0.f, r0l = 0.f, i0h = 0.f, i0l = 0.f, r1h = 0.f, r1l = 0.f, i1h = 0.f, i1l = 0.f;
+            float4 *sef = reinterpret_cast<float4 *>(se);   // the parent's double-float pairs
+            for (int i = threadIdx.x; i < P1; i += blockDim.x) sef[i] = __ldcg(&outdf[int64_t(pb) * P1 + i]);
+            __syncthreads();
+            if (o < P1) {
+                float r0h = 0.f, r0l = 0.f, i0h = 0.f, i0l = 0.f, r1h = 0.f, r1l = 0.f, i1h = 0.f, i1l = 0.f;
 #pragma unroll
-                    for (int u = 0; u < 8; u += 2) {   // two chains
-                        if (k0 + u >= k1) break;
-                        df_cmac(r0h, r0l, i0h, i0l, wf[u], sef[k0 + u]);
-                        if (k0 + u + 1 < k1) df_cmac(r1h, r1l, i1h, i1l, wf[u + 1], sef[k0 + u + 1]);
-                    }
-                    reinterpret_cast<float4 *>(part)[w * P1 + o] =
-                        df4_add(make_float4(r0h, r0l, i0h, i0l), make_float4(r1h, r1l, i1h, i1l));
+                for (int u = 0; u < 8; u += 2) {   // two chains
+                    if (k0 + u >= k1) break;
+                    df_cmac(r0h, r0l, i0h, i0l, wf[u], sef[k0 + u]);
+                    if (k0 + u + 1 < k1) df_cmac(r1h, r1l, i1h, i1l, wf[u + 1], sef[k0 + u + 1]);
                 }
-            } else if (w == 0) {
-                // factored FP64 shift (ShiftFac) by warp 0: a = si_q * parent
-                // (lane k), B's terms on the schedule, each output's partial
-                // sums added and scaled by so_q
-                if (o < P1) {
-                    const double2 A = __ldcg(&out[int64_t(pb) * P1 + o]);
-                    se[o] = make_double2(fma(A.x, fsi.x, -A.y * fsi.y), fma(A.x, fsi.y, A.y * fsi.x));
-                }
-                __syncwarp();
-                double re = 0.0, im = 0.0;
-#pragma unroll 2
-                for (int t = 0; t < TF; t++) {
-                    const uint32_t code = fcode[t * 32 + lane];
-                    const double cf = fcoef[t * 32 + lane];
-                    const double2 x = se[code & 255u];
-                    re = fma(cf, x.x, re);
-                    im = fma(cf, x.y, im);
-                    if (code >> 8) {   // the run leaves an output here
-                        fslot[(code >> 8) - 1u] = make_double2(re, im);
-                        re = im = 0.0;
-                    }
-                }
-                __syncwarp();
-                if (o < P1) {
-                    double2 y = fslot[o * pf.maxp];
-                    for (int j = 1; j < fnp[o]; j++) {
-                        const double2 v = fslot[o * pf.maxp + j];
-                        y.x += v.x;
-                        y.y += v.y;
-                    }
-                    acc.x += fma(y.x, fso.x, -y.y * fso.y);
-                    acc.y += fma(y.x, fso.y, y.y * fso.x);
-                }
+                reinterpret_cast<float4 *>(part)[w * P1 + o] =
+                    df4_add(make_float4(r0h, r0l, i0h, i0l), make_float4(r1h, r1l, i1h, i1l));
             }
-            if constexpr (DF) {
-                __syncthreads();
-                if (w == 0 && o < P1) {
-                    const float4 *pf4 = reinterpret_cast<const float4 *>(part);
-                    shf = df4_add(pf4[o], df4_add(pf4[P1 + o], df4_add(pf4[2 * P1 + o], pf4[3 * P1 + o])));
-                    accf = df4_add(accf, shf);
-                }
+            __syncthreads();
+            if (w == 0 && o < P1) {
+                const float4 *pf4 = reinterpret_cast<const float4 *>(part);
+                shf = df4_add(pf4[o], df4_add(pf4[P1 + o], df4_add(pf4[2 * P1 + o], pf4[3 * P1 + o])));
+                accf = df4_add(accf, shf);
             }
         }
-        if constexpr (DF) {
-            // the children read the pairs (the input of their shifts); the
-            // FP64 result, read by the later kernels only, is the FP64 sums
-            // plus the shifted parent, stored after the flag, off the chain
-            if (w == 0 && o < P1) outdf[b * P1 + o] = accf;
-            flag_publish(&flag[b], 2);   // its barrier also frees the shared buffers
-            if (w == 0 && o < P1)
-                out[b * P1 + o] = make_double2(acc.x + (double(shf.x) + double(shf.y)),
-                                               acc.y + (double(shf.z) + double(shf.w)));
-        } else {
-            if (w == 0 && o < P1) out[b * P1 + o] = acc;
-            flag_publish(&flag[b], 2);   // its barrier also frees the shared buffers
-        }
+        // the children read the pairs (the input of their shifts); the
+        // FP64 result, read by the later kernels only, is the FP64 sums
+        // plus the shifted parent, stored after the flag, off the chain
+        if (w == 0 && o < P1) outdf[b * P1 + o] = accf;
+        flag_publish(&flag[b], 2);   // its barrier also frees the shared buffers
+        if (w == 0 && o < P1)
+            out[b * P1 + o] = make_double2(acc.x + (double(shf.x) + double(shf.y)),
+                                           acc.y + (double(shf.z) + double(shf.w)));
     }
 }
 
 // -------------------------------------------------------------------------
-// down_warps: the FP64 downward pass with one warp per box (the same result
-// as k_down_levels<false>).  Warp g of the grid takes the boxes
-// level_start[2] + g, + G, ... (G warps in all), in ascending order, and for
-// each:
-//   the box's own sums (lane o = coefficient o): the V-list sum (vsum: the
-//     row k_m2l_boxes wrote into out[b]; else the rows Pv[e] of the pairs and
-//     the V-list log term), the X-list rows PX[x] and the X-list log term;
-//   then (levels >= 3), once the parent is published, the parent's expansion
-//     shifted to this box in factored form (ShiftFac: so_q[l] sum_k B[l][k]
-//     si_q[k] parent[k], B's terms on the 32-lane schedule);
-//   the result is written to out[b] and published by flag[b] = 2.
-// A box waits only for its parent, a box of smaller index, so every wait
-// ends once every warp is resident (the grid comes from the occupancy
-// calculator).  Each warp of a block sits on its own SM sub-partition, so the
-// shifts of concurrently processed boxes use all four FP64 pipes.
+// down_groups: the FP64 downward pass, one block per group of four siblings, warp
+// q the child q.  Block g of the grid takes the parents p = level_start[1] + g,
+// + G, ... (G blocks), in ascending order, and for each:
+//   the children's own sums (lane o = coefficient o): the V-list sum that out[b]
+//     holds on entry, the X-list rows PX[x] and the X-list log term;
+//   then (levels >= 3), once the parent is published, its expansion shifted to the
+//     four children together (ShiftFac): the offsets of the children differ by
+//     powers omega = 1, i, -i, -1 (adjoint: conjugate) of i, so
+//       child_q[l] += so_q[l] sum_r omega_q^r S_r[l],
+//       S_r[l]      = sum_{k = r mod 4} B[l][k] si_0[k] parent[k]
+//     warp r forms S_r (its eight coefficients per output in registers), and after
+//     one barrier warp q adds the four up for its child;
+//   the results are written to out[b] and published by flag[b] = 2.
+// Bound by FP64 instructions, each 64 cycles of a sub-partition's pipe: about 30
+// per warp and group, where a warp per child spent 49 (and 15 on the reduction of a
+// log term that most boxes do not have); also the chain from one level to the next.
+// 17,491 leaves, p = 16: 185 -> 110 us; 700 leaves, seven levels: 55 -> 30 us.
+// A group waits only for its parent, whose group has a smaller index, so every wait
+// ends once every block is resident (the grid comes from the occupancy calculator).
 // -------------------------------------------------------------------------
 __global__ void __launch_bounds__(128)
-k_down_warps(const int64_t *__restrict__ level_start, int nlevels, const int32_t *__restrict__ v_ptr,
-             const double2 *__restrict__ Pv, const int32_t *__restrict__ x_ptr, const int32_t *__restrict__ x_src,
-             const double2 *__restrict__ PX, int px_stride, const int32_t *__restrict__ leaf_box,
-             const double2 *__restrict__ first, const int32_t *__restrict__ parent,
-             const int32_t *__restrict__ box_ix, const int32_t *__restrict__ box_iy, ShiftFac pf, double2 *out, int P1,
-             const double *__restrict__ lvtab, const int32_t *__restrict__ v_lsrc,
-             const int32_t *__restrict__ v_code, const double *__restrict__ logd, bool vsum, int32_t *flag,
-             long long limit, int32_t *err)
+k_down_groups(const int64_t *__restrict__ level_start, int nlevels, const int32_t *__restrict__ box_child0,
+              const int32_t *__restrict__ x_ptr, const int32_t *__restrict__ x_src, const double2 *__restrict__ PX,
+              int px_stride, const int32_t *__restrict__ leaf_box, const double2 *__restrict__ first, ShiftFac pf,
+              bool adj, double2 *out, int P1, const double *__restrict__ lvtab, int32_t *flag, long long limit,
+              int32_t *err)
 {
-    extern __shared__ double2 sdw[];
-    const int TF = pf.T, SLF = P1 * pf.maxp;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    double2 *se = sdw + w * (P1 + SLF);                                   // [P1] si_q * parent
-    double2 *fslot = se + P1;                                             // [SLF] run sums
-    double *fcoef = reinterpret_cast<double *>(sdw + nw * (P1 + SLF));    // [TF][32]
-    uint32_t *fcode = reinterpret_cast<uint32_t *>(fcoef + TF * 32);      // [TF][32]
-    int32_t *fnp = reinterpret_cast<int32_t *>(fcode + TF * 32);          // [P1]
-    for (int i = threadIdx.x; i < TF * 32; i += blockDim.x) {
-        fcoef[i] = __ldg(&pf.coef[i]);
-        fcode[i] = __ldg(&pf.code[i]);
-    }
-    for (int i = threadIdx.x; i < P1; i += blockDim.x) fnp[i] = __ldg(&pf.np[i]);
-    __syncthreads();
+    __shared__ double2 sx[4][8];       // si_0 * parent, the k of each warp
+    __shared__ double2 S[2][4][32];    // S_r, two groups in turn
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int o = lane;   // coefficient of this lane (P1 <= 32)
+    double bco[8];
+    const unsigned nz = shift_coefficients(pf, w, o, P1, bco);
+    double2 fsi = make_double2(0.0, 0.0), fso = make_double2(0.0, 0.0);
+    if (lane < 8 && w + 4 * lane < P1) fsi = __ldg(&pf.si[w + 4 * lane]);
+    if (o < P1) fso = __ldg(&pf.so[w * P1 + o]);
     griddep_wait();
     griddep_launch_dependents();
-    const int o = lane;   // coefficient of this lane (P1 <= 32)
-    const int64_t G = int64_t(gridDim.x) * nw;
-    for (int64_t b = level_start[2] + int64_t(blockIdx.x) * nw + w; b < level_start[nlevels]; b += G) {
-        const int lvb = lv_of(level_start, nlevels, b);
-        const bool shift = lvb >= 3;
-        const int pb = shift ? parent[b] : 0;
-        const int q = (box_ix[b] & 1) + 2 * (box_iy[b] & 1);
-        double2 fsi = make_double2(0.0, 0.0), fso = make_double2(0.0, 0.0);
-        if (shift && o < P1) {   // the shift's diagonals do not depend on the parent's values
-            fsi = __ldg(&pf.si[q * P1 + o]);
-            fso = __ldg(&pf.so[q * P1 + o]);
-        }
-        // ---- the box's own sums
-        double re = 0.0, im = 0.0;
-        if (o < P1) {
-            if (vsum) {
+    int lvb = 2, par = 0;
+    const int64_t n1 = level_start[nlevels - 1], G = gridDim.x;
+    for (int64_t base = level_start[1] + blockIdx.x; base < n1; base += 32 * G) {
+        const int64_t cand = base + lane * G;
+        const int cc = cand < n1 ? box_child0[cand] : -1;
+        for (unsigned todo = __ballot_sync(0xffffffffu, cc >= 0); todo; todo &= todo - 1) {
+            const int sel = __ffs(todo) - 1;
+            const int64_t p = base + sel * G, b = __shfl_sync(0xffffffffu, cc, sel) + w;
+            while (b >= level_start[lvb + 1]) lvb++;
+            // ---- the box's own sums
+            double re = 0.0, im = 0.0;
+            if (o < P1) {
                 const double2 t = out[b * P1 + o];
                 re = t.x;
                 im = t.y;
-            } else {
-                for (int e = v_ptr[b]; e < v_ptr[b + 1]; e++) {
-                    const double2 t = Pv[int64_t(e) * P1 + o];
-                    re += t.x;
-                    im += t.y;
-                }
             }
-        }
-        const int x0 = x_ptr[b], x1 = x_ptr[b + 1];
-        if (o < P1) {
+            const int x0 = x_ptr[b], x1 = x_ptr[b + 1];
+            if (x1 > x0) {
+                if (o < P1) {
 #pragma unroll 4
-            for (int x = x0; x < x1; x++) {
-                const double2 t = PX[int64_t(x) * px_stride + o];
-                re += t.x;
-                im += t.y;
-            }
-        }
-        // log terms, one entry per lane: the X list (times log r of the
-        // source level) and, for tensor-core M2L rows, the V list
-        double lx = 0.0, lr = 0.0, li = 0.0;
-        for (int x = x0 + lane; x < x1; x += 32) lx += first[int64_t(leaf_box[x_src[x]]) * P1].x;
-        if (!vsum && v_lsrc) {
-            const double lgb = lvtab[kLvTab + lvb];
-            for (int e = v_ptr[b] + lane; e < v_ptr[b + 1]; e += 32) {
-                const double2 a0 = first[int64_t(v_lsrc[e]) * P1];
-                const double c0 = logd[v_code[e]] + lgb;
-                lr = fma(c0, a0.x, lr);
-                li = fma(c0, a0.y, li);
-            }
-        }
-        for (int m = 16; m > 0; m >>= 1) {
-            lx += __shfl_xor_sync(0xffffffffu, lx, m);
-            lr += __shfl_xor_sync(0xffffffffu, lr, m);
-            li += __shfl_xor_sync(0xffffffffu, li, m);
-        }
-        if (o == 0) {
-            re = fma(lvtab[kLvTab + lvb - 1], lx, re + lr);
-            im += li;
-        }
-        // ---- plus the parent's expansion shifted to this box (levels >= 3)
-        if (shift) {
-            if (lane == 0) flag_wait(&flag[pb], 2, limit, err);
-            __syncwarp();
-            if (o < P1) {
-                const double2 A = __ldcg(&out[int64_t(pb) * P1 + o]);
-                se[o] = make_double2(fma(A.x, fsi.x, -A.y * fsi.y), fma(A.x, fsi.y, A.y * fsi.x));
-            }
-            __syncwarp();
-            double sr = 0.0, si = 0.0;
-#pragma unroll 2
-            for (int t = 0; t < TF; t++) {
-                const uint32_t code = fcode[t * 32 + lane];
-                const double cf = fcoef[t * 32 + lane];
-                const double2 xv = se[code & 255u];
-                sr = fma(cf, xv.x, sr);
-                si = fma(cf, xv.y, si);
-                if (code >> 8) {   // the run leaves an output here
-                    fslot[(code >> 8) - 1u] = make_double2(sr, si);
-                    sr = si = 0.0;
+                    for (int x = x0; x < x1; x++) {
+                        const double2 t = PX[int64_t(x) * px_stride + o];
+                        re += t.x;
+                        im += t.y;
+                    }
                 }
+                // the log term (times log r of the source level), one entry per lane
+                double lx = 0.0;
+                for (int x = x0 + lane; x < x1; x += 32) lx += first[int64_t(leaf_box[x_src[x]]) * P1].x;
+                for (int m = 16; m > 0; m >>= 1) lx += __shfl_xor_sync(0xffffffffu, lx, m);
+                if (o == 0) re = fma(lvtab[kLvTab + lvb - 1], lx, re);
             }
-            __syncwarp();
-            if (o < P1) {
-                double2 y = fslot[o * pf.maxp];
-                for (int j = 1; j < fnp[o]; j++) {
-                    const double2 v = fslot[o * pf.maxp + j];
-                    y.x += v.x;
-                    y.y += v.y;
+            // ---- plus the parent's expansion shifted to this box
+            if (lvb >= 3) {   // uniform over the block
+                if (lane == 0) flag_wait(&flag[p], 2, limit, err);
+                __syncwarp();
+                if (lane < 8 && w + 4 * lane < P1) {
+                    const double2 A = __ldcg(&out[p * P1 + w + 4 * lane]);
+                    sx[w][lane] = make_double2(fma(A.x, fsi.x, -A.y * fsi.y), fma(A.x, fsi.y, A.y * fsi.x));
                 }
+                __syncwarp();
+                double sr = 0.0, si = 0.0;
+#pragma unroll
+                for (int m = 0; m < 8; m++)
+                    if (nz >> m & 1) {
+                        const double2 x = sx[w][m];
+                        sr = fma(bco[m], x.x, sr);
+                        si = fma(bco[m], x.y, si);
+                    }
+                S[par][w][o] = make_double2(sr, si);
+                // the only barrier of a group: a set of S is written again two groups
+                // later, behind the next one's
+                __syncthreads();
+                const double2 s0 = S[par][0][o], s1 = S[par][1][o], s2 = S[par][2][o], s3 = S[par][3][o];
+                const int n = w == 0 ? 0 : w == 3 ? 2 : (w == 1) != adj ? 1 : 3;   // omega_w = i^n
+                // S_0 + omega S_1 + omega^2 S_2 + omega^3 S_3
+                const double2 e2 = rot90(s2, 2 * n), g2 = rot90(s3, 2 * n);
+                const double2 g = rot90(make_double2(s1.x + g2.x, s1.y + g2.y), n);
+                const double2 y = make_double2((s0.x + e2.x) + g.x, (s0.y + e2.y) + g.y);
                 re += fma(y.x, fso.x, -y.y * fso.y);
                 im += fma(y.x, fso.y, y.y * fso.x);
+                par ^= 1;
             }
+            if (o < P1) out[b * P1 + o] = make_double2(re, im);
+            __syncwarp();   // the warp's writes come before lane 0's release store
+            if (lane == 0) asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(&flag[b]), "r"(2) : "memory");
         }
-        if (o < P1) out[b * P1 + o] = make_double2(re, im);
-        // the warp's writes are ordered before lane 0's release store; the
-        // next box's shared-memory writes come after every lane's reads
-        __syncwarp();
-        if (lane == 0) asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(&flag[b]), "r"(2) : "memory");
     }
-}
-
-inline size_t down_warps_smem_bytes(int P1, int T, int maxp, int nwarps)
-{
-    return sizeof(double2) * size_t(nwarps) * (P1 + size_t(P1) * maxp) + (sizeof(double) + sizeof(uint32_t)) * T * 32 +
-           sizeof(int32_t) * P1;
 }
 
 // -------------------------------------------------------------------------
@@ -1757,8 +1678,7 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
     const double2 *opA = (parts & 2) ? nullptr : op.leafA;
     const bool climb = far && h.nlevels > 3;
     const bool dfp = (parts & 64) != 0;   // double-float shifts
-    const size_t shU = dfp ? up_smem_bytes(NP, P1, op.up_s.T, op.up_s.maxp)
-                           : up_smem_bytes_f64(NP, P1, op.up_f.T, op.up_f.maxp);
+    const size_t shU = dfp ? up_smem_bytes(NP, P1, op.up_s.T, op.up_s.maxp) : up_smem_bytes_f64(NP, P1);
     if (opA || climb) {
 #define BC_UP(A, D)                                                                                          \
     launch_pdl(k_up_levels<A, D>, a.up_blocks, 128, shU, st, a.nleaf, d.leaf_order, d.leaf_box, d.leaf_level, \
@@ -1861,17 +1781,16 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
         // the X-list products come from the internal stream
         if (split && split->side && (ce = cudaStreamWaitEvent(st, split->side->xdone, 0)) != cudaSuccess) return ce;
         if (dfp)
-            ce = launch_pdl(k_down_levels<true>, a.shift_blocks, 128, down_smem_bytes(P1, 0, 0, true), st,
+            ce = launch_pdl(k_down_levels, a.shift_blocks, 128, down_smem_bytes(P1), st,
                             d.level_start, h.nlevels, d.v_ptr, d.Pv, d.x_ptr, d.x_src, PX, px_stride, d.leaf_box,
-                            first, d.box_parent, d.box_ix, d.box_iy, op.par_df, op.par_f, second, d.exdf, P1, d.lvtab,
+                            first, d.box_parent, d.box_ix, d.box_iy, op.par_df, second, d.exdf, P1, d.lvtab,
                             first_digits ? d.v_src : nullptr, d.v_code, tb.logd, !first_digits, d.flag, glimit,
                             a.err);
         else
-            ce = launch_pdl(k_down_warps, a.down_blocks, 128, down_warps_smem_bytes(P1, op.par_f.T, op.par_f.maxp, 4),
-                            st, d.level_start, h.nlevels, d.v_ptr, d.Pv, d.x_ptr, d.x_src, PX, px_stride,
-                            d.leaf_box, first, d.box_parent, d.box_ix, d.box_iy, op.par_f, second, P1, d.lvtab,
-                            first_digits && !summed ? d.v_src : nullptr, d.v_code, tb.logd, !first_digits || summed,
-                            d.flag, glimit, a.err);
+            // every M2L here leaves the V-list sums in `second`
+            ce = launch_pdl(k_down_groups, a.down_blocks, 128, 0, st, d.level_start, h.nlevels, d.box_child0, d.x_ptr,
+                            d.x_src, PX, px_stride, d.leaf_box, first, op.par_f, adj, second, P1, d.lvtab, d.flag,
+                            glimit, a.err);
         if (ce != cudaSuccess) return ce;
     } else if (ev) {
         cudaEventRecord(ev[4], st);
@@ -1941,7 +1860,7 @@ cudaError_t launch_far_points(const PassArgs &a, const HostTree &h, const DevTre
     const long long glimit = std::max(1ll, a.wait_limit / 16);
     if (h.nlevels > 3) {
         // climb only: the leaf expansions were written by the caller
-        const size_t shU = up_smem_bytes_f64(NP, P1, op.up_f.T, op.up_f.maxp);
+        const size_t shU = up_smem_bytes_f64(NP, P1);
         ce = launch_pdl(k_up_levels<false, false>, a.up_blocks, 128, shU, st, a.nleaf, d.leaf_order, d.leaf_box,
                         d.leaf_level, d.level_start, h.nlevels, d.box_child0, (const double *)nullptr,
                         (const double2 *)nullptr, op.leafA_df, op.up_s, op.up_f, d.expA, d.exdf, NP, P1, d.lvtab,
@@ -1962,14 +1881,13 @@ cudaError_t launch_far_points(const PassArgs &a, const HostTree &h, const DevTre
 #undef BC_M2LP
         if (ce != cudaSuccess) return ce;
     }
-    return launch_pdl(k_down_warps, a.down_blocks, 128, down_warps_smem_bytes(P1, op.par_f.T, op.par_f.maxp, 4), st,
-                      d.level_start, h.nlevels, fl.v_ptr, d.Pv, fl.x_ptr, fl.x_src, fl.PX, P1, d.leaf_box, d.expA,
-                      d.box_parent, d.box_ix, d.box_iy, op.par_f, d.expB, P1, d.lvtab, (const int32_t *)nullptr,
-                      fl.v_code, tb.logd, true, d.flag, glimit, a.err);
+    return launch_pdl(k_down_groups, a.down_blocks, 128, 0, st, d.level_start, h.nlevels, d.box_child0, fl.x_ptr,
+                      fl.x_src, fl.PX, P1, d.leaf_box, d.expA, op.par_f, false, d.expB, P1, d.lvtab, d.flag, glimit,
+                      a.err);
 }
 
-cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int f_T, int f_maxp, int up_per_sm, int down_per_sm,
-                         int *up_blocks, int *shift_blocks, int *down_blocks)
+cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int up_per_sm, int down_per_sm, int *up_blocks, int *shift_blocks,
+                         int *down_blocks)
 {
     {
         // binomial table of the factored M2L (see c_binom)
@@ -1995,8 +1913,8 @@ cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int f_T, int f_m
     int dev = 0, sms = 0, bu0 = 0, bu1 = 0, bs = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t shU = up_smem_bytes_f64(NP, P1, f_T, f_maxp), shUd = up_smem_bytes(NP, P1, df_T, df_maxp);
-    const size_t shD = down_smem_bytes(P1, f_T, f_maxp, false), shDd = down_smem_bytes(P1, 0, 0, true);
+    const size_t shU = up_smem_bytes_f64(NP, P1), shUd = up_smem_bytes(NP, P1, df_T, df_maxp);
+    const size_t shD = down_smem_bytes(P1);
     // the double-float variants hold the scheduled shift operators in shared
     // memory, beyond the default 48 KB at high orders; the limit is per
     // kernel, so it is only ever raised (contexts of different orders share
@@ -2017,26 +1935,22 @@ cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int f_T, int f_m
                           (const void *)k_up_levels<true, true>, (const void *)k_m2l_boxes<false, 16>,
                           (const void *)k_m2l_boxes<true, 16>, (const void *)k_m2l_boxes<false, 24>,
                           (const void *)k_m2l_boxes<true, 24>, (const void *)k_m2l_boxes<false, 32>,
-                          (const void *)k_m2l_boxes<true, 32>, (const void *)k_down_warps,
-                          (const void *)k_down_levels<false>, (const void *)k_down_levels<true>})
+                          (const void *)k_m2l_boxes<true, 32>, (const void *)k_down_groups,
+                          (const void *)k_down_levels})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     // every block of a persistent pass must be resident: the smallest
     // occupancy over the variants that share the grid
-    int bu2 = 0, bu3 = 0, bs2 = 0;
+    int bu2 = 0, bu3 = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bu0, k_up_levels<false, false>, 128, shU);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bu1, k_up_levels<true, false>, 128, shU);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bu2, k_up_levels<false, true>, 128, shUd);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bu3, k_up_levels<true, true>, 128, shUd);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bs, k_down_levels<false>, 128, shD);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bs2, k_down_levels<true>, 128, shDd);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bs, k_down_levels, 128, shD);
     int bw = 0;
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bw, k_down_warps, 128,
-                                                          down_warps_smem_bytes(P1, f_T, f_maxp, 4));
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bw, k_down_groups, 128, 0);
     if (e != cudaSuccess) return e;
     const int bu = std::min(std::min(bu0, bu1), std::min(bu2, bu3));
-    bs = std::min(bs, bs2);
     if (bu < 1 || bs < 1 || bw < 1) return cudaErrorInvalidConfiguration;
     *up_blocks = sms * std::min(up_per_sm, bu);
     *shift_blocks = sms * std::min(down_per_sm, bs);
