@@ -21,9 +21,10 @@
 //        L_l = sum (-1)^l (2w)^-l [ -c_q / l + (c_m / r_c) / w ]
 //   M2P  (W list) and L2P as for the volume potential, near field direct;
 // with c_q = -q / (2 pi), c_m = -m / (2 pi).  A source that coincides with a
-// target node contributes nothing.  FP64 throughout, except the L2P (the volume
+// target node contributes nothing.  FP64 and (logarithms) fixed point, except the L2P (the volume
 // apply's group-E tensor tiles over the same locals: 7 digits in the FP64 mode, 5
-// in the split one; 1.86 -> NN ms at 17,584 leaves, 4,096 nodes, FP64).
+// in the split one; 1.86 -> 1.63 ms at 17,584 leaves, 4,096 nodes, FP64).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -138,76 +139,151 @@ __global__ void k_layer_gather(int64_t n, const int32_t *__restrict__ perm, cons
     }
 }
 
-// Sum over the warp of each coefficient k < P1 (butterfly, the same order on
-// every lane); lane k writes coefficient k to out[k].
-template <int PMAX>
-__device__ __forceinline__ void warp_sum_store(double2 (&acc)[PMAX], int P1, int lane, double2 *__restrict__ out)
+// Sum over the warp of each of 32 coefficients, lane k ends with coefficient k: the
+// lanes of each half hand the other half its coefficients, 62 additions in all (a
+// butterfly of each coefficient takes 310).
+__device__ __forceinline__ double2 warp_sums(double2 (&acc)[32], int lane)
 {
 #pragma unroll
-    for (int k = 0; k < PMAX; k++) {
-        if (k < P1) {   // uniform over the warp
-            double re = acc[k].x, im = acc[k].y;
+    for (int h = 16; h > 0; h >>= 1) {
+        const bool up = lane & h;   // keeps the upper half
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                re += __shfl_xor_sync(0xffffffffu, re, o);
-                im += __shfl_xor_sync(0xffffffffu, im, o);
-            }
-            if (lane == k) out[k] = make_double2(re, im);
+        for (int i = 0; i < h; i++) {
+            const double2 keep = up ? acc[i + h] : acc[i], give = up ? acc[i] : acc[i + h];
+            acc[i].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, h);
+            acc[i].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, h);
         }
+    }
+    return acc[0];
+}
+
+// e^n, 0 <= n < 32, n per lane (repeated squaring).
+__device__ __forceinline__ double2 cpow(double2 e, int n)
+{
+    double2 r = n & 1 ? e : make_double2(1.0, 0.0);
+#pragma unroll
+    for (int b = 1; b < 5; b++) {
+        e = make_double2(fma(e.x, e.x, -e.y * e.y), (e.x + e.x) * e.y);
+        if (n >> b & 1) r = cmul(r, e);
+    }
+    return r;
+}
+
+// P2M: a cluster of four blocks (16 warps on four SMs) per leaf with sources; the
+// warps' partial sums meet in distributed shared memory.  A curve's sources crowd in a
+// few leaves, whose chains of FP64 instructions, 64 cycles of a sub-partition's pipe
+// each, set the time.
+//   Up to kP2MFew sources: lane k is coefficient k, a warp takes every 16th source and
+//   its lanes form their powers of eta by repeated squaring, about 50 FP64 instructions
+//   per source (at most eight sources per warp).
+//   More: lane s takes sources s, s + 512, ..., carries the power up the coefficients,
+//   about 310 instructions per source of a lane, then 62 for the sums.
+// 4,096 sources in 17,584 leaves: one warp per leaf, the second form alone with 680
+// instructions, 62 us; kP2MFew = 16: 51, 128: 32 to 36.
+constexpr int kP2MFew = 128, kLayerCluster = 4;
+
+// The sums of the cluster's 16 warps (part: this block's four) to out[0..P1); sum
+// alternates between two buffers from call to call.
+__device__ __forceinline__ void cluster_sum_store(const double2 (&part)[4][32], double2 *sum, int P1,
+                                                  double2 *__restrict__ out)
+{
+    auto cluster = cooperative_groups::this_cluster();
+    __syncthreads();
+    const int k = threadIdx.x;
+    if (k < P1)
+        sum[k] = make_double2((part[0][k].x + part[1][k].x) + (part[2][k].x + part[3][k].x),
+                              (part[0][k].y + part[1][k].y) + (part[2][k].y + part[3][k].y));
+    cluster.sync();
+    if (cluster.block_rank() == 0 && k < P1) {
+        const double2 a = sum[k], b = cluster.map_shared_rank(sum, 1)[k], c = cluster.map_shared_rank(sum, 2)[k],
+                      d = cluster.map_shared_rank(sum, 3)[k];
+        out[k] = make_double2((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
     }
 }
 
-// P2M: one warp per leaf, lane s the sources s, s + 32, ... of the leaf; each
-// lane carries eta^k up the coefficients (one complex multiplication per
-// term), then the warp sums each coefficient.  Every leaf box is written
-// (zero without sources: the climb reads all children).  P1 <= PMAX.
-template <int PMAX>
-__global__ void __launch_bounds__(128)
+// P2M.  Every leaf box is written (zero without sources: the climb reads all
+// children).  P1 <= 32.
+__global__ void __cluster_dims__(kLayerCluster, 1, 1) __launch_bounds__(128)
 k_layer_p2m(int64_t nleaf, const int32_t *__restrict__ src_ptr, const double2 *__restrict__ sxy,
             const double *__restrict__ cq, const double2 *__restrict__ cm, const int32_t *__restrict__ leaf_box,
             const int32_t *__restrict__ box_level, const int32_t *__restrict__ box_ix,
             const int32_t *__restrict__ box_iy, double x0, double y0, double L, int P1, double2 *__restrict__ ex)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t leaf = blockIdx.x * int64_t(blockDim.x >> 5) + (threadIdx.x >> 5); leaf < nleaf; leaf += nw) {
-        const int b = leaf_box[leaf];
-        const int j0 = src_ptr[leaf], j1 = src_ptr[leaf + 1];
-        if (j0 == j1) {   // most leaves: no source, no sums to form (uniform over the warp)
-            for (int k = lane; k < P1; k += 32) ex[int64_t(b) * P1 + k] = make_double2(0.0, 0.0);
-            continue;
-        }
+    __shared__ double2 part[4][32], sum[2][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int rank = blockIdx.x % kLayerCluster, cid = blockIdx.x / kLayerCluster, ncl = gridDim.x / kLayerCluster;
+    int par = 0;
+    const double ik = lane ? -1.0 / double(lane) : 0.0;
+    for (int64_t base = cid; base < nleaf; base += 32 * int64_t(ncl)) {   // 32 leaves at a time
+        const int64_t cand = base + lane * int64_t(ncl);
+        const bool in = cand < nleaf;
+        const int cb = in ? leaf_box[cand] : 0, cj0 = in ? src_ptr[cand] : 0, cj1 = in ? src_ptr[cand + 1] : 0;
+        const unsigned some = __ballot_sync(0xffffffffu, cj1 > cj0), any = __ballot_sync(0xffffffffu, in);
+        // most leaves: no source, no sums to form
+        for (int q = rank * 4 + w; q < 32; q += 4 * kLayerCluster)
+            if ((any & ~some) >> q & 1) {
+                const int64_t b = __shfl_sync(0xffffffffu, cb, q);
+                if (lane < P1) ex[b * P1 + lane] = make_double2(0.0, 0.0);
+            }
+        for (unsigned todo = some; todo; todo &= todo - 1) {   // uniform over the cluster
+        const int q = __ffs(todo) - 1;
+        const int b = __shfl_sync(0xffffffffu, cb, q), j0 = __shfl_sync(0xffffffffu, cj0, q),
+                  j1 = __shfl_sync(0xffffffffu, cj1, q);
         const BoxGeom g = box_geom(b, box_level, box_ix, box_iy, x0, y0, L);
         const double ir = 1.0 / g.r;
-        double2 acc[PMAX];
-#pragma unroll
-        for (int k = 0; k < PMAX; k++) acc[k] = make_double2(0.0, 0.0);
-        for (int j = j0 + lane; j < j1; j += 32) {
-            const double2 y = sxy[j];
-            const double2 eta = make_double2((y.x - g.cx) * ir, (y.y - g.cy) * ir);
-            const double c = cq[j];
-            const double2 cmr = make_double2(cm[j].x * ir, cm[j].y * ir);   // c_m / r
-            acc[0].x += c;
-            double2 pw = make_double2(1.0, 0.0);   // eta^(k-1)
-#pragma unroll
-            for (int k = 1; k < PMAX; k++) {
-                if (k < P1) {
-                    const double2 d = cmul(cmr, pw);
-                    pw = cmul(pw, eta);
-                    const double ck = -c * (1.0 / double(k));
-                    acc[k].x += fma(ck, pw.x, d.x);
-                    acc[k].y += fma(ck, pw.y, d.y);
+        if (j1 - j0 <= kP2MFew) {
+            double2 acc = make_double2(0.0, 0.0);
+            for (int j = j0 + 4 * rank + w; j < j1; j += 4 * kLayerCluster) {
+                const double2 y = sxy[j];
+                const double2 eta = make_double2((y.x - g.cx) * ir, (y.y - g.cy) * ir);
+                const double c = cq[j], ck = c * ik;
+                // (c_m / r - (c_q / k) eta) eta^(k-1)
+                const double2 t = make_double2(fma(ck, eta.x, cm[j].x * ir), fma(ck, eta.y, cm[j].y * ir));
+                const double2 pw = cpow(eta, lane ? lane - 1 : 0);
+                if (lane == 0) {
+                    acc.x += c;
+                } else {
+                    acc.x = fma(pw.x, t.x, fma(-pw.y, t.y, acc.x));
+                    acc.y = fma(pw.x, t.y, fma(pw.y, t.x, acc.y));
                 }
             }
+            part[w][lane] = acc;
+        } else {
+            double2 acc[32];
+#pragma unroll
+            for (int k = 0; k < 32; k++) acc[k] = make_double2(0.0, 0.0);
+            for (int j = j0 + 128 * rank + int(threadIdx.x); j < j1; j += 128 * kLayerCluster) {
+                const double2 y = sxy[j];
+                const double2 eta = make_double2((y.x - g.cx) * ir, (y.y - g.cy) * ir);
+                const double c = cq[j];
+                const double2 cmr = make_double2(cm[j].x * ir, cm[j].y * ir);   // c_m / r
+                acc[0].x += c;
+                double2 pw = make_double2(1.0, 0.0);   // eta^(k-1)
+#pragma unroll
+                for (int k = 1; k < 32; k++) {
+                    if (k < P1) {
+                        const double ck = c * (-1.0 / double(k));
+                        const double2 t = make_double2(fma(ck, eta.x, cmr.x), fma(ck, eta.y, cmr.y));
+                        acc[k].x = fma(pw.x, t.x, fma(-pw.y, t.y, acc[k].x));
+                        acc[k].y = fma(pw.x, t.y, fma(pw.y, t.x, acc[k].y));
+                        pw = cmul(pw, eta);
+                    }
+                }
+            }
+            part[w][lane] = j0 + 128 * rank + 32 * w < j1 ? warp_sums(acc, lane) : acc[0];
         }
-        warp_sum_store(acc, P1, lane, ex + int64_t(b) * P1);
+        cluster_sum_store(part, sum[par], P1, ex + int64_t(b) * P1);
+        par ^= 1;
+        }
     }
+    cooperative_groups::this_cluster().sync();   // the last sums have been read
 }
 
 // P2L of the X list: one warp per entry, lane s the sources s, s + 32, ... of
 // the source leaf; each lane carries t^l = (-1/(2w))^l up the coefficients,
-// then the warp sums each coefficient.  P1 <= PMAX.
-template <int PMAX>
+// then the warp sums each coefficient.  P1 <= 32.  (Entries of 65 to 128 sources as
+// a rule: four blocks per entry, as for P2M, repeat the log and the division and took
+// 70 us instead of 43 for 288 entries; an FP64 butterfly of every coefficient made it 60.)
 __global__ void __launch_bounds__(128)
 k_layer_p2l(int64_t nx, const int32_t *__restrict__ x_box, const int32_t *__restrict__ x_src,
             const int32_t *__restrict__ src_ptr, const double2 *__restrict__ sxy, const double *__restrict__ cq,
@@ -223,9 +299,9 @@ k_layer_p2l(int64_t nx, const int32_t *__restrict__ x_box, const int32_t *__rest
         const BoxGeom gb = box_geom(x_box[x], box_level, box_ix, box_iy, x0, y0, L);
         const double ir = 1.0 / gc.r;
         const double2 e = make_double2((gb.cx - gc.cx) * ir, (gb.cy - gc.cy) * ir);
-        double2 acc[PMAX];
+        double2 acc[32];
 #pragma unroll
-        for (int l = 0; l < PMAX; l++) acc[l] = make_double2(0.0, 0.0);
+        for (int l = 0; l < 32; l++) acc[l] = make_double2(0.0, 0.0);
         for (int j = src_ptr[leaf] + lane; j < src_ptr[leaf + 1]; j += 32) {
             const double2 y = sxy[j];
             const double2 w = make_double2(e.x - (y.x - gc.cx) * ir, e.y - (y.y - gc.cy) * ir);
@@ -237,16 +313,17 @@ k_layer_p2l(int64_t nx, const int32_t *__restrict__ x_box, const int32_t *__rest
             const double2 t = make_double2(-0.5 * iw.x, -0.5 * iw.y);   // -1 / (2w)
             double2 pw = make_double2(1.0, 0.0);
 #pragma unroll
-            for (int l = 1; l < PMAX; l++) {
+            for (int l = 1; l < 32; l++) {
                 if (l < P1) {
                     pw = cmul(pw, t);
-                    const double2 v = cmul(pw, make_double2(dm.x - c * (1.0 / double(l)), dm.y));
-                    acc[l].x += v.x;
-                    acc[l].y += v.y;
+                    const double vx = fma(c, -1.0 / double(l), dm.x);
+                    acc[l].x = fma(pw.x, vx, fma(-pw.y, dm.y, acc[l].x));
+                    acc[l].y = fma(pw.x, dm.y, fma(pw.y, vx, acc[l].y));
                 }
             }
         }
-        warp_sum_store(acc, P1, lane, PX + x * P1);
+        const double2 s = warp_sums(acc, lane);
+        if (lane < P1) PX[x * P1 + lane] = s;
     }
 }
 
@@ -379,12 +456,12 @@ cudaError_t launch_layer(const PassArgs &a, const HostTree &h, const DevTree &d,
         k_layer_gather<<<grid_cap((ly.n + 255) / 256, 152 * 8), 256, 0, st>>>(ly.n, ly.perm, q, m, ly.cq, ly.cm);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    k_layer_p2m<32><<<grid_cap((a.nleaf + 3) / 4, 152 * 8), 128, 0, st>>>(
+    k_layer_p2m<<<kLayerCluster * grid_cap(a.nleaf, 152 * 4), 128, 0, st>>>(
         a.nleaf, ly.src_ptr, ly.sxy, ly.cq, ly.cm, d.leaf_box, d.box_level, d.box_ix, d.box_iy, h.x0, h.y0, h.L, P1,
         d.expA);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (ly.nx > 0) {
-        k_layer_p2l<32><<<grid_cap((ly.nx + 3) / 4, 152 * 8), 128, 0, st>>>(
+        k_layer_p2l<<<grid_cap((ly.nx + 3) / 4, 152 * 8), 128, 0, st>>>(
             ly.nx, ly.x_box, ly.x_src, ly.src_ptr, ly.sxy, ly.cq, ly.cm, d.leaf_box, d.box_level, d.box_ix, d.box_iy,
             h.x0, h.y0, h.L, P1, ly.PX);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
