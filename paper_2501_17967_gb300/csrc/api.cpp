@@ -1052,7 +1052,7 @@ bool build_wide_tree(bc_tree *t)
 int wide_parts(const bc_ctx *ctx) { return ctx->m2l_tri || ctx->m2l_kind ? kSplitTableParts : kWideParts; }
 
 // The split mode's M2L: on 7-digit products (as accurate as the FP64 kernels,
-// which take 0.87 ms of the FP64 pipe where the tiles take 0.25), unless an
+// which take 0.87 ms of the FP64 pipe where tiles and sums take 0.24), unless an
 // option chooses the products or another M2L, or the tiles do not fit.
 void split_m2l(bc_ctx *ctx, bc_tree *t, int prec, SplitLaunch &sl)
 {
@@ -1165,7 +1165,60 @@ bc_status apply_impl(bc_ctx *ctx, const bc_tree *tree, const double *vin, double
 }  // namespace
 
 bc_status prepare_split_tree(bc_tree *t) { return build_split_tree(t); }
-bool prepare_wide_tree(bc_tree *t) { return build_wide_tree(t); }
+// Tiles of a layer's L2P on 7 digits: the tree's own where an apply has set them up, else
+// (the same products) the expansion-to-leaf part alone: ordering all the lists and
+// the room for their rows took 1.3 ms of a first layer apply on 17,584 leaves (2.04
+// ms; 0.98 so).
+// nullptr: they do not fit.
+const SplitTree *prepare_wide_l2p(bc_tree *t)
+try {
+    if (t->wide_ready) return &t->spw;
+    if (t->spl.PE) return &t->spl;
+    if (t->wide_off || !t->ctx->wide_ready) return nullptr;
+    const SplitTables &T = t->ctx->wide;
+    const HostTree &h = t->h;
+    const int64_t nbox = int64_t(h.box_level.size());
+    std::vector<int32_t> leaves;
+    for (int32_t k = 0; k < int32_t(h.nleaf); k++)
+        if (h.leaf_level[k] >= 2) leaves.push_back(k);
+    std::vector<SplitTile> tiles;
+    add_tiles(tiles, T.e_op[0], 0, int64_t(leaves.size()), T.tileN, true);
+    SplitTree n;
+    int32_t *perm = nullptr;
+    n.ntE = n.ntL = int(tiles.size());
+    DevArena up;
+    up.add(&n.tE, tiles);
+    up.add(&perm, leaves);
+    up.room(&n.PE, size_t(h.nleaf) * T.np);
+    up.room(&n.edig, size_t(2 * nbox) * T.slices * kSplitKE);
+    up.room(&n.eexp, size_t(2 * nbox));
+    up.room(&n.cE[0], leaves.size());
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    cudaError_t e = ensure_side(t);
+    if (e == cudaSuccess && (e = up.commit(t->d.allocs, t->side.side)) == cudaSuccess) {
+        ColLists cl;
+        cl.nleaf = h.nleaf;
+        cl.leaf_level = t->d.leaf_level;
+        cl.leaf_box = t->d.leaf_box;
+        cl.box_level = t->d.box_level;
+        if (!leaves.empty())
+            cl.seg[cl.nseg++] = ColSeg{ColKind::L2P, 0, int64_t(leaves.size()), perm, n.cE[0], n.PE, int64_t(T.np), nbox};
+        if (cl.nseg) e = launch_make_cols(cl, t->side.side);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(t->side.side);
+        if (e != cudaSuccess) {
+            cudaFree(t->d.allocs.back());
+            t->d.allocs.pop_back();
+        }
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    n.err = t->ctx->dev_err;
+    t->spl = n;
+    return &t->spl;
+} catch (const std::bad_alloc &) {
+    return nullptr;
+}
 
 void set_error(const char *fmt, ...)
 {

@@ -477,9 +477,9 @@ cudaError_t layer_log_init();
 cudaError_t launch_log_inv_check(const double *x, int64_t n, double *lg, double *inv, cudaStream_t st);
 // The tiles of a tree in one digit format (built on first use; api.cpp).
 bc_status prepare_split_tree(struct bc_tree *t);
-// The same for the 7-digit products of the FP64 mode; false: not available
-// (the caller takes the FP64 kernels).
-bool prepare_wide_tree(struct bc_tree *t);
+// The expansion-to-leaf tiles of the 7-digit products; nullptr: not available (the
+// caller takes the FP64 kernels).
+const SplitTree *prepare_wide_l2p(struct bc_tree *t);
 // Strip solve, blocks up to 32 x 32 (kernels_strip.cu): nsys block-cyclic-
 // tridiagonal systems, workspace strip_work_doubles(N, m, r) each.
 size_t strip_work_doubles(int64_t N, int m, int r);
@@ -541,6 +541,7 @@ struct bc_tree {
     bc::DevTree d;
     bc::TileOrder order;      // list entries by operator
     bc::SplitTree sp, spw;    // tiles of the 5-digit and the 7-digit products
+    bc::SplitTree spl;        // of the latter the expansion-to-leaf part alone (a layer before any such apply)
     bc::SideStream side;
     bool split_ready = false, wide_ready = false;
     bool m2l_ready = false;   // tensor-core M2L tiles and rows (BC_SPLIT_BF16_ALL)

@@ -238,9 +238,9 @@ bc_status bc_layer_apply(bc_ctx *ctx, bc_layer *layer, const double *q, const do
         if (bs != BC_OK) return bs;
         sl.tree = &tree->sp;
         split = &sl;
-    } else if (prepare_wide_tree(tree)) {   // FP64: the L2P on 7 digits (else on the FP64 pipe)
+    } else if (const SplitTree *wt = prepare_wide_l2p(tree)) {   // FP64: the L2P on 7 digits (else on the FP64 pipe)
         sl.tables = &ctx->wide;
-        sl.tree = &tree->spw;
+        sl.tree = wt;
         split = &sl;
     }
     const size_t nu = size_t(tree->h.nleaf) * ctx->NP, n = size_t(layer->n);

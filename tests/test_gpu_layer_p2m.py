@@ -32,3 +32,18 @@ def test_source_counts(n):
     err = np.abs(u[far] - ref[far]).max() / np.abs(ref[far]).max()
     print(f"{n} sources, {far.sum()} leaves: {err:.1e}")
     assert far.sum() >= 40 and err <= 1e-10
+
+
+# the L2P's tiles made by the layer itself, and the tree's after an apply: same products
+@pytest.mark.parametrize("level", [0, 1, 3])
+def test_before_and_after_an_apply(level):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ctx = bc.Context(p=16, nterms=30, device=0)
+    tree = bc.Tree(ctx, *synth.uniform_leaves(level))
+    rng = np.random.default_rng(3)
+    layer = bc.Layer(tree, rng.uniform(-0.9, 0.9, (40, 2)))
+    q, m = torch.from_numpy(rng.standard_normal(40)).cuda(), torch.from_numpy(rng.standard_normal((40, 2))).cuda()
+    before = layer.apply(q, m)
+    bc.apply(tree, torch.ones(tree.nleaf, 16, 16, device="cuda", dtype=torch.float64))
+    assert torch.equal(before, layer.apply(q, m))
