@@ -12,9 +12,10 @@ eps = 1e-11) and 2:1 balanced: 14,191 leaves, 15 levels, 3.63M leaf nodes.
 A step is one forward apply u = A f and one adjoint apply h = A^T g of the
 whole tree; value = leaf nodes / (time of a step).  The headline precision
 ("split") takes the fixed-operator products (near field, P2M, L2P, W and X
-lists) on BF16 tensor cores as exact digit products and keeps the
-multipole-to-local translations, the M2M/L2L shifts, the log terms and
-every sum in native FP64.  The same JSON line carries the native FP64 path,
+lists) on BF16 tensor cores as exact digit products of 40-bit operands, the
+multipole-to-local translations as products of 56-bit ones (as accurate as
+FP64), and keeps the M2M/L2L shifts and the log terms in native FP64.  The same
+JSON line carries the FP64 path (every product of 56-bit operands),
 the all-tensor split variant and the 20-Gaussian workload as extra keys, and
 the error against the oracle per level, forward and adjoint.
 With --gpus N every rank runs its own replica (the path does not shard; no
@@ -51,11 +52,12 @@ WORKLOADS = {
 }
 PRECISIONS = {"fp64": 0, "split": 1, "split_all": 2}
 DTYPES = {
-    0: "f64",
+    0: "f64 (fixed-operator products as 7 bf16 digits per operand, 56 bits, exact FP32 accumulation; the error is "
+       "FP64's)",
     1: "bf16 digits (5 slices, exact FP32 accumulation) for the near field, P2M, L2P, W and X lists; "
-       "f64 for M2L, M2M/L2L, log terms and sums",
-    2: "bf16 digits for every fixed-operator product including M2L; double-float (2 x f32) M2M/L2L; "
-       "f64 log terms and sums",
+       "7 slices (56 bits, FP64's error) for the M2L; f64 for M2M/L2L and log terms",
+    2: "bf16 digits (5 slices) for every fixed-operator product including M2L; double-float (2 x f32) M2M/L2L; "
+       "f64 log terms",
 }
 
 
@@ -243,66 +245,44 @@ STAGE_KERNELS = {
     "tensor_v": "k_split_vec + k_split_gemm<256> (leaf-to-expansion; X list and near field too in line)",
     "clear": "k_clear_flags",
     "upward": "k_up_levels",
-    "m2l": "k_m2l_boxes (FP64 M2L per target box; FP64 path also k_x_entries) | "
-           "k_split_exp + k_split_gemm<64> (all-tensor split)",
-    "down_levels": "k_down_warps | k_down_levels<double-float> (all-tensor split)",
-    "tensor_e": "k_split_exp + k_split_gemm<64> (L2P and W list)",
-    "leaf_output": "k_leaf_out",
+    "m2l": "k_split_exp + k_gemm64 + k_v_sums (all-tensor split: without the sums)",
+    "down_levels": "k_down_groups | k_down_levels (double-float, all-tensor split)",
+    "tensor_e": "k_split_exp + k_gemm64 (L2P and W list)",
+    "leaf_output": "k_leaf_sums",
     "tensor_near": "k_split_gemm<256> (X list, then near field, on the internal stream)",
 }
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of each stage's
 # kernel in the bench configuration, keyed by (workload, nterms, precision):
 # filled from the ncu captures of the unchanged kernels, null otherwise
-# (the FP64 M2L: mean of one forward and one adjoint launch)
-TRAFFIC = {("adaptive200", 24, "split"): {"m2l": 10043776}}
+TRAFFIC = {}
 
 
 def stage_work(st, nleaf, nleaf_far, P1, NP, prec):
     """Algorithmic work of each stage of one apply, counted from the tree's
-    lists: (amount, kind), kind "tensor" (BF16 flops of the 15 digit products,
-    rows x K x columns of the real operators), "fp64" (FP64 flops; a real x
-    complex term counts 4, a complex x complex term 8) or "bytes"."""
+    lists: (amount, kind), kind "tensor" (BF16 flops of the digit products, 15 with
+    five digits, 34 with seven; rows x K x columns of the real operators), "fp64"
+    (FP64 flops; a real x complex term counts 4) or "bytes"."""
     R = 2 * P1
-    m2l64 = (4.0 * P1 * P1 + 14.0 * P1) * st["n_v"]          # factored form, per V pair
-    shift64 = 4.0 * (P1 * (P1 + 1) / 2) + 12.0 * P1           # factored shift per child: binomial + diagonals
-    up64 = 4 * shift64 * st["n_nonleaf"]
-    down64 = shift64 * st["n_down"] + 2.0 * P1 * st["n_x"]
-    if prec == 0:
-        return {
-            "tensor_v": (0.0, "tensor"), "tensor_near": (0.0, "tensor"), "clear": (0.0, "fp64"),
-            "upward": (4.0 * P1 * NP * nleaf + up64, "fp64"),
-            "m2l": (m2l64 + 4.0 * P1 * NP * st["n_x"], "fp64"),
-            "down_levels": (down64, "fp64"),
-            "tensor_e": (0.0, "tensor"),
-            "leaf_output": (2.0 * NP * NP * st["n_near"] + 4.0 * P1 * NP * (nleaf_far + st["n_w"]), "fp64"),
-        }
-    w = {
-        "tensor_v": (15 * 2.0 * NP * R * (nleaf + st["n_x"]), "tensor"),
-        "tensor_near": (15 * 2.0 * NP * NP * st["n_near"], "tensor"),
+    dig = 34 if prec == 0 else 15
+    tri = 4.0 * (P1 * (P1 + 1) / 2)                           # the binomial triangle, shared by four siblings
+    return {
+        "tensor_v": (dig * 2.0 * NP * R * (nleaf + st["n_x"]), "tensor"),
+        "tensor_near": (dig * 2.0 * NP * NP * st["n_near"], "tensor"),
         "clear": (0.0, "fp64"),
-        "upward": (up64, "fp64"),
-        "m2l": (m2l64, "fp64"),
-        "down_levels": (down64, "fp64"),
-        "tensor_e": (15 * 2.0 * R * NP * (nleaf_far + st["n_w"]), "tensor"),
+        "upward": ((tri + 56.0 * P1) * st["n_nonleaf"], "fp64"),
+        "m2l": ((15 if prec == 2 else 34) * 2.0 * R * R * st["n_v"], "tensor"),
+        "down_levels": ((tri + 62.0 * P1) * st["n_down"] / 4 + 2.0 * P1 * st["n_x"], "fp64"),
+        "tensor_e": (dig * 2.0 * R * NP * (nleaf_far + st["n_w"]), "tensor"),
         "leaf_output": (8.0 * NP * (st["n_near"] + st["n_w"] + nleaf_far + nleaf), "bytes"),
     }
-    if prec == 2:
-        w["m2l"] = (15 * 2.0 * R * R * st["n_v"], "tensor")
-    return w
 
 
 def launches_per_apply(prec, overlap, st):
     """Kernels of one apply (trees of more than three levels), as the launch
     list of the profiles shows them."""
-    if prec == 0:
-        return 1 + 1 + 1 + (1 if st["n_x"] > 0 else 0) + 1 + 2   # clear, up, M2L, X, down, leaf logs + leaf
-    if prec == 1:
-        # digits + P2M tiles, clear, up, FP64 M2L, down, L2P digits + tiles, logs + leaf; beside the M2L:
-        # X tiles, multipole digits + W tiles, near field
-        return 2 + 1 + 1 + 1 + 1 + 2 + 2 + (4 if overlap else 0)
-    # all-tensor: digits + group V, clear, up, M2L digits + tiles, down, E digits + tiles, logs + leaf;
-    # X tiles and near field on the internal stream
-    return 2 + 1 + 1 + 2 + 1 + 2 + 2 + (2 if overlap else 0)
+    # digits + group V (P2M; in line also X list and near field), clear, up, M2L digits + tiles (+ row sums), down,
+    # E digits + tiles, logs + leaf; X tiles and near field apart on the internal stream
+    return 2 + 1 + 1 + (2 if prec == 2 else 3) + 1 + 2 + 2 + (2 if overlap else 0)
 
 
 def run_batch64(args):
@@ -437,10 +417,10 @@ def layer_line(args, dev, steps, check=True):
 def strip_line(args, dev, steps, peak_fp64, check=True):
     """The strip solve of Sec. 3.3 at the paper's size: 56 elements of 16 x 24
     nodes (N = 56 blocks of m = 384, one right-hand side), block LU of the
-    tridiagonal part plus the Woodbury corner correction, random block
+    tridiagonal part plus the bordered corner correction, random block
     diagonally dominant blocks; and the batched small-block case (608
-    systems of N = 256, m = 17, one warp each).  Algorithmic FP64 work per
-    system N m^2 (14 m / 3 + 6 R), R = r + 2m."""
+    systems of N = 256, m = 17, one CTA each).  Algorithmic FP64 work per
+    system N m^2 (14 m / 3 + 6 R), R = r + m."""
     import torch
 
     import oracle
@@ -472,17 +452,17 @@ def strip_line(args, dev, steps, peak_fp64, check=True):
         return sum(a.elapsed_time(c) for a, c in ev) / nsteps, x
 
     def work(nsys, N, m, r):
-        return nsys * N * m * m * (14.0 * m / 3.0 + 6.0 * (r + 2 * m))
+        return nsys * N * m * m * (14.0 * m / 3.0 + 6.0 * (r + m))
 
     big = make(1, 56, 384, 1, 5)
     ms, x = timed(big, max(3, steps // 2))
     ach = work(1, 56, 384, 1) / (ms * 1e-3) / 1e12
     line = {"value": 1.0 / (ms * 1e-3), "unit": "strip solves/s", "ms": ms,
             "workload": "the paper's strip size: N = 56 elements of 16 x 24 nodes (m = 384), one right-hand side; "
-                        "block LU + Woodbury, blocked LU per element over the whole GPU",
+                        "block LU + border, one cooperative launch over the whole GPU",
             "roofline": {"bound": "alu", "achieved": round(ach, 4), "peak": round(peak_fp64, 3), "unit": "TFLOP/s",
                          "frac": round(ach / peak_fp64, 4), "traffic": None,
-                         "work": "N m^2 (14 m / 3 + 6 R) FP64 flop per system, R = r + 2m"},
+                         "work": "N m^2 (14 m / 3 + 6 R) FP64 flop per system, R = r + m"},
             "dtype": "f64"}
     if check:
         A, B, C, b = big
@@ -497,7 +477,7 @@ def strip_line(args, dev, steps, peak_fp64, check=True):
     ms2, x2 = timed(small, steps)
     ach2 = work(608, 256, 17, 1) / (ms2 * 1e-3) / 1e12
     line["batched_small"] = {"value": 608 / (ms2 * 1e-3), "unit": "strip systems/s", "ms": ms2,
-                             "workload": "608 systems, N = 256, m = 17, r = 1, one warp each",
+                             "workload": "608 systems, N = 256, m = 17, r = 1, one CTA each",
                              "roofline_frac": round(ach2 / peak_fp64, 4)}
     if check:
         A, B, C, b = small
@@ -714,11 +694,11 @@ def main():
     def arrangement_work(prec, overlap=None):
         overlap = args.overlap if overlap is None else overlap
         wk = stage_work(st, tree.nleaf, nleaf_far, P1, P * P, prec)
-        if prec and not overlap:
+        if not overlap:
             wk["tensor_v"] = (wk["tensor_v"][0] + wk["tensor_near"][0], "tensor")   # one group-V launch
             wk["tensor_near"] = (0.0, "tensor")
-        elif prec:
-            xw = 15 * 2.0 * P * P * 2 * P1 * st["n_x"]   # X-list tiles run on the internal stream
+        else:
+            xw = (15 if prec else 34) * 2.0 * P * P * 2 * P1 * st["n_x"]   # X-list tiles run on the internal stream
             wk["tensor_v"] = (wk["tensor_v"][0] - xw, "tensor")
             wk["tensor_near"] = (wk["tensor_near"][0] + xw, "tensor")
         return wk

@@ -338,8 +338,10 @@ bc_status bc_table_export(const bc_ctx *ctx, int which, int64_t *count, double *
  *   "m2l_triangular" (0/1, default 0): keep only the terms with k + l <= P of
  *     each multipole-to-local translation (and exactly their transpose in the
  *     adjoint), which halves the M2L arithmetic but loses accuracy.
- *   "m2l_kernel" (0/1, default 0): the FP64 multipole-to-local kernel: 0 FP64
- *     FMAs, one block per target box; 1 the FP64 tensor cores (mma.sync f64
+ *   "m2l_kernel" (0/1, default 0): the native FP64 multipole-to-local kernel
+ *     (where the translations are not digit products: bc_apply_noalloc, layers,
+ *     m2l_triangular, trees whose tiles do not fit): 0 FP64
+ *     FMAs, one block per target box; 1, for every FP64 translation, the FP64 tensor cores (mma.sync f64
  *     tiles of the binomial matrix), one warp per target box.  Same results
  *     to rounding.
  *   "m2l_blocks_per_sm" (integer 0..32, default 0): resident blocks per SM of
@@ -347,29 +349,30 @@ bc_status bc_table_export(const bc_ctx *ctx, int which, int64_t *count, double *
  *     beside the near-field tensor launch, which fits beside them; 8 (4)
  *     otherwise).
  *   "wait_limit" (default 2^26): polls of each bounded device-side wait of the
- *     split-precision kernel before it gives up, records the failure (reported
+ *     tensor-core kernels before it gives up, records the failure (reported
  *     by bc_sync as BC_ERR_TIMEOUT), frees its tensor memory and returns; the
  *     level passes' box flags poll a sixteenth of it and report the same way.
  *   "split_overlap" (0..3, default 1): the X-list and near-field tensor-core
- *     launches of a split-precision apply run on an internal stream and are
+ *     launches of an apply run on an internal stream and are
  *     joined before the downward pass (X list) and the leaf output (near
  *     field) (1; 2 in the forward apply only, 3 in the adjoint only), or in
- *     line on the apply's stream (0).  With the M2L in FP64
- *     (BC_SPLIT_BF16) they start after the upward pass and run beside the
- *     FP64 M2L (they use the tensor cores, it the FP64 units); with the
- *     tensor-core M2L (BC_SPLIT_BF16_ALL) they start at once, beside the
- *     latency-bound level passes.
+ *     line on the apply's stream (0).  With the M2L on the tensor cores they
+ *     start at once, beside the latency-bound level passes; with the native
+ *     FP64 M2L they start after the upward pass and run beside it (they use the
+ *     tensor cores, it the FP64 units).
  *   "split_overlap_ctas" (integer >= 0, default 0): CTAs (one per SM) of
  *     that near-field launch; 0 takes every SM beside the FP64 M2L and three
  *     quarters of them beside the level passes.
  *   "debug_split_parts" (integer -1..127, default -1): diagnostics; which
- *     products of a split-precision apply use the tensor-core results (bits:
+ *     products of a split-precision apply use the 5-digit results (bits:
  *     1 near field, 2 leaf-to-expansion, 4 X list, 8 expansion-to-leaf,
- *     16 W list, 32 M2L translations); the others are evaluated in FP64.
+ *     16 W list, 32 M2L translations); the others are evaluated by the native FP64
+ *     kernels; 0 is the BC_FP64 apply.
  *     Bit 64: the shifts of the upward and downward level passes, and with
  *     bit 2 off the leaf-to-expansion step, in double-float arithmetic (pairs
  *     of FP32 numbers, about 48 bits) instead of FP64.  -1 takes the set of
- *     the precision mode: 31 for BC_SPLIT_BF16, 127 for BC_SPLIT_BF16_ALL.
+ *     the precision mode: 31 for BC_SPLIT_BF16 (with the M2L on 7 digits), 127
+ *     for BC_SPLIT_BF16_ALL.
    "debug_withhold_copy" (0/1, default 0): diagnostics; the split-precision
  *     kernel never starts its table copy, so its first wait runs out (tests of
  *     the timeout path).
@@ -380,18 +383,18 @@ bc_status bc_set_option(bc_ctx *ctx, const char *name, double value);
  * evaluates: bit 0 the near field (leaf-to-leaf tables), bit 1 the far field
  * (expansions); 3 = the full operator (default).  timing != 0 records a CUDA
  * event at each stage boundary:
- *   0 tensor group V, far part (split precision: digits of the input,
+ *   0 tensor group V, far part (digits of the input,
  *     leaf-to-expansion; in line also the X list and the near field),
- *     1 flag clearing, 2 upward pass (FP64: with the leaf-to-expansion step),
- *     3 M2L (FP64 path: and the X-list products), 4 downward level pass (sums,
- *     shifts), 5 tensor group E (split precision: digits of the expansions,
+ *     1 flag clearing, 2 upward pass (native FP64: with the leaf-to-expansion
+ *     step), 3 M2L (native FP64: and the X-list products), 4 downward level pass
+ *     (sums, shifts), 5 tensor group E (digits of the expansions,
  *     expansion-to-leaf and W list), 6 leaf output; 7 the X-list and
  *     near-field tensor launches when they run apart on the internal stream
- *     (split_overlap: beside stage 3 with the FP64 M2L, beside stages 1-4
- *     otherwise; in line stage 7 is empty);
+ *     (split_overlap: beside stages 1-4, or stage 3 with the native FP64 M2L;
+ *     in line stage 7 is empty);
  * bc_debug_stage_times then waits for the last events of the most recent
  * forward (adjoint = 0) or adjoint apply and writes the eight stage durations
- * in milliseconds to ms[8] (stages 0, 5 and 7 are empty for FP64 applies). */
+ * in milliseconds to ms[8] (stages 0, 5 and 7 are empty where an apply runs on the native FP64 kernels). */
 bc_status bc_debug_set(bc_ctx *ctx, int pass_mask, int timing);
 bc_status bc_debug_stage_times(bc_ctx *ctx, int adjoint, double *ms);
 /* The term schedule of the double-float upward shift of BC_SPLIT_BF16_ALL, for

@@ -702,7 +702,7 @@ inline int m2l_threads(int P1) { return (m2l_groups(P1) * P1 + 31) / 32 * 32; }
 // below its last, so 32 terms fit in 63 bits and each loses less than 2^-5 of the
 // last place of the largest term, where an FP64 addition rounds to half of one.
 // Groups with an infinity or a NaN, near the ends of the range, or all zero are added
-// in FP64.  k_v_sums (300,000 pairs, 31 coefficients): 84 -> 53 us.
+// in FP64.  k_v_sums (403,338 pairs, 30 coefficients): 84 -> 53 us.
 // -------------------------------------------------------------------------
 struct RowSum {
     double v = 0.0;
@@ -764,7 +764,7 @@ struct RowSum {
 // out the log term), one warp per box, lane o = coefficient o:
 //   out[b][o] = sum_{e in V(b)} [ Pv[e][o] + (o = 0) (log|d_e| + log r_b) first[s_e][0] ]
 // Apart from the downward pass, whose chain of boxes would wait for the ~27
-// dependent row loads of each.  16 P1 bytes per pair (197 MB at 300,000 pairs, 29 us);
+// dependent row loads of each.  16 P1 bytes per pair (194 MB at 403,338 pairs, 29 us);
 // bound by the additions: kVRows rows in flight, summed by RowSum, with 64 registers
 // per thread (12 rows took 90, two blocks per SM and 67 us instead of 53).
 // -------------------------------------------------------------------------
@@ -1337,7 +1337,7 @@ __global__ void k_leaf_out(int64_t nleaf, const int32_t *__restrict__ order,
 // per leaf); kLeafRows of them in flight, the next leaf's lists read before the
 // sums.  Of each four rows one is added in FP64 and three by RowSum: the FP64 pipe
 // and the integer pipe work side by side, neither alone keeps up with memory.
-// 17,491 leaves, p = 16 (500 MB, 74 us at the copy rate): all additions in FP64 139 us
+// 17,491 leaves, p = 16 (468 MB, 69 us at the copy rate): all additions in FP64 139 us
 // (forward) and 161 (adjoint), all by RowSum 137, one in four 99.
 // -------------------------------------------------------------------------
 constexpr int kLeafRows = 12;

@@ -21,9 +21,11 @@
 //        L_l = sum (-1)^l (2w)^-l [ -c_q / l + (c_m / r_c) / w ]
 //   M2P  (W list) and L2P as for the volume potential, near field direct;
 // with c_q = -q / (2 pi), c_m = -m / (2 pi).  A source that coincides with a
-// target node contributes nothing.  FP64 and (logarithms) fixed point, except the L2P (the volume
-// apply's group-E tensor tiles over the same locals: 7 digits in the FP64 mode, 5
-// in the split one; 1.86 -> 1.63 ms at 17,584 leaves, 4,096 nodes, FP64).
+// target node contributes nothing.  FP64 accuracy throughout: the near sums'
+// logarithm and reciprocal in fixed point, the L2P on the volume apply's group-E
+// tensor tiles over the same locals (7 digits in the FP64 mode, 5 in the split one).
+// 17,584 leaves, 4,096 nodes, FP64: 1.86 -> 1.63 ms by the L2P; 0.74 with the near
+// sums, level passes and P2M as they are now.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -52,7 +54,8 @@ __device__ __forceinline__ double2 cinv(double2 a)
 // TOMS 16, 1990) in fixed point.  An FP64 operation holds a sub-partition's FP64
 // pipe for 64 cycles per warp, 30 of them per (node, source) pair bound the sums
 // (13 for the logarithm, 8 for the reciprocal); integer and FP32 operations take 1 or
-// 2 cycles, and only the two conversions are left on the FP64 pipe.  With
+// 2 cycles, and ten FP64 operations per pair are left (17,584 leaves, 4,096 sources:
+// leaf output 1160 -> 408 us).  With
 // x = 2^e m, m in [1, 2), and j the top kLogBits bits of m's fraction, c_j is
 // 1 / (1 + (j + 1/2) / 2^kLogBits) rounded to 11 bits, so that m c_j is an exact 64-bit
 // integer and r = m c_j - 1 an exact multiple of 2^-63, |r| < 7.4e-4; then

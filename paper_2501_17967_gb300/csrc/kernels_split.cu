@@ -476,7 +476,9 @@ struct GemmShape {
     static constexpr int N = Fmt<S>::N, L = Fmt<S>::L;
     static constexpr int KC = KD > 144 ? kSplitKC : KD;   // K columns per operator chunk and B buffer
     static constexpr int NKC = KD / KC;
-    // operator chunk buffers: three, two where the shared memory is short (KD = 144:
+    // operator chunk buffers of 128 columns: each chunk costs some 500 cycles beside its
+    // MMAs (six of 64 columns in the same memory: near field of 17,491 leaves, 7 digits,
+    // 550 -> 821 us); three, two where the shared memory is short (KD = 144:
     // two whole tiles of B) or left to the FP64 M2L's blocks beside (ICVT)
     static constexpr int NB = KD == 144 || ICVT ? 2 : 3;
     static constexpr int kBSlice = N * KC * 2;         // bytes of one B digit slice of a chunk
@@ -911,7 +913,11 @@ k_split_gemm(const __grid_constant__ SplitGemm gm, double inv_alpha0, int inv_al
 // only where it changes.  Streamed through three chunk buffers like the larger
 // ones, a tile took 5.2 us, four times its MMAs: each chunk's copy latency
 // stood between short MMA runs.  17,491 leaves, 30 terms, 7 digits, alone: the
-// M2L's tiles 427 -> 262 us, expansion-to-leaf and W list 168 -> 134 us.
+// M2L's tiles 427 -> 262 us, expansion-to-leaf and W list 168 -> 134 us (176 and 87
+// with the epilogue of four columns side by side: per M2L tile 4,100 cycles, its MMAs
+// 2,400, its epilogue 2,600-3,500; per expansion-to-leaf tile 6,600, the epilogue
+// 5,700.  Loading a batch's levels before the last one was stored spilled registers:
+// 241 and 107 us).
 //   warp 0      MMAs: per tile one chain per operator digit, issued back to back
 //   warp 1      operator copies
 //   warps 2-7   column metadata and digits: 192 / N threads per column, each with
