@@ -430,15 +430,22 @@ inline int grid_cap(int64_t n, int cap) { return int(n < cap ? (n > 0 ? n : 1) :
 
 cudaError_t layer_log_init()
 {
-    // c_j to 11 bits, -log c_j from the host's extended-precision logarithm
-    unsigned long long t[kLogN];
-    for (int j = 0; j < kLogN; j++) {
-        const double c = std::nearbyint(2048.0 / (1.0 + (j + 0.5) / kLogN));
-        const long double l = -logl(static_cast<long double>(c) / 2048.0L);
-        t[j] = static_cast<unsigned long long>(c - 1024.0) << 53 |
-               static_cast<unsigned long long>(l * 9007199254740992.0L + 0.5L);
-    }
-    return cudaMemcpyToSymbol(g_logtab, t, sizeof t);
+    // c_j to 11 bits, -log c_j from the host's extended-precision logarithm (once per
+    // process: half a millisecond where that is done in software)
+    struct Table {
+        unsigned long long t[kLogN];
+        Table()
+        {
+            for (int j = 0; j < kLogN; j++) {
+                const double c = std::nearbyint(2048.0 / (1.0 + (j + 0.5) / kLogN));
+                const long double l = -logl(static_cast<long double>(c) / 2048.0L);
+                t[j] = static_cast<unsigned long long>(c - 1024.0) << 53 |
+                       static_cast<unsigned long long>(l * 9007199254740992.0L + 0.5L);
+            }
+        }
+    };
+    static const Table tab;
+    return cudaMemcpyToSymbol(g_logtab, tab.t, sizeof tab.t);
 }
 
 cudaError_t launch_log_inv_check(const double *x, int64_t n, double *lg, double *inv, cudaStream_t st)
