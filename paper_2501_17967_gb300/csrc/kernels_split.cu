@@ -545,6 +545,7 @@ __device__ __forceinline__ void epilogue_columns(const SplitGemm &gm, const Spli
 {
     constexpr int kL = Fmt<S>::L, kN = Fmt<S>::N, kQ = 4;   // columns per batch
     for (int c0 = cb; c0 < ce; c0 += kQ) {   // uniform over the warp
+        __syncwarp();   // the lanes part ways below, by their results: tcgen05.ld wants the whole warp
         uint32_t d[kL][kQ];
 #pragma unroll
         for (int g = 0; g < kL; g++) tmem_ld4(ta0 + uint32_t(g * kN + c0), d[g]);

@@ -91,6 +91,19 @@ def test_magnitudes(kind, adjoint):
         assert err <= BAR
 
 
+@pytest.mark.parametrize("p", [8, 12, 16])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_results_about_the_end_of_the_normal_range(p, adjoint):
+    """Rows of which some entries are subnormal: lanes of one epilogue warp scale their results in different ways.
+    Bar: the FP64 kernels' and the rounding of some forty partial results to multiples of 2^-1074."""
+    tree, x = make(p, 24)
+    u1 = kernels(tree, x, adjoint)
+    scale = 2.0 ** (-1015 - round(np.log2(u1.abs().max().item())))
+    u = digits(tree, x * scale, adjoint)
+    err = (u / scale - u1).abs().max().item()
+    assert (u.abs() < 2.0 ** -1022).any() and err <= BAR * u1.abs().max().item() + 64 * 2.0 ** -1074 / scale
+
+
 @pytest.mark.parametrize("adjoint", [False, True])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
 def test_non_finite_values(bad, adjoint):
