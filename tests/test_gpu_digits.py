@@ -94,14 +94,15 @@ def test_magnitudes(kind, adjoint):
 @pytest.mark.parametrize("p", [8, 12, 16])
 @pytest.mark.parametrize("adjoint", [False, True])
 def test_results_about_the_end_of_the_normal_range(p, adjoint):
-    """Rows of which some entries are subnormal: lanes of one epilogue warp scale their results in different ways.
-    Bar: the FP64 kernels' and the rounding of some forty partial results to multiples of 2^-1074."""
+    """Products of which some entries are subnormal (a leaf's rows carry its r^2, higher coefficients are smaller):
+    lanes of one epilogue warp scale their results in different ways.  The level passes lose bits there too, in
+    either path: the bar is BAR above twice what the FP64 kernels lose on the same input."""
     tree, x = make(p, 24)
     u1 = kernels(tree, x, adjoint)
-    scale = 2.0 ** (-1015 - round(np.log2(u1.abs().max().item())))
-    u = digits(tree, x * scale, adjoint)
-    err = (u / scale - u1).abs().max().item()
-    assert (u.abs() < 2.0 ** -1022).any() and err <= BAR * u1.abs().max().item() + 64 * 2.0 ** -1074 / scale
+    top = u1.abs().max().item()
+    scale = 2.0 ** (-1015 - round(np.log2(top)))
+    u, v = digits(tree, x * scale, adjoint), kernels(tree, x * scale, adjoint)
+    assert (u / scale - u1).abs().max().item() <= BAR * top + 2.0 * (v / scale - u1).abs().max().item()
 
 
 @pytest.mark.parametrize("adjoint", [False, True])
