@@ -295,6 +295,16 @@ void bc_layer_destroy(bc_layer *layer);
 bc_status bc_strip_workspace(int64_t nsys, int64_t N, int m, int r, int64_t *bytes);
 bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B, const double *C,
                          const double *b, double *x, void *work, int32_t *status, void *stream);
+/* Diagnostics: bc_strip_solve with the order of events in the large-block solve
+ * (m > 32; smaller blocks: no effect) disturbed.  All zero: as bc_strip_solve.
+ *   stall_ns: blocks that own right-hand columns only wait so long (at most 1 ms)
+ *     before each factored panel they apply. */
+typedef struct {
+    int32_t stall_ns;
+} bc_strip_debug;
+bc_status bc_debug_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B,
+                               const double *C, const double *b, double *x, void *work, int32_t *status,
+                               const bc_strip_debug *debug, void *stream);
 
 /* Batched applies: many independent densities on different trees (all of
  * this context's p and root side L) in one launch per pass.  Not in the

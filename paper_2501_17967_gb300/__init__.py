@@ -54,6 +54,10 @@ class _Stats(ctypes.Structure):
                                                "n_nonleaf", "n_down")]
 
 
+class _StripDebug(ctypes.Structure):
+    _fields_ = [("stall_ns", ctypes.c_int32)]
+
+
 DENSITY_FN = ctypes.CFUNCTYPE(None, ctypes.POINTER(ctypes.c_double), ctypes.c_int64,
                               ctypes.POINTER(ctypes.c_double), ctypes.c_void_p)
 
@@ -93,6 +97,8 @@ SIGNATURES = [
     ("bc_strip_workspace", ctypes.c_int, [_I64, _I64, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int64)]),
     ("bc_strip_solve", ctypes.c_int, [_I64, _I64, ctypes.c_int, ctypes.c_int, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
                                       _VP]),
+    ("bc_debug_strip_solve", ctypes.c_int, [_I64, _I64, ctypes.c_int, ctypes.c_int, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
+                                            ctypes.POINTER(_StripDebug), _VP]),
     ("bc_batch_create", ctypes.c_int, [_VP, ctypes.POINTER(_VP), ctypes.c_int, ctypes.POINTER(_VP)]),
     ("bc_batch_destroy", None, [_VP]),
     ("bc_batch_nleaf", _I64, [_VP]),

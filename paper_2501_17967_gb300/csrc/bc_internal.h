@@ -489,7 +489,8 @@ cudaError_t launch_strip(int64_t nsys, int64_t N, int m, int r, const double *A,
 // Larger blocks (kernels_strip_large.cu): one system, one cooperative launch.
 size_t strip_large_work_doubles(int64_t N, int m, int r);
 cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const double *B, const double *C, const double *b,
-                               double *x, double *work, int32_t *status, cudaStream_t stream);
+                               double *x, double *work, int32_t *status, cudaStream_t stream,
+                               const bc_strip_debug &dbg);
 // Batched applies: copy the per-tree arrays into / out of the union's vectors.
 constexpr int kBatchChunk = 96;   // trees per gather/scatter launch (pointer tables go by value)
 struct BatchPtrs {

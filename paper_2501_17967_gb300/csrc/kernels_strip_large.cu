@@ -43,8 +43,9 @@ constexpr int kMaxM = 448;
 constexpr int kMaxD = 3, kMaxR = 4;   // columns of a kind per worker (m = 448, r = 32 on 150 workers)
 constexpr int kPollLimit = 1 << 22;
 
-// counters in the workspace (zeroed before the launch), 128 bytes apart
-enum { kCtrPanel = 0, kCtrCols = 16, kCtrInv = 32, kCtrDone = 48, kCtrGrid = 64, kCtrAbort = 80, kCtrWords = 96 };
+// counters in the workspace (zeroed before the launch), 64 bytes apart
+// (kCtrDone: one per parity of the element)
+enum { kCtrPanel = 0, kCtrCols = 16, kCtrInv = 32, kCtrDone = 48, kCtrGrid = 80, kCtrAbort = 96, kCtrWords = 112 };
 
 struct LargeArgs {
     int64_t N;
@@ -57,6 +58,7 @@ struct LargeArgs {
     int32_t *perm;             // [2][np][m] row (within the panel's rows) that ends at each position
     uint32_t *ctr;
     int32_t *status;
+    int stall_ns;              // diagnostics: workers without a matrix column wait so long before each background panel
 };
 
 __device__ __forceinline__ uint32_t ctr_load(const uint32_t *p)
@@ -551,8 +553,12 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
         double *F = a.F + size_t(par) * mm;
         const double *Li = a.Linv + size_t(par) * np * kW * kW;
         const int32_t *pm = a.perm + size_t(par) * np * m;
-        // F of this parity was last read in element e - 2
-        if (e >= 2 && !cta_wait(a, kCtrDone, uint32_t((e - 1) * a.nw), &S.ok)) return false;
+        // F of this parity was last read in element e - 2, which every worker has to
+        // have left: each adds one per element to its parity's count.  (One count for
+        // both would not do: a worker without a matrix column holds up no panel, so it
+        // may lag while the others' counts run ahead.)
+        uint32_t *const done = a.ctr + kCtrDone + 16 * par;
+        if (e >= 2 && !cta_wait(a, int(done - a.ctr), uint32_t((e / 2) * a.nw), &S.ok)) return false;
         auto panel_of = [&](int i) { return (w + i * a.nw) / kW; };   // of own D column i
         auto deliver = [&](int p) {   // own columns of panel p into F
             int n = 0;
@@ -607,6 +613,7 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
                 tile++;
                 __syncthreads();
             } else if (pB < np && pB < avail && tile >= ntile && !urgent) {
+                if (a.stall_ns > 0 && nD == 0) __nanosleep(a.stall_ns);
                 with_count(nbg, [&](auto n) {
                     apply_panel<decltype(n)::value>(a, F, Li + pB * kW * kW, pm + size_t(pB) * m, pB, bg, S);
                 });
@@ -630,7 +637,7 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
         with_count(nbg, [&](auto n) {
             back_substitute<decltype(n)::value>(a, F, a.Uinv + size_t(par) * np * kW * kW, bg, S);
         });
-        cta_signal(a, kCtrDone, 1);
+        cta_signal(a, int(done - a.ctr), 1);
         return true;
     };
 
@@ -767,7 +774,7 @@ size_t strip_large_work_doubles(int64_t N, int m, int r)
 }
 
 cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const double *B, const double *C, const double *b,
-                               double *x, double *work, int32_t *status, cudaStream_t st)
+                               double *x, double *work, int32_t *status, cudaStream_t st, const bc_strip_debug &dbg)
 {
     if (m > kMaxM) return cudaErrorInvalidValue;
     int dev = 0, sms = 0;
@@ -793,6 +800,7 @@ cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const d
     a.perm = reinterpret_cast<int32_t *>(w); w += size_t(a.np) * m;
     a.ctr = reinterpret_cast<uint32_t *>(w); w += kCtrWords / 2;
     a.status = status ? status : reinterpret_cast<int32_t *>(w);
+    a.stall_ns = dbg.stall_ns;
     e = cudaMemsetAsync(a.ctr, 0, kCtrWords * sizeof(uint32_t), st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_strip_large, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;

@@ -36,23 +36,8 @@ size_t strip_scratch_doubles(int64_t nsys, int64_t N, int m, int r)
     return m <= kSmallM ? size_t(nsys) * strip_work_doubles(N, m, r) : strip_large_work_doubles(N, m, r);
 }
 
-}  // namespace
-}  // namespace bc
-
-using namespace bc;
-
-bc_status bc_strip_workspace(int64_t nsys, int64_t N, int m, int r, int64_t *bytes)
-{
-    if (!bytes || !strip_shape_ok(nsys, N, m, r)) {
-        set_error("bc_strip_workspace: need nsys >= 0, N >= 1, 1 <= m <= 448, 1 <= r <= 32");
-        return BC_ERR_ARG;
-    }
-    *bytes = int64_t(sizeof(double) * strip_scratch_doubles(nsys, N, m, r));
-    return BC_OK;
-}
-
-bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B, const double *C,
-                         const double *b, double *x, void *work, int32_t *status, void *stream)
+bc_status strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B, const double *C,
+                      const double *b, double *x, void *work, int32_t *status, const bc_strip_debug &dbg, void *stream)
 {
     if (!strip_shape_ok(nsys, N, m, r)) {
         set_error("bc_strip_solve: need nsys >= 0, N >= 1, 1 <= m <= 448, 1 <= r <= 32");
@@ -73,7 +58,7 @@ bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A,
         const size_t mm = size_t(m) * m;
         for (int64_t s = 0; s < nsys && e == cudaSuccess; s++)
             e = launch_strip_large(N, m, r, A + s * N * mm, B + s * N * mm, C + s * N * mm, b + s * N * m * r,
-                                   x + s * N * m * r, wk, status ? status + s : nullptr, st);
+                                   x + s * N * m * r, wk, status ? status + s : nullptr, st, dbg);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -81,4 +66,36 @@ bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A,
         return BC_ERR_CUDA;
     }
     return BC_OK;
+}
+
+}  // namespace
+}  // namespace bc
+
+using namespace bc;
+
+bc_status bc_strip_workspace(int64_t nsys, int64_t N, int m, int r, int64_t *bytes)
+{
+    if (!bytes || !strip_shape_ok(nsys, N, m, r)) {
+        set_error("bc_strip_workspace: need nsys >= 0, N >= 1, 1 <= m <= 448, 1 <= r <= 32");
+        return BC_ERR_ARG;
+    }
+    *bytes = int64_t(sizeof(double) * strip_scratch_doubles(nsys, N, m, r));
+    return BC_OK;
+}
+
+bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B, const double *C,
+                         const double *b, double *x, void *work, int32_t *status, void *stream)
+{
+    return strip_solve(nsys, N, m, r, A, B, C, b, x, work, status, bc_strip_debug{}, stream);
+}
+
+bc_status bc_debug_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B,
+                               const double *C, const double *b, double *x, void *work, int32_t *status,
+                               const bc_strip_debug *debug, void *stream)
+{
+    if (!debug || debug->stall_ns < 0 || debug->stall_ns > 1000000) {
+        set_error("bc_debug_strip_solve: need stall_ns in [0, 1000000]");
+        return BC_ERR_ARG;
+    }
+    return strip_solve(nsys, N, m, r, A, B, C, b, x, work, status, *debug, stream);
 }
