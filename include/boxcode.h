@@ -289,7 +289,9 @@ void bc_layer_destroy(bc_layer *layer);
  * bc_strip_workspace() bytes, owned by the caller.  status: NULL or device
  * int32 [nsys], set to 1 where a pivot of the block LU (the diagonal blocks
  * D_0 .. D_{N-2} and the Schur complement of x[N-1] are factored with partial
- * pivoting) was zero or not finite, else 0; no pivoting across blocks, so the systems
+ * pivoting) was zero or not finite, to 2 where a bounded device-side wait of a
+ * large-block solve gave up (its x then holds NaN), else 0; no pivoting across
+ * blocks, so the systems
  * should be block diagonally dominant, as collocation strips with their
  * continuity rows are.  Host pointers: BC_ERR_ARG.  Stream-ordered. */
 bc_status bc_strip_workspace(int64_t nsys, int64_t N, int m, int r, int64_t *bytes);
@@ -297,10 +299,13 @@ bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A,
                          const double *b, double *x, void *work, int32_t *status, void *stream);
 /* Diagnostics: bc_strip_solve with the order of events in the large-block solve
  * (m > 32; smaller blocks: no effect) disturbed.  All zero: as bc_strip_solve.
+ *   wait_polls: polls of a device-side wait without progress (0: 2^22) before the
+ *     solve gives up;
+ *   withhold_panels: no panel is factored, so that the first wait for one runs out;
  *   stall_ns: blocks that own right-hand columns only wait so long (at most 1 ms)
  *     before each factored panel they apply. */
 typedef struct {
-    int32_t stall_ns;
+    int32_t wait_polls, withhold_panels, stall_ns;
 } bc_strip_debug;
 bc_status bc_debug_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B,
                                const double *C, const double *b, double *x, void *work, int32_t *status,

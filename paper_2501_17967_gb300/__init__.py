@@ -55,7 +55,7 @@ class _Stats(ctypes.Structure):
 
 
 class _StripDebug(ctypes.Structure):
-    _fields_ = [("stall_ns", ctypes.c_int32)]
+    _fields_ = [(n, ctypes.c_int32) for n in ("wait_polls", "withhold_panels", "stall_ns")]
 
 
 DENSITY_FN = ctypes.CFUNCTYPE(None, ctypes.POINTER(ctypes.c_double), ctypes.c_int64,
@@ -484,8 +484,9 @@ def strip_solve(A, B, C, b, stream=None, return_status=False, out=None, work=Non
     """Batched strip systems of Sec. 3.3 (block tridiagonal with periodic
     corners): C[k] x[k-1] + A[k] x[k] + B[k] x[k+1] = b[k], indices mod N.
     A, B, C: float64 device tensors [nsys, N, m, m]; b: [nsys, N, m, r].
-    Returns x (and the per-system status if asked: 1 = zero pivot); out, work
-    and status may be passed in."""
+    Returns x (and the per-system status if asked: 1 = zero or non-finite pivot,
+    2 = a device-side wait gave up, x holds NaN); out, work and status may be
+    passed in."""
     import torch
     A, B, C, b = (t.contiguous() for t in (A, B, C, b))
     if b.dim() != 4 or A.shape != B.shape or A.shape != C.shape or A.shape[:3] != b.shape[:3] \

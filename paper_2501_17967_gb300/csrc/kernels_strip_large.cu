@@ -20,8 +20,11 @@
 // products C_k G and the panels' updates of B_k and the right-hand columns, which
 // may lag (F keeps all panels of an element).  F is doubled by the parity of
 // the element.
-// Every wait is bounded: one that runs out raises the abort word, at which all
-// CTAs leave; the status word then says 1.
+// Every wait is bounded by progress: it gives up after kPollLimit polls during which
+// no worker finished an element of the backward sweep (the only phase that a wait
+// spans whole, and one as long as the strip).  A wait that runs out raises the abort
+// word, at which all CTAs leave, the workers with NaN in the solution; the status
+// word then says 2.
 // The paper's strip (N = 56, m = 384, r = 1): 216 ms as some 8,000 launches (panel,
 // exchange, triangular solve and DGEMM kernels, recorded again for new arguments;
 // 170 ms replayed), 55 ms so: per element 0.87 ms, of which the 24 panels take 19 us
@@ -41,11 +44,12 @@ namespace {
 constexpr int kW = 16;         // panel width
 constexpr int kMaxM = 448;
 constexpr int kMaxD = 3, kMaxR = 4;   // columns of a kind per worker (m = 448, r = 32 on 150 workers)
-constexpr int kPollLimit = 1 << 22;
+constexpr int kPollLimit = 1 << 22;   // polls of several hundred cycles: a second or two
 
 // counters in the workspace (zeroed before the launch), 64 bytes apart
-// (kCtrDone: one per parity of the element)
-enum { kCtrPanel = 0, kCtrCols = 16, kCtrInv = 32, kCtrDone = 48, kCtrGrid = 80, kCtrAbort = 96, kCtrWords = 112 };
+// (kCtrDone: one per parity of the element; kCtrBeat: elements that the workers have
+// finished in the backward sweep)
+enum { kCtrPanel = 0, kCtrCols = 16, kCtrInv = 32, kCtrDone = 48, kCtrGrid = 80, kCtrAbort = 96, kCtrBeat = 112, kCtrWords = 128 };
 
 struct LargeArgs {
     int64_t N;
@@ -58,6 +62,8 @@ struct LargeArgs {
     int32_t *perm;             // [2][np][m] row (within the panel's rows) that ends at each position
     uint32_t *ctr;
     int32_t *status;
+    int polls;                 // polls of a wait without progress
+    int withhold;              // diagnostics: the panel CTA factors nothing (the first wait for a panel runs out)
     int stall_ns;              // diagnostics: workers without a matrix column wait so long before each background panel
 };
 
@@ -72,15 +78,26 @@ __device__ __forceinline__ void ctr_add(uint32_t *p, uint32_t n)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(n) : "memory");
 }
 
+// Whether a wait goes on after its poll `it` (reset where the backward sweep has moved).
+__device__ __forceinline__ bool keep_waiting(const LargeArgs &a, int &it, uint32_t &beat)
+{
+    if (++it >= a.polls) {
+        const uint32_t b = ctr_load(a.ctr + kCtrBeat);
+        if (b == beat) return false;
+        beat = b;
+        it = 0;
+    }
+    return (it & 63) != 63 || !ctr_load(a.ctr + kCtrAbort);
+}
+
 // Thread 0 waits until *p >= want; all threads of the CTA get the outcome.
 __device__ bool cta_wait(const LargeArgs &a, int word, uint32_t want, int *s_ok)
 {
     if (threadIdx.x == 0) {
-        int ok = 0;
-        for (int it = 0; it < kPollLimit && !ok; it++) {
-            if (ctr_load(a.ctr + word) >= want) ok = 1;
-            else if ((it & 63) == 63 && ctr_load(a.ctr + kCtrAbort)) break;
-        }
+        int ok = 0, it = 0;
+        uint32_t beat = ctr_load(a.ctr + kCtrBeat);
+        do ok = ctr_load(a.ctr + word) >= want;
+        while (!ok && keep_waiting(a, it, beat));
         if (!ok) atomicExch(a.ctr + kCtrAbort, 1u);
         *s_ok = ok;
     }
@@ -269,13 +286,14 @@ __device__ void panel_cta(const LargeArgs &a, double *Ls)
         for (int p = 0; p < a.np && ok; p++) {
             ok = cta_wait(a, kCtrCols, uint32_t(e * a.m + min(a.m, (p + 1) * kW)), &s_ok);
             if (!ok) break;
+            if (a.withhold) continue;   // diagnostics: the waits for this panel run out
             if ((p + 1) * kW <= a.m) panel_factor<true>(a, F, Li + p * kW * kW, pm + size_t(p) * a.m, p, S, Ls, &s_bad);
             else panel_factor<false>(a, F, Li + p * kW * kW, pm + size_t(p) * a.m, p, S, Ls, &s_bad);
             cta_signal(a, kCtrPanel, 1);
         }
     }
     if (ok) ok = grid_barrier(a, phase, &s_ok);
-    if (threadIdx.x == 0) *a.status = (s_bad || !ok || ctr_load(a.ctr + kCtrAbort)) ? 1 : 0;
+    if (threadIdx.x == 0) *a.status = !ok || ctr_load(a.ctr + kCtrAbort) ? 2 : s_bad ? 1 : 0;
 }
 
 // The helper CTA: the inverse of each published panel's upper diagonal block
@@ -524,7 +542,8 @@ __device__ void back_substitute(const LargeArgs &a, const double *F, const doubl
     }
 }
 
-__device__ void worker_cta(const LargeArgs &a, double *sh)
+// false: a wait ran out
+__device__ bool worker_cta(const LargeArgs &a, double *sh)
 {
     __shared__ WorkShared S;
     const int m = a.m, r = a.r, R = a.R, np = a.np, t = threadIdx.x, w = int(blockIdx.x) - 2;
@@ -620,12 +639,9 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
                 pB++;
                 idle = 0;
             } else {
-                if (t == 0) {
-                    S.ok = 1;
-                    if (++idle >= kPollLimit || ((idle & 63) == 63 && ctr_load(a.ctr + kCtrAbort))) {
-                        atomicExch(a.ctr + kCtrAbort, 1u);
-                        S.ok = 0;
-                    }
+                if (t == 0) {   // (no backward sweep runs beside a factorization: nothing resets this one)
+                    S.ok = ++idle < a.polls && ((idle & 63) != 63 || !ctr_load(a.ctr + kCtrAbort));
+                    if (!S.ok) atomicExch(a.ctr + kCtrAbort, 1u);
                 }
                 __syncthreads();
                 const bool go = S.ok != 0;
@@ -664,9 +680,9 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
             for (int k = t; k < m; k += blockDim.x) a.G[(size_t(e) * R + wr + i * a.nw) * m + k] = now[i * m + k];
         cur ^= 1;
     }
-    if (!ok) return;
+    if (!ok) return false;
     if (Nt > 0) {
-        if (!grid_barrier(a, phase, &S.ok)) return;   // every H is written
+        if (!grid_barrier(a, phase, &S.ok)) return false;   // every H is written
         // ---- backward: X_k = G_k - H_k X_{k+1}, thread t row t; sixteen columns
         // of H_k at a time, the next sixteen on their way
         for (int64_t k = Nt - 2; k >= 0; k--) {
@@ -696,8 +712,9 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
             });
             cur ^= 1;
             __syncthreads();
+            if (t == 0) asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(a.ctr + kCtrBeat) : "memory");
         }
-        if (!grid_barrier(a, phase, &S.ok)) return;   // every X is written
+        if (!grid_barrier(a, phase, &S.ok)) return false;   // every X is written
     }
     // ---- border: S = A - B Z_0 - C Z_{N-2} (N = 1: A + B + C) in D, s likewise in
     // R0 (own right-hand columns below r); H and R1 hold the columns of Z and Y
@@ -724,10 +741,10 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
         __syncthreads();
     }
     ok = factor(Nt, R0, nS, nullptr, nullptr, nullptr);
-    if (!ok) return;
+    if (!ok) return false;
     for (int i = 0; i < nS; i++)
         for (int k = t; k < m; k += blockDim.x) a.x[(size_t(Nt) * m + k) * r + wr + i * a.nw] = R0[i * m + k];
-    if (!grid_barrier(a, phase, &S.ok)) return;   // x_{N-1} is written
+    if (!grid_barrier(a, phase, &S.ok)) return false;   // x_{N-1} is written
     // ---- x_k = Y_k - Z_k x_{N-1}: element and right-hand side per pass, thread t row t
     for (int64_t job = w; job < Nt * r; job += a.nw) {
         const int64_t k = job / r;
@@ -746,6 +763,7 @@ __device__ void worker_cta(const LargeArgs &a, double *sh)
         }
         __syncthreads();
     }
+    return true;
 }
 
 __global__ void __launch_bounds__(512, 1) k_strip_large(const __grid_constant__ LargeArgs a)
@@ -753,7 +771,12 @@ __global__ void __launch_bounds__(512, 1) k_strip_large(const __grid_constant__ 
     extern __shared__ double sh[];
     if (blockIdx.x == 0) panel_cta(a, sh);
     else if (blockIdx.x == 1) helper_cta(a);
-    else worker_cta(a, sh);
+    else if (!worker_cta(a, sh)) {
+        // nothing of an unfinished solution passes for one
+        const int64_t n = a.N * a.m * a.r;
+        for (int64_t i = (int64_t(blockIdx.x) - 2) * blockDim.x + threadIdx.x; i < n; i += int64_t(a.nw) * blockDim.x)
+            a.x[i] = nan("");
+    }
 }
 
 int strip_panels(int m) { return (m + kW - 1) / kW; }
@@ -800,6 +823,8 @@ cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const d
     a.perm = reinterpret_cast<int32_t *>(w); w += size_t(a.np) * m;
     a.ctr = reinterpret_cast<uint32_t *>(w); w += kCtrWords / 2;
     a.status = status ? status : reinterpret_cast<int32_t *>(w);
+    a.polls = dbg.wait_polls > 0 ? dbg.wait_polls : kPollLimit;
+    a.withhold = dbg.withhold_panels;
     a.stall_ns = dbg.stall_ns;
     e = cudaMemsetAsync(a.ctr, 0, kCtrWords * sizeof(uint32_t), st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_strip_large, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));

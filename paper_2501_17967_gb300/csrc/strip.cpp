@@ -93,8 +93,8 @@ bc_status bc_debug_strip_solve(int64_t nsys, int64_t N, int m, int r, const doub
                                const double *C, const double *b, double *x, void *work, int32_t *status,
                                const bc_strip_debug *debug, void *stream)
 {
-    if (!debug || debug->stall_ns < 0 || debug->stall_ns > 1000000) {
-        set_error("bc_debug_strip_solve: need stall_ns in [0, 1000000]");
+    if (!debug || debug->wait_polls < 0 || debug->wait_polls > (1 << 22) || debug->stall_ns < 0 || debug->stall_ns > 1000000) {
+        set_error("bc_debug_strip_solve: need wait_polls in [0, 2^22], stall_ns in [0, 1000000]");
         return BC_ERR_ARG;
     }
     return strip_solve(nsys, N, m, r, A, B, C, b, x, work, status, *debug, stream);

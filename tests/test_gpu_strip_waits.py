@@ -39,3 +39,23 @@ def test_blocks_without_a_matrix_column_may_lag(N, m, r):
     want = bc.strip_solve(*args)
     x, status = debug_solve(*args, stall_ns=300000)
     assert status == [0] and torch.equal(x, want)
+
+
+@pytest.mark.parametrize("N,m,r", [(1, 40, 2), (3, 48, 1), (2, 150, 3)])
+def test_a_wait_that_runs_out(N, m, r):
+    """A panel that never comes: every block leaves, the status says 2, no number passes for a solution, and the next
+    solve is sound."""
+    args = system(2, N, m, r)
+    x, status = debug_solve(*args, wait_polls=2000, withhold_panels=1)
+    assert status == [2, 2] and torch.isnan(x).all()
+    want, st = bc.strip_solve(*args, return_status=True)
+    assert st.cpu().tolist() == [0, 0] and torch.isfinite(want).all()
+
+
+def test_a_long_strip_outlasts_the_polls():
+    """The panel block waits through the whole backward sweep: a limit that covers some hundred elements (4,000 polls of
+    about 0.4 us) does not end a sweep of 6,000 (10 us or so each, as long as the sweep moves)."""
+    args = system(1, 6000, 33, 1)
+    want = bc.strip_solve(*args)
+    x, status = debug_solve(*args, wait_polls=4000)
+    assert status == [0] and torch.equal(x, want)
