@@ -67,6 +67,8 @@ struct Walk {
     }
 };
 
+constexpr int kMaxM = 32, kMaxR = 32;   // largest block and number of right-hand sides
+
 struct StripPivot {
     int row, bad;
     double inv;
@@ -341,7 +343,10 @@ cudaError_t launch_strip(int64_t nsys, int64_t N, int m, int r, const double *A,
                          const double *b, double *x, double *work, int32_t *status, cudaStream_t st)
 {
     const size_t sm = strip_smem_bytes(m, r);
-    const cudaError_t ce = cudaFuncSetAttribute(k_strip_small, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+    // the limit of the largest shape in every call: it belongs to the kernel, and a
+    // smaller one would fail another thread's launch
+    const cudaError_t ce = cudaFuncSetAttribute(k_strip_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                int(strip_smem_bytes(kMaxM, kMaxR)));
     if (ce != cudaSuccess) return ce;
     // Warps per system, by the entries of the augmented block and the systems an
     // SM gets.  Measured (ms at 1 / 2 / 4 / 8 warps): m = 8, 608 systems 4.8 / 3.9 /

@@ -781,6 +781,9 @@ __global__ void __launch_bounds__(512, 1) k_strip_large(const __grid_constant__ 
 
 int strip_panels(int m) { return (m + kW - 1) / kW; }
 
+// What a launch may ask for.  The limit belongs to the kernel, not to the launch, so
+// every call sets this one: a smaller one would fail another thread's launch.
+constexpr size_t kMaxSmem = 200 * 1024;
 size_t large_smem(int m, int r, int nw)
 {
     const size_t nD = size_t(m + nw - 1) / nw, nR = size_t(m + r + nw - 1) / nw;
@@ -811,7 +814,7 @@ cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const d
     a.nw = std::min(sms - 2, m + r);
     const int nD = (m + a.nw - 1) / std::max(a.nw, 1), nR = (a.R + a.nw - 1) / std::max(a.nw, 1);
     const size_t smem = large_smem(m, r, std::max(a.nw, 1));
-    if (a.nw < kW || nD > kMaxD || nR > kMaxR || smem > 200 * 1024) return cudaErrorInvalidConfiguration;
+    if (a.nw < kW || nD > kMaxD || nR > kMaxR || smem > kMaxSmem) return cudaErrorInvalidConfiguration;
     a.A = A; a.B = B; a.C = C; a.b = b; a.x = x;
     const size_t nt = size_t(std::max<int64_t>(N - 1, 1));
     double *w = work;
@@ -827,7 +830,7 @@ cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const d
     a.withhold = dbg.withhold_panels;
     a.stall_ns = dbg.stall_ns;
     e = cudaMemsetAsync(a.ctr, 0, kCtrWords * sizeof(uint32_t), st);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_strip_large, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_strip_large, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMaxSmem));
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_strip_large), dim3(unsigned(a.nw + 2)),

@@ -59,3 +59,33 @@ def test_a_long_strip_outlasts_the_polls():
     want = bc.strip_solve(*args)
     x, status = debug_solve(*args, wait_polls=4000)
     assert status == [0] and torch.equal(x, want)
+
+
+@pytest.mark.parametrize("big,small", [((1, 3, 448, 32), (1, 3, 33, 1)), ((2, 3, 32, 32), (2, 3, 30, 1))])
+def test_shapes_from_two_threads(big, small):
+    """Solves that want much and little shared memory, from two threads at once: every launch is accepted."""
+    import threading
+    args = [system(*s) for s in (big, small)]
+    want = [bc.strip_solve(*a) for a in args]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(i):
+        try:
+            st, out = torch.cuda.Stream(), torch.empty_like(want[i])
+            mem = bc.strip_workspace(*args[i][3].shape, "cuda")
+            status = torch.zeros(len(out), dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            for _ in range(300):
+                bc.strip_solve(*args[i], out=out, work=mem, status=status, stream=st)
+            st.synchronize()
+            assert torch.equal(out, want[i])
+        except Exception as e:
+            failed.append(e)
+
+    th = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not failed, failed
