@@ -89,3 +89,18 @@ def test_shapes_from_two_threads(big, small):
     for t in th:
         t.join()
     assert not failed, failed
+
+
+def test_memory_of_a_solve_on_another_stream():
+    """What strip_solve allocates for itself is not handed out again while the solve runs on the caller's stream."""
+    args = system(1, 8, 100, 1)
+    want = bc.strip_solve(*args)
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    for _ in range(20):
+        out = torch.empty_like(want)
+        x, status = bc.strip_solve(*args, out=out, stream=st, return_status=True)
+        junk = [torch.full((n,), float("nan"), device="cuda", dtype=torch.float64) for n in (64, 1 << 12, 1 << 16, 1 << 18)]
+        del junk
+        st.synchronize()
+        assert torch.equal(x, want) and status.cpu().tolist() == [0]
