@@ -802,6 +802,7 @@ bc_status build_split_tables(bc_ctx *ctx)
     if (s == BC_OK) s = build_digit_tables(ctx, ctx->wide, kWideSlices, &ctx->wide_ready);
     if (s != BC_OK) return s;
     cudaError_t e = split_prepare();
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->setup, cudaStreamNonBlocking);
     return e == cudaSuccess ? BC_OK : cuda_fail(e, "split kernel attributes");
 }
 
@@ -883,7 +884,7 @@ cudaError_t build_tile_order(bc_tree *t)
     up.add(&o.w, w);
     up.add(&o.v, v);
     up.add(&o.l2p, l2p);
-    const cudaError_t e = up.commit(t->d.allocs, t->side.side);
+    const cudaError_t e = up.commit(t->d.allocs, t->ctx->setup);
     o.ready = e == cudaSuccess;
     return e;
 }
@@ -966,7 +967,7 @@ try {
         if (!Pv) up.room(&Pv, size_t(nv) * P1);
         for (int dir = 0; dir < 2; dir++) up.room(&n.cM[dir], size_t(nv));
     }
-    if ((e = up.commit(t->d.allocs, t->side.side)) != cudaSuccess) return e;
+    if ((e = up.commit(t->d.allocs, t->ctx->setup)) != cudaSuccess) return e;
     ColLists cl;
     cl.nleaf = h.nleaf;
     cl.near_ptr = t->d.near_ptr; cl.near_src = t->d.near_src;
@@ -991,8 +992,8 @@ try {
         }
         if (m2l) seg(ColKind::V, dir, nv, o.v, n.cM[dir], reinterpret_cast<double *>(Pv), 2 * P1, f0);
     }
-    e = launch_make_cols(cl, t->side.side);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(t->side.side);
+    e = launch_make_cols(cl, t->ctx->setup);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(t->ctx->setup);
     if (e != cudaSuccess) {
         cudaFree(t->d.allocs.back());
         t->d.allocs.pop_back();
@@ -1029,7 +1030,8 @@ bc_status build_split_m2l(bc_tree *t)
 // 7-digit tiles of the FP64 mode, on first use.  They take device memory that
 // the FP64 kernels do not need; where that is not to be had the FP64 kernels
 // serve (and are asked for again only with another tree).  The set-up runs on
-// the tree's own stream, so it neither joins nor breaks a stream capture.
+// the context's set-up stream, which no apply uses (the tree's internal stream may be
+// part of the caller's capture), so it neither joins nor breaks a stream capture.
 bool build_wide_tree(bc_tree *t)
 {
     if (t->wide_ready) return true;
@@ -1040,7 +1042,7 @@ bool build_wide_tree(bc_tree *t)
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        t->wide_off = true;
+        t->wide_off = e == cudaErrorMemoryAllocation;
         return false;
     }
     t->wide_ready = true;
@@ -1195,8 +1197,8 @@ try {
     up.room(&n.cE[0], leaves.size());
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    cudaError_t e = ensure_side(t);
-    if (e == cudaSuccess && (e = up.commit(t->d.allocs, t->side.side)) == cudaSuccess) {
+    cudaError_t e = up.commit(t->d.allocs, t->ctx->setup);
+    if (e == cudaSuccess) {
         ColLists cl;
         cl.nleaf = h.nleaf;
         cl.leaf_level = t->d.leaf_level;
@@ -1204,8 +1206,8 @@ try {
         cl.box_level = t->d.box_level;
         if (!leaves.empty())
             cl.seg[cl.nseg++] = ColSeg{ColKind::L2P, 0, int64_t(leaves.size()), perm, n.cE[0], n.PE, int64_t(T.np), nbox};
-        if (cl.nseg) e = launch_make_cols(cl, t->side.side);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(t->side.side);
+        if (cl.nseg) e = launch_make_cols(cl, t->ctx->setup);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(t->ctx->setup);
         if (e != cudaSuccess) {
             cudaFree(t->d.allocs.back());
             t->d.allocs.pop_back();
@@ -1357,6 +1359,7 @@ void bc_destroy(bc_ctx *ctx)
     for (auto &dir : ctx->ev)
         for (auto &e : dir)
             if (e) cudaEventDestroy(e);
+    if (ctx->setup) cudaStreamDestroy(ctx->setup);
     free_all(ctx->dt.allocs);
     free_all(ctx->split_allocs);
     delete ctx;

@@ -527,6 +527,7 @@ struct bc_ctx {
     bc::DevTables dt;
     bc::SplitTables split, wide;   // 5-digit (split modes) and 7-digit (FP64 mode) operators
     std::vector<void *> split_allocs;
+    cudaStream_t setup = nullptr;   // set-up of trees' tiles; never part of an apply or a capture
     bool split_ready = false, wide_ready = false;
     int32_t *dev_err = nullptr;   // device flag set by kernels whose bounded waits gave up
     int up_blocks = 0, shift_blocks = 0, down_blocks = 0;   // grids of the persistent passes

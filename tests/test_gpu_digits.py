@@ -139,6 +139,38 @@ def test_first_apply_inside_a_capture():
     assert relerr(y, want) <= BAR
 
 
+@pytest.mark.parametrize("first", ["fp64", "split", "layer"])
+def test_first_use_of_the_tiles_later_in_a_capture(first):
+    """The 7-digit tiles of a tree made while its internal stream is part of the capture, by an earlier apply (of
+    the all-tensor mode, which does not use them)."""
+    tree, x = make(16, 24, max_level=5)
+    y, z, src = torch.zeros_like(x), torch.zeros_like(x), torch.zeros_like(x)
+    bc.apply(tree, x, out=y, precision=bc.SPLIT_BF16_ALL)
+    if first == "split":       # the 5-digit tiles exist, the 7-digit M2L's do not
+        fn = lambda t, v, out: bc.apply(t, v, out=out, precision=bc.SPLIT_BF16)   # noqa: E731
+    elif first == "layer":
+        curve = np.stack([0.5 * np.cos(np.arange(100)), 0.5 * np.sin(np.arange(100))], 1)
+        m = torch.zeros(100, 2, device="cuda", dtype=torch.float64)
+        fn = lambda t, v, out: layers[id(t)].apply(v.reshape(-1)[:100], m, out=out.reshape(-1))   # noqa: E731
+        layers = {id(tree): bc.Layer(tree, curve)}
+    else:
+        fn = lambda t, v, out: bc.apply(t, v, out=out)   # noqa: E731
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        bc.apply(tree, src, out=y, precision=bc.SPLIT_BF16_ALL)
+        fn(tree, src, z)
+    src.copy_(x)
+    g.replay()
+    torch.cuda.synchronize()
+    want = torch.empty_like(x)
+    assert torch.equal(y, bc.apply(tree, x, precision=bc.SPLIT_BF16_ALL))
+    fn(tree, x, want)
+    assert torch.equal(z, want)
+    if first == "fp64":        # by the digits, not by the kernels that serve where they do not fit
+        assert not torch.equal(z, kernels(tree, x, False)) and relerr(z, kernels(tree, x, False)) <= BAR
+
+
 def test_trees_on_their_own_streams():
     """Applies of different trees of one context, from several threads and streams at once."""
     import threading
