@@ -285,7 +285,8 @@ void bc_layer_destroy(bc_layer *layer);
  * cooperative launch over the whole GPU (all its SMs: a solve on another stream
  * waits).  Layout, all FP64 row-major device arrays: A, B,
  * C [nsys][N][m][m]; b, x [nsys][N][m][r].  Shapes: N >= 1, 1 <= m <= 448,
- * 1 <= r <= 32.  work: device scratch of
+ * 1 <= r <= 32 (large blocks on fewer than 122 SMs: BC_ERR_UNSUPPORTED where a
+ * block's columns are too many for them).  work: device scratch of
  * bc_strip_workspace() bytes, owned by the caller.  status: NULL or device
  * int32 [nsys], set to 1 where a pivot of the block LU (the diagonal blocks
  * D_0 .. D_{N-2} and the Schur complement of x[N-1] are factored with partial
@@ -303,9 +304,10 @@ bc_status bc_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A,
  *     solve gives up;
  *   withhold_panels: no panel is factored, so that the first wait for one runs out;
  *   stall_ns: blocks that own right-hand columns only wait so long (at most 1 ms)
- *     before each factored panel they apply. */
+ *     before each factored panel they apply;
+ *   max_blocks: at most so many blocks, as on a part with so many SMs (0: all). */
 typedef struct {
-    int32_t wait_polls, withhold_panels, stall_ns;
+    int32_t wait_polls, withhold_panels, stall_ns, max_blocks;
 } bc_strip_debug;
 bc_status bc_debug_strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, const double *B,
                                const double *C, const double *b, double *x, void *work, int32_t *status,

@@ -55,7 +55,7 @@ class _Stats(ctypes.Structure):
 
 
 class _StripDebug(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_int32) for n in ("wait_polls", "withhold_panels", "stall_ns")]
+    _fields_ = [(n, ctypes.c_int32) for n in ("wait_polls", "withhold_panels", "stall_ns", "max_blocks")]
 
 
 DENSITY_FN = ctypes.CFUNCTYPE(None, ctypes.POINTER(ctypes.c_double), ctypes.c_int64,

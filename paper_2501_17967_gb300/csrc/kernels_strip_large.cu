@@ -43,7 +43,9 @@ namespace {
 
 constexpr int kW = 16;         // panel width
 constexpr int kMaxM = 448;
-constexpr int kMaxD = 3, kMaxR = 4;   // columns of a kind per worker (m = 448, r = 32 on 150 workers)
+// columns of a kind per worker: three and four for m = 448, r = 32 on 150 workers,
+// four of each from 120 workers on
+constexpr int kMaxD = 4, kMaxR = 4;
 constexpr int kPollLimit = 1 << 22;   // polls of several hundred cycles: a second or two
 
 // counters in the workspace (zeroed before the launch), 64 bytes apart
@@ -358,7 +360,7 @@ struct WorkShared {
 template <class F>
 __device__ __forceinline__ void with_count(int n, F &&f)   // f of an integral constant
 {
-    static_assert(kMaxD + kMaxR == 7, "cases below");
+    static_assert(kMaxD + kMaxR == 8, "cases below");
     switch (n) {
     case 1: f(std::integral_constant<int, 1>()); break;
     case 2: f(std::integral_constant<int, 2>()); break;
@@ -367,6 +369,7 @@ __device__ __forceinline__ void with_count(int n, F &&f)   // f of an integral c
     case 5: f(std::integral_constant<int, 5>()); break;
     case 6: f(std::integral_constant<int, 6>()); break;
     case 7: f(std::integral_constant<int, 7>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
     default: break;
     }
 }
@@ -812,9 +815,10 @@ cudaError_t launch_strip_large(int64_t N, int m, int r, const double *A, const d
     a.np = strip_panels(m);
     // one CTA per SM; no more workers than there are columns of the larger kind
     a.nw = std::min(sms - 2, m + r);
+    if (dbg.max_blocks > 0) a.nw = std::min(a.nw, dbg.max_blocks - 2);
     const int nD = (m + a.nw - 1) / std::max(a.nw, 1), nR = (a.R + a.nw - 1) / std::max(a.nw, 1);
     const size_t smem = large_smem(m, r, std::max(a.nw, 1));
-    if (a.nw < kW || nD > kMaxD || nR > kMaxR || smem > kMaxSmem) return cudaErrorInvalidConfiguration;
+    if (a.nw < kW || nD > kMaxD || nR > kMaxR || smem > kMaxSmem) return cudaErrorNotSupported;
     a.A = A; a.B = B; a.C = C; a.b = b; a.x = x;
     const size_t nt = size_t(std::max<int64_t>(N - 1, 1));
     double *w = work;

@@ -60,6 +60,10 @@ bc_status strip_solve(int64_t nsys, int64_t N, int m, int r, const double *A, co
             e = launch_strip_large(N, m, r, A + s * N * mm, B + s * N * mm, C + s * N * mm, b + s * N * m * r,
                                    x + s * N * m * r, wk, status ? status + s : nullptr, st, dbg);
     }
+    if (e == cudaErrorNotSupported) {
+        set_error("bc_strip_solve: blocks of m = %d with r = %d need more SMs than there are (122 for every m and r)", m, r);
+        return BC_ERR_UNSUPPORTED;
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("bc_strip_solve: %s (%s)", cudaGetErrorName(e), cudaGetErrorString(e));
@@ -93,8 +97,8 @@ bc_status bc_debug_strip_solve(int64_t nsys, int64_t N, int m, int r, const doub
                                const double *C, const double *b, double *x, void *work, int32_t *status,
                                const bc_strip_debug *debug, void *stream)
 {
-    if (!debug || debug->wait_polls < 0 || debug->wait_polls > (1 << 22) || debug->stall_ns < 0 || debug->stall_ns > 1000000) {
-        set_error("bc_debug_strip_solve: need wait_polls in [0, 2^22], stall_ns in [0, 1000000]");
+    if (!debug || debug->wait_polls < 0 || debug->wait_polls > (1 << 22) || debug->stall_ns < 0 || debug->stall_ns > 1000000 || debug->max_blocks < 0) {
+        set_error("bc_debug_strip_solve: need wait_polls in [0, 2^22], stall_ns in [0, 1000000], max_blocks >= 0");
         return BC_ERR_ARG;
     }
     return strip_solve(nsys, N, m, r, A, B, C, b, x, work, status, *debug, stream);

@@ -104,3 +104,15 @@ def test_memory_of_a_solve_on_another_stream():
         del junk
         st.synchronize()
         assert torch.equal(x, want) and status.cpu().tolist() == [0]
+
+
+@pytest.mark.parametrize("blocks,m,r", [(148, 448, 32), (148, 439, 1), (122, 448, 32), (132, 391, 5)])
+def test_the_whole_range_on_fewer_blocks(blocks, m, r):
+    """Four columns of a kind per block, as on a part with fewer SMs: every documented shape from 122 blocks on."""
+    args = system(1, 3, m, r)
+    want = bc.strip_solve(*args)
+    x, status = debug_solve(*args, max_blocks=blocks)
+    assert status == [0] and (x - want).abs().max() <= 1e-12 * want.abs().max()
+    with pytest.raises(bc.BoxCodeError) as e:
+        debug_solve(*args, max_blocks=80)
+    assert e.value.status == -6
