@@ -743,6 +743,11 @@ def main():
             line[pname[other]] = {"value": world * N / (ms_o * 1e-3), "ms_per_step": ms_o, "dtype": DTYPES[other],
                                   "roofline": dominant(ps),
                                   "stage_ms": {k: v["ms"] for k, v in ps.items()}}
+        # every step in native FP64 (option fp64_native)
+        ctx.set_option("fp64_native", 1)
+        ms_n, _ = run.timed(bc.FP64, max(3, args.steps // 4), args.warmup, stages=False)
+        ctx.set_option("fp64_native", 0)
+        line["fp64_native"] = {"value": world * N / (ms_n * 1e-3), "ms_per_step": ms_n, "dtype": "f64"}
         # the 20-Gaussian workload in the headline precision
         if args.workload != "adaptive20":
             g2 = density("adaptive20")

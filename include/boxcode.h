@@ -70,10 +70,12 @@ typedef enum {
                               multipole-to-local translations) on 7 digits,
                               vectors with an infinity or a NaN in FP64; the
                               M2M and L2L shifts, the log terms and all sums in
-                              native FP64.  Trees whose tiles do not fit in
-                              device memory, and the options m2l_triangular and
-                              m2l_kernel (M2L only), take the native FP64
-                              kernels, as bc_apply_noalloc does (every p) */
+                              native FP64.  The tiles of a tree take device
+                              memory from its first such apply to its end (about
+                              44 KB per leaf at p = 16); where they do not fit,
+                              with the option fp64_native, and (M2L only) with
+                              m2l_triangular and m2l_kernel, every step is in
+                              native FP64, as in bc_apply_noalloc (every p) */
     BC_SPLIT_BF16 = 1,     /* 5 digits for the fixed-operator products: the
                               near-field tables, P2M, L2P, the W list (M2P) and
                               the X list (P2L), and their adjoints.  The rest as
@@ -355,9 +357,13 @@ bc_status bc_table_export(const bc_ctx *ctx, int which, int64_t *count, double *
  *   "m2l_triangular" (0/1, default 0): keep only the terms with k + l <= P of
  *     each multipole-to-local translation (and exactly their transpose in the
  *     adjoint), which halves the M2L arithmetic but loses accuracy.
+ *   "fp64_native" (0/1, default 0): 1 keeps BC_FP64 (applies, batches captured
+ *     from then on, layers) and BC_SPLIT_BF16's multipole-to-local translations
+ *     in native FP64, without 7-digit tiles and their memory (set it before a
+ *     tree's first apply: tiles that are there stay).
  *   "m2l_kernel" (0/1, default 0): the native FP64 multipole-to-local kernel
  *     (where the translations are not digit products: bc_apply_noalloc, layers,
- *     m2l_triangular, trees whose tiles do not fit): 0 FP64
+ *     fp64_native, m2l_triangular, trees whose tiles do not fit): 0 FP64
  *     FMAs, one block per target box; 1, for every FP64 translation, the FP64 tensor cores (mma.sync f64
  *     tiles of the binomial matrix), one warp per target box.  Same results
  *     to rounding.

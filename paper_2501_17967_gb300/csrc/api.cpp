@@ -1034,6 +1034,7 @@ bc_status build_split_m2l(bc_tree *t)
 // part of the caller's capture), so it neither joins nor breaks a stream capture.
 bool build_wide_tree(bc_tree *t)
 {
+    if (t->ctx->fp64_native) return false;
     if (t->wide_ready) return true;
     if (t->wide_off || !t->ctx->wide_ready) return false;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -1174,6 +1175,7 @@ bc_status prepare_split_tree(bc_tree *t) { return build_split_tree(t); }
 // nullptr: they do not fit.
 const SplitTree *prepare_wide_l2p(bc_tree *t)
 try {
+    if (t->ctx->fp64_native) return nullptr;
     if (t->wide_ready) return &t->spw;
     if (t->spl.PE) return &t->spl;
     if (t->wide_off || !t->ctx->wide_ready) return nullptr;
@@ -1963,6 +1965,14 @@ bc_status bc_set_option(bc_ctx *ctx, const char *name, double value)
             return BC_ERR_ARG;
         }
         ctx->overlap_ctas = int(value);
+        return BC_OK;
+    }
+    if (std::strcmp(name, "fp64_native") == 0) {
+        if (value != 0.0 && value != 1.0) {
+            set_error("bc_set_option: fp64_native must be 0 (7-digit products) or 1 (FP64 kernels)");
+            return BC_ERR_ARG;
+        }
+        ctx->fp64_native = value != 0.0;
         return BC_OK;
     }
     if (std::strcmp(name, "m2l_kernel") == 0) {

@@ -520,6 +520,7 @@ struct bc_ctx {
     int split_overlap = 1;      // near-field tensor launch on the side stream (1) or inline (0)
     int overlap_ctas = 0;       // CTAs of that launch (0: by arrangement, see near_ctas_for)
     int m2l_bps = 0;            // resident blocks per SM of the FP64 M2L kernel (0: by arrangement)
+    bool fp64_native = false;   // FP64 products on the FP64 kernels, not on 7 digits
     int m2l_kind = 0;           // FP64 M2L kernel: 0 FMA, 1 tensor-core MMA (see PassArgs)
     bool timing = false;        // record CUDA events around each stage
     cudaEvent_t ev[2][bc::kNumEvents] = {};   // [forward, adjoint]

@@ -196,3 +196,31 @@ def test_trees_on_their_own_streams():
     for w, o in zip(want, outs):
         assert torch.equal(w, o)
     assert np.isfinite(relerr(outs[0], want[0]))
+
+
+@pytest.mark.parametrize("p", [7, 16])
+def test_native_fp64_on_request(p):
+    """fp64_native: BC_FP64 on the FP64 kernels alone, bit for bit bc_apply_noalloc, without the tiles' memory."""
+    tree, x = make(p, 30)
+    tree.ctx.set_option("fp64_native", 1)
+    for adjoint in (False, True):
+        assert torch.equal(digits(tree, x, adjoint), kernels(tree, x, adjoint))
+    batch = bc.Batch(tree.ctx, [tree, tree])
+    outs = [torch.empty_like(x) for _ in range(2)]
+    batch.run([x, x], outs)
+    assert torch.equal(outs[0], kernels(tree, x, False)) and torch.equal(outs[1], outs[0])
+    curve = np.stack([0.5 * np.cos(np.arange(200)), 0.5 * np.sin(np.arange(200))], 1)
+    layer, q, m = bc.Layer(tree, curve), x.reshape(-1)[:200], x.reshape(-1)[200:600].reshape(200, 2)
+    native = layer.apply(q, m)
+    batch.close()
+    split = bc.apply(tree, x, precision=bc.SPLIT_BF16) if p == 16 else None   # its M2L follows: no 7-digit tiles
+    free = torch.cuda.mem_get_info()[0]
+    tree.ctx.set_option("fp64_native", 0)
+    if p == 16:
+        assert relerr(bc.apply(tree, x, precision=bc.SPLIT_BF16), split) <= 1e-10
+        assert torch.cuda.mem_get_info()[0] < free
+    u = digits(tree, x, False)
+    assert not torch.equal(u, kernels(tree, x, False)) and relerr(u, kernels(tree, x, False)) <= BAR
+    assert relerr(layer.apply(q, m), native) <= BAR
+    with pytest.raises(bc.BoxCodeError):
+        tree.ctx.set_option("fp64_native", 2)
