@@ -799,8 +799,15 @@ bc_status build_split_tables(bc_ctx *ctx)
     if (ctx->device < 0 || 2 * ctx->P1 > kSplitKE) return BC_OK;
     bc_status s = BC_OK;
     if (ctx->p == 8 || ctx->p == 12 || ctx->p == 16) s = build_digit_tables(ctx, ctx->split, kSplitSlices, &ctx->split_ready);
-    if (s == BC_OK) s = build_digit_tables(ctx, ctx->wide, kWideSlices, &ctx->wide_ready);
     if (s != BC_OK) return s;
+    // the FP64 mode does not depend on its digits: where they don't fit, the FP64 kernels serve
+    try {
+        s = build_digit_tables(ctx, ctx->wide, kWideSlices, &ctx->wide_ready);
+    } catch (const std::bad_alloc &) {
+        s = BC_ERR_OOM;
+    }
+    if (s != BC_OK && s != BC_ERR_OOM) return s;
+    cudaGetLastError();
     cudaError_t e = split_prepare();
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->setup, cudaStreamNonBlocking);
     return e == cudaSuccess ? BC_OK : cuda_fail(e, "split kernel attributes");
