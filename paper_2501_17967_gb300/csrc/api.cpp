@@ -607,10 +607,12 @@ struct DevArena {
             total += std::max<size_t>((it.bytes + 255) & ~size_t(255), 256);
             if (it.src) up = total;
         }
+        // what may throw comes before anything is held
+        std::vector<uint8_t> host(up);
+        allocs.reserve(allocs.size() + 1);
         void *base = nullptr;
         cudaError_t e = cudaMalloc(&base, std::max<size_t>(total, 256));
         if (e != cudaSuccess) return e;
-        std::vector<uint8_t> host(up);
         for (size_t i = 0; i < items.size(); i++)
             if (items[i].src && items[i].bytes) std::memcpy(host.data() + off[i], items[i].src, items[i].bytes);
         if (up) e = cudaMemcpyAsync(base, host.data(), up, cudaMemcpyHostToDevice, st);
@@ -1034,6 +1036,26 @@ bc_status build_split_m2l(bc_tree *t)
     return BC_OK;
 }
 
+// Allocations and copies of a set-up are allowed while some stream of the caller's is
+// being captured; the thread's mode is put back at the end, also past an exception.
+class RelaxedCapture {
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+    const bool ok_;
+
+public:
+    RelaxedCapture() : ok_(cudaThreadExchangeStreamCaptureMode(&mode_) == cudaSuccess)
+    {
+        if (!ok_) cudaGetLastError();
+    }
+    ~RelaxedCapture()
+    {
+        if (ok_) cudaThreadExchangeStreamCaptureMode(&mode_);
+    }
+    RelaxedCapture(const RelaxedCapture &) = delete;
+    RelaxedCapture &operator=(const RelaxedCapture &) = delete;
+    bool ok() const { return ok_; }
+};
+
 // 7-digit tiles of the FP64 mode, on first use.  They take device memory that
 // the FP64 kernels do not need; where that is not to be had the FP64 kernels
 // serve (and are asked for again only with another tree).  The set-up runs on
@@ -1044,10 +1066,9 @@ bool build_wide_tree(bc_tree *t)
     if (t->ctx->fp64_native) return false;
     if (t->wide_ready) return true;
     if (t->wide_off || !t->ctx->wide_ready) return false;
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return false; }
+    const RelaxedCapture relaxed;
+    if (!relaxed.ok()) return false;
     const cudaError_t e = build_digit_tree(t, t->ctx->wide, t->spw, true);
-    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
         cudaGetLastError();
         t->wide_off = e == cudaErrorMemoryAllocation;
@@ -1204,8 +1225,8 @@ try {
     up.room(&n.edig, size_t(2 * nbox) * T.slices * kSplitKE);
     up.room(&n.eexp, size_t(2 * nbox));
     up.room(&n.cE[0], leaves.size());
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    const RelaxedCapture relaxed;
+    if (!relaxed.ok()) return nullptr;
     cudaError_t e = up.commit(t->d.allocs, t->ctx->setup);
     if (e == cudaSuccess) {
         ColLists cl;
@@ -1222,7 +1243,6 @@ try {
             t->d.allocs.pop_back();
         }
     }
-    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) { cudaGetLastError(); return nullptr; }
     n.err = t->ctx->dev_err;
     t->spl = n;
