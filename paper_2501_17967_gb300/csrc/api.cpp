@@ -2,12 +2,14 @@
 // trees, applies.  Device memory is plain cudaMalloc; every entry point
 // returns a bc_status and records a message for bc_last_error().
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <complex>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
 #include <exception>
+#include <functional>
 #include <new>
 #include <system_error>
 #include <thread>
@@ -514,10 +516,10 @@ uint16_t bf16_of_int(int d)
 // digits, row exponents and (7 digits) the FP64 entries.
 struct OpGroup {
     int S = kSplitSlices, K = 0, kvalid = 0;   // digits, padded and valid inner dimension
+    size_t ndig = 0, nex = 0, nf = 0;          // room taken by the operators so far
     std::vector<uint16_t> dig;
     std::vector<int32_t> ex;
     std::vector<double> f;
-    bool exact = true;   // every row keeps the accumulation bound of the format
 };
 
 // f(0) .. f(n-1), on threads of their own where they can be had; an exception
@@ -541,50 +543,49 @@ template <class F> void in_parallel(int n, const F &f)
         if (e) std::rethrow_exception(e);
 }
 
-// Appends the BF16 digits of a real operator (rows x K, row-major) in the
-// chunk layout [digit a][row half h][K chunk kc] x (128 rows x KC) of
-// canonical K-major core matrices, its row exponents and (7 digits) its
-// entries [k][row].
-SplitOp add_split_op(OpGroup &G, const std::vector<double> &m, int rows)
+// Room for a real operator of `rows` rows in its group: its digits, in the chunk layout
+// [digit a][row half h][K chunk kc] x (128 rows x KC) of canonical K-major core
+// matrices, its row exponents and (7 digits) its entries [k][row].
+SplitOp add_split_op(OpGroup &G, int rows)
 {
-    const int K = G.K, S = G.S, KC = K > 144 ? kSplitKC : K, nkc = K / KC, mh = rows > 128 ? 2 : 1;
-    const size_t chunk = size_t(128) * KC;   // elements per chunk
+    const int K = G.K, KC = K > 144 ? kSplitKC : K, nkc = K / KC, mh = rows > 128 ? 2 : 1;
     SplitOp op;
-    op.a_off = int64_t(G.dig.size()) * int64_t(sizeof(uint16_t));
+    op.a_off = int64_t(G.ndig) * int64_t(sizeof(uint16_t));
     op.rows = rows;
-    op.exp_off = int32_t(G.ex.size());
-    op.f_off = int64_t(G.f.size());
-    const size_t base = G.dig.size();
-    G.dig.resize(base + size_t(S) * mh * nkc * chunk, 0);
-    G.ex.resize(G.ex.size() + size_t(mh) * 128, 0);
-    if (S == kWideSlices) {
-        G.f.resize(G.f.size() + size_t(G.kvalid) * rows);
-        for (int k = 0; k < G.kvalid; k++)
-            for (int i = 0; i < rows; i++) G.f[size_t(op.f_off) + size_t(k) * rows + i] = m[size_t(i) * K + k];
-    }
-    auto part = [&, base](int i0, int i1, bool *ok) {
-        std::vector<int16_t> dg(size_t(S) * K);
-        for (int i = i0; i < i1; i++) {
-            long long sum = 0;
-            G.ex[size_t(op.exp_off) + i] = split_row(&m[size_t(i) * K], K, S, dg.data(), &sum);
-            if (sum > (1ll << 17)) *ok = false;
-            const int h = i / 128, rg = (i % 128) / 8, r = i % 8;
-            for (int a = 0; a < S; a++)
-                for (int k = 0; k < K; k++) {
-                    const int kc = k / KC, kg = (k % KC) / 8, e = k % 8;
-                    const size_t off = base + ((size_t(a) * mh + h) * nkc + kc) * chunk +
-                                       (size_t(rg) * (KC / 8) + kg) * 64 + size_t(r) * 8 + e;
-                    G.dig[off] = bf16_of_int(dg[size_t(a) * K + k]);
-                }
-        }
-    };
-    // the 256 x 256 near tables take a few ms each: the rows in parallel
-    const int nt = size_t(rows) * K > 8192 ? 8 : 1;
-    bool ok[8];
-    std::fill(ok, ok + 8, true);
-    in_parallel(nt, [&](int t) { part(rows * t / nt, rows * (t + 1) / nt, &ok[t]); });
-    for (bool v : ok) G.exact = G.exact && v;
+    op.exp_off = int32_t(G.nex);
+    op.f_off = int64_t(G.nf);
+    G.ndig += size_t(G.S) * mh * nkc * 128 * KC;
+    G.nex += size_t(mh) * 128;
+    if (G.S == kWideSlices) G.nf += size_t(G.kvalid) * rows;
     return op;
+}
+
+// The operator m (rows x K, row-major) in its place; whether every row keeps the
+// accumulation bound.
+bool fill_split_op(OpGroup &G, const SplitOp &op, const std::vector<double> &m)
+{
+    const int K = G.K, S = G.S, KC = K > 144 ? kSplitKC : K, nkc = K / KC, mh = op.rows > 128 ? 2 : 1;
+    const size_t chunk = size_t(128) * KC, base = size_t(op.a_off) / sizeof(uint16_t);   // elements
+    if (S == kWideSlices) {
+        for (int k = 0; k < G.kvalid; k++)
+            for (int i = 0; i < op.rows; i++) G.f[size_t(op.f_off) + size_t(k) * op.rows + i] = m[size_t(i) * K + k];
+    }
+    std::vector<int16_t> dg(size_t(S) * K);
+    bool ok = true;
+    for (int i = 0; i < op.rows; i++) {
+        long long sum = 0;
+        G.ex[size_t(op.exp_off) + i] = split_row(&m[size_t(i) * K], K, S, dg.data(), &sum);
+        ok = ok && sum <= (1ll << 17);
+        const int h = i / 128, rg = (i % 128) / 8, r = i % 8;
+        for (int a = 0; a < S; a++)
+            for (int k = 0; k < K; k++) {
+                const int kc = k / KC, kg = (k % KC) / 8, e = k % 8;
+                const size_t off = base + ((size_t(a) * mh + h) * nkc + kc) * chunk +
+                                   (size_t(rg) * (KC / 8) + kg) * 64 + size_t(r) * 8 + e;
+                G.dig[off] = bf16_of_int(dg[size_t(a) * K + k]);
+            }
+    }
+    return ok;
 }
 
 // Device memory of one set-up in a single allocation: the uploaded arrays
@@ -653,81 +654,91 @@ bc_status build_digit_tables(bc_ctx *ctx, SplitTables &T, int slices, bool *read
         const double wm = *std::max_element(ht.w.begin(), ht.w.end());
         for (int k = 0; k < NP; k++) vs[k] = std::ldexp(1.0, int(std::lround(std::log2(std::max(ht.w[k] / wm, 1e-12)))));
     }
+    // Column scales of group E.  The rounding error of output j is about
+    // 2^-40 (max_k |A'_jk| sum_k |x'_k| + max_k |x'_k| sum_k |A'_jk|) with
+    // A' = A / s, x' = s x; it is smallest for s_k = sqrt(alpha_k / beta_k),
+    // alpha_k ~ |A_jk| and beta_k ~ |x_k| the profiles of coefficient k.
+    // Expansion-to-leaf (L2P, P2M^H): the operator grows like (sqrt 2)^l
+    // (nodes up to a corner of the box) and its inputs (local coefficients,
+    // adjoint multipoles) decay at least like 3^-l (sources two box widths
+    // away), so s = 2^l; the W list (M2P, P2L^H): operator ~ 3^-l, inputs
+    // (multipoles, adjoint locals) ~ (sqrt 2)^l, so s = 2^-l.
+    std::vector<double> se(KE), sw(KE);
+    for (int k = 0; k < KE; k++) {
+        se[k] = std::ldexp(1.0, k / 2);
+        sw[k] = std::ldexp(1.0, -(k / 2));
+    }
+    // The operators take their places here and are filled in by all threads below:
+    // each is a zeroed matrix (rows x K, row-major) that `fill` sets.
+    struct Job {
+        OpGroup *G;
+        SplitOp op;
+        std::function<void(std::vector<double> &)> fill;
+    };
+    std::vector<Job> jobs;
+    auto add = [&](OpGroup &G, int rows, std::function<void(std::vector<double> &)> fill) {
+        jobs.push_back({&G, add_split_op(G, rows), std::move(fill)});
+        return jobs.back().op;
+    };
     for (int dir = 0; dir < 2; dir++) {
         OpGroup &V = gv[dir], &E = ge[dir];
         V.S = E.S = slices;
         V.K = KV; V.kvalid = NP;
         E.K = KE; E.kvalid = R;
-        std::vector<double> m;
-        auto cscale = [&](int k) { return dir == 0 ? 1.0 / vs[k] : 1.0; };
+        auto cscale = [&vs, dir](int k) { return dir == 0 ? 1.0 / vs[k] : 1.0; };
         // group V
         T.near_op[dir].assign(kNumNear, SplitOp());
-        m.assign(size_t(NP) * KV, 0.0);
         for (int tab = 0; tab < kNumNear; tab++) {
-            NearGeom g = near_table_geometry(tab);
+            const NearGeom g = near_table_geometry(tab);
             if (!g.valid) continue;
-            for (int i = 0; i < NP; i++)
-                for (int k = 0; k < NP; k++)
-                    m[size_t(i) * KV + k] = cscale(k) * (dir == 0 ? ht.T[(size_t(tab) * NP + i) * NP + k]
-                                                                  : ht.T[(size_t(g.rev) * NP + k) * NP + i]);
-            T.near_op[dir][tab] = add_split_op(V, m, NP);
+            T.near_op[dir][tab] = add(V, NP, [&ht, NP, KV, tab, g, dir, cscale](std::vector<double> &m) {
+                for (int i = 0; i < NP; i++)
+                    for (int k = 0; k < NP; k++)
+                        m[size_t(i) * KV + k] = cscale(k) * (dir == 0 ? ht.T[(size_t(tab) * NP + i) * NP + k]
+                                                                      : ht.T[(size_t(g.rev) * NP + k) * NP + i]);
+            });
         }
-        m.assign(size_t(R) * KV, 0.0);
-        for (int l = 0; l < P1; l++)
-            for (int j = 0; j < NP; j++) {
-                cplx z = dir == 0 ? at2(ht.Q, size_t(l) * NP + j) : std::conj(at2(ht.E, size_t(j) * P1 + l));
-                m[size_t(2 * l) * KV + j] = cscale(j) * z.real();
-                m[size_t(2 * l + 1) * KV + j] = cscale(j) * z.imag();
-            }
-        T.leafA_op[dir] = add_split_op(V, m, R);
+        // (Re, Im) rows of a complex operator z(l, j) on the leaf values
+        auto leaf_rows = [&, cscale](auto z) {
+            return [=](std::vector<double> &m) {
+                for (int l = 0; l < P1; l++)
+                    for (int j = 0; j < NP; j++) {
+                        const cplx v = z(l, j);
+                        m[size_t(2 * l) * KV + j] = cscale(j) * v.real();
+                        m[size_t(2 * l + 1) * KV + j] = cscale(j) * v.imag();
+                    }
+            };
+        };
+        T.leafA_op[dir] = add(V, R, leaf_rows([&ht, NP, P1, dir](int l, int j) {
+            return dir == 0 ? at2(ht.Q, size_t(l) * NP + j) : std::conj(at2(ht.E, size_t(j) * P1 + l));
+        }));
         T.x_op[dir].assign(kNumWX, SplitOp());
-        for (int c = 0; c < kNumWX; c++) {
-            for (int l = 0; l < P1; l++)
-                for (int j = 0; j < NP; j++) {
-                    cplx z = dir == 0 ? at2(ht.P2L, (size_t(c) * P1 + l) * NP + j)
-                                      : std::conj(at2(ht.M2P, (size_t(c) * NP + j) * P1 + l));
-                    m[size_t(2 * l) * KV + j] = cscale(j) * z.real();
-                    m[size_t(2 * l + 1) * KV + j] = cscale(j) * z.imag();
-                }
-            T.x_op[dir][c] = add_split_op(V, m, R);
-        }
+        for (int c = 0; c < kNumWX; c++)
+            T.x_op[dir][c] = add(V, R, leaf_rows([&ht, NP, P1, dir, c](int l, int j) {
+                return dir == 0 ? at2(ht.P2L, (size_t(c) * P1 + l) * NP + j)
+                                : std::conj(at2(ht.M2P, (size_t(c) * NP + j) * P1 + l));
+            }));
         // group E: out_j = Re(sum_l Op(j,l) b_l) = sum_l Re Op(j,l) Re b_l - Im Op(j,l) Im b_l;
         // columns rescaled by powers of two (the expansion digits carry the inverse scale)
-        std::vector<double> me(size_t(NP) * KE, 0.0);
-        std::vector<std::vector<double>> mw(kNumWX, std::vector<double>(size_t(NP) * KE, 0.0));
-        for (int j = 0; j < NP; j++)
-            for (int l = 0; l < P1; l++) {
-                cplx z = dir == 0 ? at2(ht.E, size_t(j) * P1 + l) : std::conj(at2(ht.Q, size_t(l) * NP + j));
-                me[size_t(j) * KE + 2 * l] = z.real();
-                me[size_t(j) * KE + 2 * l + 1] = -z.imag();
-                for (int c = 0; c < kNumWX; c++) {
-                    cplx w = dir == 0 ? at2(ht.M2P, (size_t(c) * NP + j) * P1 + l)
-                                      : std::conj(at2(ht.P2L, (size_t(c) * P1 + l) * NP + j));
-                    mw[c][size_t(j) * KE + 2 * l] = w.real();
-                    mw[c][size_t(j) * KE + 2 * l + 1] = -w.imag();
-                }
-            }
-        // Column scales.  The rounding error of output j is about
-        // 2^-40 (max_k |A'_jk| sum_k |x'_k| + max_k |x'_k| sum_k |A'_jk|) with
-        // A' = A / s, x' = s x; it is smallest for s_k = sqrt(alpha_k / beta_k),
-        // alpha_k ~ |A_jk| and beta_k ~ |x_k| the profiles of coefficient k.
-        // Expansion-to-leaf (L2P, P2M^H): the operator grows like (sqrt 2)^l
-        // (nodes up to a corner of the box) and its inputs (local coefficients,
-        // adjoint multipoles) decay at least like 3^-l (sources two box widths
-        // away), so s = 2^l; the W list (M2P, P2L^H): operator ~ 3^-l, inputs
-        // (multipoles, adjoint locals) ~ (sqrt 2)^l, so s = 2^-l.
-        std::vector<double> se(KE), sw(KE);
-        for (int k = 0; k < KE; k++) {
-            se[k] = std::ldexp(1.0, k / 2);
-            sw[k] = std::ldexp(1.0, -(k / 2));
-            for (int j = 0; j < NP; j++) {
-                me[size_t(j) * KE + k] /= se[k];
-                for (int c = 0; c < kNumWX; c++) mw[c][size_t(j) * KE + k] /= sw[k];
-            }
-        }
-        T.e_op[dir] = add_split_op(E, me, NP);
+        auto node_rows = [&](auto z, const std::vector<double> &s) {
+            return [=, &s](std::vector<double> &m) {
+                for (int j = 0; j < NP; j++)
+                    for (int l = 0; l < P1; l++) {
+                        const cplx v = z(j, l);
+                        m[size_t(j) * KE + 2 * l] = v.real() / s[2 * l];
+                        m[size_t(j) * KE + 2 * l + 1] = -v.imag() / s[2 * l + 1];
+                    }
+            };
+        };
+        T.e_op[dir] = add(E, NP, node_rows([&ht, NP, P1, dir](int j, int l) {
+            return dir == 0 ? at2(ht.E, size_t(j) * P1 + l) : std::conj(at2(ht.Q, size_t(l) * NP + j));
+        }, se));
         T.w_op[dir].assign(kNumWX, SplitOp());
-        for (int c = 0; c < kNumWX; c++) T.w_op[dir][c] = add_split_op(E, mw[c], NP);
+        for (int c = 0; c < kNumWX; c++)
+            T.w_op[dir][c] = add(E, NP, node_rows([&ht, NP, P1, dir, c](int j, int l) {
+                return dir == 0 ? at2(ht.M2P, (size_t(c) * NP + j) * P1 + l)
+                                : std::conj(at2(ht.P2L, (size_t(c) * P1 + l) * NP + j));
+            }, sw));
         // Group M: M2L per V code in real form (rows 2l, 2l+1 = Re, Im of
         // output coefficient l; column 2k, 2k+1 = Re, Im of input k):
         //   forward (l,k) = M2L_c[l][k];  adjoint (l,k) = conj(M2L_{-d}[k][l]),
@@ -738,24 +749,21 @@ bc_status build_digit_tables(bc_ctx *ctx, SplitTables &T, int slices, bool *read
         // its input grows at most like (sqrt 2)^k, so the rescaled rows stay
         // within a few powers of two.
         T.m2l_op[dir].assign(kNumV, SplitOp());
-        {
-            std::vector<double> mm(size_t(R) * KE, 0.0);
-            for (int c = 0; c < kNumV; c++) {
-                const int dx = c % 7 - 3, dy = c / 7 - 3, cr = kNumV - 1 - c;
-                if (std::max(std::abs(dx), std::abs(dy)) < 2) continue;
-                std::fill(mm.begin(), mm.end(), 0.0);
+        for (int c = 0; c < kNumV; c++) {
+            const int dx = c % 7 - 3, dy = c / 7 - 3, cr = kNumV - 1 - c;
+            if (std::max(std::abs(dx), std::abs(dy)) < 2) continue;
+            T.m2l_op[dir][c] = add(E, R, [&ht, &sw, P1, dir, c, cr](std::vector<double> &m) {
                 for (int l = 0; l < P1; l++)
                     for (int k = 0; k < P1; k++) {
                         cplx z = dir == 0 ? at2(ht.M2L, (size_t(c) * P1 + l) * P1 + k)
                                           : std::conj(at2(ht.M2L, (size_t(cr) * P1 + k) * P1 + l));
                         if (l == 0 && k == 0) z = 0.0;
-                        mm[size_t(2 * l) * KE + 2 * k] = z.real() / sw[2 * k];
-                        mm[size_t(2 * l) * KE + 2 * k + 1] = -z.imag() / sw[2 * k + 1];
-                        mm[size_t(2 * l + 1) * KE + 2 * k] = z.imag() / sw[2 * k];
-                        mm[size_t(2 * l + 1) * KE + 2 * k + 1] = z.real() / sw[2 * k + 1];
+                        m[size_t(2 * l) * KE + 2 * k] = z.real() / sw[2 * k];
+                        m[size_t(2 * l) * KE + 2 * k + 1] = -z.imag() / sw[2 * k + 1];
+                        m[size_t(2 * l + 1) * KE + 2 * k] = z.imag() / sw[2 * k];
+                        m[size_t(2 * l + 1) * KE + 2 * k + 1] = z.real() / sw[2 * k + 1];
                     }
-                T.m2l_op[dir][c] = add_split_op(E, mm, R);
-            }
+            });
         }
         // expA is the W source (first) in the forward apply and the P2M^H input
         // (second) in the adjoint; expB the other way round
@@ -764,8 +772,26 @@ bc_status build_digit_tables(bc_ctx *ctx, SplitTables &T, int slices, bool *read
             scl[dir][k] = dir == 0 ? sw[k] : se[k];
             scl[dir][KE + k] = dir == 0 ? se[k] : sw[k];
         }
-        if (wide && !(V.exact && E.exact)) return BC_OK;   // not ready: the FP64 kernels serve
     }
+    for (OpGroup *G : {&gv[0], &gv[1], &ge[0], &ge[1]}) {
+        G->dig.assign(G->ndig, 0);
+        G->ex.assign(G->nex, 0);
+        G->f.assign(G->nf, 0.0);
+    }
+    // Some 330 operators of up to 256 x 256 (p = 16), 60 ns an entry: one thread took
+    // most of a context's creation.
+    std::atomic<size_t> next{0};
+    std::atomic<bool> exact{true};   // every row keeps the accumulation bound of the format
+    in_parallel(int(std::min(16u, std::max(1u, std::thread::hardware_concurrency()))), [&](int) {
+        std::vector<double> m;
+        for (size_t q; (q = next++) < jobs.size();) {
+            const Job &jb = jobs[q];
+            m.assign(size_t(jb.op.rows) * jb.G->K, 0.0);
+            jb.fill(m);
+            if (!fill_split_op(*jb.G, jb.op, m)) exact = false;
+        }
+    });
+    if (wide && !exact) return BC_OK;   // not ready: the FP64 kernels serve
     uint16_t *d[2][2];
     int32_t *x[2][2];
     double *f[2][2], *sc[2], *pv = nullptr;
