@@ -73,7 +73,8 @@ typedef enum {
                               native FP64.  The tiles of a tree take device
                               memory from its first such apply to its end (about
                               44 KB per leaf at p = 16); where they do not fit,
-                              with the option fp64_native, and (M2L only) with
+                              for trees of at most 256 nodes at p <= 8, with the
+                              option fp64_native, and (M2L only) with
                               m2l_triangular and m2l_kernel, every step is in
                               native FP64, as in bc_apply_noalloc (every p) */
     BC_SPLIT_BF16 = 1,     /* 5 digits for the fixed-operator products: the

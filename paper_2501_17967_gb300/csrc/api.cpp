@@ -1062,6 +1062,13 @@ bc_status build_split_m2l(bc_tree *t)
     return BC_OK;
 }
 
+// Trees so small that the FP64 kernels serve: up to 256 nodes of at most 64 a leaf (1 or
+// 4 leaves up to p = 8, 16 at p = 4).  An apply takes 15 to 26 us there (4 leaves, p = 4,
+// 6, 7, 8: 15.2, 19.6, 22.8, 25.6 us; 16 leaves, p = 4: 43.5) where the digits take 24 to
+// 26 (24.4, 26.2, 24.4, 24.9; 41.9), and a tree's first one goes without the tiles'
+// set-up of some 60 us (p = 4, 4 and 16 leaves: 31 and 63 us against 91 and 112).
+bool wide_too_small(const bc_tree *t) { return t->ctx->p <= 8 && t->h.nleaf * t->ctx->NP <= 256; }
+
 // Allocations and copies of a set-up are allowed while some stream of the caller's is
 // being captured; the thread's mode is put back at the end, also past an exception.
 class RelaxedCapture {
@@ -1089,7 +1096,7 @@ public:
 // part of the caller's capture), so it neither joins nor breaks a stream capture.
 bool build_wide_tree(bc_tree *t)
 {
-    if (t->ctx->fp64_native) return false;
+    if (t->ctx->fp64_native || wide_too_small(t)) return false;
     if (t->wide_ready) return true;
     if (t->wide_off || !t->ctx->wide_ready) return false;
     const RelaxedCapture relaxed;
@@ -1229,7 +1236,7 @@ bc_status prepare_split_tree(bc_tree *t) { return build_split_tree(t); }
 // nullptr: they do not fit.
 const SplitTree *prepare_wide_l2p(bc_tree *t)
 try {
-    if (t->ctx->fp64_native) return nullptr;
+    if (t->ctx->fp64_native || wide_too_small(t)) return nullptr;
     if (t->wide_ready) return &t->spw;
     if (t->spl.PE) return &t->spl;
     if (t->wide_off || !t->ctx->wide_ready) return nullptr;

@@ -198,6 +198,25 @@ def test_trees_on_their_own_streams():
     assert np.isfinite(relerr(outs[0], want[0]))
 
 
+# 256 nodes of at most 64 a leaf: the FP64 kernels serve; above, or with larger leaves, the digits
+@pytest.mark.parametrize("p,level,native", [(4, 0, True), (4, 1, True), (4, 2, True), (5, 1, True), (5, 2, False), (8, 0, True),
+                                            (8, 1, True), (9, 0, False), (9, 1, False), (16, 0, False), (4, 3, False)])
+def test_small_trees_of_small_orders(p, level, native):
+    tree = bc.Tree(bc.Context(p=p, nterms=20, device=0), *synth.uniform_leaves(level))
+    x = torch.randn(tree.nleaf, p, p, device="cuda", dtype=torch.float64, generator=torch.Generator(device="cuda").manual_seed(p))
+    for adjoint in (False, True):
+        u, v = digits(tree, x, adjoint), kernels(tree, x, adjoint)
+        assert torch.equal(u, v) if native else relerr(u, v) <= BAR
+    x[0, 0, 0] = float("inf")
+    assert torch.equal(torch.isfinite(digits(tree, x, False)), torch.isfinite(kernels(tree, x, False)))
+    batch = bc.Batch(tree.ctx, [tree, tree])     # the union may be above the line where its trees are not
+    xs = [torch.randn_like(x) for _ in range(2)]
+    outs = [torch.empty_like(x) for _ in range(2)]
+    batch.run(xs, outs)
+    for a, u in zip(xs, outs):
+        assert relerr(u, kernels(tree, a, False)) <= BAR
+
+
 @pytest.mark.parametrize("p", [7, 16])
 def test_native_fp64_on_request(p):
     """fp64_native: BC_FP64 on the FP64 kernels alone, bit for bit bc_apply_noalloc, without the tiles' memory."""
