@@ -589,8 +589,10 @@ bool fill_split_op(OpGroup &G, const SplitOp &op, const std::vector<double> &m)
 }
 
 // Device memory of one set-up in a single allocation: the uploaded arrays
-// (one copy) and the uninitialised ones.
+// (one copy, done when `st` is; the arena keeps its source until then) and the
+// uninitialised ones.
 struct DevArena {
+    std::vector<uint8_t> host;
     struct Item { void **dst; const void *src; size_t bytes; };
     std::vector<Item> items;
     template <class T> void add(T **dst, const std::vector<T> &v)
@@ -609,7 +611,7 @@ struct DevArena {
             if (it.src) up = total;
         }
         // what may throw comes before anything is held
-        std::vector<uint8_t> host(up);
+        host.assign(up, 0);
         allocs.reserve(allocs.size() + 1);
         void *base = nullptr;
         cudaError_t e = cudaMalloc(&base, std::max<size_t>(total, 256));
@@ -617,7 +619,6 @@ struct DevArena {
         for (size_t i = 0; i < items.size(); i++)
             if (items[i].src && items[i].bytes) std::memcpy(host.data() + off[i], items[i].src, items[i].bytes);
         if (up) e = cudaMemcpyAsync(base, host.data(), up, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { cudaFree(base); return e; }
         allocs.push_back(base);
         for (size_t i = 0; i < items.size(); i++) *items[i].dst = static_cast<uint8_t *>(base) + off[i];
@@ -806,6 +807,7 @@ bc_status build_digit_tables(bc_ctx *ctx, SplitTables &T, int slices, bool *read
     }
     arena.add(&pv, vs);
     cudaError_t e = arena.commit(ctx->split_allocs, cudaStreamPerThread);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamPerThread);
     if (e != cudaSuccess) return cuda_fail(e, "digit tables upload");
     for (int dir = 0; dir < 2; dir++) {
         T.escale[dir] = sc[dir];
@@ -896,32 +898,29 @@ std::vector<int32_t> order_by_code(const std::vector<int32_t> &code, int ncodes,
     return out;
 }
 
-cudaError_t build_tile_order(bc_tree *t)
+// The entries of the tree's lists ordered by operator, added to an arena whose upload
+// completes them (`lists`: theirs until then).
+void add_tile_order(bc_tree *t, DevArena &up, std::vector<int32_t> (&lists)[5])
 {
     TileOrder &o = t->order;
-    if (o.ready) return cudaSuccess;
     const HostTree &h = t->h;
-    std::vector<int32_t> near, x, w, v, l2p;
-    auto rest = [&] {
+    auto &[near, x, w, v, l2p] = lists;
+    auto rest = [&, &near = near, &x = x, &w = w, &l2p = l2p] {
         near = order_by_code(h.near_tab, kNumNear, o.n_near);
         x = order_by_code(h.x_code, kNumWX, o.n_x);
         w = order_by_code(h.w_code, kNumWX, o.n_w);
         for (int32_t k : h.leaf_order)
             if (h.leaf_level[k] >= 2) l2p.push_back(k);
     };
-    auto vlist = [&] { v = order_by_code(h.v_code, kNumV, o.n_v); };   // the longest list, beside the others
+    auto vlist = [&, &v = v] { v = order_by_code(h.v_code, kNumV, o.n_v); };   // the longest list, beside the others
     in_parallel(h.v_code.size() > 50000 ? 2 : 1, [&](int i) { if (i) vlist(); else rest(); });
     if (h.v_code.size() <= 50000) vlist();
     o.n_l2p = int64_t(l2p.size());
-    DevArena up;
     up.add(&o.near, near);
     up.add(&o.x, x);
     up.add(&o.w, w);
     up.add(&o.v, v);
     up.add(&o.l2p, l2p);
-    const cudaError_t e = up.commit(t->d.allocs, t->ctx->setup);
-    o.ready = e == cudaSuccess;
-    return e;
 }
 
 // Tiles, digit buffers and result rows of a tree in the format of T (the two
@@ -935,9 +934,11 @@ try {
     const int64_t nn = int64_t(h.near_src.size()), nx = int64_t(h.x_src.size()), nw = int64_t(h.w_src.size());
     const int64_t nv = int64_t(h.v_src.size()), nbox = int64_t(h.box_level.size());
     cudaError_t e = ensure_side(t);
-    if (e == cudaSuccess) e = build_tile_order(t);
     if (e != cudaSuccess) return e;
-    const TileOrder &o = t->order;
+    TileOrder &o = t->order;
+    DevArena up;
+    std::vector<int32_t> lists[5];
+    if (!o.ready) add_tile_order(t, up, lists);
     const size_t NP = size_t(T.np), KV = size_t(T.kv);   // nodes per leaf, group-V K
     std::vector<SplitTile> vn, en, mn;
     SplitTree n;
@@ -971,15 +972,10 @@ try {
     n.ntM = int(mn.size());
     const SplitTree &other = &s == &t->sp ? t->spw : t->sp;
     double2 *Pv = t->d.Pv;
-    DevArena up;
-    up.add(&n.tVN, vn);
-    up.add(&n.tE, en);
     if (m2l) up.add(&n.tM, mn);
     if (s.Pnear) {   // set up before without the M2L
         n = SplitTree(s);
         n.ntM = int(mn.size());
-        up.items.clear();
-        up.add(&n.tM, mn);
     } else if (other.Pnear) {
         n.Pnear = other.Pnear; n.PX = other.PX; n.PE = other.PE; n.PW = other.PW;
     } else {
@@ -989,6 +985,8 @@ try {
         up.room(&n.PW, size_t(nw) * NP);
     }
     if (!s.Pnear) {
+        up.add(&n.tVN, vn);
+        up.add(&n.tE, en);
         up.room(&n.vdig, size_t(h.nleaf) * S * KV);
         up.room(&n.vexp, size_t(h.nleaf));
         up.room(&n.edig, size_t(2 * nbox) * S * kSplitKE);
@@ -1037,6 +1035,7 @@ try {
     n.err = t->ctx->dev_err;
     s = n;
     t->d.Pv = Pv;
+    o.ready = true;
     return cudaSuccess;
 } catch (const std::bad_alloc &) {
     return cudaErrorMemoryAllocation;
