@@ -63,8 +63,7 @@ __device__ __forceinline__ double2 cinv(double2 a)
 //     1/x   = 2^-e c_j / (1 + r),           1/(1+r)  = 1 - r + r^2 + r^3 (-1 + r - r^2),
 // the linear and square terms as 64-bit integers (r^2 to 2^-62), the cubic ones, below
 // 4e-10, in FP32 (2e-17), the series cut below 2e-19.  Errors before the last rounding:
-// logarithm 2^-53 absolute, reciprocal 2^-54 relative.  From 1 to 1 + 2^-7 the
-// logarithm is formed in FP64 from x - 1 (exact), within an ulp or so of itself.  Valid for normal x with 1/x
+// logarithm 2^-53 absolute, reciprocal 2^-54 relative.  Valid for normal x with 1/x
 // normal (|e| <= 1021), which the near sums' squared distances meet.  Table:
 // g_logtab[j] = (c_j 2^11 - 1024) in 11 bits, -log c_j in units of 2^-53 in 53 bits (set by
 // layer_log_init).
@@ -103,17 +102,6 @@ __device__ __forceinline__ void log_inv(double x, const unsigned long long *__re
                         ((static_cast<long long>(e) * kLn2Lo) >> 32);
     const long long lb = int_bits(static_cast<unsigned long long>(l < 0 ? -l : l), -53);
     lg = l ? __longlong_as_double(lb | (l & (1ll << 63))) : 0.0;
-    if (static_cast<unsigned long long>(bits - 0x3FF0000000000000ll) < (1ull << 45)) {   // x - 1 below 2^-7: rare
-        const double d = x - 1.0;
-        double q = fma(d, 1.0 / 9.0, -0.125);   // log1p(d) = d + d^2 q(d), cut below 2^-59 of d
-        q = fma(q, d, 1.0 / 7.0);
-        q = fma(q, d, -1.0 / 6.0);
-        q = fma(q, d, 0.2);
-        q = fma(q, d, -0.25);
-        q = fma(q, d, 1.0 / 3.0);
-        q = fma(q, d, -0.5);
-        lg = fma(d * d, q, d);
-    }
     const unsigned long long s = (1ull << 63) - r + (w >> 19) + 4ll * ci;   // 1 / (1 + r), units 2^-63
     const unsigned cw = c << 20;
     inv = __longlong_as_double(int_bits((s >> 32) * cw + __umulhi(unsigned(s), cw), -62 - e));   // from units 2^-62
