@@ -186,3 +186,19 @@ def test_near_sum_log_against_cuda():
     ei = ((inv - ref_i).abs() / ref_i.abs()).max().item()
     print(f"table log: max error {el / 2.0 ** -53:.2f} units of 2^-53 (scaled); reciprocal {ei / 2.0 ** -53:.2f}")
     assert el <= 2.0 ** -51 and ei <= 2.0 ** -51, (el, ei)
+
+
+def test_near_sum_log_at_every_interval_boundary():
+    """Both sides of the 1,024 table interval boundaries over 41 binades; the bars of test_near_sum_log_against_cuda."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    e, j = np.meshgrid(np.arange(-20, 21), np.arange(1024), indexing="ij")
+    b = np.ldexp(1.0 + j / 1024.0, e).ravel()
+    x = torch.from_numpy(np.concatenate([b, np.nextafter(b, 0.0), np.nextafter(b, np.inf)])).cuda()
+    lg, inv = torch.empty_like(x), torch.empty_like(x)
+    bc._check(bc._load().bc_debug_log_inv(0, ctypes.c_void_p(x.data_ptr()), x.numel(), ctypes.c_void_p(lg.data_ptr()),
+                                         ctypes.c_void_p(inv.data_ptr()), None))
+    torch.cuda.synchronize()
+    ref_l, ref_i = torch.log(x), 1.0 / x
+    assert ((lg - ref_l).abs() / ref_l.abs().clamp(min=1.0)).max().item() <= 2.0 ** -51
+    assert ((inv - ref_i).abs() / ref_i).max().item() <= 2.0 ** -51
