@@ -924,10 +924,11 @@ void add_tile_order(bc_tree *t, DevArena &up, std::vector<int32_t> (&lists)[5])
 }
 
 // Tiles, digit buffers and result rows of a tree in the format of T (the two
-// formats share the result rows), with the M2L's where m2l is set.  The host
-// orders the lists and cuts them into tiles; the columns (16 bytes per entry
-// and direction) are written by the device.
-cudaError_t build_digit_tree(bc_tree *t, const SplitTables &T, SplitTree &s, bool m2l)
+// formats share the result rows): those of the leaf products (`leaf`) and of the
+// M2L (`m2l`), as far as they are not there.  The host orders the lists and cuts
+// them into tiles; the columns (16 bytes per entry and direction) are written by
+// the device.
+cudaError_t build_digit_tree(bc_tree *t, const SplitTables &T, SplitTree &s, bool leaf, bool m2l)
 try {
     const HostTree &h = t->h;
     const int P1 = t->ctx->P1, S = T.slices;
@@ -935,70 +936,71 @@ try {
     const int64_t nv = int64_t(h.v_src.size()), nbox = int64_t(h.box_level.size());
     cudaError_t e = ensure_side(t);
     if (e != cudaSuccess) return e;
+    leaf = leaf && !s.tVN;
+    m2l = m2l && !s.tM;
     TileOrder &o = t->order;
     DevArena up;
     std::vector<int32_t> lists[5];
     if (!o.ready) add_tile_order(t, up, lists);
     const size_t NP = size_t(T.np), KV = size_t(T.kv);   // nodes per leaf, group-V K
     std::vector<SplitTile> vn, en, mn;
-    SplitTree n;
-    int64_t p0 = 0;
-    for (int c = 0; c < kNumNear; c++) {
-        if (o.n_near[c]) add_tiles(vn, T.near_op[0][c], p0, o.n_near[c], T.tileN, KV == 64);
-        p0 += o.n_near[c];
-    }
-    n.ntN = int(vn.size());
-    add_tiles(vn, T.leafA_op[0], p0, h.nleaf, T.tileN, KV == 64);
-    n.ntA = int(vn.size()) - n.ntN;
-    p0 += h.nleaf;
-    for (int c = 0; c < kNumWX; c++) {
-        if (o.n_x[c]) add_tiles(vn, T.x_op[0][c], p0, o.n_x[c], T.tileN, KV == 64);
-        p0 += o.n_x[c];
-    }
-    n.ntVN = int(vn.size());
-    add_tiles(en, T.e_op[0], 0, o.n_l2p, T.tileN, true);
-    n.ntL = int(en.size());
-    p0 = o.n_l2p;
-    for (int c = 0; c < kNumWX; c++) {
-        if (o.n_w[c]) add_tiles(en, T.w_op[0][c], p0, o.n_w[c], T.tileN, true);
-        p0 += o.n_w[c];
-    }
-    n.ntE = int(en.size());
-    p0 = 0;
-    for (int c = 0; c < kNumV && m2l; c++) {
-        if (o.n_v[c]) add_tiles(mn, T.m2l_op[0][c], p0, o.n_v[c], T.tileN, true);
-        p0 += o.n_v[c];
-    }
-    n.ntM = int(mn.size());
-    const SplitTree &other = &s == &t->sp ? t->spw : t->sp;
+    SplitTree n = s;
     double2 *Pv = t->d.Pv;
-    if (m2l) up.add(&n.tM, mn);
-    if (s.Pnear) {   // set up before without the M2L
-        n = SplitTree(s);
-        n.ntM = int(mn.size());
-    } else if (other.Pnear) {
-        n.Pnear = other.Pnear; n.PX = other.PX; n.PE = other.PE; n.PW = other.PW;
-    } else {
-        up.room(&n.Pnear, size_t(nn) * NP);
-        up.room(&n.PX, size_t(nx) * kSplitKE);
-        up.room(&n.PE, size_t(h.nleaf) * NP);
-        up.room(&n.PW, size_t(nw) * NP);
-    }
-    if (!s.Pnear) {
+    if (leaf) {
+        int64_t p0 = 0;
+        for (int c = 0; c < kNumNear; c++) {
+            if (o.n_near[c]) add_tiles(vn, T.near_op[0][c], p0, o.n_near[c], T.tileN, KV == 64);
+            p0 += o.n_near[c];
+        }
+        n.ntN = int(vn.size());
+        add_tiles(vn, T.leafA_op[0], p0, h.nleaf, T.tileN, KV == 64);
+        n.ntA = int(vn.size()) - n.ntN;
+        p0 += h.nleaf;
+        for (int c = 0; c < kNumWX; c++) {
+            if (o.n_x[c]) add_tiles(vn, T.x_op[0][c], p0, o.n_x[c], T.tileN, KV == 64);
+            p0 += o.n_x[c];
+        }
+        n.ntVN = int(vn.size());
+        add_tiles(en, T.e_op[0], 0, o.n_l2p, T.tileN, true);
+        n.ntL = int(en.size());
+        p0 = o.n_l2p;
+        for (int c = 0; c < kNumWX; c++) {
+            if (o.n_w[c]) add_tiles(en, T.w_op[0][c], p0, o.n_w[c], T.tileN, true);
+            p0 += o.n_w[c];
+        }
+        n.ntE = int(en.size());
         up.add(&n.tVN, vn);
         up.add(&n.tE, en);
+        const SplitTree &other = &s == &t->sp ? t->spw : t->sp;
+        if (other.Pnear) {
+            n.Pnear = other.Pnear; n.PX = other.PX; n.PE = other.PE; n.PW = other.PW;
+        } else {
+            up.room(&n.Pnear, size_t(nn) * NP);
+            up.room(&n.PX, size_t(nx) * kSplitKE);
+            up.room(&n.PE, size_t(h.nleaf) * NP);
+            up.room(&n.PW, size_t(nw) * NP);
+        }
         up.room(&n.vdig, size_t(h.nleaf) * S * KV);
         up.room(&n.vexp, size_t(h.nleaf));
-        up.room(&n.edig, size_t(2 * nbox) * S * kSplitKE);
-        up.room(&n.eexp, size_t(2 * nbox));
         for (int dir = 0; dir < 2; dir++) {
             up.room(&n.cVN[dir], size_t(nn + h.nleaf + nx));
             up.room(&n.cE[dir], size_t(o.n_l2p + nw));
         }
     }
     if (m2l) {
+        int64_t p0 = 0;
+        for (int c = 0; c < kNumV; c++) {
+            if (o.n_v[c]) add_tiles(mn, T.m2l_op[0][c], p0, o.n_v[c], T.tileN, true);
+            p0 += o.n_v[c];
+        }
+        n.ntM = int(mn.size());
+        up.add(&n.tM, mn);
         if (!Pv) up.room(&Pv, size_t(nv) * P1);
         for (int dir = 0; dir < 2; dir++) up.room(&n.cM[dir], size_t(nv));
+    }
+    if (!s.edig) {
+        up.room(&n.edig, size_t(2 * nbox) * S * kSplitKE);
+        up.room(&n.eexp, size_t(2 * nbox));
     }
     if ((e = up.commit(t->d.allocs, t->ctx->setup)) != cudaSuccess) return e;
     ColLists cl;
@@ -1016,7 +1018,7 @@ try {
         // expA holds the multipoles (adjoint: the second array), expB the locals
         double *first = reinterpret_cast<double *>(dir ? t->d.expB : t->d.expA);
         const int64_t f0 = dir ? nbox : 0, s0 = dir ? 0 : nbox;
-        if (!s.Pnear) {
+        if (leaf) {
             seg(ColKind::Near, dir, nn, o.near, n.cVN[dir], n.Pnear, int64_t(NP), 0);
             seg(ColKind::LeafA, dir, h.nleaf, t->d.leaf_order, n.cVN[dir] + nn, first, 2 * P1, 0);
             seg(ColKind::X, dir, nx, o.x, n.cVN[dir] + nn + h.nleaf, n.PX, kSplitKE, 0);
@@ -1044,7 +1046,7 @@ try {
 bc_status build_split_tree(bc_tree *t)
 {
     if (t->split_ready) return BC_OK;
-    const cudaError_t e = build_digit_tree(t, t->ctx->split, t->sp, false);
+    const cudaError_t e = build_digit_tree(t, t->ctx->split, t->sp, true, false);
     if (e != cudaSuccess) return cuda_fail(e, "split tree upload");
     t->split_ready = true;
     return BC_OK;
@@ -1055,7 +1057,7 @@ bc_status build_split_tree(bc_tree *t)
 bc_status build_split_m2l(bc_tree *t)
 {
     if (t->m2l_ready) return BC_OK;
-    const cudaError_t e = build_digit_tree(t, t->ctx->split, t->sp, true);
+    const cudaError_t e = build_digit_tree(t, t->ctx->split, t->sp, true, true);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core M2L tiles");
     t->m2l_ready = true;
     return BC_OK;
@@ -1088,25 +1090,27 @@ public:
     bool ok() const { return ok_; }
 };
 
-// 7-digit tiles of the FP64 mode, on first use.  They take device memory that
+// 7-digit tiles on first use: of the FP64 mode, or (leaf = false) of the M2L alone, for
+// the split mode.  They take device memory that
 // the FP64 kernels do not need; where that is not to be had the FP64 kernels
 // serve (and are asked for again only with another tree).  The set-up runs on
 // the context's set-up stream, which no apply uses (the tree's internal stream may be
 // part of the caller's capture), so it neither joins nor breaks a stream capture.
-bool build_wide_tree(bc_tree *t)
+bool build_wide_tree(bc_tree *t, bool leaf = true)
 {
     if (t->ctx->fp64_native || wide_too_small(t)) return false;
-    if (t->wide_ready) return true;
+    if (leaf ? t->wide_ready : t->wide_m2l) return true;
     if (t->wide_off || !t->ctx->wide_ready) return false;
     const RelaxedCapture relaxed;
     if (!relaxed.ok()) return false;
-    const cudaError_t e = build_digit_tree(t, t->ctx->wide, t->spw, true);
+    const cudaError_t e = build_digit_tree(t, t->ctx->wide, t->spw, leaf, true);
     if (e != cudaSuccess) {
         cudaGetLastError();
         t->wide_off = e == cudaErrorMemoryAllocation;
         return false;
     }
-    t->wide_ready = true;
+    t->wide_m2l = true;
+    t->wide_ready = t->wide_ready || leaf;
     return true;
 }
 
@@ -1119,7 +1123,7 @@ int wide_parts(const bc_ctx *ctx) { return ctx->m2l_tri || ctx->m2l_kind ? kSpli
 // option chooses the products or another M2L, or the tiles do not fit.
 void split_m2l(bc_ctx *ctx, bc_tree *t, int prec, SplitLaunch &sl)
 {
-    if (prec != BC_SPLIT_BF16 || ctx->split_parts >= 0 || wide_parts(ctx) != kWideParts || !build_wide_tree(t)) return;
+    if (prec != BC_SPLIT_BF16 || ctx->split_parts >= 0 || wide_parts(ctx) != kWideParts || !build_wide_tree(t, false)) return;
     sl.parts |= 32;
     sl.m2l_tables = &ctx->wide;
     sl.m2l_tree = &t->spw;

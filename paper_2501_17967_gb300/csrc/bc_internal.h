@@ -546,7 +546,7 @@ struct bc_tree {
     bc::SplitTree sp, spw;    // tiles of the 5-digit and the 7-digit products
     bc::SplitTree spl;        // of the latter the expansion-to-leaf part alone (a layer before any such apply)
     bc::SideStream side;
-    bool split_ready = false, wide_ready = false;
+    bool split_ready = false, wide_ready = false, wide_m2l = false;   // wide_m2l: the M2L's part of the 7-digit tiles
     bool m2l_ready = false;   // tensor-core M2L tiles and rows (BC_SPLIT_BF16_ALL)
     bool wide_off = false;    // the 7-digit set-up did not fit: FP64 kernels
 };

@@ -243,3 +243,22 @@ def test_native_fp64_on_request(p):
     assert relerr(layer.apply(q, m), native) <= BAR
     with pytest.raises(bc.BoxCodeError):
         tree.ctx.set_option("fp64_native", 2)
+
+
+@pytest.mark.parametrize("order", [("split", "fp64"), ("fp64", "split"), ("split", "all", "fp64"), ("all", "layer", "split", "fp64")])
+def test_parts_of_the_tiles_in_any_order(order):
+    """A tree sets up its tiles as its calls need them (the split mode the M2L's part of the 7-digit ones only): every
+    order of first use gives what a fresh tree gives."""
+    curve = np.stack([0.5 * np.cos(np.arange(300)), 0.5 * np.sin(np.arange(300))], 1)
+
+    def run(tree, x, what):
+        if what == "layer":
+            return bc.Layer(tree, curve).apply(x.reshape(-1)[:300], x.reshape(-1)[300:900].reshape(300, 2))
+        prec = {"fp64": bc.FP64, "split": bc.SPLIT_BF16, "all": bc.SPLIT_BF16_ALL}[what]
+        return torch.cat([bc.apply(tree, x, precision=prec), bc.apply_adjoint(tree, x, precision=prec)])
+
+    tree, x = make(16, 24, max_level=5)
+    for what in order + order:
+        fresh, _ = make(16, 24, max_level=5)
+        assert torch.equal(run(tree, x, what), run(fresh, x, what)), what
+    bc._check(bc._load().bc_sync(tree.ctx.handle, None))
