@@ -72,7 +72,8 @@ typedef enum {
                               M2M and L2L shifts, the log terms and all sums in
                               native FP64.  The tiles of a tree take device
                               memory from its first such apply to its end (about
-                              44 KB per leaf at p = 16); where they do not fit,
+                              44 KB per leaf at p = 16); where they do not fit
+                              (bc_last_error() then says so after the call),
                               for trees of at most 256 nodes at p <= 8, with the
                               option fp64_native, and (M2L only) with
                               m2l_triangular and m2l_kernel, every step is in

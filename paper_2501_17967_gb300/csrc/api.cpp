@@ -1107,6 +1107,9 @@ bool build_wide_tree(bc_tree *t, bool leaf = true)
     if (e != cudaSuccess) {
         cudaGetLastError();
         t->wide_off = e == cudaErrorMemoryAllocation;
+        if (t->wide_off)   // served all the same, but a good deal slower: the caller can find out
+            set_error("the 7-digit tiles of a tree of %lld leaves do not fit in memory: its FP64 products stay on the FP64 kernels",
+                      (long long)t->h.nleaf);
         return false;
     }
     t->wide_m2l = true;

@@ -37,6 +37,8 @@ os.environ["REFUSE_ABOVE"] = "{limit}"
 if "{what}" == "tables":
     tree, x = d.make(9, 30)
 u, h = d.digits(tree, x, False), d.digits(tree, x, True)
+if "{what}" == "tiles":
+    assert "FP64 kernels" in bc._load().bc_last_error().decode()
 assert torch.equal(u, d.kernels(tree, x, False)) and torch.equal(h, d.kernels(tree, x, True))
 del os.environ["REFUSE_ABOVE"]
 tree, x = d.make(9, 30)
