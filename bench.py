@@ -15,8 +15,8 @@ whole tree; value = leaf nodes / (time of a step).  The headline precision
 lists) on BF16 tensor cores as exact digit products of 40-bit operands, the
 multipole-to-local translations as products of 56-bit ones (as accurate as
 FP64), and keeps the M2M/L2L shifts and the log terms in native FP64.  The same
-JSON line carries the FP64 path (every product of 56-bit operands),
-the all-tensor split variant and the 20-Gaussian workload as extra keys, and
+JSON line carries the FP64 path (every product of 56-bit operands, and once more
+with every step in native FP64), the all-tensor split variant and the 20-Gaussian workload as extra keys, and
 the error against the oracle per level, forward and adjoint.
 With --gpus N every rank runs its own replica (the path does not shard; no
 collective on the data path) and value is the total over ranks.
@@ -390,7 +390,7 @@ def layer_line(args, dev, steps, check=True):
         torch.cuda.synchronize()
         return sum(a.elapsed_time(b) for a, b in ev) / steps, u.cpu().numpy().reshape(-1, P * P)
 
-    # split: the L2P at every leaf on the tensor cores; FP64: all of it in FP64
+    # the L2P at every leaf on the tensor cores, split: 5 digits, FP64: 7
     ms, un = timed(bc.SPLIT_BF16)
     if not check:
         return {"value": tree.nleaf * P * P / (ms * 1e-3), "ms": ms, "profile_run": True}

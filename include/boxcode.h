@@ -63,14 +63,17 @@ typedef enum {
  * the tensor cores (tcgen05, FP32 accumulation, exact), and the recombination
  * is integer/FP64.  The rounding of the operands is the only error: with 5
  * digits about 2^-40 of sum |A_ik v_k| per output, with 7 digits about a tenth
- * of the rounding of the same sum in FP64 arithmetic. */
+ * of the rounding of the same sum in FP64 arithmetic.  (Relative to the largest
+ * entry of a row or a vector: one below an eighth of it keeps fewer than 53 bits of
+ * its own.)  Rows of partial results are summed by aligned integers of 58 bits and
+ * FP64 additions, which together round less than FP64 additions alone. */
 typedef enum {
     BC_FP64 = 0,           /* FP64 accuracy throughout: every operator product
                               (near-field tables, P2M, L2P, W and X lists, the
                               multipole-to-local translations) on 7 digits,
                               vectors with an infinity or a NaN in FP64; the
-                              M2M and L2L shifts, the log terms and all sums in
-                              native FP64.  The tiles of a tree take device
+                              M2M and L2L shifts and the log terms in native
+                              FP64, sums of rows at FP64's accuracy.  The tiles of a tree take device
                               memory from its first such apply to its end (about
                               44 KB per leaf at p = 16); where they do not fit
                               (bc_last_error() then says so after the call),
@@ -82,10 +85,12 @@ typedef enum {
                               near-field tables, P2M, L2P, the W list (M2P) and
                               the X list (P2L), and their adjoints.  The rest as
                               in BC_FP64: the multipole-to-local translations on
-                              7 digits, the M2M and L2L shifts, every log-kernel
-                              scaling term and every sum of partial results in
-                              native FP64 (p = 8, 12 and 16, nterms <= 32; other
-                              orders BC_ERR_UNSUPPORTED) */
+                              7 digits (native FP64 with the option
+                              fp64_native), the M2M and L2L shifts and every
+                              log-kernel scaling term in native FP64, sums of
+                              partial results at FP64's accuracy (p = 8, 12 and
+                              16, nterms <= 32; other orders
+                              BC_ERR_UNSUPPORTED) */
     BC_SPLIT_BF16_ALL = 2  /* BC_SPLIT_BF16 with the multipole-to-local
                               translations on 5 digits (their log terms stay
                               FP64) and the M2M / L2L shifts in double-float
@@ -220,7 +225,8 @@ bc_status bc_apply_adjoint(bc_ctx *ctx, const bc_tree *tree, const double *g, do
 
 /* out[k] = interpolant of the leaf-node values u at point xy[k]: v_bulk off
  * the grid, as the glue step needs it on the fictitious curve (Sec. 3.4)
- * (barycentric Chebyshev interpolation on the leaf containing the point; a point on a
+ * (Chebyshev interpolation on the leaf containing the point, its Lagrange factors
+ * formed as products of node differences, without divisions; a point on a
  * shared edge belongs to the leaf on its +x / +y side, the root's far edges to
  * the last leaf).  Points outside the root give BC_ERR_ARG on the host path;
  * on the device path they produce NaN.  u, xy, out: device or host (all of the
@@ -230,8 +236,8 @@ bc_status bc_eval_points(bc_ctx *ctx, const bc_tree *tree, const double *u, cons
 
 /* Value and gradient at points: val[k] as in bc_eval_points and
  * grad[2k], grad[2k+1] = the x and y derivatives of the same leaf
- * interpolant at xy[k] (barycentric differentiation, free of cancellation as
- * a point nears a node).  The glue step of Sec. 3.4 needs v_bulk and its
+ * interpolant at xy[k] (the same products differentiated, free of cancellation
+ * as a point nears a node).  The glue step of Sec. 3.4 needs v_bulk and its
  * normal derivative n . grad v_bulk on the fictitious curve (the jumps tau
  * and sigma of Alg. 1).  u, xy, val, grad: device or host (all of the same
  * kind); points outside the root: BC_ERR_ARG on the host path, NaN on the

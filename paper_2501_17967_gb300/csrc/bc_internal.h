@@ -269,7 +269,7 @@ struct SplitGemm {
     int ntiles = 0;
     const uint8_t *ops = nullptr;
     const int32_t *op_exp = nullptr;
-    const uint16_t *dig = nullptr;     // [nvec][5][K] BF16 digit bits
+    const uint16_t *dig = nullptr;     // [nvec][slices][K] BF16 digit bits
     const int32_t *dexp = nullptr;     // [nvec]
     int max_ctas = 0;                  // CTAs of the launch at most (0: one per SM)
     // 7 digits: the vectors in FP64 (vec < nsplit: src0 + vec kvalid, scales
@@ -336,8 +336,9 @@ int split_sm_count();          // SMs of the device (after split_prepare)
 // stream; on the 20-Gaussian workload the leaf step in the upward pass
 // doubles that pass, since each block streams the 98 KB operator for its ~4
 // leaves before it can climb).
-// BC_SPLIT_BF16 takes the fixed-operator products (bits 1-16: the M2L, the
-// shifts, the log terms and the sums stay FP64), BC_SPLIT_BF16_ALL every part.
+// BC_SPLIT_BF16 takes the fixed-operator products (bits 1-16; the M2L is on 7
+// digits beside them, the shifts and the log terms stay FP64), BC_SPLIT_BF16_ALL
+// every part.
 constexpr int kSplitAllParts = 127;
 constexpr int kSplitTableParts = 31;
 constexpr int kWideParts = 63;   // FP64 mode: every product but the shifts, on 7 digits
@@ -397,8 +398,7 @@ struct PassArgs {
 PassArgs pass_args(const bc_ctx *ctx, const bc_tree *t);
 // Largest grids of the persistent FP64 passes whose blocks are all resident
 // (occupancy calculator), capped at `per_sm` blocks per SM.
-// (df_T, df_maxp: the double-float climb's schedule; f_T, f_maxp: the largest
-// factored FP64 shift schedule of the context.)
+// (df_T, df_maxp: the double-float climb's schedule.)
 cudaError_t fp64_prepare(int NP, int P1, int df_T, int df_maxp, int up_per_sm, int down_per_sm,
                          int *up_blocks, int *shift_blocks, int *down_blocks);
 

@@ -1692,12 +1692,11 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
     if (late && (ce = side_launches()) != cudaSuccess) return ce;
     if (ev) cudaEventRecord(ev[3], st);
     bool first_digits = false;   // digits of `first` taken (tensor-core M2L)
-    bool summed = false;         // its rows already summed per box
     if (far && h.nlevels > 2) {
         // M2L: per V pair on the tensor cores (part 32; results one row per
-        // pair, summed by the downward pass), else every box's V-list sum in
-        // FP64, written into its row of `second`; then (FP64) the X-list
-        // products, then the level-by-level sum
+        // pair, summed per box by k_v_sums, or in the double-float pass), else every
+        // box's V-list sum by the FP64 kernels; either leaves it in the box's row of
+        // `second`; then (FP64) the X-list products, then the level-by-level sum
         const int64_t npairs = int64_t(h.v_src.size());
         if (npairs > 0 && (parts & 32)) {
             // tensor group M: digits of `first` (times alpha0 in the adjoint),
@@ -1716,7 +1715,6 @@ cudaError_t launch_apply(const PassArgs &a, const HostTree &h, const DevTree &d,
                                 h.level_start[2], a.nbox, d.v_ptr, d.v_src, d.v_code, d.box_level, tb.logd, d.lvtab,
                                 d.Pv, first, second, P1);
                 if (ce != cudaSuccess) return ce;
-                summed = true;
             }
         } else if (a.m2l_kind == 1) {
             // FP64 tensor cores, one warp per target box; beside the
