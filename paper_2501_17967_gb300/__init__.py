@@ -372,6 +372,13 @@ def _on_stream(stream):
     return torch.cuda.stream(stream)
 
 
+def _contiguous(x, stream):
+    if x.is_contiguous():
+        return x
+    with _on_stream(stream):
+        return x.contiguous()
+
+
 def _check_tensor(x, tree: Tree, name):
     import torch
     n = tree.nleaf * tree.ctx.p * tree.ctx.p
@@ -409,8 +416,7 @@ def eval_points(tree: Tree, u, xy, out=None, stream=None):
     """Interpolate leaf-node values u at points xy[n, 2] (device tensors)."""
     import torch
     _check_tensor(u, tree, "u")
-    with _on_stream(stream):
-        xy = xy.contiguous()
+    xy = _contiguous(xy, stream)
     n = xy.shape[0]
     if out is None:
         out = torch.empty(n, dtype=torch.float64, device=xy.device)
@@ -425,8 +431,7 @@ def eval_points_grad(tree: Tree, u, xy, stream=None):
     (device tensors): returns (val[n], grad[n, 2])."""
     import torch
     _check_tensor(u, tree, "u")
-    with _on_stream(stream):
-        xy = xy.contiguous()
+    xy = _contiguous(xy, stream)
     n = xy.shape[0]
     val = torch.empty(n, dtype=torch.float64, device=xy.device)
     grad = torch.empty((n, 2), dtype=torch.float64, device=xy.device)
@@ -462,9 +467,7 @@ class Layer:
         m[n, 2]; device tensors (on `stream`) or host tensors.  precision FP64,
         or SPLIT_BF16: the L2P at every leaf on the tensor cores (p = 8, 12, 16)."""
         import torch
-        with _on_stream(stream):
-            q = q.contiguous()
-            m = m.contiguous()
+        q, m = _contiguous(q, stream), _contiguous(m, stream)
         if q.dtype != torch.float64 or m.dtype != torch.float64 or q.numel() != self.n or m.numel() != 2 * self.n:
             raise ValueError("q must be float64 [n] and m float64 [n, 2]")
         NP = self.tree.ctx.p ** 2
@@ -503,19 +506,19 @@ def strip_solve(A, B, C, b, stream=None, return_status=False, out=None, work=Non
     2 = a device-side wait gave up, x holds NaN); out, work and status may be
     passed in."""
     import torch
-    with _on_stream(stream):
-        A, B, C, b = (t.contiguous() for t in (A, B, C, b))
+    A, B, C, b = (_contiguous(t, stream) for t in (A, B, C, b))
     if b.dim() != 4 or A.shape != B.shape or A.shape != C.shape or A.shape[:3] != b.shape[:3] \
             or A.shape[2] != A.shape[3] or any(t.dtype != torch.float64 for t in (A, B, C, b)):
         raise ValueError("A, B, C must be float64 [nsys, N, m, m] and b float64 [nsys, N, m, r]")
     nsys, N, m, r = (int(v) for v in b.shape)
     lib = _load()
     x = torch.empty_like(b) if out is None else out
-    with _on_stream(stream):
-        if work is None:
-            work = strip_workspace(nsys, N, m, r, b.device)
-        if status is None:
-            status = torch.zeros(max(1, nsys), dtype=torch.int32, device=b.device)
+    if work is None or status is None:
+        with _on_stream(stream):
+            if work is None:
+                work = strip_workspace(nsys, N, m, r, b.device)
+            if status is None:
+                status = torch.zeros(max(1, nsys), dtype=torch.int32, device=b.device)
     _check(lib.bc_strip_solve(nsys, N, m, r, ctypes.c_void_p(A.data_ptr()), ctypes.c_void_p(B.data_ptr()),
                               ctypes.c_void_p(C.data_ptr()), ctypes.c_void_p(b.data_ptr()),
                               ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(work.data_ptr()),
